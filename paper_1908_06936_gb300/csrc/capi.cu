@@ -31,9 +31,25 @@ exa_status cuda_err(exa_ctx* c, cudaError_t e, const char* what) {
   return set_err(c, EXA_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+exa_status ensure_side(exa_ctx* c) {
+  if (c->side) return EXA_OK;
+  if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->la_ev[0], cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->la_ev[1], cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    return set_err(c, EXA_ERR_CUDA, "look-ahead stream creation failed");
+  }
+  return EXA_OK;
+}
+
 // Grow-only device buffer with the context's memory bound enforced.
-exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name) {
+// `optional`: the caller does without.  A request that is not optional and cannot be met otherwise takes the digit
+// operands' memory back.
+exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool optional) {
   if (bytes <= b.bytes) return EXA_OK;
+  if (!optional && c->digits_held && c->ws_limit && c->held_bytes - b.bytes + bytes > c->ws_limit) {
+    release_digits(c);
+  }
   const size_t held = c->held_bytes - b.bytes;
   if (c->ws_limit && held + bytes > c->ws_limit)
     return set_err(c, EXA_ERR_NOMEM, "workspace %s needs %zu bytes; context bound is %zu (held %zu)", name, bytes,
@@ -47,6 +63,11 @@ exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name) {
   }
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
+  if (e != cudaSuccess && !optional && c->digits_held) {
+    cudaGetLastError();
+    release_digits(c);
+    e = cudaMalloc(&p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_err(c, EXA_ERR_NOMEM, "cudaMalloc(%zu) for %s: %s", bytes, name, cudaGetErrorString(e));
@@ -86,6 +107,11 @@ exa_status reset_status(exa_ctx* c) {
 exa_status factor_fp64(exa_ctx* c, double* a, int64_t ld, int64_t npad, int nb) {
   const int T = (int)(npad / nb);
   exa_status st;
+  if (nb == 128) {
+    bool done = false;
+    st = factor_digits(c, a, ld, npad, &done);
+    if (st != EXA_OK || done) return st;
+  }
   if ((st = ensure(c, c->w_all, (size_t)T * nb * nb * sizeof(double), "inverted diagonal tiles")) != EXA_OK) return st;
   if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   if ((st = ensure(c, c->logdet_part, (size_t)T * sizeof(double), "log-det partials")) != EXA_OK) return st;

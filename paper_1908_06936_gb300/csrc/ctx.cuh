@@ -18,6 +18,9 @@ struct DevBuf {
 
 constexpr int kNumEvents = 8;
 constexpr int kMixPanel = 512;     // panel width of the mixed-precision factorisation
+constexpr int kDiagCtas = 64;      // CTAs of one diagonal-block launch at most
+constexpr int kDigSideSMs = 32;    // SMs left to the look-ahead stream of the FP64 factorisation ...
+constexpr int64_t kDigLateRows = 16384;  // ... while at least this many rows remain (kDiagCtas below)
 constexpr int kRedPartials = 512;  // partial sums of one two-stage reduction
 
 inline int64_t kPartialDoubles(int64_t npad, int nb) { return 2 * kRedPartials + (npad / 1024 + 2) * (int64_t)nb; }
@@ -53,6 +56,7 @@ struct exa_ctx {
   exa::DevBuf mx_split4;
   exa::DevBuf mx_split_b;   // split-precision operands (B role: inverse diagonal block / test B)
   exa::SplitOperand sp_a, sp_a2, sp_a3, sp_a4, sp_b;
+  bool digits_held = false; // the buffers of reserve_digits are the FP64 path's: given up for requests that need the room
   exa::DevBuf mx_vec;       // refinement vectors
   exa::DevBuf mx_w2;        // inverse of the panel-wide diagonal block (row-major)
   exa::DevBuf mx_wall;      // every panel's diagonal-block inverse, T x 512 x 512 (kept for the gradient)
@@ -104,11 +108,19 @@ namespace exa {
 
 exa_status set_err(exa_ctx* c, exa_status st, const char* fmt, ...);
 exa_status cuda_err(exa_ctx* c, cudaError_t e, const char* what);
-exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name);
+exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool optional = false);
 exa_status check_theta(exa_ctx* c, const double theta[3]);
 exa_status reset_status(exa_ctx* c);
 exa_status read_status(exa_ctx* c);
 exa_status factor_fp64(exa_ctx* c, double* a, int64_t ld, int64_t npad, int nb);
+// The same on the tensor cores (npad a multiple of 128); *done = false: its workspace could not be had.
+exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* done);
+// Its digit operands for a matrix of npad rows (in the split-operand buffers of the mixed path); false: they cannot
+// be had, and those buffers are released.
+bool reserve_digits(exa_ctx* c, int64_t npad);
+void release_digits(exa_ctx* c);
+// The look-ahead stream and its events.
+exa_status ensure_side(exa_ctx* c);
 exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_prec prec, int band, int far_thr);
 // Generate Sigma into `sigma_keep` (or straight into the factor buffer) and factor it in mixed precision.
 exa_status mixed_generate_factor(exa_ctx* c, const double* d_locs, int64_t n, const double theta[3], int64_t npad,

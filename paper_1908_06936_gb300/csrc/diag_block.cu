@@ -48,6 +48,7 @@ struct DiagArgs {
   double* w2;           // 512 x 512 row-major inverse
   double* scr;          // kDiagScratch doubles
   DevStatus* st;
+  int size;             // rows of the block, a multiple of 128 up to 512
 };
 
 // Grid-wide barrier of the cooperative launch (all CTAs co-resident): CTA leader arrives on a
@@ -288,9 +289,10 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
   // it during the rest of (c) (look-ahead), so the serial leaves overlap the updates.
   if (b == 0) diag_leaf(g, 0, S);
   sync_all();
-  for (int j = 0; j < kDSteps; ++j) {
+  const int size = g.size, nsteps = size / kDW;
+  for (int j = 0; j < nsteps; ++j) {
     const int64_t c0 = k0 + (int64_t)j * kDW;
-    const int below = kDB - (j + 1) * kDW;  // rows of the block below step j
+    const int below = size - (j + 1) * kDW;  // rows of the block below step j
     const int ns = below / kDT;             // 32-row strips
     const double* V = g.scr + (int64_t)j * kDW * kDW;
     // (b) P(r, c) = sum_k A(c0 + 64 + r, c0 + k) V(c, k): one task per strip and 32-column half
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
     }
     lead_target += (unsigned int)foreign;
     if (b == 0) {
-      if (j + 1 < kDSteps) {
+      if (j + 1 < nsteps) {
         if (tid == 0) {
           const long long t0 = clock64();
           while (*(volatile unsigned int*)leadcnt < lead_target && !*abort) {
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
   }
 
   // ---------------- log-determinant parts, leaves of the inverse ----------------
-  for (int s4 = b; s4 < 4 && tid == 0; s4 += G) {
+  for (int s4 = b; s4 < size / 128 && tid == 0; s4 += G) {
     double s = 0.0;
     for (int i = 0; i < 128; ++i) {
       const int64_t r = k0 + 128 * s4 + i;
@@ -385,8 +387,9 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
   }
   double* w2 = g.w2;
   // W2 <- zero above the diagonal, the 64-inverses on the diagonal (other lower entries later)
-  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < (int64_t)kDB * kDB; idx += (int64_t)G * kDThreads) {
+  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < (int64_t)size * kDB; idx += (int64_t)G * kDThreads) {
     const int r = (int)(idx / kDB), c = (int)(idx % kDB);
+    if (c >= size) continue;
     if (c > r) {
       w2[idx] = 0.0;
     } else if (r / kDW == c / kDW) {
@@ -398,8 +401,9 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
 
   // ---------------- inverse by doubling: widths h = 64, 128, 256 ----------------
   double* T = g.scr + kDiagT;  // h x h product, row-major
-  for (int h = kDW; h < kDB; h *= 2) {
-    const int pairs = kDB / (2 * h);             // blocks of width 2h
+  // (a smaller block is the last of its matrix: only its 128 sub-tile inverses are wanted)
+  for (int h = kDW; h < (size == kDB ? kDB : 128); h *= 2) {
+    const int pairs = size / (2 * h);             // blocks of width 2h
     const int tiles = (h / kDT) * (h / kDT);     // 32 x 32 tiles of one h x h product
     // first product: T_p = L_BA W_A  (L_BA: rows p 2h + h .., columns p 2h ..; W_A lower, row-major in w2)
     for (int t = b; t < pairs * tiles; t += G) {
@@ -437,7 +441,7 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
   }
 
   // ---------------- the four 128 sub-tile inverses (diagonal blocks of W2) ----------------
-  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < 4 * 128 * 128; idx += (int64_t)G * kDThreads) {
+  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < (int64_t)size * 128; idx += (int64_t)G * kDThreads) {
     const int s = (int)(idx / (128 * 128)), rc = (int)(idx % (128 * 128)), r = rc / 128, c = rc % 128;
     g.w_sub[idx] = __ldcg(w2 + (int64_t)(128 * s + r) * kDB + 128 * s + c);
   }
@@ -446,7 +450,7 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
 size_t diag_block_scratch_doubles() { return (size_t)kDiagScratch; }
 
 cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0, double* w_sub, double* logdet_part,
-                              double* w2, double* scratch, DevStatus* st, int grid) {
+                              double* w2, double* scratch, DevStatus* st, int grid, int size) {
   // at least 116 KB of shared memory, so that no SM holds two CTAs (the FP64 pipe of an SM is
   // the resource: two CTAs on one SM would leave another idle)
   size_t smem = (size_t)(kLeafSmem + 2 * kDT * (kDT + 1)) * sizeof(double);
@@ -459,7 +463,7 @@ cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0,
   if (grid < 2) grid = 2;  // CTA 0 runs the leaves; the updates need at least one more CTA
   e = cudaMemsetAsync(scratch + kDiagBar, 0, 2 * sizeof(double), s);
   if (e != cudaSuccess) return e;
-  DiagArgs g{a, ld, k0, w_sub, logdet_part, w2, scratch, st};
+  DiagArgs g{a, ld, k0, w_sub, logdet_part, w2, scratch, st, size};
   void* args[] = {&g};
   // cooperative launch: every CTA is resident at once, so the grid barriers cannot wait on an
   // unscheduled CTA

@@ -1,0 +1,519 @@
+// FP64 contractions on the fifth-generation tensor cores (steps a2, a7 and the prediction variance).
+//
+// FP64 units issue 1.26 TFLOP/s on this part, BF16 tensor cores 1,870: one 1,490th.  A product of two FP64
+// matrices is therefore formed from BF16 ones.  Each row is scaled by a power of two so that |a| < 1 and cut
+// into S = 8 signed 7-bit digits, a = sum_s d_s 2^(-6-7s), |d_s| <= 64, exact in BF16 (the error-free splitting
+// of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).  Digit products are integers up to 2^12; group
+// g = s + t sums at most 8 of them for each of K <= 512 columns, so every partial sum stays within 2^24 and FP32
+// accumulation in TMEM is exact whatever its order.  The 36 products with g <= 7 are formed.  What is left out is
+// a rounding-like error of about 2^-52 of the product of the two row maxima per pass, without a sign of its own
+// except on the diagonal of A A^T, where the squares of the left-out digits add up to a bias: there the split's
+// row sums sq put the left-out group g = 8 back.
+#include "digits.cuh"
+
+#include <cuda_bf16.h>
+
+#include "ctx.cuh"
+#include "tc_common.cuh"
+
+namespace exa {
+
+using namespace tc;
+
+namespace dig {
+constexpr int TM = 128, TN = kDigTN;
+constexpr int kEpiWarps = 8, kThreads = 64 + 32 * kEpiWarps;
+
+template <int S>
+struct Cfg {
+  static constexpr int A_BYTES = TM * 32, B_BYTES = TN * 32;  // one digit plane of a 16-column step
+  static constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = S == kDigSlices ? 4 : 12;
+  static constexpr int SMEM = STAGES * STAGE_BYTES + 512;
+  static constexpr int TMEM_COLS = S * TN;  // group g in columns [TN g, TN g + TN)
+};
+static_assert(Cfg<kDigSlices>::SMEM <= 232448 && Cfg<kDigLow>::SMEM <= 232448, "stages fit in shared memory");
+
+// Shared-memory descriptor of a K-major operand without swizzling: 8-row core matrices of 128 bytes, the two of
+// a 16-column step 128 bytes apart (leading offset), 8-row groups 256 bytes apart (stride offset).
+__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// Lower-triangle enumeration of 128 x TN tiles: bands of kBand row blocks, each a rectangle left of the band's
+// diagonal square (column tiles outer, rows inner: the tiles of one wave share operand rows in L2) and then the
+// square's own lower tiles.  Row block b holds 2 (b + 1) column tiles.
+constexpr int kBand = 16;
+__device__ __forceinline__ void lower_tile(long long t, int mt, int& bi, int& bj) {
+  int q = (int)(sqrtf((float)t) / kBand);  // t >= R (R + 1) with R = kBand q
+  while (q > 0 && (long long)kBand * q * (kBand * q + 1) > t) --q;
+  while ((long long)kBand * (q + 1) * (kBand * (q + 1) + 1) <= t) ++q;
+  const int R = kBand * q, h = mt - R < kBand ? mt - R : kBand;
+  t -= (long long)R * (R + 1);
+  const long long rect = (long long)h * 2 * R;
+  if (t < rect) {
+    bj = (int)(t / h);
+    bi = R + (int)(t % h);
+    return;
+  }
+  const int u = (int)(t - rect);  // the square: row block R + b holds column tiles 2 R .. 2 (R + b) + 1
+  int b = (int)sqrtf((float)u);
+  while (b > 0 && b * (b + 1) > u) --b;
+  while ((b + 1) * (b + 2) <= u) ++b;
+  bi = R + b;
+  bj = 2 * R + u - b * (b + 1);
+}
+
+struct Args {
+  double* C;
+  const double* Cin;
+  int64_t ldc, ldcin;
+  const uint8_t *A, *B;           // first plane, at the operand's row origin
+  int64_t a_plane, b_plane;       // bytes between planes
+  const int *ea, *eb, *sq;
+  int mt, nt;                     // row blocks, column tiles
+  int shape, tri;
+  int k16;
+  uint32_t sign;                  // sign bit of the product's factor
+  long long t0, ntiles;           // tiles [t0, ntiles)
+  DevStatus* st;
+};
+
+__device__ __forceinline__ void tile_of(const Args& g, long long t, int& bi, int& bj) {
+  if (g.shape == kDigRect) {
+    bi = (int)(t % g.mt);
+    bj = (int)(t / g.mt);
+  } else {
+    lower_tile(t, g.mt, bi, bj);
+  }
+}
+
+__device__ __forceinline__ void timeout(DevStatus* st, volatile int* abort, int site) {
+  *abort = 1;
+  if (atomicExch(&st->timeout, 1) == 0) st->timeout_where = site;
+}
+
+// v an integer, |v| < 2^51, as a double: its bits added to those of 1.5 2^52, the constant taken off again.
+__device__ __forceinline__ double int_to_f64(long long v) {
+  return __longlong_as_double(v + 0x4338000000000000ll) - 6755399441055744.0;
+}
+
+// One CTA per SM, persistent: warp 0 copies operand planes into a ring of 16-column stages, one thread of warp 1
+// issues the MMAs, warps 2-9 drain TMEM into C.  The S B planes of a stage lie one after another and group g
+// follows group g - 1 in TMEM, so A digit s against B digits 0 .. S-1-s is one run of columns (two MMAs where
+// N > 256): 12 MMAs a step instead of 36.
+//
+// Bound: the tensor pipe (36 BF16 products per FP64 one: 52 TFLOP/s at the 1,872 of a burst).  Eight groups of a
+// 128 x 64 tile fill TMEM (512 columns), and the tile has to be that large: each 16-column step moves 48 KB into
+// shared memory for 1,152 cycles of MMA, 42 bytes a cycle, against the ~46 an SM was seen to take in.  So there is
+// one accumulator set, and the drain's first part (TMEM to integers, four 32-bit words an output) is not hidden.
+template <int S>
+__global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_constant__ Args g) {
+  using C_ = Cfg<S>;
+  constexpr int A_BYTES = C_::A_BYTES, B_BYTES = C_::B_BYTES, STAGES = C_::STAGES, STAGE_BYTES = C_::STAGE_BYTES;
+  extern __shared__ __align__(256) uint8_t smem[];
+  uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accfull = empty + STAGES;
+  uint64_t* accempty = accfull + 1;
+  uint32_t* tmem_slot = (uint32_t*)(accempty + 1);
+  volatile int* abort = (volatile int*)(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(accfull, 1);
+    mbar_init(accempty, 32 * kEpiWarps);
+    *abort = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(tmem_slot, C_::TMEM_COLS);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp == 0) {
+    // ---------------- copies: lane s < S brings A plane s, lane S + s B plane s ----------------
+    int stage = 0;
+    uint32_t phase = 0;
+    int last_par[STAGES];
+    for (int s = 0; s < STAGES; ++s) last_par[s] = -1;
+    bool ok = true;  // the same for every lane
+    for (long long t = g.t0 + blockIdx.x; t < g.ntiles && ok; t += gridDim.x) {
+      int bi, bj;
+      tile_of(g, t, bi, bj);
+      const int steps = g.tri ? min(g.k16, (bj + 1) * (TN / 16)) : g.k16;
+      const bool isA = lane < S;
+      const uint8_t* src = isA ? g.A + (int64_t)lane * g.a_plane + (int64_t)bi * A_BYTES
+                               : g.B + (int64_t)(lane - S) * g.b_plane + (int64_t)bj * B_BYTES;
+      const int64_t step_bytes = S * (isA ? g.a_plane : g.b_plane);
+      const uint32_t off = isA ? lane * A_BYTES : S * A_BYTES + (lane - S) * B_BYTES;
+      for (int kc = 0; kc < steps; ++kc) {
+        if (lane == 0) {
+          ok = mbar_wait(&empty[stage], phase ^ 1, abort);
+          if (ok) mbar_expect_tx(&full[stage], STAGE_BYTES);
+          else timeout(g.st, abort, 81);
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        if (lane < 2 * S)
+          bulk_load(smem_u32(smem + stage * STAGE_BYTES) + off, src, isA ? A_BYTES : B_BYTES, smem_u32(&full[stage]));
+        src += step_bytes;
+        last_par[stage] = (int)phase;
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+    }
+    if (!ok || *abort) {  // let every copy of this warp land before the CTA exits
+      for (int s = 0; s < STAGES; ++s)
+        if (last_par[s] >= 0) {
+          volatile int never = 0;
+          mbar_wait(&full[s], (uint32_t)last_par[s], &never);
+        }
+    }
+  } else if (warp == 1 && lane == 0) {
+    // ---------------- MMA issue ----------------
+    int stage = 0;
+    uint32_t phase = 0, it = 0;
+    for (long long t = g.t0 + blockIdx.x; t < g.ntiles && !*abort; t += gridDim.x) {
+      int bi, bj;
+      tile_of(g, t, bi, bj);
+      const int steps = g.tri ? min(g.k16, (bj + 1) * (TN / 16)) : g.k16;
+      if (!mbar_wait(accempty, (it & 1) ^ 1, abort)) {
+        timeout(g.st, abort, 82);
+        break;
+      }
+      fence_after();
+      bool ok = true;
+      for (int kc = 0; kc < steps; ++kc) {
+        if (!mbar_wait(&full[stage], phase, abort)) {
+          timeout(g.st, abort, 83);
+          ok = false;
+          break;
+        }
+        fence_after();
+        const uint32_t sb = smem_u32(smem + stage * STAGE_BYTES);
+        const uint64_t b0 = sdesc(sb + S * A_BYTES);
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          const uint64_t a = sdesc(sb + s * A_BYTES);
+          const int n = TN * (S - s);
+          // the first step's s = 0 writes every group, all others add
+          const uint32_t acc = (kc | s) ? 1u : 0u;
+          if (n > 256) {
+            const int h = n / 2;  // a multiple of 32
+            mma_bf16(tmem + s * TN, a, b0, idesc(kFmtBF16, TM, h), acc);
+            mma_bf16(tmem + s * TN + h, a, b0 + (uint64_t)(h * 32 >> 4), idesc(kFmtBF16, TM, h), acc);
+          } else {
+            mma_bf16(tmem + s * TN, a, b0, idesc(kFmtBF16, TM, n), acc);
+          }
+        }
+        mma_commit(&empty[stage]);
+        if (++stage == STAGES) {
+          stage = 0;
+          phase ^= 1;
+        }
+      }
+      if (!ok) break;
+      mma_commit(accfull);
+      ++it;
+    }
+  } else if (warp >= 2) {
+    // ---------------- drain: warp w takes TMEM lanes 32 (w % 4).. and column half (w - 2) / 4 ----------------
+    const int quad = warp & 3, half = (warp - 2) >> 2;
+    const int r = quad * 32 + lane;
+    constexpr int CH = TN / 2, P = S / 2;
+    uint32_t it = 0;
+    for (long long t = g.t0 + blockIdx.x; t < g.ntiles; t += gridDim.x) {
+      int bi, bj;
+      tile_of(g, t, bi, bj);
+      const int64_t row = (int64_t)bi * TM + r, col0 = (int64_t)bj * TN + half * CH;
+      const int er = g.ea[row];
+      const bool lower = g.shape == kDigLower;
+      if (!__all_sync(0xffffffffu, mbar_wait(accfull, it & 1, abort))) {
+        if (lane == 0) timeout(g.st, abort, 84);
+        break;
+      }
+      fence_after();
+      // groups 2p and 2p + 1 hold exact integers of weights 2^(-12-14p), 2^(-19-14p): one 32-bit word for both
+      int w[P][CH];
+      const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + half * CH;
+#pragma unroll
+      for (int p = 0; p < P; ++p) {
+#pragma unroll
+        for (int h = 0; h < CH; h += 16) {
+          uint32_t x0[16], x1[16];
+          tmem_ld16(ta + (2 * p) * TN + h, x0);
+          tmem_ld16(ta + (2 * p + 1) * TN + h, x1);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            w[p][h + j] = __float2int_rn(__uint_as_float(x0[j])) * 128 + __float2int_rn(__uint_as_float(x1[j]));
+        }
+      }
+      fence_before();
+      mbar_arrive(accempty);
+      ++it;
+      const int base = er - 12 - 7 * (S - 1);  // weight of the last group, without the column's exponent
+#pragma unroll
+      for (int j0 = 0; j0 < CH; j0 += 8) {
+        double cv[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          cv[j] = g.Cin && !(lower && col0 + j0 + j > row) ? g.Cin[row + (col0 + j0 + j) * g.ldcin] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int64_t col = col0 + j0 + j;
+          if (lower && col > row) continue;
+          const int ec = g.eb[col];
+          // x = sum of the groups, in units of the last one
+          double x;
+          if constexpr (S == 2) {
+            x = int_to_f64(w[0][j0 + j]);
+          } else {
+            const double hi = int_to_f64((long long)w[0][j0 + j] * 16384 + w[1][j0 + j]);
+            double lo = int_to_f64((long long)w[P - 2][j0 + j] * 16384 + w[P - 1][j0 + j]);
+            if (lower && row == col) lo = fma((double)g.sq[row], 1.0 / 128.0, lo);
+            x = fma(hi, 268435456.0, lo);
+          }
+          const int sh = base + ec;
+          double v;
+          if (er == kDigBad || ec == kDigBad) {
+            v = __longlong_as_double(0x7FF8000000000000ll);
+          } else if (sh >= -1000 && sh <= 900) {
+            v = fma(x, __hiloint2double((int)((uint32_t)(sh + 1023) << 20 | g.sign), 0), cv[j]);
+          } else {
+            v = g.sign ? cv[j] - scalbn(x, sh) : cv[j] + scalbn(x, sh);
+          }
+          g.C[row + col * g.ldc] = v;
+        }
+      }
+    }
+  }
+  fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    fence_after();
+    tmem_dealloc(tmem, C_::TMEM_COLS);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Split: 16 rows per CTA through shared memory (row stride odd in doubles), row maxima on the bit patterns, then
+// every thread cuts 8 consecutive columns of one row and stores 16 bytes per digit; a warp's stores of one digit
+// are two 256-byte runs.  Bound: HBM (8 bytes read, 2 S written per value) and the integer pipe.
+// ---------------------------------------------------------------------------
+constexpr int kRows = 16, kSplitThreads = 256;
+
+// v 2^c on the exponent field (0, infinities and NaNs as they are; below the normal range 0, above it infinity).
+__device__ __forceinline__ double scale_exp(double v, int c) {
+  const unsigned long long D = (unsigned long long)__double_as_longlong(v);
+  const int E = (int)((D >> 52) & 0x7FF);
+  if (E == 0 || E == 0x7FF) return v;
+  const int F = E + c;
+  const unsigned long long rest = D & 0x800FFFFFFFFFFFFFull, sign = D & 0x8000000000000000ull;
+  return __longlong_as_double((long long)(F <= 0      ? sign
+                                          : F >= 0x7FF ? sign | 0x7FF0000000000000ull
+                                                       : rest | ((unsigned long long)F << 52)));
+}
+
+template <int S>
+__global__ void __launch_bounds__(kSplitThreads) digit_split_kernel(const double* __restrict__ src, int64_t rs,
+                                                                    int64_t cs, int64_t rows, int K, int lower,
+                                                                    const int* __restrict__ colex, int colsign,
+                                                                    DigitOperand op, int64_t out_row0) {
+  extern __shared__ double tile[];
+  __shared__ int s_e[kRows];
+  __shared__ int s_sq[kRows];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ld = K + 1;
+  const int64_t r0 = (int64_t)blockIdx.x * kRows;
+  for (int base = 0; base < kRows * K; base += 8 * kSplitThreads) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int idx = base + u * kSplitThreads + tid;
+      const int r = cs == 1 ? idx / K : idx % kRows, k = cs == 1 ? idx % K : idx / kRows;
+      v[u] = idx < kRows * K && r0 + r < rows && !(lower && k > r0 + r) ? src[(r0 + r) * rs + (int64_t)k * cs] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int idx = base + u * kSplitThreads + tid;
+      const int r = cs == 1 ? idx / K : idx % kRows, k = cs == 1 ? idx % K : idx / kRows;
+      if (idx >= kRows * K) continue;
+      if (colex) v[u] = scale_exp(v[u], colsign * colex[k]);
+      tile[r * ld + k] = v[u];
+    }
+  }
+  if (tid < kRows) s_sq[tid] = 0;
+  __syncthreads();
+  for (int r = warp; r < kRows; r += kSplitThreads / 32) {
+    unsigned long long mx = 0;  // non-negative doubles order like their bits
+    for (int k = lane; k < K; k += 32) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(tile[r * ld + k]) & 0x7FFFFFFFFFFFFFFFull;
+      mx = b > mx ? b : mx;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = ob > mx ? ob : mx;
+    }
+    // the row's values are below 2^e in magnitude; a subnormal maximum counts as 2^-1022
+    if (lane == 0) {
+      const int be = (int)(mx >> 52);
+      s_e[r] = be == 0x7FF ? kDigBad : mx == 0 ? 0 : be ? be - 1022 : -1021;
+    }
+  }
+  __syncthreads();
+  const int octets = K / 8;
+  for (int u = tid; u < kRows * octets; u += kSplitThreads) {
+    const int r = (u & 7) + 8 * ((u >> 3) / octets), o = (u >> 3) % octets;
+    if (r0 + r >= rows) continue;
+    const int e = s_e[r];
+    uint32_t out[S][4];
+    int sq = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const unsigned long long D = (unsigned long long)__double_as_longlong(tile[r * ld + 8 * o + j]);
+      // N = a 2^(7S-1-e) rounded, |N| <= 2^(7S-1): a = M 2^(E-1075) with its 53-bit significand M
+      long long N = 0;
+      const int E = (int)((D >> 52) & 0x7FF);
+      if (E != 0 && e != kDigBad) {
+        const unsigned long long M = (D & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+        const int sh = 1075 - (7 * S - 1) + e - E;  // right shift, at least 53 - (7S - 1)
+        if (sh >= 64) N = 0;
+        else if (sh > 0) N = (long long)((M + (1ull << (sh - 1))) >> sh);
+        else N = (long long)(M << (-sh));
+        if (D >> 63) N = -N;
+      }
+      // balanced digits in base 128 from the least significant end, the leading one takes the rest
+      int d[S];
+#pragma unroll
+      for (int s = S - 1; s >= 1; --s) {
+        const int q = (((int)N + 64) & 127) - 64;
+        d[s] = q;
+        N = (N - q) >> 7;
+      }
+      d[0] = (int)N;
+      if constexpr (S == 8) sq += 2 * (d[1] * d[7] + d[2] * d[6] + d[3] * d[5]) + d[4] * d[4];
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        const uint32_t b = __float_as_uint((float)d[s]) >> 16;  // exact in BF16
+        out[s][j >> 1] = (j & 1) ? out[s][j >> 1] | (b << 16) : b;
+      }
+    }
+    if constexpr (S == 8) atomicAdd(&s_sq[r], sq);
+    const int64_t orow = out_row0 + r0 + r;
+    uint8_t* p = op.dig + ((int64_t)(o >> 1) * S * op.rows) * 32 + (orow >> 3) * 256 + (o & 1) * 128 + (orow & 7) * 16;
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      *reinterpret_cast<uint4*>(p + (int64_t)s * op.rows * 32) = make_uint4(out[s][0], out[s][1], out[s][2], out[s][3]);
+  }
+  __syncthreads();
+  if (tid < kRows && r0 + tid < rows) {
+    op.ex[out_row0 + r0 + tid] = s_e[tid];
+    op.sq[out_row0 + r0 + tid] = s_sq[tid];
+  }
+}
+
+}  // namespace dig
+
+size_t digit_bytes(int64_t rows, int K, int S) {
+  rows = round_up(rows, 8);
+  return (size_t)(K / 16) * S * rows * 32 + 2 * (size_t)round_up(rows, 64) * sizeof(int);
+}
+
+void digit_layout(DigitOperand& op, void* base, int64_t rows, int K, int S) {
+  rows = round_up(rows, 8);
+  op.rows = rows;
+  op.dig = (uint8_t*)base;
+  op.ex = (int*)(op.dig + (size_t)(K / 16) * S * rows * 32);
+  op.sq = op.ex + round_up(rows, 64);
+}
+
+template <int S>
+static cudaError_t split_impl(cudaStream_t s, const double* src, int64_t rs, int64_t cs, int64_t rows, int K,
+                              bool lower, const int* colex, int colsign, const DigitOperand& op, int64_t out_row0) {
+  static PerDeviceOnce once;
+  cudaError_t e = once([] {
+    return cudaFuncSetAttribute(dig::digit_split_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                dig::kRows * (kDigMaxK + 1) * (int)sizeof(double));
+  });
+  if (e != cudaSuccess) return e;
+  dig::digit_split_kernel<S><<<(unsigned)ceil_div(rows, dig::kRows), dig::kSplitThreads,
+                               (size_t)dig::kRows * (K + 1) * sizeof(double), s>>>(src, rs, cs, rows, K, lower, colex,
+                                                                                colsign, op, out_row0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_digit_split(cudaStream_t s, const double* src, int64_t rs, int64_t cs, int64_t rows, int K, int S,
+                               const DigitOperand& op, int64_t out_row0, bool lower, const int* colex, int colsign) {
+  if (rows <= 0) return cudaSuccess;
+  if (K <= 0 || K % 16 || K > kDigMaxK || out_row0 % 8 || out_row0 + rows > op.rows) return cudaErrorInvalidValue;
+  if (S == kDigSlices) return split_impl<kDigSlices>(s, src, rs, cs, rows, K, lower, colex, colsign, op, out_row0);
+  if (S == kDigLow) return split_impl<kDigLow>(s, src, rs, cs, rows, K, lower, colex, colsign, op, out_row0);
+  return cudaErrorInvalidValue;
+}
+
+template <int S>
+static cudaError_t gemm_impl(cudaStream_t s, const dig::Args& a, int max_ctas) {
+  static PerDeviceOnce once;
+  cudaError_t e = once([] {
+    return cudaFuncSetAttribute(dig::gemm_digits_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                dig::Cfg<S>::SMEM);
+  });
+  if (e != cudaSuccess) return e;
+  int cap = tc_num_sms();
+  if (max_ctas > 0 && max_ctas < cap) cap = max_ctas;
+  if (a.ntiles <= a.t0) return cudaSuccess;
+  const int grid = (int)(a.ntiles - a.t0 < cap ? a.ntiles - a.t0 : cap);
+  dig::gemm_digits_kernel<S><<<grid, dig::kThreads, dig::Cfg<S>::SMEM, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gemm_digits(cudaStream_t s, const DigitGemm& g, int max_ctas) {
+  if (g.m <= 0 || g.n <= 0) return cudaSuccess;
+  if (g.m % dig::TM || g.n % dig::TN || g.K <= 0 || g.K % 16 || g.K > kDigMaxK || g.a_row0 % 8 || g.b_row0 % 8 ||
+      g.a_row0 + g.m > g.A.rows || g.b_row0 + g.n > g.B.rows || (g.shape == kDigLower && g.m != g.n) || g.skip % dig::TM ||
+      g.skip > (g.shape == kDigLower ? dig::kBand * dig::TM : 0))
+    return cudaErrorInvalidValue;
+  dig::Args a{};
+  a.C = g.C;
+  a.Cin = g.Cin;
+  a.ldc = g.ldc;
+  a.ldcin = g.ldcin;
+  a.A = g.A.dig + g.a_row0 * 32;
+  a.B = g.B.dig + g.b_row0 * 32;
+  a.a_plane = g.A.rows * 32;
+  a.b_plane = g.B.rows * 32;
+  a.ea = g.A.ex + g.a_row0;
+  a.eb = g.B.ex + g.b_row0;
+  a.sq = g.A.sq + g.a_row0;
+  a.mt = (int)(g.m / dig::TM);
+  a.nt = (int)(g.n / dig::TN);
+  a.shape = g.shape;
+  a.tri = g.tri;
+  a.k16 = g.K / 16;
+  a.ntiles = g.shape == kDigLower ? (long long)a.mt * (a.mt + 1) : (long long)a.mt * a.nt;
+  a.sign = g.neg ? 0x80000000u : 0u;
+  const long long skip = g.skip / dig::TM;  // within the first band, where tiles go row block by row block
+  a.t0 = skip * (skip + 1);
+  a.st = g.st;
+  if (g.S == kDigSlices) return gemm_impl<kDigSlices>(s, a, max_ctas);
+  if (g.S == kDigLow) return gemm_impl<kDigLow>(s, a, max_ctas);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace exa

@@ -669,7 +669,8 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   } else {
     // the factor's own buffer is requested first, so the test below sees what remains
     if ((st = ensure(c, c->mat, nn_bytes, "matrix")) != EXA_OK) return st;
-    st = ensure(c, c->gr_part, nn_bytes, "inverse covariance");
+    if (nb == 128) reserve_digits(c, npad);  // worth more than the second buffer
+    st = ensure(c, c->gr_part, nn_bytes, "inverse covariance", true);
     if (st == EXA_ERR_NOMEM) {
       one_buffer = true;
       c->err[0] = 0;
@@ -698,6 +699,7 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   const long long t64n = one_buffer ? npad / 64 : (n + 63) / 64;
   const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
   if ((st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials")) != EXA_OK) return st;
+  if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   if (!one_buffer) {
     if (e == cudaSuccess) e = sigma_inverse_fp64(c, npad, nb, S);
     // fused regeneration of dSigma/dtheta and reduction
@@ -846,6 +848,7 @@ extern "C" exa_status exa_fisher(exa_ctx* c, const double* d_locs, const double 
   if (e != cudaSuccess) return cuda_err(c, e, "generation launch");
   if ((st = factor_fp64(c, A, npad, npad, nb)) != EXA_OK) return st;
   if ((st = read_status(c)) != EXA_OK) return st;
+  if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   e = sigma_inverse_fp64(c, npad, nb, S);
   if (e == cudaSuccess) {
     mirror_lower_kernel<<<dim3((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)npad), 256, 0,

@@ -24,7 +24,6 @@ constexpr int kLookaheadSMs = 20;         // SMs left to the look-ahead stream d
 constexpr int64_t kFuseMinRows = 40960;   // two panels per trailing pass down to this many rows
 constexpr int64_t kLateRows = 61440;      // one-panel phase: the look-ahead share grows below this many rows
 constexpr int kLateSMs = 48;              // ... up to this many SMs
-constexpr int kDiagMaxCtas = 64;          // CTAs of one diagonal-block launch at most
 constexpr double kExactThreshold = 0.8;  // tiles holding |Sigma_ij| >= 0.8 sigma^2 get exact products
 constexpr double kSmoothNu = 1.2;        // above this smoothness every tile gets exact products
 constexpr double kWideBandNu = 0.75;     // from this smoothness one more panel of the band is exact
@@ -55,10 +54,10 @@ cudaError_t split_layout(SplitOperand& op, void* base_p, int64_t rows, int K, bo
 }
 
 exa_status ensure_split(exa_ctx* c, SplitOperand& op, DevBuf& buf, int64_t rows, int K, bool t3, bool oz) {
-  void* old = buf.p;
   exa_status st = ensure(c, buf, split_bytes(rows, K, t3, oz) + 1024, "split operands");
   if (st != EXA_OK) return st;
-  const bool same = (old == buf.p) && op.rows == rows && op.K == K && ((op.hi != nullptr) == t3) &&
+  // the buffers serve the FP64 digits as well (chol_digits.cu), which may have moved this one since
+  const bool same = (t3 ? (void*)op.hi : op.dig) == buf.p && op.rows == rows && op.K == K && ((op.hi != nullptr) == t3) &&
                     ((op.dig != nullptr) == oz);
   if (same) return EXA_OK;
   const cudaError_t e = split_layout(op, buf.p, rows, K, t3, oz);
@@ -106,7 +105,7 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   {
     // one CTA per SM of the look-ahead share, 64 at most (the block's parallel phases gain
     // little beyond: 1.45 ms on 32 CTAs, 1.33 ms on 64)
-    const int grid = ctas > 0 ? (ctas < kDiagMaxCtas ? ctas : kDiagMaxCtas) : kDiagMaxCtas;
+    const int grid = ctas > 0 ? (ctas < kDiagCtas ? ctas : kDiagCtas) : kDiagCtas;
     const double nb3 = (double)NB * NB * NB;
     ProfScope ps(c, PK_POTRF, 2.0 * nb3 / 3.0, 8.0 * (3.0 * NB * NB + 4.0 * nb * nb), 1, s, true);
     e = launch_diag_block(s, a, ld, k0, W + (k0 / nb) * (int64_t)nb * nb, LD + k0 / nb, W2, (double*)c->mx_dscr.p,
@@ -324,6 +323,7 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   const int64_t fuse_rows = c->fuse_min_rows < 0 ? kFuseMinRows : c->fuse_min_rows;
   // the fused phase runs while rows (k + 4) NB .. npad number at least fuse_rows, from k = 0
   const bool fuse = fuse_rows > 0 && c->tc_pairs && T >= 4 && npad - 4 * (int64_t)NB >= fuse_rows;
+  c->digits_held = false;
   SplitOperand* buf[4] = {&c->sp_a, &c->sp_a2, &c->sp_a3, &c->sp_a4};
   DevBuf* mem[4] = {&c->mx_split, &c->mx_split2, &c->mx_split3, &c->mx_split4};
   for (int i = 0; i < (fuse ? 4 : 2); ++i)
@@ -336,14 +336,7 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   if (c->keep_block_inverses &&
       (st = ensure(c, c->mx_wall, (size_t)T * NB * NB * sizeof(double), "diagonal block inverses")) != EXA_OK)
     return st;
-  if (!c->side) {
-    if (cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->la_ev[0], cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->la_ev[1], cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      return set_err(c, EXA_ERR_CUDA, "look-ahead stream creation failed");
-    }
-  }
+  if ((st = ensure_side(c)) != EXA_OK) return st;
   MixStep M{c, a, ld, npad, band, T, far_thr};
   cudaStream_t ms = c->stream, ss = c->side;
   const int sms = tc_num_sms();
@@ -684,6 +677,7 @@ extern "C" exa_status exa_gemm_update(exa_ctx* c, exa_gemm_kind kind, int64_t m,
                    (long long)k);
   const int k1 = (int)(k < kSplitMaxK ? k : kSplitMaxK), k2 = (int)(k - k1);
   exa_status st;
+  c->digits_held = false;
   if ((st = ensure_split(c, c->sp_a, c->mx_split, m, k1, !oz, oz)) != EXA_OK) return st;
   if ((st = ensure_split(c, c->sp_b, c->mx_split_b, n, k1, !oz, oz)) != EXA_OK) return st;
   if (k2 > 0) {

@@ -8,7 +8,7 @@ namespace exa {
 
 static const char* kNames[PK_COUNT] = {"matern_gen", "potrf_diag_fp64", "trsm_panel_fp64", "syrk_update_fp64",
                                        "dgemm_small_fp64", "split_rows", "gemm_tf32x3_tc", "gemm_tf32x3_pair",
-                                       "gemm_ozaki_tc",
+                                       "gemm_ozaki_tc", "gemm_fp64_digits",
                                        "trsv", "symv_residual", "gradient", "batched_chol", "other"};
 
 const char* prof_name(int kind) { return (kind >= 0 && kind < PK_COUNT) ? kNames[kind] : "?"; }

@@ -20,6 +20,7 @@ enum ProfKind : int {
   PK_GEMM_T3,       // tcgen05 TF32x3 products, one CTA per 128 x 128 tile
   PK_GEMM_T3_PAIR,  // tcgen05 TF32x3 products on CTA pairs (256 x 256 tiles): the trailing update
   PK_GEMM_OZ,       // tcgen05 exact digit-slice products
+  PK_GEMM_DIG,      // tcgen05 FP64 products from eight digits
   PK_TRSV,          // triangular solves
   PK_SYMV,          // refinement residual
   PK_GRAD,          // gradient kernels

@@ -1,0 +1,86 @@
+"""The FP64 factorisation on the tensor cores (eight 7-bit digits per value, 512-wide panels) at the edges of its
+tiles and panels, against A itself and against the FP64-unit factorisation (a context with 64-wide tiles).
+
+Bound of a factor's residual |L L^T - A|_ij, in units of sqrt(A_ii A_jj) (no row of L exceeds sqrt(A_ii)): each
+512-column pass may be off by 512 (2^-55 + 2^-53) 4 = 2,560 u of the two row maxima (u = 2^-53: values rounded at
+2^-56 of a row bound that is at most twice the maximum, and the left-out digit products, at most 7 2^-56 + ... <
+2^-53), and FP64 rounding in the diagonal blocks and in forming L L^T adds (n + 1) u twice.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -53
+
+
+def spd(n, seed, exps=0):
+    """G G^T + I, symmetrically scaled by powers of two 2^k, |k| <= exps; returns (matrix, scales)."""
+    rng = np.random.default_rng(seed)
+    g = rng.standard_normal((n, max(2, n // 2))) / np.sqrt(max(2, n // 2))
+    a = g @ g.T + np.eye(n)
+    a = 0.5 * (a + a.T)
+    d = 2.0 ** rng.integers(-exps, exps + 1, n).astype(np.float64)
+    return a * d[:, None] * d[None, :], d
+
+
+def factor(ctx, a, ld):
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    n = len(a)
+    buf = torch.full((n, ld), 7.0, dtype=torch.float64, device="cuda")  # column j of the matrix is row j here
+    buf[:, :n] = torch.as_tensor(a, device="cuda")
+    ctx.check(exa.exa_potrf(ctx.handle, buf, n, ld))
+    out = buf.cpu().numpy()
+    assert np.all(out[:, n:] == 7.0) and np.array_equal(np.tril(out[:, :n], -1), np.tril(a, -1))
+    return np.triu(out[:, :n]).T
+
+
+@pytest.mark.parametrize("n,pad,exps", [(1, 0, 0), (127, 3, 0), (128, 0, 0), (129, 0, 0), (511, 0, 0), (512, 0, 0),
+                                        (513, 5, 0), (640, 0, 480), (769, 0, 0), (1024, 0, 0), (1025, 1, 480),
+                                        (1664, 0, 0), (2200, 0, 60), (4500, 0, 0)])
+def test_factor_residual(n, pad, exps):
+    import paper_1908_06936_gb300 as exa
+
+    a, d = spd(n, n, exps)
+    root = np.sqrt(np.diag(a) / d / d)
+    bound = (-(-n // 512) * 2560 + 2 * (n + 1)) * U * np.outer(root, root)
+    with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as general:
+        l = factor(c, a, n + pad)
+        assert np.array_equal(l, factor(c, a, n + pad))  # repeatable to the bit
+        l64 = factor(general, a, n + pad) / d[:, None]
+    l = l / d[:, None]
+    assert np.all(np.abs(l @ l.T - a / d[:, None] / d[None, :]) <= bound)
+    # both factors are exact for matrices within the bound of A, and cond(A) <= 8 here: they agree to a few times it
+    assert np.max(np.abs(l - l64)) <= 32 * np.max(bound)
+
+
+@pytest.mark.parametrize("n,row", [(900, 700), (1300, 511), (1300, 512), (1300, 1299)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -1.0])
+def test_failing_pivot_is_reported(n, row, bad):
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    a, _ = spd(n, 3)
+    if bad < 0:
+        a[row, row] = bad
+    else:
+        a[row, 5] = a[5, row] = bad
+    with exa.Context() as c:
+        assert exa.exa_potrf(c.handle, torch.as_tensor(a, device="cuda"), n, n) == exa.EXA_ERR_NOT_SPD
+        assert exa.exa_last_pivot(c.handle) == row
+        good, _ = spd(n, 4)
+        c.check(exa.exa_potrf(c.handle, torch.as_tensor(good, device="cuda"), n, n))
+
+
+def test_workspace_bound_takes_the_fp64_units():
+    # 16 MB hold the padded matrix (10.6 MB) and the panels of the FP64-unit factorisation, not the digits
+    import paper_1908_06936_gb300 as exa
+
+    a, _ = spd(1100, 5)
+    with exa.Context(workspace_bytes=16 << 20) as c, exa.Context() as free:
+        l = factor(c, a, 1100)
+        assert exa.exa_workspace_bytes(c.handle) <= 16 << 20
+        ref = factor(free, a, 1100)
+    assert np.max(np.abs(l - ref)) <= 1e-11
