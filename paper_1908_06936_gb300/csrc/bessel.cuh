@@ -211,8 +211,8 @@ __device__ __forceinline__ int table_segment(double s) {
 
 // Table construction.  Segment sgi covers [lo, lo + w) of s with lo = 2^e (1 + sub / kTabSub),
 // w = 2^e / kTabSub.  Node id = sgi (kTabDeg + 1) + k is f at the k-th Chebyshev point.
-__device__ __forceinline__ void segment_geometry(int sgi, double& centre, double& half) {
-  const int e = kTabE0 + sgi / kTabSub, sub = sgi % kTabSub;
+__device__ __forceinline__ void segment_geometry(int sgi, double& centre, double& half, int e0 = kTabE0) {
+  const int e = e0 + sgi / kTabSub, sub = sgi % kTabSub;
   const double lo = ldexp(1.0 + (double)sub / kTabSub, e);
   const double w = ldexp(1.0 / kTabSub, e);
   centre = lo + 0.5 * w;
@@ -229,11 +229,9 @@ __device__ __forceinline__ double table_node_value(const MaternParams& P, int id
   return P.sigma2 * matern_ratio(P, sqrt(centre + half * tk));
 }
 
-// Chebyshev coefficients of segment sgi from its nodes, then their monomial form in t.
-__device__ __forceinline__ void table_segment_coefs(const double* __restrict__ nodes, int sgi,
-                                                    MaternTable* __restrict__ T) {
+// Values at the kTabDeg + 1 Chebyshev points of a segment -> coefficients of the interpolating polynomial in t.
+__device__ __forceinline__ void segment_polynomial(const double* __restrict__ q, double* __restrict__ out) {
   constexpr int N = kTabDeg + 1;
-  const double* q = nodes + sgi * N;
   double cheb[N];
   for (int j = 0; j < N; ++j) {
     double s = 0.0;
@@ -255,11 +253,16 @@ __device__ __forceinline__ void table_segment_coefs(const double* __restrict__ n
       t0[i] = t1[i];
     }
   }
+  for (int i = 0; i < N; ++i) out[i] = a[i];
+}
+
+__device__ __forceinline__ void table_segment_coefs(const double* __restrict__ nodes, int sgi,
+                                                    MaternTable* __restrict__ T) {
+  segment_polynomial(nodes + sgi * (kTabDeg + 1), T->a[sgi]);
   double centre, half;
   segment_geometry(sgi, centre, half);
   T->ih[sgi] = 1.0 / half;
   T->mc[sgi] = -centre / half;
-  for (int i = 0; i < N; ++i) T->a[sgi][i] = a[i];
 }
 
 // The exact routine as an out-of-line call for the table's rare out-of-range entries, so that

@@ -73,6 +73,7 @@ struct exa_ctx {
   exa::DevBuf gr_xsplit;    // mixed gradient: digit planes of every 512-row block of X = L^-1
   exa::DevBuf gr_lsplit;    // mixed gradient: digit planes of one 512-row block of L
   exa::DevBuf gr_t;         // mixed gradient: 512 x n product of one row block
+  exa::DevBuf gr_table;     // per-theta interpolation table of dSigma/dtheta and its node values
   exa::DevBuf gr_blocks;    // per-block gradient partial sums
   exa::DevBuf pr_c, pr_y;   // prediction: cross-covariance block and its solve block
   exa::DevBuf fs_m;         // Fisher information: Sigma^-1 D_k for k = 0, 1, 2

@@ -235,10 +235,99 @@ __device__ __forceinline__ void matern_derivs(const GradParams& G, double r, dou
   d2 = sig * (lnx - 0.69314718055994530942 - G.psi_nu) + P.sigma2 * exp(base - x) * dknu_dnu_scaled(P.nu, x);
 }
 
+// Per-theta interpolation table of the three derivatives in s = (r / beta)^2, laid out as the generator's (degree-8
+// polynomials on 1/64 octave pieces) over a longer range: 2^-24 <= s < 2^16, x = r / beta from 2^-12 to 256.  The
+// exact derivatives take a quadrature of ~100 exponentials an entry (3.1 ns an entry, 156 ms at n = 10,000); from
+// the table an entry is ~33 FP64 operations.  Below and above the range the exact routine applies.
+constexpr int kDerE0 = -24, kDerOct = 40, kDerSeg = kDerOct * kTabSub;
+struct DerivTable {
+  double seg[kDerSeg][2];                 // -centre / half-width, 1 / half-width
+  double a[kDerSeg][3][kTabDeg + 1];
+};
+constexpr int kDerNodes = kDerSeg * (kTabDeg + 1);
+// Building it costs ~23,000 exact evaluations; below this many entries they are evaluated one by one.
+constexpr int64_t kDerMinEntries = 4 * (int64_t)kDerNodes;
+
+__global__ void __launch_bounds__(64) deriv_nodes_kernel(const __grid_constant__ GradParams G,
+                                                         double* __restrict__ nodes) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= kDerNodes) return;
+  const int sgi = id / (kTabDeg + 1), k = id % (kTabDeg + 1);
+  double centre, half, d0, d1, d2;
+  segment_geometry(sgi, centre, half, kDerE0);
+  const double tk = cos(3.14159265358979323846 * (k + 0.5) / (kTabDeg + 1));
+  matern_derivs(G, sqrt(centre + half * tk) * G.m.beta, d0, d1, d2);
+  nodes[id] = d0;
+  nodes[kDerNodes + id] = d1;
+  nodes[2 * kDerNodes + id] = d2;
+}
+
+__global__ void __launch_bounds__(64) deriv_coef_kernel(const double* __restrict__ nodes,
+                                                        DerivTable* __restrict__ T) {
+  const int id = blockIdx.x * blockDim.x + threadIdx.x;
+  if (id >= 3 * kDerSeg) return;
+  const int f = id / kDerSeg, sgi = id % kDerSeg;
+  segment_polynomial(nodes + f * kDerNodes + sgi * (kTabDeg + 1), T->a[sgi][f]);
+  if (f == 0) {
+    double centre, half;
+    segment_geometry(sgi, centre, half, kDerE0);
+    T->seg[sgi][0] = -centre / half;
+    T->seg[sgi][1] = 1.0 / half;
+  }
+}
+
+static __device__ __noinline__ void matern_derivs_exact(const GradParams& G, double r2, double* d) {
+  matern_derivs(G, sqrt(r2), d[0], d[1], d[2]);
+}
+
+// Derivatives [K0, K1) of (sigma^2, beta, nu) at squared distance r2, from the table where there is one.
+template <int K0, int K1>
+__device__ __forceinline__ void matern_derivs_tab(const GradParams& G, const DerivTable* __restrict__ T, double r2,
+                                                  double (&d)[K1 - K0]) {
+  const double s = r2 * G.m.ib2;
+  const unsigned int se = (unsigned int)((unsigned long long)__double_as_longlong(s) >> 52);
+  // negative, zero, subnormal, infinite and NaN values all fall outside
+  if (!T || se - (unsigned int)(1023 + kDerE0) >= (unsigned int)kDerOct) {
+    double e[3];
+    matern_derivs_exact(G, r2, e);
+#pragma unroll
+    for (int k = K0; k < K1; ++k) d[k - K0] = e[k];
+    return;
+  }
+  const int sgi = (int)((unsigned long long)__double_as_longlong(s) >> (52 - kTabSubBits)) -
+                  ((1023 + kDerE0) << kTabSubBits);
+  const double t = fma(s, __ldg(&T->seg[sgi][1]), __ldg(&T->seg[sgi][0]));
+#pragma unroll
+  for (int k = K0; k < K1; ++k) {
+    const double* c = T->a[sgi][k];
+    double f = __ldg(&c[kTabDeg]);
+#pragma unroll
+    for (int q = kTabDeg - 1; q >= 0; --q) f = fma(f, t, __ldg(&c[q]));
+    d[k - K0] = f;
+  }
+}
+
+// The table for theta on the context stream, or nullptr where it does not pay or cannot be had.
+static const DerivTable* deriv_table(exa_ctx* c, const GradParams& G, int64_t entries) {
+  const size_t tab_b = (size_t)round_up(sizeof(DerivTable), 256);
+  if (entries < kDerMinEntries ||
+      ensure(c, c->gr_table, tab_b + 3 * (size_t)kDerNodes * sizeof(double), "derivative table", true) != EXA_OK) {
+    c->err[0] = 0;
+    return nullptr;
+  }
+  DerivTable* T = (DerivTable*)c->gr_table.p;
+  double* nodes = (double*)((char*)c->gr_table.p + tab_b);
+  ProfScope ps(c, PK_GRAD, 0.0, 0.0, 2);
+  deriv_nodes_kernel<<<(kDerNodes + 63) / 64, 64, 0, c->stream>>>(G, nodes);
+  deriv_coef_kernel<<<(3 * kDerSeg + 63) / 64, 64, 0, c->stream>>>(nodes, T);
+  return T;
+}
+
 // One 64 x 64 lower tile per block (as the generator), 256 threads; per-block partial
 // sums of w (a_i a_j - S_ij) D_k for k = sigma^2, beta, nu in a fixed order.
 __global__ void __launch_bounds__(256) grad_reduce_kernel(const double* __restrict__ locs, int64_t n,
                                                           const __grid_constant__ GradParams G,
+                                                          const DerivTable* __restrict__ tab,
                                                           const double* __restrict__ alpha,
                                                           const double* __restrict__ sinv, int64_t lds,
                                                           double ssign, double* __restrict__ partial) {
@@ -254,11 +343,11 @@ __global__ void __launch_bounds__(256) grad_reduce_kernel(const double* __restri
       if (j > i) continue;
       const double w = (i == j) ? 1.0 : 2.0;
       const double cij = w * (ai * alpha[j] - ssign * sinv[i + j * lds]);
-      double d0, d1, d2;
-      matern_derivs(G, sqrt(model_dist2(G.m, xi, yi, locs[2 * j], locs[2 * j + 1])), d0, d1, d2);
-      acc0 = fma(cij, d0, acc0);
-      acc1 = fma(cij, d1, acc1);
-      acc2 = fma(cij, d2, acc2);
+      double d[3];
+      matern_derivs_tab<0, 3>(G, tab, model_dist2(G.m, xi, yi, locs[2 * j], locs[2 * j + 1]), d);
+      acc0 = fma(cij, d[0], acc0);
+      acc1 = fma(cij, d[1], acc1);
+      acc2 = fma(cij, d[2], acc2);
     }
   }
   const int tid = threadIdx.x;
@@ -287,6 +376,7 @@ __global__ void __launch_bounds__(128) lauum_grad_fused_kernel(const double* __r
                                                                int64_t npad, int64_t n,
                                                                const double* __restrict__ locs,
                                                                const __grid_constant__ GradParams G,
+                                                               const DerivTable* __restrict__ tab,
                                                                const double* __restrict__ alpha,
                                                                double* __restrict__ partial, const DevStatus* st) {
   __shared__ double As[64 * gSS];
@@ -347,11 +437,11 @@ __global__ void __launch_bounds__(128) lauum_grad_fused_kernel(const double* __r
       if (j > i || j >= n) continue;
       const double w = (i == j) ? 1.0 : 2.0;
       const double cij = w * (ai * alpha[j] - Ss[r * 65 + cc]);
-      double d0, d1, d2;
-      matern_derivs(G, sqrt(model_dist2(G.m, xi, yi, locs[2 * j], locs[2 * j + 1])), d0, d1, d2);
-      acc0 = fma(cij, d0, acc0);
-      acc1 = fma(cij, d1, acc1);
-      acc2 = fma(cij, d2, acc2);
+      double d[3];
+      matern_derivs_tab<0, 3>(G, tab, model_dist2(G.m, xi, yi, locs[2 * j], locs[2 * j + 1]), d);
+      acc0 = fma(cij, d[0], acc0);
+      acc1 = fma(cij, d[1], acc1);
+      acc2 = fma(cij, d[2], acc2);
     }
   }
   red[0][tid] = acc0;
@@ -404,7 +494,9 @@ static cudaError_t launch_gradient(exa_ctx* c, const double* locs, int64_t n, in
   G.psi_nu = host_digamma(theta[2]);
   const long long t = (n + 63) / 64;
   const long long blocks = t * (t + 1) / 2;
-  grad_reduce_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(locs, n, G, alpha, sinv, npad, ssign, partial);
+  const DerivTable* tab = deriv_table(c, G, n * (n + 1) / 2);
+  ProfScope ps(c, PK_GRAD, 0.0, 4.0 * (double)n * (double)(n + 1), 2);
+  grad_reduce_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(locs, n, G, tab, alpha, sinv, npad, ssign, partial);
   grad_finish_kernel<<<3, 256, 0, c->stream>>>(partial, blocks, out);
   return cudaGetLastError();
 }
@@ -608,10 +700,7 @@ static exa_status loglik_grad_mixed(exa_ctx* c, const double* d_locs, const doub
   const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
   if ((st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials")) != EXA_OK) return st;
   cudaError_t e;
-  {
-    ProfScope ps(c, PK_GRAD, 0.0, 4.0 * (double)n * (double)(n + 1));
-    e = launch_gradient(c, d_locs, n, npad, theta, x, Sneg, ssign, (double*)c->gr_blocks.p, c->d_scalars + 8);
-  }
+  e = launch_gradient(c, d_locs, n, npad, theta, x, Sneg, ssign, (double*)c->gr_blocks.p, c->d_scalars + 8);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c->h_scalars + 8, c->d_scalars + 8, 3 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (e != cudaSuccess) return cuda_err(c, e, "gradient launch");
@@ -703,18 +792,17 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   if (!one_buffer) {
     if (e == cudaSuccess) e = sigma_inverse_fp64(c, npad, nb, S);
     // fused regeneration of dSigma/dtheta and reduction
-    if (e == cudaSuccess) {
-      ProfScope ps(c, PK_GRAD, 0.0, 4.0 * (double)n * (double)(n + 1));
+    if (e == cudaSuccess)
       e = launch_gradient(c, d_locs, n, npad, theta, y, S, 1.0, (double*)c->gr_blocks.p, c->d_scalars + 8);
-    }
   } else {
     if (e == cudaSuccess) e = factor_inverse_fp64(c, npad, nb);
     if (e == cudaSuccess) {
       GradParams G;
       model_params(c, theta, &G.m);
       G.psi_nu = host_digamma(theta[2]);
+      const DerivTable* tab = deriv_table(c, G, n * (n + 1) / 2);
       ProfScope ps(c, PK_GRAD, (double)npad * npad * npad / 3.0, 4.0 * (double)npad * (double)(npad + 1), 2);
-      lauum_grad_fused_kernel<<<(unsigned)nblocks, 128, 0, s>>>(A, npad, npad, n, d_locs, G, y,
+      lauum_grad_fused_kernel<<<(unsigned)nblocks, 128, 0, s>>>(A, npad, npad, n, d_locs, G, tab, y,
                                                                   (double*)c->gr_blocks.p, c->d_status);
       grad_finish_kernel<<<3, 256, 0, s>>>((double*)c->gr_blocks.p, (int64_t)nblocks, c->d_scalars + 8);
       e = cudaGetLastError();
@@ -745,17 +833,19 @@ __global__ void __launch_bounds__(256) mirror_lower_kernel(double* __restrict__ 
     s[i + j * ld] = s[j + i * ld];  // upper (i < j) from lower (j, i)
 }
 
+template <int K>
 __global__ void __launch_bounds__(256) deriv_matrix_kernel(const double* __restrict__ locs, int64_t n, int64_t npad,
-                                                           const __grid_constant__ GradParams G, int k,
+                                                           const __grid_constant__ GradParams G,
+                                                           const DerivTable* __restrict__ tab,
                                                            double* __restrict__ D) {
   const int64_t j = blockIdx.y;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npad; i += (int64_t)gridDim.x * blockDim.x) {
     double v = 0.0;
     if (i < n && j < n) {
-      double d[3];
-      matern_derivs(G, sqrt(model_dist2(G.m, locs[2 * i], locs[2 * i + 1], locs[2 * j], locs[2 * j + 1])), d[0], d[1],
-                    d[2]);
-      v = d[k];
+      double d[1];
+      matern_derivs_tab<K, K + 1>(G, tab, model_dist2(G.m, locs[2 * i], locs[2 * i + 1], locs[2 * j], locs[2 * j + 1]),
+                                  d);
+      v = d[0];
     }
     D[i + j * npad] = v;
   }
@@ -858,11 +948,14 @@ extern "C" exa_status exa_fisher(exa_ctx* c, const double* d_locs, const double 
   GradParams G;
   G.m = P;
   G.psi_nu = host_digamma(theta[2]);
+  const DerivTable* tab_d = deriv_table(c, G, 3 * n * n);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
     {
       ProfScope ps(c, PK_GRAD, 0.0, 8.0 * (double)nn);
-      deriv_matrix_kernel<<<dim3((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)npad), 256,
-                            0, s>>>(d_locs, n, npad, G, k, A);
+      const dim3 grid((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)npad);
+      if (k == 0) deriv_matrix_kernel<0><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
+      else if (k == 1) deriv_matrix_kernel<1><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
+      else deriv_matrix_kernel<2><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) {

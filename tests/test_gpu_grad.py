@@ -220,3 +220,30 @@ def test_mixed_gradient_bf16_and_fp32_refused(ctx):
         with pytest.raises(exa.ExaError) as ei:
             ctx.loglik_grad(to_dev(locs), to_dev(Z), (1.0, 0.1, 0.5), prec)
         assert ei.value.status == exa.EXA_ERR_ARG
+
+
+@pytest.mark.parametrize("theta", [(1.0, 0.1, 0.5), (1.3, 0.05, 1.4)])
+@pytest.mark.parametrize("m", [20, 22, 33])
+def test_gradient_table_range_edges(theta, m):
+    # m = 20 evaluates dSigma/dtheta entry by entry, larger fields from the interpolation table; pairs closer than
+    # 2^-12 beta or farther than 256 beta apart lie outside the table.  A nugget keeps Sigma well conditioned.
+    import paper_1908_06936_gb300 as exa
+
+    locs = synth.jittered_grid(m, seed=m)
+    beta = theta[1]
+    step = np.geomspace(2.0 ** -20, 2.0 ** -10, 12)[:, None] * beta
+    close = locs[:12] + step * np.array([[0.6, 0.8]])
+    far = np.geomspace(60.0, 900.0, 12)[:, None] * beta * np.array([[0.8, 0.6]])
+    locs = np.ascontiguousarray(np.concatenate([locs, close, far]))
+    z = synth.normals(len(locs), m)
+    oracle.set_model(nugget=0.1)
+    try:
+        ref = oracle.loglik_grad(locs, z, theta)
+    finally:
+        oracle.set_model()
+    with exa.Context() as c:
+        c.check(exa.exa_ctx_set_model(c.handle, 0.1))
+        l, g = c.loglik_grad(to_dev(locs), to_dev(z), theta)
+    scale = max(1.0, float(np.max(np.abs(ref["grad"]))))
+    assert abs(l - ref["l"]) <= 1e-10 * abs(ref["l"])
+    assert np.all(np.abs(g - ref["grad"]) <= 1e-8 * scale), (g, ref["grad"])
