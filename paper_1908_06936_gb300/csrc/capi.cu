@@ -107,6 +107,7 @@ exa_status reset_status(exa_ctx* c) {
 exa_status factor_fp64(exa_ctx* c, double* a, int64_t ld, int64_t npad, int nb) {
   const int T = (int)(npad / nb);
   exa_status st;
+  c->wall_kept = false;
   if (nb == 128) {
     bool done = false;
     st = factor_digits(c, a, ld, npad, &done);

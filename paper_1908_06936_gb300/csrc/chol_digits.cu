@@ -61,7 +61,8 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
   *done = true;
   double* W = (double*)c->w_all.p;
   double* LD = (double*)c->logdet_part.p;
-  double* W2 = (double*)c->mx_w2.p;
+  const bool keep = c->keep_block_inverses && c->mx_wall.bytes >= (size_t)(npad / kNB) * kNB * kNB * sizeof(double);
+  c->wall_kept = keep;
   double* X = (double*)c->mx_split2.p;
   cudaStream_t ms = c->stream, ss = c->side;
   const int sms = tc_num_sms();
@@ -76,6 +77,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     const int64_t k0 = (int64_t)k * kNB;
     const int w = (int)std::min<int64_t>(kNB, npad - k0);
     const double w3 = (double)w * w * w;
+    double* W2 = keep && w == kNB ? (double*)c->mx_wall.p + k0 * kNB : (double*)c->mx_w2.p;
     cudaError_t e;
     {
       ProfScope ps(c, PK_POTRF, (w == kNB ? 2.0 : 1.0) * w3 / 3.0, 8.0 * (3.0 * w * w), 1, s, s != ms);
@@ -190,13 +192,14 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
 
 void release_digits(exa_ctx* c) {
   cudaStreamSynchronize(c->stream);
-  for (DevBuf* b : {&c->mx_split, &c->mx_split2, &c->mx_split_b, &c->mx_w2, &c->mx_dscr}) {
+  for (DevBuf* b : {&c->mx_split, &c->mx_split2, &c->mx_split_b, &c->mx_w2, &c->mx_dscr, &c->mx_wall}) {
     if (b->p) cudaFree(b->p);
     c->held_bytes -= b->bytes;
     b->p = nullptr;
     b->bytes = 0;
   }
   c->digits_held = false;
+  c->wall_kept = false;
 }
 
 }  // namespace exa

@@ -56,6 +56,7 @@ struct exa_ctx {
   exa::DevBuf mx_split4;
   exa::DevBuf mx_split_b;   // split-precision operands (B role: inverse diagonal block / test B)
   exa::SplitOperand sp_a, sp_a2, sp_a3, sp_a4, sp_b;
+  bool wall_kept = false;   // the last FP64 factorisation left its 512-wide block inverses in mx_wall
   bool digits_held = false; // the buffers of reserve_digits are the FP64 path's: given up for requests that need the room
   exa::DevBuf mx_vec;       // refinement vectors
   exa::DevBuf mx_w2;        // inverse of the panel-wide diagonal block (row-major)
@@ -120,6 +121,10 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
 // be had, and those buffers are released.
 bool reserve_digits(exa_ctx* c, int64_t npad);
 void release_digits(exa_ctx* c);
+// Sigma^-1 on the tensor cores: room for it (allocate = false: whether it is held), and the inverse in the lower
+// triangle of c->mat from the factor there, whose block inverses were kept; x: npad^2 doubles of scratch.
+bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate = true);
+cudaError_t inverse_digits(exa_ctx* c, int64_t npad, double* x);
 // The look-ahead stream and its events.
 exa_status ensure_side(exa_ctx* c);
 exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_prec prec, int band, int far_thr);

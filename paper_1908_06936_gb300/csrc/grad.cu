@@ -18,10 +18,12 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "bessel.cuh"
 #include "ctx.cuh"
+#include "digits.cuh"
 #include "util.cuh"
 
 namespace exa {
@@ -758,7 +760,8 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   } else {
     // the factor's own buffer is requested first, so the test below sees what remains
     if ((st = ensure(c, c->mat, nn_bytes, "matrix")) != EXA_OK) return st;
-    if (nb == 128) reserve_digits(c, npad);  // worth more than the second buffer
+    // worth more than the second buffer
+    if (nb == 128 && reserve_digits(c, npad)) reserve_inverse_digits(c, npad);
     st = ensure(c, c->gr_part, nn_bytes, "inverse covariance", true);
     if (st == EXA_ERR_NOMEM) {
       one_buffer = true;
@@ -769,10 +772,16 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
       S = (double*)c->gr_part.p;
     }
   }
+  const long long t64n = one_buffer ? npad / 64 : (n + 63) / 64;
+  const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
+  if ((st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials")) != EXA_OK) return st;
   exa_result res;
   memset(&res, 0, sizeof(res));
   double* y = nullptr;
-  if ((st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y)) != EXA_OK) return st;
+  c->keep_block_inverses = nb == 128 && !one_buffer && reserve_inverse_digits(c, npad);
+  st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y);
+  c->keep_block_inverses = 0;
+  if (st != EXA_OK) return st;
   *loglik = res.loglik;
   double* A = (double*)c->mat.p;
   double* W = (double*)c->w_all.p;
@@ -785,12 +794,15 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
     ProfScope ps(c, PK_TRSV, 2.0 * rows * nb, 8.0 * rows * nb, 2);
     e = launch_trsv_bwd_step(s, A, npad, npad, nb, k, W, y, part + 2 * kRedPartials, c->d_status);
   }
-  const long long t64n = one_buffer ? npad / 64 : (n + 63) / 64;
-  const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
-  if ((st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials")) != EXA_OK) return st;
-  if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
+  const bool digits = !one_buffer && c->wall_kept && reserve_inverse_digits(c, npad, false);
+  if (!digits && (st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   if (!one_buffer) {
-    if (e == cudaSuccess) e = sigma_inverse_fp64(c, npad, nb, S);
+    if (e == cudaSuccess && digits) {
+      e = inverse_digits(c, npad, S);
+      S = A;
+    } else if (e == cudaSuccess) {
+      e = sigma_inverse_fp64(c, npad, nb, S);
+    }
     // fused regeneration of dSigma/dtheta and reduction
     if (e == cudaSuccess)
       e = launch_gradient(c, d_locs, n, npad, theta, y, S, 1.0, (double*)c->gr_blocks.p, c->d_scalars + 8);
@@ -833,21 +845,19 @@ __global__ void __launch_bounds__(256) mirror_lower_kernel(double* __restrict__ 
     s[i + j * ld] = s[j + i * ld];  // upper (i < j) from lower (j, i)
 }
 
+// Columns [j0, j0 + gridDim.y) of D_K as a full symmetric matrix, zero in the padding.
 template <int K>
 __global__ void __launch_bounds__(256) deriv_matrix_kernel(const double* __restrict__ locs, int64_t n, int64_t npad,
-                                                           const __grid_constant__ GradParams G,
+                                                           int64_t j0, const __grid_constant__ GradParams G,
                                                            const DerivTable* __restrict__ tab,
                                                            double* __restrict__ D) {
-  const int64_t j = blockIdx.y;
+  const int64_t j = j0 + blockIdx.y;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < npad; i += (int64_t)gridDim.x * blockDim.x) {
-    double v = 0.0;
-    if (i < n && j < n) {
-      double d[1];
+    double d[1] = {0.0};
+    if (i < n && j < n)
       matern_derivs_tab<K, K + 1>(G, tab, model_dist2(G.m, locs[2 * i], locs[2 * i + 1], locs[2 * j], locs[2 * j + 1]),
                                   d);
-      v = d[0];
-    }
-    D[i + j * npad] = v;
+    D[i + (int64_t)blockIdx.y * npad] = d[0];
   }
 }
 
@@ -936,10 +946,19 @@ extern "C" exa_status exa_fisher(exa_ctx* c, const double* d_locs, const double 
     e = launch_matern_gen(s, d_locs, n, npad, P, A, npad, nullptr, tab);
   }
   if (e != cudaSuccess) return cuda_err(c, e, "generation launch");
-  if ((st = factor_fp64(c, A, npad, npad, nb)) != EXA_OK) return st;
+  c->keep_block_inverses = nb == 128 && reserve_inverse_digits(c, npad);
+  st = factor_fp64(c, A, npad, npad, nb);
+  c->keep_block_inverses = 0;
+  if (st != EXA_OK) return st;
   if ((st = read_status(c)) != EXA_OK) return st;
-  if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
-  e = sigma_inverse_fp64(c, npad, nb, S);
+  const bool digits = c->wall_kept && reserve_inverse_digits(c, npad, false);
+  if (digits) {
+    e = inverse_digits(c, npad, S);
+    std::swap(A, S);  // Sigma^-1 took the factor's place
+  } else {
+    if ((st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
+    e = sigma_inverse_fp64(c, npad, nb, S);
+  }
   if (e == cudaSuccess) {
     mirror_lower_kernel<<<dim3((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)npad), 256, 0,
                           s>>>(S, npad, npad);
@@ -949,15 +968,51 @@ extern "C" exa_status exa_fisher(exa_ctx* c, const double* d_locs, const double 
   G.m = P;
   G.psi_nu = host_digamma(theta[2]);
   const DerivTable* tab_d = deriv_table(c, G, 3 * n * n);
-  for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-    {
-      ProfScope ps(c, PK_GRAD, 0.0, 8.0 * (double)nn);
-      const dim3 grid((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)npad);
-      if (k == 0) deriv_matrix_kernel<0><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
-      else if (k == 1) deriv_matrix_kernel<1><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
-      else deriv_matrix_kernel<2><<<grid, 256, 0, s>>>(d_locs, n, npad, G, tab_d, A);
-      e = cudaGetLastError();
+  // D_k(rows, [j0, j0 + cols)) into dst (ld npad)
+  auto derivative = [&](int k, int64_t j0, int64_t cols, double* dst) -> cudaError_t {
+    ProfScope ps(c, PK_GRAD, 0.0, 8.0 * (double)npad * (double)cols);
+    const dim3 grid((unsigned)((npad + 255) / 256 < 32 ? (npad + 255) / 256 : 32), (unsigned)cols);
+    if (k == 0) deriv_matrix_kernel<0><<<grid, 256, 0, s>>>(d_locs, n, npad, j0, G, tab_d, dst);
+    else if (k == 1) deriv_matrix_kernel<1><<<grid, 256, 0, s>>>(d_locs, n, npad, j0, G, tab_d, dst);
+    else deriv_matrix_kernel<2><<<grid, 256, 0, s>>>(d_locs, n, npad, j0, G, tab_d, dst);
+    return cudaGetLastError();
+  };
+  if (digits) {
+    // M_k = sum over 512-column chunks of S's and D_k's digits (both symmetric: rows of either are its columns)
+    for (int64_t j0 = 0; j0 < npad && e == cudaSuccess; j0 += kDigMaxK) {
+      const int w = (int)std::min<int64_t>(kDigMaxK, npad - j0);
+      DigitOperand Ds, Dd;
+      digit_layout(Ds, c->mx_split.p, npad, w, kDigSlices);
+      digit_layout(Dd, c->mx_split2.p, npad, w, kDigSlices);
+      {
+        ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * (double)npad * w, 1);
+        e = launch_digit_split(s, S + j0 * npad, 1, npad, npad, w, kDigSlices, Ds);
+      }
+      for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+        e = derivative(k, j0, w, A);
+        if (e == cudaSuccess) {
+          ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * (double)npad * w, 1);
+          e = launch_digit_split(s, A, 1, npad, npad, w, kDigSlices, Dd);
+        }
+        if (e != cudaSuccess) break;
+        DigitGemm g{};
+        g.C = M + k * nn;
+        g.Cin = j0 ? g.C : nullptr;
+        g.ldc = g.ldcin = npad;
+        g.m = g.n = npad;
+        g.A = Ds;
+        g.B = Dd;
+        g.K = w;
+        g.S = kDigSlices;
+        g.shape = kDigRect;
+        g.st = c->d_status;
+        ProfScope ps(c, PK_GEMM_DIG, 2.0 * (double)npad * npad * w, 16.0 * (double)nn);
+        e = launch_gemm_digits(s, g);
+      }
     }
+  }
+  for (int k = 0; k < 3 && e == cudaSuccess && !digits; ++k) {
+    e = derivative(k, 0, npad, A);
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_DGEMM_SMALL, 2.0 * (double)npad * npad * npad, 24.0 * (double)nn);
       e = launch_dgemm_nt_small(s, (int)npad, (int)npad, (int)npad, 1.0, S, 1, npad, A, 1, npad, 0.0, M + k * nn, 1,

@@ -84,3 +84,23 @@ def test_workspace_bound_takes_the_fp64_units():
         assert exa.exa_workspace_bytes(c.handle) <= 16 << 20
         ref = factor(free, a, 1100)
     assert np.max(np.abs(l - ref)) <= 1e-11
+
+
+@pytest.mark.parametrize("n", [1, 100, 129, 512, 520, 640, 1000, 1025, 1300])
+def test_gradient_and_fisher_against_the_fp64_units(n):
+    # the bars of the gradient's two forms against each other (1e-10 of the largest component) and of the Fisher
+    # information against the oracle (1e-9 of the diagonal)
+    import paper_1908_06936_gb300 as exa
+    from gpu_util import to_dev
+    from paper_1908_06936_gb300 import synth
+
+    theta = (1.2, 0.1, 0.6)
+    locs = to_dev(synth.uniform_square(n, n) if n < 4 else synth.jittered_grid(int(np.ceil(np.sqrt(n))), n)[:n])
+    z = to_dev(synth.normals(n, n))
+    with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as general:
+        l, g = c.loglik_grad(locs, z, theta)
+        l64, g64 = general.loglik_grad(locs, z, theta)
+        f, f64 = c.fisher(locs, theta), general.fisher(locs, theta)
+    assert abs(l - l64) <= 1e-10 * abs(l64)
+    assert np.all(np.abs(g - g64) <= 1e-10 * max(1.0, float(np.max(np.abs(g64))))), (g, g64)
+    assert np.all(np.abs(f - f64) <= 1e-9 * np.sqrt(np.outer(np.diag(f64), np.diag(f64))) + 1e-300), (f, f64)
