@@ -77,6 +77,7 @@ struct exa_ctx {
   exa::DevBuf gr_table;     // per-theta interpolation table of dSigma/dtheta and its node values
   exa::DevBuf gr_blocks;    // per-block gradient partial sums
   exa::DevBuf pr_c, pr_y;   // prediction: cross-covariance block and its solve block
+  exa::DevBuf pr_m;         // prediction: partial sums of the means
   exa::DevBuf fs_m;         // Fisher information: Sigma^-1 D_k for k = 0, 1, 2
   // batched
   exa::DevBuf bt_mat, bt_meta, bt_vec, bt_work, bt_mat2;
@@ -123,7 +124,12 @@ bool reserve_digits(exa_ctx* c, int64_t npad);
 void release_digits(exa_ctx* c);
 // Sigma^-1 on the tensor cores: room for it (allocate = false: whether it is held), and the inverse in the lower
 // triangle of c->mat from the factor there, whose block inverses were kept; x: npad^2 doubles of scratch.
-bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate = true);
+// rows: of the second operand where it has more than npad (prediction points).
+bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate = true, int64_t rows = 0);
+// Digits of the h x h diagonal block at k0 of the factor in c->mat (Dl) and of its inverse with column k scaled by row
+// k's exponent of Dl (Dw), in mx_split_b.
+struct DigitOperand;
+cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl);
 cudaError_t inverse_digits(exa_ctx* c, int64_t npad, double* x);
 // The look-ahead stream and its events.
 exa_status ensure_side(exa_ctx* c);

@@ -18,13 +18,14 @@ constexpr int kSub = 128;
 
 static size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 
-bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate) {
+bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t rows) {
+  if (rows < npad) rows = npad;
   struct {
     DevBuf* b;
     size_t bytes;
   } want[] = {{&c->mx_wall, (size_t)(npad / kNB) * kNB * kNB * sizeof(double)},
               {&c->mx_split, digit_bytes(npad, kNB, kDigSlices)},
-              {&c->mx_split2, digit_bytes(npad, kNB, kDigSlices)},
+              {&c->mx_split2, digit_bytes(rows, kNB, kDigSlices)},
               {&c->mx_split_b, 2 * align256(digit_bytes(kNB, kNB, kDigSlices))}};
   if (!allocate) {
     bool have = true;
@@ -37,6 +38,16 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate) {
   for (auto& w : want) ok = ok && ensure(c, *w.b, w.bytes, "digit operands", true) == EXA_OK;
   if (!ok) c->err[0] = 0;
   return ok;
+}
+
+cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl) {
+  const double* a = (const double*)c->mat.p + k0 + k0 * npad;
+  const double* w = h == kNB ? (const double*)c->mx_wall.p + k0 * kNB : (const double*)c->w_all.p + k0 * kSub;
+  digit_layout(Dl, c->mx_split_b.p, h, h, kDigSlices);
+  digit_layout(Dw, (uint8_t*)c->mx_split_b.p + align256(digit_bytes(kNB, kNB, kDigSlices)), h, h, kDigSlices);
+  cudaError_t e = launch_digit_split(c->stream, a, 1, npad, h, h, kDigSlices, Dl, 0, true);
+  if (e == cudaSuccess) e = launch_digit_split(c->stream, w, h, 1, h, h, kDigSlices, Dw, 0, true, Dl.ex, 1);
+  return e;
 }
 
 // Diagonal block <- W (row-major, h x h), strict upper triangle 0.
@@ -59,16 +70,13 @@ cudaError_t inverse_digits(exa_ctx* c, int64_t npad, double* x) {
     const double* w = h == kNB ? (const double*)c->mx_wall.p + l0 * kNB : (const double*)c->w_all.p + l0 * kSub;
     const double dh = (double)h;
     DigitOperand Dl, Dw, D, Dx;
-    digit_layout(Dl, c->mx_split_b.p, h, (int)h, kDigSlices);
-    digit_layout(Dw, (uint8_t*)c->mx_split_b.p + align256(digit_bytes(kNB, kNB, kDigSlices)), h, (int)h, kDigSlices);
     digit_layout(Dx, c->mx_split2.p, n1, (int)h, kDigSlices);
     if (l0 > 0) {
       // X_l = W_l T_l, column k of W and row k of T scaled by row k's size in L_ll (as in the panel solve)
       digit_layout(D, c->mx_split.p, l0, (int)h, kDigSlices);
       {
         ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * dh * (double)n1, 3);
-        e = launch_digit_split(s, a + l0 + l0 * ld, 1, ld, h, (int)h, kDigSlices, Dl, 0, true);
-        if (e == cudaSuccess) e = launch_digit_split(s, w, h, 1, h, (int)h, kDigSlices, Dw, 0, true, Dl.ex, 1);
+        e = split_block_inverse(c, npad, l0, (int)h, Dw, Dl);
         if (e == cudaSuccess) e = launch_digit_split(s, x + l0, ld, 1, l0, (int)h, kDigSlices, D, 0, false, Dl.ex, -1);
       }
       DigitGemm g{};

@@ -104,3 +104,20 @@ def test_gradient_and_fisher_against_the_fp64_units(n):
     assert abs(l - l64) <= 1e-10 * abs(l64)
     assert np.all(np.abs(g - g64) <= 1e-10 * max(1.0, float(np.max(np.abs(g64))))), (g, g64)
     assert np.all(np.abs(f - f64) <= 1e-9 * np.sqrt(np.outer(np.diag(f64), np.diag(f64))) + 1e-300), (f, f64)
+
+
+@pytest.mark.parametrize("n,m", [(1, 1), (100, 65), (512, 64), (513, 63), (640, 2049), (1300, 2500)])
+def test_prediction_against_the_fp64_units(n, m):
+    # the bars of test_gpu_predict: means to 1e-9 of the largest observation, variances to 1e-9 sigma^2
+    import paper_1908_06936_gb300 as exa
+    from gpu_util import to_dev
+    from paper_1908_06936_gb300 import synth
+
+    theta = (1.2, 0.1, 0.6)
+    locs = to_dev(synth.uniform_square(n, n) if n < 4 else synth.jittered_grid(int(np.ceil(np.sqrt(n))), n)[:n])
+    z, new = to_dev(synth.normals(n, n)), to_dev(synth.uniform_square(m, m + 1))
+    with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as general:
+        mean, var = (t.cpu().numpy() for t in c.predict(locs, z, theta, new))
+        mean64, var64 = (t.cpu().numpy() for t in general.predict(locs, z, theta, new))
+    assert np.all(np.abs(mean - mean64) <= 1e-9 * float(z.abs().max()))
+    assert np.all(np.abs(var - var64) <= 1e-9 * theta[0])
