@@ -231,9 +231,14 @@ exa_status exa_loglik_grad(exa_ctx* ctx, const double* d_locs, const double* d_z
 exa_status exa_ctx_set_gradient_inverse(exa_ctx* ctx, int fp64);
 
 /* Batched evaluation of nrep independent replicate fields of uneven sizes
- * (one persistent launch walks the tile tasks of every replicate; the
+ * (one persistent launch walks the tile tasks of every replicate, or one launch
+ * per kind and 128-wide tile column takes every replicate's; the
  * replicate studies of Section III, Example 2).
- *   prec      EXA_FP64: every tile task in FP64.  EXA_MIXED_FP32 (the MP
+ *   prec      EXA_FP64: FP64 throughout, step-synchronous over 128-wide tile columns
+ *             with the products formed from exact digit products on the tensor cores
+ *             (as the single-field factorisation); with a tile of 32 or a CTA count set
+ *             by exa_ctx_set_batched, or without room for the digits, in one persistent
+ *             launch on the FP64 units.  EXA_MIXED_FP32 (the MP
  *             variant of Section II-A): diagonal tiles factored in FP64, the
  *             off-diagonal TRSM and update tiles computed from FP32-rounded
  *             operands with FP32 accumulation over the tile and added to the
@@ -380,7 +385,8 @@ int exa_profile_read(exa_ctx* ctx, exa_kernel_stat* out, int max, int reset);
 
 /* Options of the batched form:
  *   tile_nb      tile of the persistent factorisation, 32 or 64 (0: 64);
- *   ctas_per_sm  persistent CTAs per SM, capped at what fits resident (0: all that fit);
+ *   ctas_per_sm  persistent CTAs per SM, capped at what fits resident (0: all that fit;
+ *                EXA_FP64 with 64 and 0 runs on the tensor cores instead);
  *   spin_cycles  bound of one dependency wait in SM clock cycles (0: 2e9, about 1 s);
  *   inject_stall test hook: non-zero adds to the work list a task whose dependency is
  *                never met, so its wait runs out and the affected replicates report
@@ -389,7 +395,8 @@ exa_status exa_ctx_set_batched(exa_ctx* ctx, int tile_nb, int ctas_per_sm, long 
 
 /* Tile autotuner of the batched form.  Runs the batch (same arguments as
  * exa_loglik_batched) with every candidate configuration -- tile 64 and 32,
- * each with the largest and the next-largest number of resident CTAs per SM --
+ * each with the largest and the next-largest number of resident CTAs per SM, and in
+ * EXA_FP64 the tensor-core form (reported as tile 64, ctas_per_sm 0) --
  * twice (plan + buffers, then a run timed with CUDA events on the context
  * stream), keeps the fastest in the context and returns it (tile_nb,
  * ctas_per_sm, best_ms: host outputs).  Synchronises the stream.  d_loglik /

@@ -35,6 +35,7 @@
 
 #include "bessel.cuh"
 #include "ctx.cuh"
+#include "digits.cuh"
 #include "gemm_tc.cuh"
 
 namespace exa {
@@ -1189,7 +1190,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
         const BMeta& m = meta[r];
         if (m.T <= k) continue;
         diag.push_back({mat + m.mo, m.npad, (int64_t)k * NB, ldpart + m.lo + k, wbuf + m.wo + (int64_t)k * NB * NB,
-                        dRst + r});
+                        dRst + r, nullptr, nullptr, nullptr});
       }
       stp.ndiag = (int)diag.size() - stp.diag_off;
       // replicates with a panel below tile k
@@ -1358,12 +1359,346 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   return EXA_OK;
 }
 
+// ---------------------------------------------------------------------------
+// FP64 on the tensor cores: the same step-synchronous form with every product formed from eight digits (digits.cu),
+// and y = L^-1 z carried along (the diagonal kernel finishes y_k, one launch per step takes L_rest,k y_k off the
+// rest), so that no refinement and no second copy of Sigma is needed.  Per step k:
+//   1. Cholesky and inverse W_k of the diagonal tiles, y_k = W_k z_k, the row exponents of L_kk;
+//   2. digits of the W_k and of the panels, column c of the panel and of W scaled by row c's exponent;
+//   3. L_ik = A_ik W_k^T, one grouped launch; 4. z_i -= L_ik y_k and the digits of L_ik;
+//   5. A_ij -= L_ik L_jk^T, one grouped launch.
+// On the FP64 units (the persistent form) 32 fields of 400 to 6,400 points took 542 ms in the factorisation.
+// ---------------------------------------------------------------------------
+struct ZTask {
+  const double* l;   // panel, column-major
+  int64_t ld, rows;
+  double* z;         // y_k, then the rest of z
+};
+
+// z_r -= sum_t L(r, t) y_t, 128 rows a CTA, two halves of the columns.
+__global__ void __launch_bounds__(256) batched_z_update_kernel(const ZTask* __restrict__ tasks) {
+  __shared__ double y[kTcNB], half1[kTcNB];
+  const ZTask t = tasks[blockIdx.y];
+  const int64_t r0 = (int64_t)blockIdx.x * kTcNB;
+  if (r0 >= t.rows) return;  // uniform over the CTA, before any barrier
+  const int row = threadIdx.x & (kTcNB - 1), h = threadIdx.x >> 7;
+  if (h == 0) y[row] = t.z[row];
+  __syncthreads();
+  const double* col = t.l + r0 + row + (int64_t)(h * 64) * t.ld;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+  for (int c = 0; c < 64; c += 4)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] = fma(col[(int64_t)(c + u) * t.ld], y[h * 64 + c + u], s[u]);
+  const double sum = (s[0] + s[1]) + (s[2] + s[3]);
+  if (h) half1[row] = sum;
+  __syncthreads();
+  if (!h) t.z[kTcNB + r0 + row] -= sum + half1[row];
+}
+
+__global__ void __launch_bounds__(256) batched_z_init_kernel(const BMeta* __restrict__ M, double* __restrict__ z) {
+  const BMeta m = M[blockIdx.y];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m.npad; i += (int64_t)gridDim.x * blockDim.x)
+    z[m.vo + i] = i < m.n ? m.z[i] : 0.0;
+}
+
+__global__ void batched_fp64_finish_kernel(int nrep, const BMeta* __restrict__ M, const DevStatus* __restrict__ rst,
+                                           const DevStatus* __restrict__ st, const double* __restrict__ ldpart,
+                                           const double* __restrict__ qpart, double* __restrict__ loglik,
+                                           int32_t* __restrict__ rstatus) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= nrep) return;
+  const BMeta m = M[r];
+  if (rstatus[r] == EXA_OK) {
+    if (st->timeout) rstatus[r] = EXA_ERR_TIMEOUT;
+    else if (rst[r].info) rstatus[r] = EXA_ERR_NOT_SPD;
+  }
+  double ldet = 0.0, q = 0.0;
+  for (int64_t k = 0; k < m.T; ++k) {
+    ldet += ldpart[m.lo + k];
+    q += qpart[m.lo + k];
+  }
+  loglik[r] = rstatus[r] == EXA_OK ? -0.5 * (double)m.n * 1.8378770664093454836 - 0.5 * (2.0 * ldet) - 0.5 * q : NAN;
+}
+
+struct DigStep {
+  int diag_off, ndiag, set_off, nset;     // DiagTileTask range; ZTask range, and the split tasks at twice its offsets
+  long long trsm_off, ntrsm, upd_off, nupd;
+  int64_t max_m;
+};
+
+struct DigPlan {
+  std::vector<int64_t> ns;
+  std::vector<DigStep> steps;
+  const void *mat = nullptr, *buf = nullptr, *task = nullptr;  // what the device lists point into
+  void* stage = nullptr;   // pinned; captured copies read it at replay, so no other form writes to it
+  size_t stage_bytes = 0;
+};
+
+// *done = false: its memory could not be had and nothing was launched.
+static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, const double* const* d_locs,
+                                     const double* const* d_z, const double* d_theta, double* d_loglik,
+                                     int32_t* d_status, bool* done) {
+  constexpr int NB = kTcNB;
+  *done = false;
+  cudaStream_t s = c->stream;
+  if (!c->dplan) c->dplan = new DigPlan();
+  DigPlan& P = *c->dplan;
+  std::vector<BMeta> meta(nrep);
+  int64_t mo = 0, wo = 0, lo = 0, vo = 0, gt = 0, ps_rows = 0;
+  int Tmax = 0;
+  for (int r = 0; r < nrep; ++r) {
+    BMeta& m = meta[r];
+    m.n = h_n[r];
+    m.npad = round_up(h_n[r], NB);
+    m.T = m.npad / NB;
+    m.mo = mo;
+    m.wo = wo;
+    m.co = 0;
+    m.lo = lo;
+    m.vo = vo;
+    m.gt = gt;
+    m.locs = d_locs[r];
+    m.z = d_z[r];
+    mo += round_up(m.npad * m.npad, 32);
+    wo += m.T * NB * NB;
+    lo += m.T;
+    vo += m.npad;
+    gt += m.T * (m.T + 1) / 2;
+    ps_rows += m.npad - NB;
+    Tmax = m.T > Tmax ? (int)m.T : Tmax;
+  }
+  if (Tmax > 32000) return EXA_OK;
+  const bool same_shape = (int)P.ns.size() == nrep && std::equal(P.ns.begin(), P.ns.end(), h_n);
+  // one buffer: meta | params | tables | statuses | row exponents | inverses | log and quadratic parts | z | digits
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t at = off;
+    off += (bytes + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_meta = take(nrep * sizeof(BMeta)), o_par = take(nrep * sizeof(MaternParams));
+  const size_t o_tab = take(nrep * sizeof(MaternTable)), o_rst = take(nrep * sizeof(DevStatus));
+  const size_t o_rex = take((size_t)nrep * NB * sizeof(int)), o_w = take(wo * sizeof(double));
+  const size_t o_ld = take(lo * sizeof(double)), o_q = take(lo * sizeof(double)), o_z = take(vo * sizeof(double));
+  const size_t o_ws = take(digit_bytes((int64_t)nrep * NB, NB, kDigSlices));
+  constexpr int64_t kNodes = kTabSeg * (kTabDeg + 1);
+  const size_t nodes_b = (size_t)nrep * kNodes * sizeof(double);  // scratch before the first panel
+  const size_t ps_b = digit_bytes(ps_rows, NB, kDigSlices);
+  const size_t o_ps = take(ps_b > nodes_b ? ps_b : nodes_b);
+  // task lists: diagonal tiles | splits (W, panel) | z | products
+  long long nd = 0, nset = 0, ntask = 0;
+  for (int r = 0; r < nrep; ++r) {
+    const long long T = meta[r].T;
+    nd += T;
+    nset += T - 1;
+    ntask += T * (T - 1) + (T - 1) * T * (T + 1) / 3;  // sum of 2 b (solves) and of b (b + 1) (updates), b < T
+  }
+  const size_t d_b = round_up(nd * (int64_t)sizeof(DiagTileTask), 256);
+  const size_t s_b = round_up(2 * nset * (int64_t)sizeof(DigitSplitTask), 256);
+  const size_t z_b = round_up(nset * (int64_t)sizeof(ZTask), 256);
+  const size_t t_b = round_up(ntask * (int64_t)sizeof(DigitTask), 256);
+  struct {
+    DevBuf* b;
+    size_t bytes;
+  } want[] = {{&c->bd_mat, (size_t)mo * sizeof(double)}, {&c->bd_buf, off}, {&c->bd_task, d_b + s_b + z_b + t_b}};
+  size_t held = c->held_bytes;
+  for (auto& w : want) held += w.bytes > w.b->bytes ? w.bytes - w.b->bytes : 0;
+  if (c->ws_limit && held > c->ws_limit) return EXA_OK;
+  for (auto& w : want)
+    if (ensure(c, *w.b, w.bytes, "batched digit form", true) != EXA_OK) {
+      c->err[0] = 0;
+      release_batched_digits(c);
+      return EXA_OK;
+    }
+  uint8_t* base = (uint8_t*)c->bd_buf.p;
+  BMeta* dM = (BMeta*)(base + o_meta);
+  MaternParams* dP = (MaternParams*)(base + o_par);
+  MaternTable* dTab = (MaternTable*)(base + o_tab);
+  DevStatus* dRst = (DevStatus*)(base + o_rst);
+  int* dRex = (int*)(base + o_rex);
+  double* wbuf = (double*)(base + o_w);
+  double* ldpart = (double*)(base + o_ld);
+  double* qpart = (double*)(base + o_q);
+  double* zbuf = (double*)(base + o_z);
+  double* mat = (double*)c->bd_mat.p;
+  DigitOperand Ws, Ps;
+  digit_layout(Ws, base + o_ws, (int64_t)nrep * NB, NB, kDigSlices);
+  digit_layout(Ps, base + o_ps, ps_rows, NB, kDigSlices);
+  uint8_t* tb = (uint8_t*)c->bd_task.p;
+  DiagTileTask* dDiag = (DiagTileTask*)tb;
+  DigitSplitTask* dSpl = (DigitSplitTask*)(tb + d_b);
+  ZTask* dZ = (ZTask*)(tb + d_b + s_b);
+  DigitTask* dTask = (DigitTask*)(tb + d_b + s_b + z_b);
+  const bool rebuild = !same_shape || P.mat != c->bd_mat.p || P.buf != c->bd_buf.p || P.task != c->bd_task.p;
+  const size_t meta_b = round_up((int64_t)nrep * sizeof(BMeta), 256);
+  const size_t stage_need = meta_b + (rebuild ? d_b + s_b + z_b + t_b : 0);
+  if (P.stage_bytes < stage_need) {
+    if (P.stage) cudaFreeHost(P.stage);
+    P.stage = nullptr;
+    P.stage_bytes = 0;
+    if (cudaMallocHost(&P.stage, stage_need) != cudaSuccess) {
+      cudaGetLastError();
+      return EXA_OK;
+    }
+    P.stage_bytes = stage_need;
+  }
+  uint8_t* hs = (uint8_t*)P.stage;
+  if (rebuild) {
+    // an earlier call's copies may still read the staging area
+    const cudaError_t es = cudaStreamSynchronize(s);
+    if (es != cudaSuccess) return cuda_err(c, es, "batched setup");
+    P.steps.clear();
+    P.ns.clear();
+    DiagTileTask* hd = (DiagTileTask*)(hs + meta_b);
+    DigitSplitTask* hp = (DigitSplitTask*)(hs + meta_b + d_b);
+    ZTask* hz = (ZTask*)(hs + meta_b + d_b + s_b);
+    DigitTask* ht = (DigitTask*)(hs + meta_b + d_b + s_b + z_b);
+    int id = 0, iset = 0;
+    long long it = 0;
+    std::vector<int> set, prow;
+    for (int k = 0; k < Tmax; ++k) {
+      DigStep stp{};
+      stp.diag_off = id;
+      stp.set_off = iset;
+      set.clear();
+      prow.clear();
+      int rows = 0;
+      for (int r = 0; r < nrep; ++r) {
+        const BMeta& m = meta[r];
+        if (m.T <= k) continue;
+        hd[id++] = {mat + m.mo, m.npad, (int64_t)k * NB, ldpart + m.lo + k, wbuf + m.wo + (int64_t)k * NB * NB,
+                    dRst + r, zbuf + m.vo + (int64_t)k * NB, qpart + m.lo + k, dRex + r * NB};
+        if (m.T == k + 1) continue;
+        set.push_back(r);
+        prow.push_back(rows);
+        rows += (int)(m.npad - (int64_t)(k + 1) * NB);
+      }
+      stp.ndiag = id - stp.diag_off;
+      stp.nset = (int)set.size();
+      for (int q = 0; q < stp.nset; ++q) {
+        const int r = set[q];
+        const BMeta& m = meta[r];
+        const int64_t mr = m.npad - (int64_t)(k + 1) * NB;
+        const double* panel = mat + m.mo + (int64_t)(k + 1) * NB + (int64_t)k * NB * m.npad;
+        // the W's at 2 set_off .., the panels after them
+        hp[2 * stp.set_off + q] = {wbuf + m.wo + (int64_t)k * NB * NB, NB, 1, NB, (int64_t)q * NB, dRex + r * NB, 1, 1};
+        hp[2 * stp.set_off + stp.nset + q] = {panel, 1, m.npad, mr, prow[q], dRex + r * NB, -1, 0};
+        hz[iset++] = {panel, m.npad, mr, zbuf + m.vo + (int64_t)k * NB};
+        stp.max_m = mr > stp.max_m ? mr : stp.max_m;
+      }
+      stp.trsm_off = it;
+      for (int q = 0; q < stp.nset; ++q) {
+        const BMeta& m = meta[set[q]];
+        double* panel = mat + m.mo + (int64_t)(k + 1) * NB + (int64_t)k * NB * m.npad;
+        for (int64_t i = 0; i < m.T - k - 1; ++i)
+          for (int h = 0; h < NB / kDigTN; ++h)
+            ht[it++] = {panel + i * NB + (int64_t)h * kDigTN * m.npad, m.npad, prow[q] + (int)i * NB,
+                        q * NB + h * kDigTN, kDigStore, 0};
+      }
+      stp.ntrsm = it - stp.trsm_off;
+      stp.upd_off = it;
+      for (int q = 0; q < stp.nset; ++q) {
+        const BMeta& m = meta[set[q]];
+        double* trail = mat + m.mo + (int64_t)(k + 1) * NB * (m.npad + 1);
+        for (int64_t i = 0; i < m.T - k - 1; ++i)
+          for (int64_t j = 0; j < 2 * (i + 1); ++j)
+            ht[it++] = {trail + i * NB + j * kDigTN * m.npad, m.npad, prow[q] + (int)i * NB, prow[q] + (int)j * kDigTN,
+                        j < 2 * i ? kDigPlain : (int)(j - 2 * i) * kDigTN, 0};
+      }
+      stp.nupd = it - stp.upd_off;
+      P.steps.push_back(stp);
+    }
+    P.ns.assign(h_n, h_n + nrep);
+    P.mat = c->bd_mat.p;
+    P.buf = c->bd_buf.p;
+    P.task = c->bd_task.p;
+  }
+  memcpy(hs, meta.data(), nrep * sizeof(BMeta));
+  *done = true;
+  cudaError_t e = cudaMemcpyAsync(dM, hs, nrep * sizeof(BMeta), cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess && rebuild)
+    e = cudaMemcpyAsync(tb, hs + meta_b, d_b + s_b + z_b + t_b, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(dRst, 0, nrep * sizeof(DevStatus), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(DevStatus), s);
+  if (e != cudaSuccess) return cuda_err(c, e, "batched setup");
+  double* dNodes = (double*)(base + o_ps);
+  {
+    ProfScope ps(c, PK_OTHER, 0.0, 0.0, 4);
+    batched_params_kernel<<<(nrep + 63) / 64, 64, 0, s>>>(nrep, d_theta, dP, d_status, c->nugget, c->metric,
+                                                          c->radius);
+    batched_table_nodes_kernel<<<dim3((unsigned)((kNodes + 127) / 128), (unsigned)nrep), 128, 0, s>>>(dP, dNodes);
+    batched_table_coef_kernel<<<dim3((kTabSeg + 127) / 128, (unsigned)nrep), 128, 0, s>>>(dNodes, dTab);
+    batched_z_init_kernel<<<dim3(4, (unsigned)nrep), 256, 0, s>>>(dM, zbuf);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) {
+    ProfScope ps(c, PK_GEN, 0.0, 8.0 * (double)gt * NB * NB / 2);
+    batched_gen_kernel<NB><<<(unsigned)gt, 256, 0, s>>>(nrep, dM, dP, dTab, mat, nullptr);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return cuda_err(c, e, "batched generation");
+  for (size_t k = 0; k < P.steps.size() && e == cudaSuccess; ++k) {
+    const DigStep& stp = P.steps[k];
+    {
+      ProfScope ps(c, PK_POTRF, (double)stp.ndiag * NB * NB * NB * 2.0 / 3.0, 0.0, 1);
+      e = launch_potrf128_tasks(s, dDiag + stp.diag_off, stp.ndiag);
+    }
+    if (e != cudaSuccess || stp.nset == 0) continue;
+    const DigitSplitTask* spl = dSpl + 2 * stp.set_off;
+    const double panel_e = (double)stp.ntrsm * NB * kDigTN;  // panel entries
+    {
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * (panel_e + (double)stp.nset * NB * NB), 2);
+      e = launch_digit_split_tasks(s, spl, stp.nset, NB, NB, Ws);
+      if (e == cudaSuccess) e = launch_digit_split_tasks(s, spl + stp.nset, stp.nset, stp.max_m, NB, Ps, true);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_GEMM_DIG, panel_e * NB, 8.0 * panel_e);
+      e = launch_gemm_digits_tasks(s, dTask + stp.trsm_off, stp.ntrsm, NB, Ps, Ws, false, c->d_status);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * panel_e);
+      e = launch_digit_split_tasks(s, spl + stp.nset, stp.nset, stp.max_m, NB, Ps, false);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_TRSV, 2.0 * panel_e, 8.0 * panel_e);
+      batched_z_update_kernel<<<dim3((unsigned)(stp.max_m / NB), (unsigned)stp.nset), 256, 0, s>>>(dZ + stp.set_off);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) {
+      const double upd = (double)stp.nupd * NB * kDigTN;
+      ProfScope ps(c, PK_GEMM_DIG, 2.0 * upd * NB, 16.0 * upd);
+      e = launch_gemm_digits_tasks(s, dTask + stp.upd_off, stp.nupd, NB, Ps, Ps, true, c->d_status);
+    }
+  }
+  if (e != cudaSuccess) return cuda_err(c, e, "batched factorisation");
+  batched_fp64_finish_kernel<<<(nrep + 127) / 128, 128, 0, s>>>(nrep, dM, dRst, c->d_status, ldpart, qpart, d_loglik,
+                                                                d_status);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_err(c, e, "batched launch");
+  return EXA_OK;
+}
+
+void release_batched_digits(exa_ctx* c) {
+  for (DevBuf* b : {&c->bd_mat, &c->bd_buf, &c->bd_task}) {
+    if (b->p) cudaFree(b->p);
+    c->held_bytes -= b->bytes;
+    b->p = nullptr;
+    b->bytes = 0;
+  }
+  if (c->dplan) c->dplan->ns.clear();
+}
+
 void release_batched(exa_ctx* c) {
   if (c->bt_stage) cudaFreeHost(c->bt_stage);
   c->bt_stage = nullptr;
   c->bt_stage_bytes = 0;
   delete c->bplan;
   c->bplan = nullptr;
+  release_batched_digits(c);
+  if (c->dplan && c->dplan->stage) cudaFreeHost(c->dplan->stage);
+  delete c->dplan;
+  c->dplan = nullptr;
 }
 
 }  // namespace exa
@@ -1382,6 +1717,13 @@ extern "C" exa_status exa_loglik_batched(exa_ctx* c, int32_t nrep, const int64_t
   if (prec != EXA_FP64 && prec != EXA_MIXED_FP32 && prec != EXA_MIXED_TF32X3)
     return set_err(c, EXA_ERR_ARG, "the batched form runs in EXA_FP64, EXA_MIXED_FP32 or EXA_MIXED_TF32X3");
   if (!c->bplan) c->bplan = new BatchPlan();
+  // FP64 with the default options goes to the tensor cores; a tile of 32, a CTA count and the test hook belong to the
+  // persistent form, which also runs where the digits do not fit
+  if (prec == EXA_FP64 && c->batched_nb == 64 && c->batched_ctas_per_sm == 0 && !c->batched_stall) {
+    bool done = false;
+    const exa_status st = batched_run_digits(c, nrep, h_n, d_locs, d_z, d_theta, d_loglik, d_status, &done);
+    if (st != EXA_OK || done) return st;
+  }
   if (prec == EXA_MIXED_TF32X3) return batched_run_tc(c, nrep, h_n, d_locs, d_z, d_theta, d_loglik, d_status);
   if (c->bplan->tc) {  // the persistent form rebuilds its own work list
     c->bplan->tc = false;
@@ -1429,9 +1771,10 @@ extern "C" exa_status exa_batched_autotune(exa_ctx* c, int32_t nrep, const int64
   const bool tc = prec == EXA_MIXED_TF32X3;
   for (int nb : {64, 32}) {
     const int top = tc ? 1 : max_ctas_per_sm(nb, mode);
-    for (int cps : {top, top - 1}) {
+    // 0 in FP64 with the default tile: the tensor-core form
+    for (int cps : {top, top - 1, prec == EXA_FP64 && nb == 64 ? 0 : -1}) {
       if (tc && (nb != 64 || cps != 1)) continue;
-      if (cps < 1 || st != EXA_OK) continue;
+      if (cps < 0 || (cps == 0 && (prec != EXA_FP64 || nb != 64)) || st != EXA_OK) continue;
       c->batched_nb = nb;
       c->batched_ctas_per_sm = cps;
       // first call builds the plan and the buffers for this tile; the second is timed

@@ -10,6 +10,7 @@
 namespace exa {
 
 struct BatchPlan;
+struct DigPlan;
 
 struct DevBuf {
   void* p = nullptr;
@@ -82,6 +83,8 @@ struct exa_ctx {
   // batched
   exa::DevBuf bt_mat, bt_meta, bt_vec, bt_work, bt_mat2;
   exa::DevBuf bt_tasks, bt_ps, bt_ws;  // tensor-core batched form: task lists, panel and inverse split operands
+  exa::DevBuf bd_mat, bd_buf, bd_task;  // FP64 batched form on the tensor cores
+  exa::DigPlan* dplan = nullptr;
   exa::BatchPlan* bplan = nullptr;  // cached work list of the last shape set
   void* bt_stage = nullptr;         // pinned host staging for the work list / metadata
   size_t bt_stage_bytes = 0;
@@ -147,6 +150,7 @@ exa_status matern_table(exa_ctx* c, const MaternParams& P, const MaternTable** t
 // matern_params plus the context's model options (nugget, metric, radius).
 void model_params(const exa_ctx* c, const double theta[3], MaternParams* P);
 void release_batched(exa_ctx* c);
+void release_batched_digits(exa_ctx* c);
 // Lay out a split operand of `rows` x K in `buf` (T3 planes and/or OZ digits) and build its TMA maps.
 exa_status ensure_split(exa_ctx* c, SplitOperand& op, DevBuf& buf, int64_t rows, int K, bool t3, bool oz);
 // Bytes of one split operand (a multiple of 1024), and its layout at `base` (1024-byte aligned)

@@ -78,6 +78,7 @@ struct Args {
   const uint8_t *A, *B;           // first plane, at the operand's row origin
   int64_t a_plane, b_plane;       // bytes between planes
   const int *ea, *eb, *sq;
+  const DigitTask* tasks;         // kDigTasks
   int mt, nt;                     // row blocks, column tiles
   int shape, tri;
   int k16;
@@ -86,13 +87,44 @@ struct Args {
   DevStatus* st;
 };
 
-__device__ __forceinline__ void tile_of(const Args& g, long long t, int& bi, int& bj) {
+// Operand rows and output of tile t.  diag: column minus row index of the tile's corner in a symmetric output, whose
+// entries with diag + column > row are left out (kNoDiag: none).
+constexpr int kNoDiag = -(1 << 30);
+struct Tile {
+  int64_t ar, br;
+  double* C;
+  const double* Cin;
+  int64_t ldc, ldcin;
+  int diag, bj;
+};
+__device__ __forceinline__ void tile_of(const Args& g, long long t, Tile& o) {
+  if (g.shape == kDigTasks) {
+    const DigitTask k = g.tasks[t];
+    o.ar = k.a_row;
+    o.br = k.b_row;
+    o.C = k.C;
+    o.Cin = k.diag == kDigStore ? nullptr : k.C;
+    o.ldc = o.ldcin = k.ldc;
+    o.diag = k.diag >= 0 ? k.diag : kNoDiag;
+    o.bj = 0;
+    return;
+  }
+  int bi, bj;
   if (g.shape == kDigRect) {
     bi = (int)(t % g.mt);
     bj = (int)(t / g.mt);
+    o.diag = kNoDiag;
   } else {
     lower_tile(t, g.mt, bi, bj);
+    o.diag = bj * TN - bi * TM;
   }
+  o.ar = (int64_t)bi * TM;
+  o.br = (int64_t)bj * TN;
+  o.C = g.C + o.ar + o.br * g.ldc;
+  o.Cin = g.Cin ? g.Cin + o.ar + o.br * g.ldcin : nullptr;
+  o.ldc = g.ldc;
+  o.ldcin = g.ldcin;
+  o.bj = bj;
 }
 
 __device__ __forceinline__ void timeout(DevStatus* st, volatile int* abort, int site) {
@@ -150,12 +182,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
     for (int s = 0; s < STAGES; ++s) last_par[s] = -1;
     bool ok = true;  // the same for every lane
     for (long long t = g.t0 + blockIdx.x; t < g.ntiles && ok; t += gridDim.x) {
-      int bi, bj;
-      tile_of(g, t, bi, bj);
-      const int steps = g.tri ? min(g.k16, (bj + 1) * (TN / 16)) : g.k16;
+      Tile o;
+      tile_of(g, t, o);
+      const int steps = g.tri ? min(g.k16, (o.bj + 1) * (TN / 16)) : g.k16;
       const bool isA = lane < S;
-      const uint8_t* src = isA ? g.A + (int64_t)lane * g.a_plane + (int64_t)bi * A_BYTES
-                               : g.B + (int64_t)(lane - S) * g.b_plane + (int64_t)bj * B_BYTES;
+      const uint8_t* src = isA ? g.A + (int64_t)lane * g.a_plane + o.ar * 32
+                               : g.B + (int64_t)(lane - S) * g.b_plane + o.br * 32;
       const int64_t step_bytes = S * (isA ? g.a_plane : g.b_plane);
       const uint32_t off = isA ? lane * A_BYTES : S * A_BYTES + (lane - S) * B_BYTES;
       for (int kc = 0; kc < steps; ++kc) {
@@ -188,9 +220,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
     int stage = 0;
     uint32_t phase = 0, it = 0;
     for (long long t = g.t0 + blockIdx.x; t < g.ntiles && !*abort; t += gridDim.x) {
-      int bi, bj;
-      tile_of(g, t, bi, bj);
-      const int steps = g.tri ? min(g.k16, (bj + 1) * (TN / 16)) : g.k16;
+      int steps = g.k16;
+      if (g.tri) {
+        Tile o;
+        tile_of(g, t, o);
+        steps = min(steps, (o.bj + 1) * (TN / 16));
+      }
       if (!mbar_wait(accempty, (it & 1) ^ 1, abort)) {
         timeout(g.st, abort, 82);
         break;
@@ -237,11 +272,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
     constexpr int CH = TN / 2, P = S / 2;
     uint32_t it = 0;
     for (long long t = g.t0 + blockIdx.x; t < g.ntiles; t += gridDim.x) {
-      int bi, bj;
-      tile_of(g, t, bi, bj);
-      const int64_t row = (int64_t)bi * TM + r, col0 = (int64_t)bj * TN + half * CH;
-      const int er = g.ea[row];
-      const bool lower = g.shape == kDigLower;
+      Tile o;
+      tile_of(g, t, o);
+      const int er = g.ea[o.ar + r];
+      const int* ebp = g.eb + o.br + half * CH;
+      double* cp = o.C + r + (int64_t)(half * CH) * o.ldc;
+      const double* cip = o.Cin ? o.Cin + r + (int64_t)(half * CH) * o.ldcin : nullptr;
+      const int last = r - o.diag - half * CH;  // columns up to this one of the half are on or below the diagonal
       if (!__all_sync(0xffffffffu, mbar_wait(accfull, it & 1, abort))) {
         if (lane == 0) timeout(g.st, abort, 84);
         break;
@@ -272,12 +309,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
         double cv[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-          cv[j] = g.Cin && !(lower && col0 + j0 + j > row) ? g.Cin[row + (col0 + j0 + j) * g.ldcin] : 0.0;
+          cv[j] = cip && j0 + j <= last ? cip[(int64_t)(j0 + j) * o.ldcin] : 0.0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int64_t col = col0 + j0 + j;
-          if (lower && col > row) continue;
-          const int ec = g.eb[col];
+          if (j0 + j > last) continue;
+          const int ec = ebp[j0 + j];
           // x = sum of the groups, in units of the last one
           double x;
           if constexpr (S == 2) {
@@ -285,7 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
           } else {
             const double hi = int_to_f64((long long)w[0][j0 + j] * 16384 + w[1][j0 + j]);
             double lo = int_to_f64((long long)w[P - 2][j0 + j] * 16384 + w[P - 1][j0 + j]);
-            if (lower && row == col) lo = fma((double)g.sq[row], 1.0 / 128.0, lo);
+            if (j0 + j == last) lo = fma((double)g.sq[o.ar + r], 1.0 / 128.0, lo);  // the diagonal
             x = fma(hi, 268435456.0, lo);
           }
           const int sh = base + ec;
@@ -297,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
           } else {
             v = g.sign ? cv[j] - scalbn(x, sh) : cv[j] + scalbn(x, sh);
           }
-          g.C[row + col * g.ldc] = v;
+          cp[(int64_t)(j0 + j) * o.ldc] = v;
         }
       }
     }
@@ -330,10 +366,9 @@ __device__ __forceinline__ double scale_exp(double v, int c) {
 }
 
 template <int S>
-__global__ void __launch_bounds__(kSplitThreads) digit_split_kernel(const double* __restrict__ src, int64_t rs,
-                                                                    int64_t cs, int64_t rows, int K, int lower,
-                                                                    const int* __restrict__ colex, int colsign,
-                                                                    DigitOperand op, int64_t out_row0) {
+__device__ __forceinline__ void split_body(const double* __restrict__ src, int64_t rs, int64_t cs, int64_t rows, int K,
+                                           int lower, const int* __restrict__ colex, int colsign,
+                                           const DigitOperand& op, int64_t out_row0) {
   extern __shared__ double tile[];
   __shared__ int s_e[kRows];
   __shared__ int s_sq[kRows];
@@ -428,6 +463,23 @@ __global__ void __launch_bounds__(kSplitThreads) digit_split_kernel(const double
   }
 }
 
+template <int S>
+__global__ void __launch_bounds__(kSplitThreads) digit_split_kernel(const double* __restrict__ src, int64_t rs,
+                                                                    int64_t cs, int64_t rows, int K, int lower,
+                                                                    const int* __restrict__ colex, int colsign,
+                                                                    DigitOperand op, int64_t out_row0) {
+  split_body<S>(src, rs, cs, rows, K, lower, colex, colsign, op, out_row0);
+}
+
+// Many pieces in one launch: blockIdx.y = piece, blockIdx.x = 16-row chunk of it.
+__global__ void __launch_bounds__(kSplitThreads) digit_split_tasks_kernel(const DigitSplitTask* __restrict__ tasks,
+                                                                          int K, int scaled, DigitOperand op) {
+  const DigitSplitTask t = tasks[blockIdx.y];
+  if ((int64_t)blockIdx.x * kRows >= t.rows) return;  // uniform over the CTA, before any barrier
+  split_body<kDigSlices>(t.src, t.rs, t.cs, t.rows, K, t.lower, scaled ? t.colex : nullptr, t.colsign, op,
+                         t.out_row0);
+}
+
 }  // namespace dig
 
 size_t digit_bytes(int64_t rows, int K, int S) {
@@ -465,6 +517,21 @@ cudaError_t launch_digit_split(cudaStream_t s, const double* src, int64_t rs, in
   if (S == kDigSlices) return split_impl<kDigSlices>(s, src, rs, cs, rows, K, lower, colex, colsign, op, out_row0);
   if (S == kDigLow) return split_impl<kDigLow>(s, src, rs, cs, rows, K, lower, colex, colsign, op, out_row0);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_digit_split_tasks(cudaStream_t s, const DigitSplitTask* d_tasks, int ntasks, int64_t max_rows,
+                                     int K, const DigitOperand& op, bool scaled) {
+  if (ntasks <= 0 || max_rows <= 0) return cudaSuccess;
+  if (K <= 0 || K % 16 || K > kDigMaxK) return cudaErrorInvalidValue;
+  static PerDeviceOnce once;
+  cudaError_t e = once([] {
+    return cudaFuncSetAttribute(dig::digit_split_tasks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                dig::kRows * (kDigMaxK + 1) * (int)sizeof(double));
+  });
+  if (e != cudaSuccess) return e;
+  dig::digit_split_tasks_kernel<<<dim3((unsigned)ceil_div(max_rows, dig::kRows), (unsigned)ntasks), dig::kSplitThreads,
+                                  (size_t)dig::kRows * (K + 1) * sizeof(double), s>>>(d_tasks, K, scaled, op);
+  return cudaGetLastError();
 }
 
 template <int S>
@@ -514,6 +581,27 @@ cudaError_t launch_gemm_digits(cudaStream_t s, const DigitGemm& g, int max_ctas)
   if (g.S == kDigSlices) return gemm_impl<kDigSlices>(s, a, max_ctas);
   if (g.S == kDigLow) return gemm_impl<kDigLow>(s, a, max_ctas);
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K,
+                                     const DigitOperand& A, const DigitOperand& B, bool neg, DevStatus* st) {
+  if (ntasks <= 0) return cudaSuccess;
+  if (K <= 0 || K % 16 || K > kDigMaxK) return cudaErrorInvalidValue;
+  dig::Args a{};
+  a.A = A.dig;
+  a.B = B.dig;
+  a.a_plane = A.rows * 32;
+  a.b_plane = B.rows * 32;
+  a.ea = A.ex;
+  a.eb = B.ex;
+  a.sq = A.sq;
+  a.tasks = d_tasks;
+  a.shape = kDigTasks;
+  a.k16 = K / 16;
+  a.ntiles = ntasks;
+  a.sign = neg ? 0x80000000u : 0u;
+  a.st = st;
+  return gemm_impl<kDigSlices>(s, a, 0);
 }
 
 }  // namespace exa

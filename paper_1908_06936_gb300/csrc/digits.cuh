@@ -35,7 +35,7 @@ cudaError_t launch_digit_split(cudaStream_t s, const double* src, int64_t rs, in
                                const DigitOperand& op, int64_t out_row0 = 0, bool lower = false,
                                const int* colex = nullptr, int colsign = 0);
 
-enum : int { kDigRect = 0, kDigLower = 1 };
+enum : int { kDigRect = 0, kDigLower = 1, kDigTasks = 2 };
 struct DigitGemm {
   // C(i, j) = Cin(i, j) +- sum_k A(a_row0 + i, k) B(b_row0 + j, k), C and Cin column-major; Cin = nullptr: 0.
   double* C;
@@ -55,5 +55,28 @@ struct DigitGemm {
 };
 // max_ctas > 0 caps the persistent grid.
 cudaError_t launch_gemm_digits(cudaStream_t s, const DigitGemm& g, int max_ctas = 0);
+
+// Grouped forms (batched replicates).  One 128 x kDigTN tile of C: rows a_row.. of A against rows b_row.. of B.
+// diag >= 0: the tile lies on the diagonal of a symmetric output (rows of A and B alike), its first column diag columns
+// right of its first row's, and only entries on or below the diagonal are written; kDigPlain: all entries; kDigStore:
+// C = A B^T without reading C.
+enum : int { kDigPlain = -1, kDigStore = -2 };
+struct DigitTask {
+  double* C;
+  int64_t ldc;
+  int a_row, b_row;
+  int diag, pad;
+};
+cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K,
+                                     const DigitOperand& A, const DigitOperand& B, bool neg, DevStatus* st);
+// One piece of a grouped split (the arguments of launch_digit_split); scaled = false: without the column exponents.
+struct DigitSplitTask {
+  const double* src;
+  int64_t rs, cs, rows, out_row0;
+  const int* colex;
+  int colsign, lower;
+};
+cudaError_t launch_digit_split_tasks(cudaStream_t s, const DigitSplitTask* d_tasks, int ntasks, int64_t max_rows,
+                                     int K, const DigitOperand& op, bool scaled = true);
 
 }  // namespace exa

@@ -151,6 +151,11 @@ struct DiagTileTask {
   double* logdet;
   double* w;
   DevStatus* st;
+  // with z != nullptr also: z (128 entries, the right-hand side here) <- y = W z, *quad = y^T y, and rex[i] the
+  // exponent e of row i of L (|L_ij| < 2^e)
+  double* z;
+  double* quad;
+  int* rex;
 };
 cudaError_t launch_potrf128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks);
 // FP64 Cholesky and inverse of the 512 x 512 diagonal block at (k0, k0) as one cooperative launch

@@ -121,3 +121,43 @@ def test_prediction_against_the_fp64_units(n, m):
         mean64, var64 = (t.cpu().numpy() for t in general.predict(locs, z, theta, new))
     assert np.all(np.abs(mean - mean64) <= 1e-9 * float(z.abs().max()))
     assert np.all(np.abs(var - var64) <= 1e-9 * theta[0])
+
+
+def batch(c, ns, tile, ctas, seed=0):
+    import torch
+    import paper_1908_06936_gb300 as exa
+    from gpu_util import to_dev
+    from paper_1908_06936_gb300 import synth
+
+    locs = [to_dev(synth.uniform_square(n, seed + r) if n < 4 else
+                   synth.jittered_grid(int(np.ceil(np.sqrt(n))), seed + r)[:n]) for r, n in enumerate(ns)]
+    z = [to_dev(synth.normals(n, seed + r)) for r, n in enumerate(ns)]
+    th = to_dev(synth.theta_perturbations((1.0, 0.1, 0.6), len(ns), seed).ravel())
+    out = torch.empty(len(ns), dtype=torch.float64, device="cuda")
+    st = torch.empty(len(ns), dtype=torch.int32, device="cuda")
+    c.check(exa.exa_ctx_set_batched(c.handle, tile, ctas, 0, 0))
+    c.check(exa.exa_loglik_batched(c.handle, len(ns), ns, locs, z, th, exa.EXA_FP64, out, st))
+    torch.cuda.synchronize()
+    assert np.all(st.cpu().numpy() == 0)
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("ns", [[1], [128, 127], [129, 1, 300, 128, 257], [1000, 400, 401, 129, 2000, 640]])
+def test_batched_fp64_against_the_persistent_form(ns):
+    # both forms are held to 1e-10 of the oracle elsewhere; a shape change and the persistent form in between leave
+    # the tensor-core form's lists right; a context without room for the digits falls back to the persistent form
+    import paper_1908_06936_gb300 as exa
+
+    with exa.Context() as c:
+        got = batch(c, ns, 0, 0)
+        ref = batch(c, ns, 32, 0)
+        batch(c, [200] + ns, 0, 0)
+        assert np.array_equal(got, batch(c, ns, 0, 0))
+    assert np.all(np.abs(got - ref) <= 1e-10 * np.abs(ref))
+    with exa.Context() as c:
+        batch(c, ns, 64, 1)
+        need = exa.exa_workspace_bytes(c.handle)
+    with exa.Context(workspace_bytes=need) as c:
+        low = batch(c, ns, 0, 0)
+        assert exa.exa_workspace_bytes(c.handle) <= need
+    assert np.all(np.abs(low - ref) <= 1e-10 * np.abs(ref))
