@@ -22,7 +22,7 @@ using namespace tc;
 
 namespace dig {
 constexpr int TM = 128, TN = kDigTN;
-constexpr int kEpiWarps = 8, kThreads = 64 + 32 * kEpiWarps;
+constexpr int kEpiWarps = 16, kThreads = 64 + 32 * kEpiWarps;
 
 template <int S>
 struct Cfg {
@@ -113,6 +113,7 @@ __device__ __forceinline__ void tile_of(const Args& g, long long t, Tile& o) {
   if (g.shape == kDigRect) {
     bi = (int)(t % g.mt);
     bj = (int)(t / g.mt);
+    if (g.tri) bj = g.nt - 1 - bj;  // the longest reductions first
     o.diag = kNoDiag;
   } else {
     lower_tile(t, g.mt, bi, bj);
@@ -132,13 +133,33 @@ __device__ __forceinline__ void timeout(DevStatus* st, volatile int* abort, int 
   if (atomicExch(&st->timeout, 1) == 0) st->timeout_where = site;
 }
 
-// v an integer, |v| < 2^51, as a double: its bits added to those of 1.5 2^52, the constant taken off again.
-__device__ __forceinline__ double int_to_f64(long long v) {
-  return __longlong_as_double(v + 0x4338000000000000ll) - 6755399441055744.0;
+// V 2^sh, rounded to nearest, for |V| < 2^63: the double is built from V's bits (FP64 instructions issue two lanes a
+// cycle on an SM: one per output is what the epilogue can hide).  Below the normal range 0, above it infinity, and NaN
+// where sh counts a row with kDigBad.
+__device__ __forceinline__ double i63_to_f64_scaled(long long V, int sh) {
+  const unsigned long long sign = (unsigned long long)V & 0x8000000000000000ull;
+  const unsigned long long m = V < 0 ? (unsigned long long)(-V) : (unsigned long long)V;
+  const int lz = __clzll((long long)m);
+  const unsigned long long r = ((m << (lz - 1)) + 0x200) >> 10;  // leading one at bit 52 (53 after a carry)
+  const int be = 1022 + 63 - lz + sh;                            // one below the biased exponent: the leading one adds it
+  if (be >= 0x7FE) return __longlong_as_double((long long)(sign | (be > kDigBad / 2 ? 0x7FF8ull : 0x7FF0ull) << 48));
+  if (m == 0 || be < 0) return __longlong_as_double((long long)sign);
+  return __longlong_as_double((long long)(sign | (((unsigned long long)be << 52) + r)));
+}
+
+// FP32 integers as integers.  F2I converts 16 lanes a cycle on an SM, which for the 65,536 accumulators of a tile is a
+// ninth of its MMA time, so half of the groups go by additions instead:
+// |a| <= 2^22: the low bits of a + 1.5 2^23;
+__device__ __forceinline__ int small_int_bits(float a) { return __float_as_int(a + 12582912.0f); }  // + 0x4B400000
+// |a| <= 2^24: the multiples of 4 from a + 1.5 2^25, then the rest.
+__device__ __forceinline__ int large_int(float a) {
+  const float u = a + 50331648.0f;
+  const float rest = a - (u - 50331648.0f);
+  return 4 * (__float_as_int(u) - 0x4C400000) + (__float_as_int(rest + 12582912.0f) - 0x4B400000);
 }
 
 // One CTA per SM, persistent: warp 0 copies operand planes into a ring of 16-column stages, one thread of warp 1
-// issues the MMAs, warps 2-9 drain TMEM into C.  The S B planes of a stage lie one after another and group g
+// issues the MMAs, warps 2-17 drain TMEM into C.  The S B planes of a stage lie one after another and group g
 // follows group g - 1 in TMEM, so A digit s against B digits 0 .. S-1-s is one run of columns (two MMAs where
 // N > 256): 12 MMAs a step instead of 36.
 //
@@ -266,10 +287,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
       ++it;
     }
   } else if (warp >= 2) {
-    // ---------------- drain: warp w takes TMEM lanes 32 (w % 4).. and column half (w - 2) / 4 ----------------
+    // ---------------- drain: warp w takes TMEM lanes 32 (w % 4).. and columns CH ((w - 2) / 4) .. ----------------
     const int quad = warp & 3, half = (warp - 2) >> 2;
     const int r = quad * 32 + lane;
-    constexpr int CH = TN / 2, P = S / 2;
+    constexpr int CH = TN * 4 / kEpiWarps;
+    static_assert(CH == 16, "two lanes per column in the prefetch");
     uint32_t it = 0;
     for (long long t = g.t0 + blockIdx.x; t < g.ntiles; t += gridDim.x) {
       Tile o;
@@ -279,61 +301,66 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
       double* cp = o.C + r + (int64_t)(half * CH) * o.ldc;
       const double* cip = o.Cin ? o.Cin + r + (int64_t)(half * CH) * o.ldcin : nullptr;
       const int last = r - o.diag - half * CH;  // columns up to this one of the half are on or below the diagonal
+      if (o.Cin)  // this warp's lines of C into L2 while the products run: lane l column l / 2, rows 16 (l % 2) ..
+        prefetch_l2(o.Cin + quad * 32 + 16 * (lane & 1) + (int64_t)(half * CH + (lane >> 1)) * o.ldcin);
       if (!__all_sync(0xffffffffu, mbar_wait(accfull, it & 1, abort))) {
         if (lane == 0) timeout(g.st, abort, 84);
         break;
       }
       fence_after();
-      // groups 2p and 2p + 1 hold exact integers of weights 2^(-12-14p), 2^(-19-14p): one 32-bit word for both
-      int w[P][CH];
+      // groups 2p and 2p + 1 hold exact integers of weights 2^(-12-14p), 2^(-19-14p): a 32-bit word for both (S = 8: at
+      // most 7 2^28 + 2^24), a 64-bit one for groups 0-3 and one for 4-7, and V for all, in units of 2^8 of the last
+      long long V[CH];
       const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + half * CH;
 #pragma unroll
-      for (int p = 0; p < P; ++p) {
+      for (int h = 0; h < CH; h += 4) {
+        constexpr int H = S < 4 ? S : 4;
+        uint32_t x[H][4];
 #pragma unroll
-        for (int h = 0; h < CH; h += 16) {
-          uint32_t x0[16], x1[16];
-          tmem_ld16(ta + (2 * p) * TN + h, x0);
-          tmem_ld16(ta + (2 * p + 1) * TN + h, x1);
+        for (int p = 0; p < H; ++p) tmem_ld4(ta + p * TN + h, x[p]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int w01 = small_int_bits(__uint_as_float(x[0][j])) * 128 + small_int_bits(__uint_as_float(x[1][j])) -
+                          (int)(129u * 0x4B400000u);
+          V[h + j] = w01;
+          if constexpr (S == 8)
+            V[h + j] = ((long long)w01 * 16384 + (__float2int_rn(__uint_as_float(x[2][j])) * 128 +
+                                                  __float2int_rn(__uint_as_float(x[3][j])))) << 20;
+        }
+        if constexpr (S == 8) {
+#pragma unroll
+          for (int p = 0; p < 4; ++p) tmem_ld4(ta + (4 + p) * TN + h, x[p]);
           tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            w[p][h + j] = __float2int_rn(__uint_as_float(x0[j])) * 128 + __float2int_rn(__uint_as_float(x1[j]));
+          for (int j = 0; j < 4; ++j) {
+            const int w45 = __float2int_rn(__uint_as_float(x[0][j])) * 128 + __float2int_rn(__uint_as_float(x[1][j]));
+            const int w67 = large_int(__uint_as_float(x[2][j])) * 128 + large_int(__uint_as_float(x[3][j]));
+            V[h + j] += ((long long)w45 * 16384 + w67 + 128) >> 8;
+          }
         }
       }
       fence_before();
       mbar_arrive(accempty);
       ++it;
-      const int base = er - 12 - 7 * (S - 1);  // weight of the last group, without the column's exponent
+      const int base = er - 12 - 7 * (S - 1) + (S == 8 ? 8 : 0);  // weight of V's unit, without the column's exponent
+      if (S == 8 && o.diag > -TM) {  // the diagonal's left-out group
+        const long long sq = (g.sq[o.ar + r] + (1 << 14)) >> 15;
 #pragma unroll
-      for (int j0 = 0; j0 < CH; j0 += 8) {
-        double cv[8];
+        for (int j = 0; j < CH; ++j) V[j] += j == last ? sq : 0;
+      }
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          cv[j] = cip && j0 + j <= last ? cip[(int64_t)(j0 + j) * o.ldcin] : 0.0;
+      for (int j0 = 0; j0 < CH; j0 += 4) {
+        asm volatile("" ::: "memory");  // four outputs at a time: more would not fit the registers
+        double cv[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          if (j0 + j > last) continue;
+        for (int j = 0; j < 4; ++j) cv[j] = cip && j0 + j <= last ? cip[(int64_t)(j0 + j) * o.ldcin] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
           const int ec = ebp[j0 + j];
-          // x = sum of the groups, in units of the last one
-          double x;
-          if constexpr (S == 2) {
-            x = int_to_f64(w[0][j0 + j]);
-          } else {
-            const double hi = int_to_f64((long long)w[0][j0 + j] * 16384 + w[1][j0 + j]);
-            double lo = int_to_f64((long long)w[P - 2][j0 + j] * 16384 + w[P - 1][j0 + j]);
-            if (j0 + j == last) lo = fma((double)g.sq[o.ar + r], 1.0 / 128.0, lo);  // the diagonal
-            x = fma(hi, 268435456.0, lo);
-          }
-          const int sh = base + ec;
-          double v;
-          if (er == kDigBad || ec == kDigBad) {
-            v = __longlong_as_double(0x7FF8000000000000ll);
-          } else if (sh >= -1000 && sh <= 900) {
-            v = fma(x, __hiloint2double((int)((uint32_t)(sh + 1023) << 20 | g.sign), 0), cv[j]);
-          } else {
-            v = g.sign ? cv[j] - scalbn(x, sh) : cv[j] + scalbn(x, sh);
-          }
-          cp[(int64_t)(j0 + j) * o.ldc] = v;
+          double x = i63_to_f64_scaled(V[j0 + j], base + ec);
+          x = __hiloint2double(__double2hiint(x) ^ (int)g.sign, __double2loint(x));
+          if (j0 + j <= last) cp[(int64_t)(j0 + j) * o.ldc] = cip ? cv[j] + x : x;
         }
       }
     }

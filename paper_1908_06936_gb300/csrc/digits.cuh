@@ -23,7 +23,7 @@ struct DigitOperand {
   int* sq = nullptr;
   int64_t rows = 0;    // rows of every plane (a multiple of 8)
 };
-constexpr int kDigBad = 0x7FFFFFFF;
+constexpr int kDigBad = 1 << 28;  // above any sum of exponents, below overflow
 
 // Bytes of an operand of `rows` x K with S digits, and its layout at `base` (256-byte aligned).
 size_t digit_bytes(int64_t rows, int K, int S);
