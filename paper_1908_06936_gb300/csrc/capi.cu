@@ -364,7 +364,7 @@ exa_status loglik_fp64(exa_ctx* c, const double* d_locs, const double* d_z, cons
   const int T = (int)(npad / nb);
   exa_status st;
   if ((st = ensure(c, c->mat, (size_t)npad * npad * sizeof(double), "matrix")) != EXA_OK) return st;
-  if ((st = ensure(c, c->vec, (size_t)3 * npad * sizeof(double), "vectors")) != EXA_OK) return st;
+  if ((st = ensure(c, c->vec, (size_t)(2 * npad + kSolveScratch) * sizeof(double), "vectors")) != EXA_OK) return st;
   if ((st = ensure(c, c->partial, (size_t)(kPartialDoubles(npad, nb)) * sizeof(double), "partials")) != EXA_OK)
     return st;
   if ((st = reset_status(c)) != EXA_OK) return st;
@@ -391,10 +391,7 @@ exa_status loglik_fp64(exa_ctx* c, const double* d_locs, const double* d_z, cons
     ProfScope ps(c, PK_OTHER, 0.0, 16.0 * (double)npad);
     e = launch_pad_vector(c->stream, d_z, n, npad, zw);
   }
-  for (int k = 0; k < T && e == cudaSuccess; ++k) {
-    ProfScope ps(c, PK_TRSV, 2.0 * (double)(npad - (int64_t)k * nb) * nb, 8.0 * (double)(npad - (int64_t)k * nb) * nb);
-    e = launch_trsv_fwd_step(c->stream, A, npad, npad, nb, k, (const double*)c->w_all.p, y, zw, c->d_status);
-  }
+  if (e == cudaSuccess) e = solve_forward(c, npad, nb, zw, y, tmp);
   if (e == cudaSuccess) {
     ProfScope ps(c, PK_OTHER, 0.0, 8.0 * (double)npad, 4);
     e = launch_sumsq(c->stream, y, npad, part, c->d_scalars + 0);

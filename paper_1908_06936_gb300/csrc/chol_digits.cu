@@ -32,6 +32,7 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
     size_t bytes;
   } want[] = {{&c->mx_w2, (size_t)kNB * kNB * sizeof(double)},
               {&c->mx_dscr, diag_block_scratch_doubles() * sizeof(double)},
+              {&c->mx_wall, (size_t)(npad / kNB) * kNB * kNB * sizeof(double)},
               {&c->mx_split, below ? align256(digit_bytes(below, kNB, kDigSlices)) : 0},
               {&c->mx_split_b, below ? 2 * block_bytes(kDigSlices) + block_bytes(kDigLow) : 0},
               {&c->mx_split2, below * kNB * sizeof(double)}};
@@ -61,8 +62,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
   *done = true;
   double* W = (double*)c->w_all.p;
   double* LD = (double*)c->logdet_part.p;
-  const bool keep = c->keep_block_inverses && c->mx_wall.bytes >= (size_t)(npad / kNB) * kNB * kNB * sizeof(double);
-  c->wall_kept = keep;
+  c->wall_kept = true;
   double* X = (double*)c->mx_split2.p;
   cudaStream_t ms = c->stream, ss = c->side;
   const int sms = tc_num_sms();
@@ -77,7 +77,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     const int64_t k0 = (int64_t)k * kNB;
     const int w = (int)std::min<int64_t>(kNB, npad - k0);
     const double w3 = (double)w * w * w;
-    double* W2 = keep && w == kNB ? (double*)c->mx_wall.p + k0 * kNB : (double*)c->mx_w2.p;
+    double* W2 = w == kNB ? (double*)c->mx_wall.p + k0 * kNB : (double*)c->mx_w2.p;
     cudaError_t e;
     {
       ProfScope ps(c, PK_POTRF, (w == kNB ? 2.0 : 1.0) * w3 / 3.0, 8.0 * (3.0 * w * w), 1, s, s != ms);
@@ -188,6 +188,45 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
   }
   if (e != cudaSuccess) return cuda_err(c, e, "Cholesky launch");
   return EXA_OK;
+}
+
+const double* block_inverse(exa_ctx* c, int64_t k0, int h) {
+  return h == kNB ? (const double*)c->mx_wall.p + k0 * kNB : (const double*)c->w_all.p + k0 * kSub;
+}
+
+cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y, double* tmp) {
+  const double* a = (const double*)c->mat.p;
+  cudaError_t e = cudaSuccess;
+  for (int64_t k0 = 0, h; k0 < npad && e == cudaSuccess; k0 += h) {
+    h = !c->wall_kept ? nb : npad - k0 >= kNB ? kNB : kSub;
+    const double rows = (double)(npad - k0);
+    ProfScope ps(c, PK_TRSV, 2.0 * rows * h, 8.0 * rows * h, c->wall_kept ? 3 + (npad - k0 > h) : 1);
+    if (c->wall_kept)
+      e = launch_block_fwd(c->stream, a + k0 + k0 * npad, npad, (int)h, npad - k0 - h, block_inverse(c, k0, (int)h),
+                           z + k0, y + k0, tmp);
+    else
+      e = launch_trsv_fwd_step(c->stream, a, npad, npad, nb, (int)(k0 / nb), (const double*)c->w_all.p, y, z,
+                               c->d_status);
+  }
+  return e;
+}
+
+cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y, double* tmp) {
+  const double* a = (const double*)c->mat.p;
+  const int64_t full = npad / kNB * kNB;  // the 128-wide blocks start here
+  cudaError_t e = cudaSuccess;
+  for (int64_t end = npad, h; end > 0 && e == cudaSuccess; end -= h) {
+    h = !c->wall_kept ? nb : end > full ? kSub : kNB;
+    const int64_t k0 = end - h;
+    const double rows = c->wall_kept ? (double)end : (double)(npad - k0);
+    ProfScope ps(c, PK_TRSV, 2.0 * rows * h, 8.0 * rows * h, c->wall_kept ? 3 + (k0 > 0) : 2);
+    if (c->wall_kept)
+      e = launch_block_bwd(c->stream, a + k0, npad, k0, (int)h, block_inverse(c, k0, (int)h), y, tmp);
+    else
+      e = launch_trsv_bwd_step(c->stream, a, npad, npad, nb, (int)(k0 / nb), (const double*)c->w_all.p, y,
+                               (double*)c->partial.p + 2 * kRedPartials, c->d_status);
+  }
+  return e;
 }
 
 void release_digits(exa_ctx* c) {

@@ -125,8 +125,15 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
 // be had, and those buffers are released.
 bool reserve_digits(exa_ctx* c, int64_t npad);
 void release_digits(exa_ctx* c);
+// y = L^-1 z (z overwritten) and y <- L^-T y with the FP64 factor in c->mat, by the block inverses its factorisation left
+// (of nb-wide tiles, or the digit path's); tmp: kSolveScratch doubles.
+constexpr int kSolveScratch = 1024;
+cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y, double* tmp);
+cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y, double* tmp);
+// The digit path's inverse of the h x h diagonal block at k0 (row-major).
+const double* block_inverse(exa_ctx* c, int64_t k0, int h);
 // Sigma^-1 on the tensor cores: room for it (allocate = false: whether it is held), and the inverse in the lower
-// triangle of c->mat from the factor there, whose block inverses were kept; x: npad^2 doubles of scratch.
+// triangle of c->mat from the factor there; x: npad^2 doubles of scratch.
 // rows: of the second operand where it has more than npad (prediction points).
 bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate = true, int64_t rows = 0);
 // Digits of the h x h diagonal block at k0 of the factor in c->mat (Dl) and of its inverse with column k scaled by row

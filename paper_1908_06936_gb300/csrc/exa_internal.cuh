@@ -184,6 +184,15 @@ cudaError_t launch_trsv_fwd_step(cudaStream_t s, const double* a, int64_t ld, in
 cudaError_t launch_trsv_bwd_step(cudaStream_t s, const double* a, int64_t ld, int64_t npad, int nb, int k,
                                  const double* w_all, double* y, double* tmp, const DevStatus* st);
 
+// One block step of either solve with the block's h x h inverse w (row-major, lower; h 128 or 512).  Forward, block at
+// lkk with `rest` rows below it: y <- L_kk^-1 z, then those rows of z (z[h ..]) -= L y; tmp: h doubles.  Backward, block
+// row at lrow (columns [0, k0 + h) of the factor's rows k0 ..): y[k0 ..] <- L_kk^-T y[k0 ..], then y[0, k0) -= L^T of
+// it; tmp: 2 h doubles.
+cudaError_t launch_block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int h, int64_t rest, const double* w,
+                             double* z, double* y, double* tmp);
+cudaError_t launch_block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, int h, const double* w,
+                             double* y, double* tmp);
+
 // Deterministic reductions: out[0] = sum(v[i]^2) ; out[0] = sum(v[i]) over n values.
 cudaError_t launch_sumsq(cudaStream_t s, const double* v, int64_t n, double* partial, double* out);
 cudaError_t launch_sum(cudaStream_t s, const double* v, int64_t n, double* partial, double* out);

@@ -744,7 +744,6 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   }
   const int nb = c->tile_nb;
   const int64_t npad = round_up(n, nb);
-  const int T = (int)(npad / nb);
   // Sigma^-1 in a second n x n buffer when it fits beside the factor; otherwise the
   // one-buffer form: X = L^-1 overwrites the factor and each tile of X^T X is formed and
   // reduced at once (lauum_grad_fused_kernel), so no second n x n buffer is needed.
@@ -778,22 +777,13 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   exa_result res;
   memset(&res, 0, sizeof(res));
   double* y = nullptr;
-  c->keep_block_inverses = nb == 128 && !one_buffer && reserve_inverse_digits(c, npad);
-  st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y);
-  c->keep_block_inverses = 0;
-  if (st != EXA_OK) return st;
+  if (nb == 128 && !one_buffer) reserve_inverse_digits(c, npad);
+  if ((st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y)) != EXA_OK) return st;
   *loglik = res.loglik;
   double* A = (double*)c->mat.p;
-  double* W = (double*)c->w_all.p;
-  double* part = (double*)c->partial.p;
   cudaStream_t s = c->stream;
-  cudaError_t e = cudaSuccess;
   // a = L^-T y (in place in y)
-  for (int k = T - 1; k >= 0 && e == cudaSuccess; --k) {
-    const double rows = (double)(npad - (int64_t)k * nb);
-    ProfScope ps(c, PK_TRSV, 2.0 * rows * nb, 8.0 * rows * nb, 2);
-    e = launch_trsv_bwd_step(s, A, npad, npad, nb, k, W, y, part + 2 * kRedPartials, c->d_status);
-  }
+  cudaError_t e = solve_backward(c, npad, nb, y, y + npad);
   const bool digits = !one_buffer && c->wall_kept && reserve_inverse_digits(c, npad, false);
   if (!digits && (st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   if (!one_buffer) {
@@ -946,10 +936,8 @@ extern "C" exa_status exa_fisher(exa_ctx* c, const double* d_locs, const double 
     e = launch_matern_gen(s, d_locs, n, npad, P, A, npad, nullptr, tab);
   }
   if (e != cudaSuccess) return cuda_err(c, e, "generation launch");
-  c->keep_block_inverses = nb == 128 && reserve_inverse_digits(c, npad);
-  st = factor_fp64(c, A, npad, npad, nb);
-  c->keep_block_inverses = 0;
-  if (st != EXA_OK) return st;
+  if (nb == 128) reserve_inverse_digits(c, npad);
+  if ((st = factor_fp64(c, A, npad, npad, nb)) != EXA_OK) return st;
   if ((st = read_status(c)) != EXA_OK) return st;
   const bool digits = c->wall_kept && reserve_inverse_digits(c, npad, false);
   if (digits) {

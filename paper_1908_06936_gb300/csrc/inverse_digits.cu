@@ -23,8 +23,7 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t row
   struct {
     DevBuf* b;
     size_t bytes;
-  } want[] = {{&c->mx_wall, (size_t)(npad / kNB) * kNB * kNB * sizeof(double)},
-              {&c->mx_split, digit_bytes(npad, kNB, kDigSlices)},
+  } want[] = {{&c->mx_split, digit_bytes(npad, kNB, kDigSlices)},
               {&c->mx_split2, digit_bytes(rows, kNB, kDigSlices)},
               {&c->mx_split_b, 2 * align256(digit_bytes(kNB, kNB, kDigSlices))}};
   if (!allocate) {
@@ -42,7 +41,7 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t row
 
 cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl) {
   const double* a = (const double*)c->mat.p + k0 + k0 * npad;
-  const double* w = h == kNB ? (const double*)c->mx_wall.p + k0 * kNB : (const double*)c->w_all.p + k0 * kSub;
+  const double* w = block_inverse(c, k0, h);
   digit_layout(Dl, c->mx_split_b.p, h, h, kDigSlices);
   digit_layout(Dw, (uint8_t*)c->mx_split_b.p + align256(digit_bytes(kNB, kNB, kDigSlices)), h, h, kDigSlices);
   cudaError_t e = launch_digit_split(c->stream, a, 1, npad, h, h, kDigSlices, Dl, 0, true);
@@ -67,7 +66,7 @@ cudaError_t inverse_digits(exa_ctx* c, int64_t npad, double* x) {
   for (int64_t l0 = 0, h; l0 < npad && e == cudaSuccess; l0 += h) {
     h = npad - l0 >= kNB ? kNB : kSub;
     const int64_t n1 = l0 + h, m = npad - n1;
-    const double* w = h == kNB ? (const double*)c->mx_wall.p + l0 * kNB : (const double*)c->w_all.p + l0 * kSub;
+    const double* w = block_inverse(c, l0, (int)h);
     const double dh = (double)h;
     DigitOperand Dl, Dw, D, Dx;
     digit_layout(Dx, c->mx_split2.p, n1, (int)h, kDigSlices);

@@ -203,25 +203,16 @@ extern "C" exa_status exa_predict(exa_ctx* c, const double* d_locs, const double
   double* y = nullptr;
   const int nb = c->tile_nb;
   const int64_t npad = round_up(n, nb);
-  // new points per block of the variance's products on the tensor cores; what they need is asked for before the
-  // factorisation, which then keeps its block inverses
+  // new points per block of the variance's products on the tensor cores
   const int64_t mc = std::min<int64_t>(round_up(m, 64), kPredColsDig);
-  c->keep_block_inverses = d_var && nb == 128 && reserve_inverse_digits(c, npad, true, mc);
-  st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y);
-  c->keep_block_inverses = 0;
-  if (st != EXA_OK) return st;
+  if (d_var && nb == 128) reserve_inverse_digits(c, npad, true, mc);
+  if ((st = loglik_fp64(c, d_locs, d_z, theta, n, &res, &y)) != EXA_OK) return st;
   const int T = (int)(npad / nb);
   double* A = (double*)c->mat.p;
   const double* W = (const double*)c->w_all.p;
-  double* part = (double*)c->partial.p;
   cudaStream_t s = c->stream;
-  cudaError_t e = cudaSuccess;
   // a = L^-T y (in place)
-  for (int k = T - 1; k >= 0 && e == cudaSuccess; --k) {
-    const double rows = (double)(npad - (int64_t)k * nb);
-    ProfScope ps(c, PK_TRSV, 2.0 * rows * nb, 8.0 * rows * nb, 2);
-    e = launch_trsv_bwd_step(s, A, npad, npad, nb, k, W, y, part + 2 * kRedPartials, c->d_status);
-  }
+  cudaError_t e = solve_backward(c, npad, nb, y, y + npad);
   if (e != cudaSuccess) return cuda_err(c, e, "prediction solve");
   MaternParams P;
   model_params(c, theta, &P);

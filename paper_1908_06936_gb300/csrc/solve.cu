@@ -638,3 +638,103 @@ cudaError_t launch_llt_solve_persistent(cudaStream_t s, const double* a, int64_t
 }
 
 }  // namespace exa
+
+namespace exa {
+
+// ---------------------------------------------------------------------------
+// Block solves of the FP64 factor with the inverses of its 512-wide diagonal blocks (128-wide at the end): per block
+// three products with the block (y = W z, r = z - L_kk y, y += W r: an explicit inverse alone would leave cond(L_kk)
+// rounding errors) and one with the panel, each spread over the GPU.  A 128-row step with one launch each (above) was
+// one CTA's work and ~48 us: 4.7 ms of an n = 12,300 evaluation, 13 ms of a prediction at n = 10,000.
+// All sums in a fixed order.
+// ---------------------------------------------------------------------------
+
+// out[r] = add[r] + sum_{t <= r} W(r, t) v[t], W row-major h x h: a warp per row.
+__global__ void __launch_bounds__(256) block_lower_kernel(const double* __restrict__ W, int h,
+                                                          const double* __restrict__ v, const double* __restrict__ add,
+                                                          double* __restrict__ out) {
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (r >= h) return;
+  double s = 0.0;
+#pragma unroll 4
+  for (int t = lane; t <= r; t += 32) s = fma(W[(int64_t)r * h + t], v[t], s);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[r] = add ? add[r] + s : s;
+}
+
+// out[t] = add[t] + sum_{u >= t} W(u, t) v[u]: 32 columns a CTA, the rows split over its warps.
+__global__ void __launch_bounds__(256) block_lower_t_kernel(const double* __restrict__ W, int h,
+                                                            const double* __restrict__ v,
+                                                            const double* __restrict__ add, double* __restrict__ out) {
+  __shared__ double part[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = blockIdx.x * 32 + lane, per = h / 8;
+  double s = 0.0;
+#pragma unroll 8
+  for (int u = warp * per; u < warp * per + per; ++u) s = fma(u >= t ? W[(int64_t)u * h + t] : 0.0, v[u], s);
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w][lane];
+    out[t] = add ? add[t] + s : s;
+  }
+}
+
+// out[r] = z[r] - sum_{t < h} L(r, t) y[t] (lower: t <= r), L column-major: 32 rows a CTA, the columns split over its
+// warps, every load of a column 256 bytes.
+__global__ void __launch_bounds__(256) block_rows_kernel(const double* __restrict__ L, int64_t ld, int h, int lower,
+                                                         const double* __restrict__ y, const double* __restrict__ z,
+                                                         double* __restrict__ out) {
+  __shared__ double part[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, per = h / 8;
+  const int64_t r = (int64_t)blockIdx.x * 32 + lane;
+  double s = 0.0;
+#pragma unroll 16
+  for (int t = warp * per; t < warp * per + per; ++t) s = fma(!lower || t <= r ? L[r + t * ld] : 0.0, y[t], s);
+  part[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w][lane];
+    out[r] = z[r] - s;
+  }
+}
+
+// out[c] = z[c] - sum_{r < h} L(r, c) x[r] (lower: r >= c), L column-major: a warp per column.
+__global__ void __launch_bounds__(256) block_cols_kernel(const double* __restrict__ L, int64_t ld, int64_t ncols, int h,
+                                                         int lower, const double* __restrict__ x,
+                                                         const double* __restrict__ z, double* __restrict__ out) {
+  const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (c >= ncols) return;
+  double s = 0.0;
+#pragma unroll 4
+  for (int r = lane; r < h; r += 32) s = fma(!lower || r >= c ? L[r + c * ld] : 0.0, x[r], s);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[c] = z[c] - s;
+}
+
+cudaError_t launch_block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int h, int64_t rest, const double* w,
+                             double* z, double* y, double* tmp) {
+  block_lower_kernel<<<h / 8, 256, 0, s>>>(w, h, z, nullptr, y);
+  block_rows_kernel<<<h / 32, 256, 0, s>>>(lkk, ld, h, 1, y, z, tmp);
+  block_lower_kernel<<<h / 8, 256, 0, s>>>(w, h, tmp, y, y);
+  if (rest > 0) block_rows_kernel<<<(unsigned)(rest / 32), 256, 0, s>>>(lkk + h, ld, h, 0, y, z + h, z + h);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, int h, const double* w,
+                             double* y, double* tmp) {
+  const double* lkk = lrow + k0 * ld;
+  double* v = y + k0;
+  double* x = tmp + h;
+  block_lower_t_kernel<<<h / 32, 256, 0, s>>>(w, h, v, nullptr, x);
+  block_cols_kernel<<<h / 8, 256, 0, s>>>(lkk, ld, h, h, 1, x, v, tmp);
+  block_lower_t_kernel<<<h / 32, 256, 0, s>>>(w, h, tmp, x, v);
+  if (k0 > 0) block_cols_kernel<<<(unsigned)(k0 / 8), 256, 0, s>>>(lrow, ld, k0, h, 0, v, y, y);
+  return cudaGetLastError();
+}
+
+}  // namespace exa
