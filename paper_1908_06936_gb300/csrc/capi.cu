@@ -42,14 +42,33 @@ exa_status ensure_side(exa_ctx* c) {
   return EXA_OK;
 }
 
+static void free_buf(exa_ctx* c, DevBuf& b) {
+  if (b.p) cudaFree(b.p);
+  c->held_bytes -= b.bytes;
+  b.p = nullptr;
+  b.bytes = 0;
+}
+
+// Gives up what its owner does without; false: nothing is held of that kind.
+static bool release_spare(exa_ctx* c) {
+  if (c->digits_held) {
+    release_digits(c);
+  } else if (c->wall_spare) {
+    cudaStreamSynchronize(c->stream);
+    free_buf(c, c->mx_wall);
+    c->wall_spare = c->wall_kept = false;
+  } else {
+    return false;
+  }
+  return true;
+}
+
 // Grow-only device buffer with the context's memory bound enforced.
-// `optional`: the caller does without.  A request that is not optional and cannot be met otherwise takes the digit
-// operands' memory back.
+// `optional`: the caller does without.  A request that is not optional and cannot be met otherwise takes the memory of
+// optional ones back.
 exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool optional) {
   if (bytes <= b.bytes) return EXA_OK;
-  if (!optional && c->digits_held && c->ws_limit && c->held_bytes - b.bytes + bytes > c->ws_limit) {
-    release_digits(c);
-  }
+  if (!optional && c->ws_limit && c->held_bytes - b.bytes + bytes > c->ws_limit) release_spare(c);
   const size_t held = c->held_bytes - b.bytes;
   if (c->ws_limit && held + bytes > c->ws_limit)
     return set_err(c, EXA_ERR_NOMEM, "workspace %s needs %zu bytes; context bound is %zu (held %zu)", name, bytes,
@@ -63,9 +82,8 @@ exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool op
   }
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess && !optional && c->digits_held) {
+  if (e != cudaSuccess && !optional && release_spare(c)) {
     cudaGetLastError();
-    release_digits(c);
     e = cudaMalloc(&p, bytes);
   }
   if (e != cudaSuccess) {
@@ -76,13 +94,6 @@ exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool op
   b.bytes = bytes;
   c->held_bytes += bytes;
   return EXA_OK;
-}
-
-static void free_buf(exa_ctx* c, DevBuf& b) {
-  if (b.p) cudaFree(b.p);
-  c->held_bytes -= b.bytes;
-  b.p = nullptr;
-  b.bytes = 0;
 }
 
 exa_status check_theta(exa_ctx* c, const double theta[3]) {

@@ -237,8 +237,7 @@ void release_digits(exa_ctx* c) {
     b->p = nullptr;
     b->bytes = 0;
   }
-  c->digits_held = false;
-  c->wall_kept = false;
+  c->digits_held = c->wall_spare = c->wall_kept = false;
 }
 
 }  // namespace exa

@@ -57,13 +57,14 @@ struct exa_ctx {
   exa::DevBuf mx_split4;
   exa::DevBuf mx_split_b;   // split-precision operands (B role: inverse diagonal block / test B)
   exa::SplitOperand sp_a, sp_a2, sp_a3, sp_a4, sp_b;
-  bool wall_kept = false;   // the last FP64 factorisation left its 512-wide block inverses in mx_wall
+  bool wall_kept = false;   // the last factorisation left its 512-wide block inverses in mx_wall
+  bool wall_spare = false;  // mx_wall is between two mixed evaluations, which do without it
   bool digits_held = false; // the buffers of reserve_digits are the FP64 path's: given up for requests that need the room
   exa::DevBuf mx_vec;       // refinement vectors
   exa::DevBuf mx_w2;        // inverse of the panel-wide diagonal block (row-major)
   exa::DevBuf mx_wall;      // every panel's diagonal-block inverse, T x 512 x 512 (kept for the gradient)
   exa::DevBuf mx_dscr;      // scratch of the cooperative diagonal-block factorisation
-  int keep_block_inverses = 0;  // mixed factorisation: write block k's inverse to mx_wall + k 512^2
+  int keep_block_inverses = 0;  // mixed factorisation: write block k's inverse to mx_wall + k 512^2 (2: if there is room)
   int ir_tight = 0;         // mixed refinement: iterate to rounding level (the gradient needs Sigma^-1 z)
   double ir_target = 0.0;   // mixed refinement: relative residual to reach (0: quadratic-form rule)
   double ir_quad_tol = 0.0; // mixed refinement: relative accuracy of q (0: the default)

@@ -97,7 +97,7 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   double* W = (double*)c->w_all.p;
   double* LD = (double*)c->logdet_part.p;
   // NB x NB inverse of the diagonal block (row-major); every block's is kept when asked
-  double* W2 = c->keep_block_inverses ? (double*)c->mx_wall.p + (size_t)k * kMixNB * kMixNB : (double*)c->mx_w2.p;
+  double* W2 = c->wall_kept ? (double*)c->mx_wall.p + (size_t)k * kMixNB * kMixNB : (double*)c->mx_w2.p;
   const int64_t k0 = (int64_t)k * NB;
   cudaError_t e = cudaSuccess;
   // 1. FP64 Cholesky of the diagonal block, its 128 sub-tile inverses and log sums, and
@@ -324,6 +324,7 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   // the fused phase runs while rows (k + 4) NB .. npad number at least fuse_rows, from k = 0
   const bool fuse = fuse_rows > 0 && c->tc_pairs && T >= 4 && npad - 4 * (int64_t)NB >= fuse_rows;
   c->digits_held = false;
+  c->wall_spare = c->wall_kept = false;
   SplitOperand* buf[4] = {&c->sp_a, &c->sp_a2, &c->sp_a3, &c->sp_a4};
   DevBuf* mem[4] = {&c->mx_split, &c->mx_split2, &c->mx_split3, &c->mx_split4};
   for (int i = 0; i < (fuse ? 4 : 2); ++i)
@@ -333,10 +334,13 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   if ((st = ensure(c, c->mx_w2, (size_t)NB * NB * sizeof(double), "diagonal block inverse")) != EXA_OK) return st;
   if ((st = ensure(c, c->mx_dscr, diag_block_scratch_doubles() * sizeof(double), "diagonal block scratch")) != EXA_OK)
     return st;
-  if (c->keep_block_inverses &&
-      (st = ensure(c, c->mx_wall, (size_t)T * NB * NB * sizeof(double), "diagonal block inverses")) != EXA_OK)
-    return st;
   if ((st = ensure_side(c)) != EXA_OK) return st;
+  if (c->keep_block_inverses) {  // last: 2 is a wish
+    st = ensure(c, c->mx_wall, (size_t)T * NB * NB * sizeof(double), "diagonal block inverses", true);
+    if (st != EXA_OK && c->keep_block_inverses == 1) return st;
+    c->wall_kept = st == EXA_OK;
+    c->err[0] = 0;
+  }
   MixStep M{c, a, ld, npad, band, T, far_thr};
   cudaStream_t ms = c->stream, ss = c->side;
   const int sms = tc_num_sms();
@@ -395,13 +399,17 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   return EXA_OK;
 }
 
-// x = (L L^T)^-1 rhs with the FP64-stored factor, on 128-wide tiles with the
-// stored inverses of the diagonal sub-tiles.
-// x = (L L^T)^-1 rhs; the upper tiles of a hold L^T.  flags: scratch for the solves' flags.
+// x = (L L^T)^-1 rhs with the FP64-stored factor: in 512-row block steps where the factorisation kept the block
+// inverses, else on 128-wide tiles with the sub-tile inverses (the upper tiles of a then hold L^T).  flags: scratch for
+// the persistent solves' flags; tmp: kSolveScratch doubles.
 static cudaError_t solve_llt(exa_ctx* c, const double* a, int64_t ld, int64_t npad, const double* rhs, double* x,
-                             double* work, int* flags) {
+                             double* work, int* flags, double* tmp) {
   cudaError_t e = cudaMemcpyAsync(work, rhs, npad * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
   if (e != cudaSuccess) return e;
+  if (c->wall_kept) {
+    e = solve_forward(c, npad, kMixSub, work, x, tmp);
+    return e == cudaSuccess ? solve_backward(c, npad, kMixSub, x, tmp) : e;
+  }
   ProfScope ps(c, PK_TRSV, 2.0 * (double)npad * (double)npad, 8.0 * (double)npad * (double)npad, 2);
   return launch_llt_solve_persistent(c->stream, a, ld, npad, (const double*)c->w_all.p, work, x, flags,
                                      c->d_status);
@@ -489,8 +497,12 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
   exa_status st;
   if ((st = ensure(c, c->mx_sigma, (size_t)npad * npad * sizeof(double), "FP64 covariance copy")) != EXA_OK)
     return st;
-  if ((st = ensure(c, c->mx_vec, (size_t)6 * npad * sizeof(double), "refinement vectors")) != EXA_OK) return st;
+  if ((st = ensure(c, c->mx_vec, (size_t)(6 * npad + kSolveScratch) * sizeof(double), "refinement vectors")) != EXA_OK)
+    return st;
   if ((st = ensure(c, c->partial, (size_t)(2 * kRedPartials + 2 * npad + 64) * sizeof(double), "partials")) != EXA_OK)
+    return st;
+  if ((st = ensure(c, c->mx_symv, (size_t)symv_tiled_partials(npad) * sizeof(double), "symmetric product partials")) !=
+      EXA_OK)
     return st;
   if ((st = reset_status(c)) != EXA_OK) return st;
   double* S = (double*)c->mx_sigma.p;
@@ -500,32 +512,36 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
   double* d = r + npad;
   double* y = d + npad;
   double* work = y + npad;
+  double* tmp = work + npad;
   double* part = (double*)c->partial.p;
   double* red = part + 2 * kRedPartials;  // the solves' flags live after the reduction partials
   cudaStream_t s = c->stream;
   cudaEventRecord(c->ev[0], s);
   int band = 0;
-  if ((st = mixed_generate_factor(c, d_locs, n, theta, npad, prec, S, &band)) != EXA_OK) return st;
+  // the solves below run four times faster with the block inverses; the gradient needs them in any case
+  const int keep = c->keep_block_inverses;
+  if (!keep) c->keep_block_inverses = 2;
+  st = mixed_generate_factor(c, d_locs, n, theta, npad, prec, S, &band);
+  c->keep_block_inverses = keep;
+  c->wall_spare = !keep && c->wall_kept;
+  if (st != EXA_OK) return st;
   cudaEventRecord(c->ev[2], s);
   cudaError_t e;
   e = launch_sum(s, (const double*)c->logdet_part.p, T128, part, c->d_scalars + 1);
   if (e == cudaSuccess) e = launch_pad_vector(s, d_z, n, npad, zp);
   if (e == cudaSuccess) e = launch_sumsq(s, zp, npad, part, c->d_scalars + 2);
   double* A = (double*)c->mat.p;
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && !c->wall_kept) {
     // L^T into the unused upper triangle: the backward solves stream contiguous columns
     ProfScope ps(c, PK_OTHER, 0.0, 8.0 * (double)npad * (double)npad);
     e = launch_transpose_lower_to_upper(s, A, npad, npad);
   }
-  if (e == cudaSuccess) e = solve_llt(c, A, npad, npad, zp, x, work, (int*)red);
+  if (e == cudaSuccess) e = solve_llt(c, A, npad, npad, zp, x, work, (int*)red, tmp);
   if (e != cudaSuccess) return cuda_err(c, e, "solve launch");
   // iterative refinement of x = Sigma^-1 z with the FP64 residual.  It stops when the
   // residual no longer halves or reaches rounding level, or once the quadratic form is final
   // to kIrQuadTol relative: a correction d changes z^T x by less than that, or the
   // second-order term r^T d of the variational estimate is below it (q is then that estimate).
-  if ((st = ensure(c, c->mx_symv, (size_t)symv_tiled_partials(npad) * sizeof(double), "symmetric product partials")) !=
-      EXA_OK)
-    return st;
   double* sp = (double*)c->mx_symv.p;
   double rel = 0.0, prev = 1e300;
   double rel_prev = 1.0;  // ||r|| / ||z|| of the step before (the residual of x = 0 is z itself)
@@ -558,7 +574,7 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
     rel_prev = rel;
     if (!(rel > (target > 0.0 ? target : 1e-15)) || it >= kMaxIt || rel > 0.5 * prev) break;
     prev = rel;
-    e = solve_llt(c, A, npad, npad, r, d, work, (int*)red);
+    e = solve_llt(c, A, npad, npad, r, d, work, (int*)red, tmp);
     // the variational estimate of q before x moves: with r = z - Sigma x and d = (L L^T)^-1 r,
     // q = z^T x + x^T r + r^T Sigma^-1 r, so q_hat = z^T x + x^T r + r^T d is off by
     // r^T (Sigma^-1 - (L L^T)^-1) r, second order in the residual (about the contraction

@@ -649,92 +649,160 @@ namespace exa {
 // All sums in a fixed order.
 // ---------------------------------------------------------------------------
 
-// out[r] = add[r] + sum_{t <= r} W(r, t) v[t], W row-major h x h: a warp per row.
-__global__ void __launch_bounds__(256) block_lower_kernel(const double* __restrict__ W, int h,
-                                                          const double* __restrict__ v, const double* __restrict__ add,
-                                                          double* __restrict__ out) {
+// All loads of a thread are issued before its first multiply-add (masked ones count as 0): in a loop with a bound of
+// its own each waited for the one before, 12 us a kernel.
+
+// out[r] = add[r] + sum_{t <= r} W(r, t) v[t], W row-major H x H: a warp per row.
+template <int H>
+__global__ void __launch_bounds__(256) block_lower_kernel(const double* __restrict__ W, const double* __restrict__ v,
+                                                          const double* __restrict__ add, double* __restrict__ out) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= h) return;
+  double w[H / 32], x[H / 32];
+#pragma unroll
+  for (int i = 0; i < H / 32; ++i) {
+    const int t = lane + 32 * i;
+    w[i] = t <= r ? W[(int64_t)r * H + t] : 0.0;
+    x[i] = v[t];
+  }
   double s = 0.0;
-#pragma unroll 4
-  for (int t = lane; t <= r; t += 32) s = fma(W[(int64_t)r * h + t], v[t], s);
+#pragma unroll
+  for (int i = 0; i < H / 32; ++i) s = fma(w[i], x[i], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) out[r] = add ? add[r] + s : s;
 }
 
-// out[t] = add[t] + sum_{u >= t} W(u, t) v[u]: 32 columns a CTA, the rows split over its warps.
-__global__ void __launch_bounds__(256) block_lower_t_kernel(const double* __restrict__ W, int h,
-                                                            const double* __restrict__ v,
-                                                            const double* __restrict__ add, double* __restrict__ out) {
-  __shared__ double part[8][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, t = blockIdx.x * 32 + lane, per = h / 8;
-  double s = 0.0;
-#pragma unroll 8
-  for (int u = warp * per; u < warp * per + per; ++u) s = fma(u >= t ? W[(int64_t)u * h + t] : 0.0, v[u], s);
-  part[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int w = 1; w < 8; ++w) s += part[w][lane];
-    out[t] = add ? add[t] + s : s;
+// Sum of v over the CTA's 256 / R threads with the same tid mod R (R = 8, 32 or 128), on thread tid < R; fixed order.
+template <int R>
+__device__ __forceinline__ double sum_over_groups(double v) {
+  constexpr int NP = R == 128 ? 2 : 8;  // partials per value after the shuffles
+  __shared__ double part[NP][R];
+  const int tid = threadIdx.x;
+  if constexpr (R == 8) {
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if ((tid & 31) < 8) part[tid >> 5][tid & 7] = v;
+  } else {
+    part[tid / R][tid % R] = v;
   }
+  __syncthreads();
+  if (tid >= R) return 0.0;
+  double s = part[0][tid];
+#pragma unroll
+  for (int w = 1; w < NP; ++w) s += part[w][tid];
+  return s;
 }
 
-// out[r] = z[r] - sum_{t < h} L(r, t) y[t] (lower: t <= r), L column-major: 32 rows a CTA, the columns split over its
-// warps, every load of a column 256 bytes.
-__global__ void __launch_bounds__(256) block_rows_kernel(const double* __restrict__ L, int64_t ld, int h, int lower,
+// out[t] = add[t] + sum_{u >= t} W(u, t) v[u], W row-major H x H: eight columns a CTA, the rows split 32 ways (32
+// columns a CTA would be 4 us of one SM's FP64 pipe).
+template <int H>
+__global__ void __launch_bounds__(256) block_lower_t_kernel(const double* __restrict__ W, const double* __restrict__ v,
+                                                            const double* __restrict__ add, double* __restrict__ out) {
+  constexpr int N = H / 32;
+  const int t = blockIdx.x * 8 + (threadIdx.x & 7), u0 = (threadIdx.x >> 3) * N;
+  double w[N], x[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    w[i] = u0 + i >= t ? W[(int64_t)(u0 + i) * H + t] : 0.0;
+    x[i] = v[u0 + i];
+  }
+  double s = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) s = fma(w[i], x[i], s);
+  s = sum_over_groups<8>(s);
+  if (threadIdx.x < 8) out[t] = add ? add[t] + s : s;
+}
+
+// out[r] = z[r] - sum_{t < H} L(r, t) y[t] (lower: t <= r), L column-major, R rows a CTA, the columns split 256 / R
+// ways: 8 rows where there are too few for the GPU's FP64 pipes otherwise, 128 (1 KB of every column) for long panels.
+template <int H, int R>
+__global__ void __launch_bounds__(256) block_rows_kernel(const double* __restrict__ L, int64_t ld, int lower,
                                                          const double* __restrict__ y, const double* __restrict__ z,
                                                          double* __restrict__ out) {
-  __shared__ double part[8][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, per = h / 8;
-  const int64_t r = (int64_t)blockIdx.x * 32 + lane;
+  constexpr int per = H * R / 256, N = per < 16 ? per : 16;
+  const int64_t r = (int64_t)blockIdx.x * R + threadIdx.x % R;
+  const int t0 = (threadIdx.x / R) * per;
   double s = 0.0;
-#pragma unroll 16
-  for (int t = warp * per; t < warp * per + per; ++t) s = fma(!lower || t <= r ? L[r + t * ld] : 0.0, y[t], s);
-  part[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0) {
+#pragma unroll 1
+  for (int c = 0; c < per; c += N) {
+    double l[N], x[N];
 #pragma unroll
-    for (int w = 1; w < 8; ++w) s += part[w][lane];
-    out[r] = z[r] - s;
+    for (int i = 0; i < N; ++i) {
+      const int t = t0 + c + i;
+      l[i] = !lower || t <= r ? L[r + t * ld] : 0.0;
+      x[i] = y[t];
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) s = fma(l[i], x[i], s);
   }
+  s = sum_over_groups<R>(s);
+  if (threadIdx.x < R) out[r] = z[r] - s;
 }
 
-// out[c] = z[c] - sum_{r < h} L(r, c) x[r] (lower: r >= c), L column-major: a warp per column.
-__global__ void __launch_bounds__(256) block_cols_kernel(const double* __restrict__ L, int64_t ld, int64_t ncols, int h,
-                                                         int lower, const double* __restrict__ x,
-                                                         const double* __restrict__ z, double* __restrict__ out) {
+// out[c] = z[c] - sum_{r < H} L(r, c) x[r] (lower: r >= c), L column-major: a warp per column.
+template <int H>
+__global__ void __launch_bounds__(256) block_cols_kernel(const double* __restrict__ L, int64_t ld, int lower,
+                                                         const double* __restrict__ x, const double* __restrict__ z,
+                                                         double* __restrict__ out) {
   const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (c >= ncols) return;
+  double l[H / 32], v[H / 32];
+#pragma unroll
+  for (int i = 0; i < H / 32; ++i) {
+    const int r = lane + 32 * i;
+    l[i] = !lower || r >= c ? L[r + c * ld] : 0.0;
+    v[i] = x[r];
+  }
   double s = 0.0;
-#pragma unroll 4
-  for (int r = lane; r < h; r += 32) s = fma(!lower || r >= c ? L[r + c * ld] : 0.0, x[r], s);
+#pragma unroll
+  for (int i = 0; i < H / 32; ++i) s = fma(l[i], v[i], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) out[c] = z[c] - s;
 }
 
+template <int H>
+static cudaError_t block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int64_t rest, const double* w, double* z,
+                             double* y, double* tmp) {
+  block_lower_kernel<H><<<H / 8, 256, 0, s>>>(w, z, nullptr, y);
+  block_rows_kernel<H, 8><<<H / 8, 256, 0, s>>>(lkk, ld, 1, y, z, tmp);
+  block_lower_kernel<H><<<H / 8, 256, 0, s>>>(w, tmp, y, y);
+  const double* l = lkk + H;
+  double* zr = z + H;
+  if (rest >= 32768)  // more than one 128-row CTA per SM
+    block_rows_kernel<H, 128><<<(unsigned)(rest / 128), 256, 0, s>>>(l, ld, 0, y, zr, zr);
+  else if (rest >= 4864)  // one 32-row CTA per SM
+    block_rows_kernel<H, 32><<<(unsigned)(rest / 32), 256, 0, s>>>(l, ld, 0, y, zr, zr);
+  else if (rest > 0)
+    block_rows_kernel<H, 8><<<(unsigned)(rest / 8), 256, 0, s>>>(l, ld, 0, y, zr, zr);
+  return cudaGetLastError();
+}
+
+template <int H>
+static cudaError_t block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, const double* w, double* y,
+                             double* tmp) {
+  const double* lkk = lrow + k0 * ld;
+  double* v = y + k0;
+  double* x = tmp + H;
+  block_lower_t_kernel<H><<<H / 8, 256, 0, s>>>(w, v, nullptr, x);
+  block_cols_kernel<H><<<H / 8, 256, 0, s>>>(lkk, ld, 1, x, v, tmp);
+  block_lower_t_kernel<H><<<H / 8, 256, 0, s>>>(w, tmp, x, v);
+  if (k0 > 0) block_cols_kernel<H><<<(unsigned)(k0 / 8), 256, 0, s>>>(lrow, ld, 0, v, y, y);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int h, int64_t rest, const double* w,
                              double* z, double* y, double* tmp) {
-  block_lower_kernel<<<h / 8, 256, 0, s>>>(w, h, z, nullptr, y);
-  block_rows_kernel<<<h / 32, 256, 0, s>>>(lkk, ld, h, 1, y, z, tmp);
-  block_lower_kernel<<<h / 8, 256, 0, s>>>(w, h, tmp, y, y);
-  if (rest > 0) block_rows_kernel<<<(unsigned)(rest / 32), 256, 0, s>>>(lkk + h, ld, h, 0, y, z + h, z + h);
-  return cudaGetLastError();
+  if (h == 512) return block_fwd<512>(s, lkk, ld, rest, w, z, y, tmp);
+  if (h == 128) return block_fwd<128>(s, lkk, ld, rest, w, z, y, tmp);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, int h, const double* w,
                              double* y, double* tmp) {
-  const double* lkk = lrow + k0 * ld;
-  double* v = y + k0;
-  double* x = tmp + h;
-  block_lower_t_kernel<<<h / 32, 256, 0, s>>>(w, h, v, nullptr, x);
-  block_cols_kernel<<<h / 8, 256, 0, s>>>(lkk, ld, h, h, 1, x, v, tmp);
-  block_lower_t_kernel<<<h / 32, 256, 0, s>>>(w, h, tmp, x, v);
-  if (k0 > 0) block_cols_kernel<<<(unsigned)(k0 / 8), 256, 0, s>>>(lrow, ld, k0, h, 0, v, y, y);
-  return cudaGetLastError();
+  if (h == 512) return block_bwd<512>(s, lrow, ld, k0, w, y, tmp);
+  if (h == 128) return block_bwd<128>(s, lrow, ld, k0, w, y, tmp);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace exa
