@@ -1642,7 +1642,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     const DigStep& stp = P.steps[k];
     {
       ProfScope ps(c, PK_POTRF, (double)stp.ndiag * NB * NB * NB * 2.0 / 3.0, 0.0, 1);
-      e = launch_potrf128_tasks(s, dDiag + stp.diag_off, stp.ndiag);
+      e = launch_diag128_tasks(s, dDiag + stp.diag_off, stp.ndiag);
     }
     if (e != cudaSuccess || stp.nset == 0) continue;
     const DigitSplitTask* spl = dSpl + 2 * stp.set_off;

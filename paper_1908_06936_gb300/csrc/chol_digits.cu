@@ -48,6 +48,25 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
   return ok;
 }
 
+// Grids of the diagonal block and what it takes on them (512 rows, measured): beyond 104 CTAs nothing is gained.
+constexpr struct { int ctas; double us; } kDiagGrids[] = {{104, 426.0}, {64, 464.0}, {32, 698.0}, {16, 1180.0}};
+
+// The look-ahead stream's share of the GPU beside a trailing update of m rows (m^2 512 operations at 42 TFLOP/s on the
+// whole GPU): the grid with which the later of the two ends first.
+static int side_share(int64_t m, int sms) {
+  const double update_us = (double)m * (double)m * kNB / 42e6;
+  int best = kDiagGrids[0].ctas;
+  double best_us = 0.0;
+  for (const auto& g : kDiagGrids) {
+    const double us = std::max(g.us, update_us * sms / (sms - g.ctas));
+    if (best_us == 0.0 || us < best_us) {
+      best_us = us;
+      best = g.ctas;
+    }
+  }
+  return best;
+}
+
 // The factorisation of `a` (npad a multiple of 128).  *done = false: the workspace could not be had and nothing was
 // launched.
 exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* done) {
@@ -92,7 +111,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     }
     return e;
   };
-  cudaError_t e = diagonal(ms, 0, kDiagCtas);
+  cudaError_t e = diagonal(ms, 0, kDiagGrids[0].ctas);
   for (int k = 0; k + 1 < T && e == cudaSuccess; ++k) {
     const int64_t k0 = (int64_t)k * kNB, r0 = k0 + kNB, m = npad - r0;
     const double dm = (double)m;
@@ -173,9 +192,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     if (e != cudaSuccess) break;
     cudaEventRecord(c->la_ev[0], ms);
     cudaStreamWaitEvent(ss, c->la_ev[0], 0);
-    // The look-ahead stream's share of the GPU: the diagonal block takes ~1.4 ms on 32 to 64 SMs whatever the
-    // matrix, the trailing update ~m^2 512 / 42 TFLOP/s, so a long update gives up few of them.
-    const int side = m > kDigLateRows ? kDigSideSMs : kDiagCtas;
+    const int side = side_share(m, sms);
     e = diagonal(ss, k + 1, side);
     cudaEventRecord(c->la_ev[1], ss);
     if (e == cudaSuccess && m > w1) {

@@ -342,34 +342,6 @@ __global__ void __launch_bounds__(256) potrf_inv128_tasks_kernel(const DiagTileT
     }
     __syncthreads();
   }
-  if (!t.z) return;
-  // y = W z with a warp per row, and the row exponents of L
-  double* zs = T;
-  if (tid < NB) {
-    zs[tid] = t.z[tid];
-    int hi = 0;
-    for (int j = 0; j <= tid; ++j) hi = max(hi, __double2hiint(S[tid * sd + j]) & 0x7FFFFFFF);
-    t.rex[tid] = (hi >> 20) - 1022;
-  }
-  __syncthreads();
-  double qs = 0.0;
-  for (int r = warp; r < NB; r += 8) {
-    double s = 0.0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) s = fma(W[r * NB + lane + 32 * q], zs[lane + 32 * q], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) t.z[r] = s;
-    qs = fma(s, s, qs);
-  }
-  __syncthreads();
-  if (lane == 0) zs[warp] = qs;
-  __syncthreads();
-  if (tid == 0) {
-    double s = 0.0;
-    for (int w = 0; w < 8; ++w) s += zs[w];
-    *t.quad = s;
-  }
 }
 
 cudaError_t launch_potrf128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks) {

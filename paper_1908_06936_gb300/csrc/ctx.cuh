@@ -19,9 +19,7 @@ struct DevBuf {
 
 constexpr int kNumEvents = 8;
 constexpr int kMixPanel = 512;     // panel width of the mixed-precision factorisation
-constexpr int kDiagCtas = 64;      // CTAs of one diagonal-block launch at most
-constexpr int kDigSideSMs = 32;    // SMs left to the look-ahead stream of the FP64 factorisation ...
-constexpr int64_t kDigLateRows = 16384;  // ... while at least this many rows remain (kDiagCtas below)
+constexpr int kDiagCtas = 64;      // CTAs of one diagonal-block launch at most (mixed path)
 constexpr int kRedPartials = 512;  // partial sums of one two-stage reduction
 
 inline int64_t kPartialDoubles(int64_t npad, int nb) { return 2 * kRedPartials + (npad / 1024 + 2) * (int64_t)nb; }

@@ -1,55 +1,54 @@
-// FP64 factorisation and inversion of one diagonal block of up to 512 rows: the diagonal tiles that the MP variant of
-// Section II-A, Fig. 1(d), keeps in double precision, and the serial part of the FP64 factorisation.  ONE cooperative
-// launch on a few SMs.
+// FP64 factorisation and inversion of diagonal blocks: of up to 512 rows on a cooperative grid (the tiles that the MP
+// variant of Section II-A, Fig. 1(d), keeps in double precision, and the serial part of the FP64 factorisation), and of
+// many 128 x 128 tiles at once, a thread-block cluster each (the batched paths).
 //
-// Every CTA of a cooperative grid works through the same steps, separated by grid-wide barriers (bounded waits; every
-// CTA reaches every barrier; a failed pivot only turns values into NaN and is recorded in the status):
+// The CTAs of a group (the grid, or a cluster) work through the same steps, separated by group-wide barriers (a failed
+// pivot only turns values into NaN and is recorded in the status, so every CTA reaches every barrier).  In 32-wide
+// steps j (c0 = 32 j):
+//     (b) L_rj = A_rj D_j^-T for the rows below by substitution, 8 or 16 rows a task; W_j-1 = V_j-1 T_j-1 (see below)
+//     (c) A_rc -= L_rj L_cj^T: the next leaf first, on a few CTAs, which CTA 0 then factors, D_j+1 =
+//         chol(A_j+1,j+1) (diag_leaf), while the others apply the rest in 32 x 16 tiles and the last ones form V_j = D_j^-1
+//   The inverse W = L^-1 keeps pace, one step behind: row block i of W starts as zero and (c) adds
+//   T_i -= L_i,j-1 W_j-1 in tiles of the same shape; then W_i = V_i T_i.  After the last leaf only the last row blocks
+//   are left.
 //
-//   Cholesky, right-looking in 32-wide steps j (c0 = 32 j):
-//     (a) CTA 0: D = chol(A_jj) (diag_leaf)
-//     (b) L_rj = A_rj D^-T for the rows below by substitution, 8 rows a task, also into a scratch panel P
-//     (c) A_rc -= L_rj L_cj^T: the next leaf first, on CTAs 0-3, which CTA 0 then factors while the others apply the
-//         rest in 32 x 16 tasks (look-ahead) and the last CTA forms V_j = D^-1
-//   Inverse W = L^-1 by doubling: a 2b block [[X_A, 0], [L_BA, X_B]] has inverse [[W_A, 0], [-W_B (L_BA W_A), W_B]],
-//   formed for b = 32, 64, 128, 256 as two steps of 8 x 32 product tasks each.
+// Bound: the chain of (b) and (c), 26 us a step: leaf 14, rows 4.3, two barriers 2.8, the next leaf's update and its
+// hand-over 4.1.  An FP64 instruction keeps its SM quarter busy for 64 cycles here, so FP64 work on one SM does 2
+// multiply-adds a cycle: a wide leaf is throughput bound (64 wide with its inverse: 88 us) and a narrow one pays for
+// barriers.  A 512 block takes 427 us on 104 CTAs, 464 on 64, 698 on 32, 1,180 on 16; with the columns of a leaf dealt
+// out one by one and the inverse by doubling after the last leaf, 610 on 64.  A 128 tile on a cluster of 4 takes 128 us;
+// on one CTA, as a blocked factorisation and then the inverse, 570.
 //
-// Bound: the chain of (a) and (b).  A dependent FP64 instruction costs 64 cycles here (an SM quarter issues half a lane
-// a cycle) and FP64 work on one SM 2 multiply-adds a cycle, so a wide leaf is throughput bound (64 wide with its
-// inverse: 88 us) and a narrow one pays for barriers (~1.5 us each).
-//
-// Outputs: L in the block's lower triangle (upper triangle untouched), log L_ii summed in a
-// fixed order per 128 sub-tile, the 128 x 128 sub-tile inverses (row-major, zero above the
-// diagonal) and, for a 512 block, its inverse (row-major, zero above the diagonal).
+// Outputs: L in the block's lower triangle (upper triangle untouched), log L_ii summed in a fixed order per 128
+// sub-tile, the 128 x 128 sub-tile inverses (row-major, zero above the diagonal) and, for a 512 block, its inverse
+// (row-major, zero above the diagonal).
 #include <math.h>
 
-#include <type_traits>
-
 #include "exa_internal.cuh"
+#include "gemm_tc.cuh"
 #include "tc_common.cuh"
 
 namespace exa {
 
 constexpr int kDB = 512;        // largest block, leading dimension of its inverse
-constexpr int kDW = 32;         // Cholesky step / inverse leaf
+constexpr int kDSub = 128;      // sub-tile
+constexpr int kDW = 32;         // step
 constexpr int kDThreads = 256;
 constexpr int kDLd = kDW + 1;   // row stride of 32-wide tiles in shared memory (odd in doubles)
-// scratch (doubles): the 32-inverses, the 256 x 256 product of the widest inverse step, then the current step's panel
-constexpr int64_t kDiagT = (int64_t)(kDB / kDW) * kDW * kDW;
-constexpr int64_t kDiagP = kDiagT + 256 * 256;
-constexpr int64_t kDiagR = kDiagP + (int64_t)(kDB - kDW) * kDW;  // 1 / L_cc
-constexpr int64_t kDiagBar = kDiagR + kDB;  // barrier counter, abort flag, lead counter
-constexpr int64_t kDiagScratch = kDiagBar + 2;
+constexpr int kDLead = 8;       // CTAs of a leaf's last update, at most (4 rows each)
+constexpr int64_t kDiagScratch = 2;  // doubles: barrier counter, abort flag, lead counter
 constexpr long long kDiagSpin = 2000000000LL;  // bound of one barrier wait, SM clock cycles (~1 s)
 
 struct DiagArgs {
-  double* a;            // column-major matrix, element (i, j) at a[i + j * ld]
-  int64_t ld, k0;       // block origin (k0, k0)
-  double* w_sub;        // 128 x 128 row-major sub-tile inverses (w_all + (k0 / 128) 128^2)
-  double* logdet;       // sub-tile log sums (logdet_part + k0 / 128)
-  double* w2;           // 512 x 512 row-major inverse
-  double* scr;          // kDiagScratch doubles
+  double* a;        // column-major matrix, element (i, j) at a[i + j * ld]
+  int64_t ld, k0;   // block origin (k0, k0)
+  double* w;        // inverse, row-major, size x size, leading dimension ldw
+  int ldw;
+  int inv;          // the inverse is formed within diagonal blocks of this width: size, or kDSub
+  double* w_sub;    // also the 128 x 128 sub-tile inverses (row-major), or null
+  double* logdet;   // sub-tile log sums
   DevStatus* st;
-  int size;             // rows of the block, a multiple of 128 up to 512
+  int size;         // rows of the block, a multiple of 128 up to 512
 };
 
 // Waits, bounded, until *count >= target (every later wait is released by *abort).
@@ -65,19 +64,63 @@ __device__ __forceinline__ void wait_at_least(const unsigned int* count, unsigne
   __threadfence();
 }
 
-// Grid-wide barrier of the cooperative launch (all CTAs co-resident) on a monotone counter.  On
-// time-out the status records it, the abort flag releases every later wait, and the
-// (then meaningless) results are discarded by the caller through the status.
-__device__ __forceinline__ void grid_barrier(unsigned int* count, volatile int* abort, unsigned int target,
-                                             DevStatus* st) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(count, 1u);
-    wait_at_least(count, target, abort, st, 71);
+// The CTAs of a cooperative grid (all co-resident), with barriers on a monotone counter.  On time-out the status
+// records it, the abort flag releases every later wait, and the (then meaningless) results are discarded by the caller
+// through the status.
+struct GridGroup {
+  unsigned int *bar, *leadcnt;  // leadcnt: lead tasks finished by CTAs other than 0 (monotone)
+  volatile int* abort;
+  DevStatus* st;
+  unsigned int nbar = 0, nlead = 0;
+  __device__ GridGroup(double* scr, DevStatus* s)
+      : bar((unsigned int*)scr), leadcnt((unsigned int*)scr + 2), abort((volatile int*)scr + 1), st(s) {}
+  __device__ int size() const { return (int)gridDim.x; }
+  __device__ int rank() const { return (int)blockIdx.x; }
+  __device__ void sync() {
+    ++nbar;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      atomicAdd(bar, 1u);
+      wait_at_least(bar, nbar * gridDim.x, abort, st, 71);
+    }
+    __syncthreads();
   }
-  __syncthreads();
-}
+  // CTA 0 goes on once the others have finished their part of the next leaf; no other waits
+  __device__ void lead_sync() {
+    const unsigned int foreign = min(gridDim.x, (unsigned int)kDLead) - 1;
+    nlead += foreign;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (blockIdx.x == 0) {
+        wait_at_least(leadcnt, nlead, abort, st, 72);
+      } else if (blockIdx.x <= foreign) {
+        __threadfence();
+        atomicAdd(leadcnt, 1u);
+      }
+    }
+    __syncthreads();
+  }
+};
+
+// A thread-block cluster.
+struct ClusterGroup {
+  __device__ int size() const {
+    unsigned int n;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+    return (int)n;
+  }
+  __device__ int rank() const {
+    unsigned int r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return (int)r;
+  }
+  __device__ void sync() {
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  __device__ void lead_sync() { sync(); }
+};
 
 // d positive, finite and not subnormal, on its bits (an FP64 comparison costs 64 cycles).
 __device__ __forceinline__ bool normal_positive(double d) {
@@ -118,47 +161,6 @@ __device__ __forceinline__ double rsqrt_int(double d) {
   return __longlong_as_double((long long)(((Z + 256) >> 9) + ((unsigned long long)(unsigned int)((1021 - k) << 20) << 32)));
 }
 
-// acc[u] += sum_k A(r + 8 u, k) B(c, k), k < K (a multiple of 32), for r = warp, c = lane: an 8 H x 32 tile with
-// A(i, k) = pa[i ars + k acs], B(c, k) = pb[c brs + k bcs].  sA: 8 H x 33, sB: 32 x 33.
-template <int H>
-__device__ __forceinline__ void tile_gemm(double (&acc)[H], const double* pa, int64_t ars, int64_t acs,
-                                          const double* pb, int64_t brs, int64_t bcs, int K, double* sA, double* sB) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int k0 = 0; k0 < K; k0 += kDW) {
-    __syncthreads();  // the previous chunk (or the caller's use of sA / sB) is finished
-    // consecutive threads walk the dimension with the smaller stride; L2 loads (ld.global.cg): the operands were
-    // written by other CTAs since the last barrier
-    double va[H], vb[4];
-#pragma unroll
-    for (int u = 0; u < H; ++u) {
-      const int idx = tid + u * kDThreads, i = acs == 1 ? idx >> 5 : idx % (8 * H), k = acs == 1 ? idx & 31 : idx / (8 * H);
-      va[u] = __ldcg(pa + i * ars + (k0 + k) * acs);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = tid + u * kDThreads, c = bcs == 1 ? idx >> 5 : idx & 31, k = bcs == 1 ? idx & 31 : idx >> 5;
-      vb[u] = __ldcg(pb + c * brs + (k0 + k) * bcs);
-    }
-#pragma unroll
-    for (int u = 0; u < H; ++u) {
-      const int idx = tid + u * kDThreads, i = acs == 1 ? idx >> 5 : idx % (8 * H), k = acs == 1 ? idx & 31 : idx / (8 * H);
-      sA[i * kDLd + k] = va[u];
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = tid + u * kDThreads, c = bcs == 1 ? idx >> 5 : idx & 31, k = bcs == 1 ? idx & 31 : idx >> 5;
-      sB[c * kDLd + k] = vb[u];
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kDW; ++k) {
-      const double b = sB[lane * kDLd + k];
-#pragma unroll
-      for (int u = 0; u < H; ++u) acc[u] = fma(sA[(warp + 8 * u) * kDLd + k], b, acc[u]);
-    }
-  }
-}
-
 // A flag in shared memory between warps of one CTA: what was written before post is seen after await, which polls (a
 // few tens of cycles; an mbarrier wait takes longer to wake) and gives up after ~2^24 polls.
 __device__ __forceinline__ void post(int* flag, int v) {
@@ -172,306 +174,436 @@ __device__ __forceinline__ void await(const int* flag, int v) {
   }
 }
 
-// (a) of step j on one CTA: chol of the 32 x 32 block at c0, with a lane per row and the columns spread over four warps,
-// one per SM quarter (column c in register c / 4 of warp c mod 4).  The owner of column c scales it by
-// r_c = 1 / sqrt(d_c) and publishes it in shared memory (done[c] = j + 1); every warp then
-// subtracts it from its own columns, the owner of column c + 1 that one first, which it publishes before the others:
-// the chain per column is one multiply-add, one shuffle, one reciprocal square root and one product.
+// D_j = chol of the 32 x 32 block at step j, on one CTA: a lane per row, the columns on four warps, one per SM quarter:
+// warp w holds columns 4 w .. 4 w + 3 and 16 + 4 w .. 16 + 4 w + 3.  Finished columns go to shared memory, where the
+// other warps wait for them (done[c] = j + 1) and subtract them from their own.  The chain per column is a product, a
+// multiply-add, a shuffle and a reciprocal square root (~500 cycles), within one warp but for every fourth column; with
+// the columns dealt out one by one the hand-over cost ~300 cycles at each.  1 / L_cc goes to the diagonal of w.
 __device__ void diag_leaf(const DiagArgs& g, int j, double* S, int* done) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t c0 = g.k0 + (int64_t)j * kDW;
   double* A = g.a + c0 + c0 * g.ld;
   const int epoch = j + 1;
   // S[c kDLd + i] = A(i, c), later L(i, c)
-  for (int idx = tid; idx < kDW * kDW; idx += kDThreads) {
-    const int i = idx & (kDW - 1), c = idx / kDW;
-    S[c * kDLd + i] = i >= c ? __ldcg(A + i + (int64_t)c * g.ld) : 0.0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = warp + 8 * u;
+    S[c * kDLd + lane] = lane >= c ? __ldcg(A + lane + (int64_t)c * g.ld) : 0.0;
   }
   __syncthreads();
   if (warp < 4) {
-    double a[8];
+    double x0[4], x1[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) a[u] = S[(warp + 4 * u) * kDLd + lane];
-    // column c, in a0 of this warp: pivot, scale, publish
-    auto publish = [&](int c, double a0) {
-      const double d = __shfl_sync(0xffffffffu, a0, c);
-      double r;
-      if (normal_positive(d)) {  // uniform across the warp
-        r = rsqrt_int(d);
-      } else if (d > 0.0 && isfinite(d)) {
-        r = rsqrt(d);
-      } else {
-        if (lane == 0) {
-          atomicMin(&g.st->pivot, (long long)(c0 + c));
-          atomicExch(&g.st->info, 1);
-        }
-        r = NAN;  // the rest becomes NaN; every barrier is still reached
-      }
-      S[c * kDLd + lane] = lane >= c ? a0 * r : 0.0;
-      __syncwarp();
-      if (lane == 0) {
-        post(done + c, epoch);
-        g.scr[kDiagR + j * kDW + c] = r;
-      }
-    };
-    if (warp == 0) publish(0, a[0]);
-    // columns 4 q4 .. 4 q4 + 3, of which this warp's is a[0]; N: registers that may hold later columns (a predicated-off
-    // multiply-add takes its 64 cycles too, so the count is a constant of the code, in four versions)
-    auto quad = [&](auto width, int q4) {
-      constexpr int N = decltype(width)::value;
+    for (int u = 0; u < 4; ++u) {
+      x0[u] = S[(4 * warp + u) * kDLd + lane];
+      x1[u] = S[(16 + 4 * warp + u) * kDLd + lane];
+    }
+    __syncwarp();
+    // x(columns cb ..) minus the contributions of columns 4 q .. 4 q + 3
+    auto subtract = [&](double (&x)[4], int cb, int q) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int c = 4 * q4 + q;
-        if (warp != q) await(done + c, epoch);
+      for (int v = 0; v < 4; ++v) {
+        const int c = 4 * q + v;
+        await(done + c, epoch);
         const double* col = S + c * kDLd;
         const double lic = col[lane];
-        // the next column's owner: warp q + 1 (its a[0]), or warp 0 (its a[1]) at the end of the four
-        const int nextw = (q + 1) & 3;
-        constexpr int kLast = N > 1 ? 1 : 0;
-        const int nu = q == 3 ? kLast : 0;
-        if (warp == nextw && c + 1 < kDW) {
-          a[nu] = fma(-lic, col[c + 1], a[nu]);
-          publish(c + 1, a[nu]);
-        }
-        if (warp > nextw && q < 3) a[0] = fma(-lic, col[warp + 4 * q4], a[0]);  // still to come in these four
 #pragma unroll
-        for (int u = 1; u < N; ++u)
-          if (!(q == 3 && u == 1 && warp == 0)) a[u] = fma(-lic, col[min(warp + 4 * (q4 + u), kDW - 1)], a[u]);
+        for (int u = 0; u < 4; ++u) x[u] = fma(-lic, col[cb + u], x[u]);
       }
-#pragma unroll
-      for (int u = 0; u + 1 < N; ++u) a[u] = a[u + 1];
     };
-    for (int q4 = 0; q4 < 2; ++q4) quad(std::integral_constant<int, 8>{}, q4);
-    for (int q4 = 2; q4 < 4; ++q4) quad(std::integral_constant<int, 6>{}, q4);
-    for (int q4 = 4; q4 < 6; ++q4) quad(std::integral_constant<int, 4>{}, q4);
-    for (int q4 = 6; q4 < 8; ++q4) quad(std::integral_constant<int, 2>{}, q4);
+    double rr = 0.0;  // 1 / L_cc of column c = lane, if it is one of this warp's
+    auto factor = [&](double (&x)[4], int cb) {
+      // (the next column's pivot and its reciprocal root come before everything else that follows from a column)
+      double d = __shfl_sync(0xffffffffu, x[0], cb), r = rsqrt_int(d);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = cb + u;
+        if (!normal_positive(d)) {  // uniform across the warp
+          r = rsqrt(d);
+          if (!(d > 0.0) || !isfinite(d)) {
+            if (lane == 0) {
+              atomicMin(&g.st->pivot, (long long)(c0 + c));
+              atomicExch(&g.st->info, 1);
+            }
+            r = NAN;  // the rest becomes NaN; every barrier is still reached
+          }
+        }
+        const double t = x[u] * r;
+        const double l = lane >= c ? t : 0.0;
+        if (lane == c) rr = r;
+        S[c * kDLd + lane] = l;
+        if (u < 3) {
+          d = __shfl_sync(0xffffffffu, fma(-l, l, x[u + 1]), c + 1);
+          r = rsqrt_int(d);
+        }
+#pragma unroll
+        for (int v = u + 1; v < 4; ++v) x[v] = fma(-l, __shfl_sync(0xffffffffu, l, cb + v), x[v]);
+        __syncwarp();
+        if (lane == 0) post(done + c, epoch);
+      }
+    };
+    // the columns that this warp factors next come first; the later ones fill the time while other warps factor
+    for (int q = 0; q < warp; ++q) {
+      subtract(x0, 4 * warp, q);
+      if (q + 1 < warp) subtract(x1, 16 + 4 * warp, q);
+    }
+    factor(x0, 4 * warp);
+    for (int q = max(warp - 1, 0); q < 4 + warp; ++q) subtract(x1, 16 + 4 * warp, q);
+    factor(x1, 16 + 4 * warp);
+    if ((lane & 15) >> 2 == warp) g.w[(int64_t)(j * kDW + lane) * (g.ldw + 1)] = rr;
   }
   __syncthreads();
-  for (int idx = tid; idx < kDW * kDW; idx += kDThreads) {
-    const int i = idx & (kDW - 1), c = idx / kDW;
-    if (i >= c) A[i + (int64_t)c * g.ld] = S[c * kDLd + i];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = warp + 8 * u;
+    if (lane >= c) A[lane + (int64_t)c * g.ld] = S[c * kDLd + lane];
   }
 }
 
-// V_j = D^-1 of the factored block j (row-major, zero above the diagonal), on one CTA: the eliminations applied to the
-// identity, a lane per row and four columns a warp, B_i -= (L_ic r_c) B_c; rows of V are r_i B_i.  S: 32 x 33.
-__device__ void diag_leaf_inverse(const DiagArgs& g, int j, double* S) {
+// Element (r, c) of the inverse, both counted within the block.
+__device__ __forceinline__ void put_inverse(const DiagArgs& g, int r, int c, double v) {
+  g.w[(int64_t)r * g.ldw + c] = v;
+  if (g.w_sub && r / kDSub == c / kDSub) g.w_sub[(int64_t)r * kDSub + c % kDSub] = v;
+}
+
+// Columns 8 q .. 8 q + 7 of V_j = D_j^-1 into the diagonal block of w: the eliminations applied to the identity, a lane
+// per row and a column a warp, B_i -= (L_ic r_c) B_c; rows of V are r_i B_i.  S: 32 x 33.
+__device__ void diag_leaf_inverse(const DiagArgs& g, int j, int q, double* S) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t c0 = g.k0 + (int64_t)j * kDW;
   const double* A = g.a + c0 + c0 * g.ld;
-  const double* R = g.scr + kDiagR + j * kDW;
+  const double* R = g.w + (int64_t)(j * kDW) * (g.ldw + 1);  // the diagonal: 1 / L_cc
   __syncthreads();
-  for (int idx = tid; idx < kDW * kDW; idx += kDThreads) {
-    const int i = idx & (kDW - 1), c = idx / kDW;
-    S[c * kDLd + i] = i > c ? __ldcg(A + i + (int64_t)c * g.ld) * __ldcg(R + c) : 0.0;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int c = warp + 8 * u;
+    S[c * kDLd + lane] = lane > c ? __ldcg(A + lane + (int64_t)c * g.ld) * __ldcg(R + (int64_t)c * (g.ldw + 1)) : 0.0;
   }
-  const double ri = __ldcg(R + lane);
+  const double ri = __ldcg(R + (int64_t)lane * (g.ldw + 1));
   __syncthreads();
-  double b[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) b[u] = lane == warp + 8 * u ? 1.0 : 0.0;
-  for (int c = 0; c < kDW; ++c) {
-    const double t = S[c * kDLd + lane];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (warp + 8 * u <= c) b[u] = fma(-t, __shfl_sync(0xffffffffu, b[u], c), b[u]);
-  }
-  double* Vg = g.scr + (int64_t)j * kDW * kDW;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) Vg[lane * kDW + warp + 8 * u] = warp + 8 * u <= lane ? b[u] * ri : 0.0;
+  const int col = 8 * q + warp;
+  double b = lane == col ? 1.0 : 0.0;
+#pragma unroll 8
+  for (int c = 8 * q; c < kDW; ++c) b = fma(-S[c * kDLd + lane], __shfl_sync(0xffffffffu, b, c), b);
+  put_inverse(g, j * kDW + lane, j * kDW + col, col <= lane ? b * ri : 0.0);
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_constant__ DiagArgs g) {
-  __shared__ double S[kDW * kDLd];         // the leaf, or its inverse
-  __shared__ double sA[16 * kDLd], sB[kDW * kDLd];
-  __shared__ int done[kDW];
-  const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  unsigned int* bar = (unsigned int*)(g.scr + kDiagBar);
-  volatile int* abort = (volatile int*)(bar + 1);
-  unsigned int* leadcnt = bar + 2;  // lead tasks finished by CTAs other than 0 (monotone)
-  unsigned int nbar = 0, lead_target = 0;
-  auto sync_all = [&]() { grid_barrier(bar, abort, (++nbar) * (unsigned int)G, g.st); };
+struct DiagSmem {
+  double S[kDW * kDLd];  // the leaf, or its inverse
+  double A[16 * kDLd], B[kDW * kDLd], R[kDW];
+  int done[kDW];
+};
+
+template <class Group>
+__device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
+  const int G = grp.size(), b = grp.rank(), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t ld = g.ld, k0 = g.k0;
+  const int ldw = g.ldw, size = g.size, nsteps = size / kDW, per = g.inv / kDW;
   double* a = g.a;
-  double* P = g.scr + kDiagP;  // the current step's panel below the leaf, row-major, 32 wide
-  if (tid < kDW) done[tid] = 0;
+  double* w = g.w;
+  double *sA = sm.A, *sB = sm.B;
+  const int nl = min(G, kDLead);    // CTAs of the next leaf's update
+  const int nv = min(G - 1, 4);     // CTAs of V_j
+  if (tid < kDW) sm.done[tid] = 0;
   __syncthreads();
 
-  // ---------------- Cholesky in 32-wide steps ----------------
-  if (b == 0) diag_leaf(g, 0, S, done);
-  sync_all();
-  const int size = g.size, nsteps = size / kDW;
-  for (int j = 0; j + 1 < nsteps; ++j) {
+  // the first leaf; the 32 x 32 blocks of the inverse off the diagonal start as zero
+  if (b == 0) diag_leaf(g, 0, sm.S, sm.done);
+  for (int r = G > 1 ? b - 1 : 0; r < size; r += G > 1 ? G - 1 : 1) {
+    if (r < 0) break;
+    const int g0 = r / g.inv * g.inv;
+    for (int c = g0 + tid; c < g0 + g.inv; c += kDThreads)
+      if (c / kDW != r / kDW) put_inverse(g, r, c, 0.0);
+  }
+  grp.sync();
+
+  for (int j = 0; j < nsteps; ++j) {
     const int64_t c0 = k0 + (int64_t)j * kDW, r0 = c0 + kDW;
     const int below = size - (j + 1) * kDW;  // rows of the block below step j
-    // (b) x D^T = A(r, c0 ..) row by row, eight rows a task: warps 0-3 (an SM quarter each) take two rows, 16 lanes a
-    //     row with columns q and q + 16; step c: x_c = a_c r_c, then a_l -= x_c L_lc for l > c
-    for (int t = b; t < below / 8; t += G) {
-      double* rows = a + r0 + 8 * t + c0 * ld;
+    const int i1 = j > 0 ? (j - 1) / per * per : 0;  // first step of the block of width inv that j - 1 lies in
+    // ---- (b) x D^T = A(r, c0 ..) row by row.  Step c takes x_c as it stands and subtracts x_c (r_c L_lc) from the
+    //      columns l > c; at the end x_c r_c.  Eight rows a task, sixteen where there are more tasks than CTAs.
+    const int lg = below / 8 > G ? 4 : 3, rows = 1 << lg, nsub = below >> lg;
+    for (int t = b; t < nsub; t += G) {
+      double* src = a + r0 + (int64_t)rows * t + c0 * ld;
       __syncthreads();
       {
-        const double v = __ldcg(rows + (tid & 7) + (int64_t)(tid >> 3) * ld);
-        double vv[4];
+        double v[2], vv[4], rc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) vv[u] = __ldcg(a + c0 + lane + (c0 + warp + 8 * u) * ld);  // D(lane, warp + 8 u)
-        sA[(tid & 7) * kDLd + (tid >> 3)] = v;
+        for (int u = 0; u < 2; ++u) {
+          const int idx = tid + u * kDThreads;
+          v[u] = idx < rows * kDW ? __ldcg(src + (idx & (rows - 1)) + (int64_t)(idx >> lg) * ld) : 0.0;
+        }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) sB[(warp + 8 * u) * kDLd + lane] = vv[u];
-        if (warp == 7) sA[8 * kDLd + lane] = __ldcg(g.scr + kDiagR + j * kDW + lane);
+        for (int u = 0; u < 4; ++u) {
+          vv[u] = __ldcg(a + c0 + lane + (c0 + warp + 8 * u) * ld);  // D(lane, warp + 8 u)
+          rc[u] = __ldcg(w + (int64_t)(j * kDW + warp + 8 * u) * (ldw + 1));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int idx = tid + u * kDThreads;
+          if (idx < rows * kDW) sA[(idx & (rows - 1)) * kDLd + (idx >> lg)] = v[u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double m = vv[u] * rc[u];
+          sB[(warp + 8 * u) * kDLd + lane] = lane > warp + 8 * u ? m : 0.0;
+          if (lane == 0) sm.R[warp + 8 * u] = rc[u];
+        }
       }
       __syncthreads();
-      if (warp < 4) {
+      if (rows == 8) {  // a row a warp: the shorter chain
+        double x = sA[warp * kDLd + lane];
+#pragma unroll
+        for (int c = 0; c < kDW; ++c) x = fma(-__shfl_sync(0xffffffffu, x, c), sB[c * kDLd + lane], x);
+        sA[warp * kDLd + lane] = x * sm.R[lane];
+      } else {  // two rows a warp, 16 lanes a row with columns q and q + 16: fewer instructions a row
         const int r = 2 * warp + (lane >> 4), q = lane & 15;
         double x0 = sA[r * kDLd + q], x1 = sA[r * kDLd + q + 16];
 #pragma unroll
         for (int c = 0; c < kDW; ++c) {
-          const double rc = sA[8 * kDLd + c];
           const double* col = sB + c * kDLd;
           if (c < 16) {
-            const double l0 = q > c ? col[q] : 0.0, l1 = col[q + 16];
-            if (q == c) x0 *= rc;
             const double xc = __shfl_sync(0xffffffffu, x0, c, 16);
-            x0 = fma(-xc, l0, x0);
-            x1 = fma(-xc, l1, x1);
+            x0 = fma(-xc, col[q], x0);
+            x1 = fma(-xc, col[q + 16], x1);
           } else {
-            const double l1 = q + 16 > c ? col[q + 16] : 0.0;
-            if (q + 16 == c) x1 *= rc;
-            x1 = fma(-__shfl_sync(0xffffffffu, x1, c - 16, 16), l1, x1);
+            x1 = fma(-__shfl_sync(0xffffffffu, x1, c - 16, 16), col[q + 16], x1);
           }
         }
-        sA[r * kDLd + q] = x0;
-        sA[r * kDLd + q + 16] = x1;
+        sA[r * kDLd + q] = x0 * sm.R[q];
+        sA[r * kDLd + q + 16] = x1 * sm.R[q + 16];
       }
       __syncthreads();
-      P[(8 * t + warp) * kDW + lane] = sA[warp * kDLd + lane];
-      rows[(tid & 7) + (int64_t)(tid >> 3) * ld] = sA[(tid & 7) * kDLd + (tid >> 3)];
+      for (int idx = tid; idx < rows * kDW; idx += kDThreads)
+        src[(idx & (rows - 1)) + (int64_t)(idx >> lg) * ld] = sA[(idx & (rows - 1)) * kDLd + (idx >> lg)];
     }
-    sync_all();
-    // (c) the next leaf: rows 8 q .. of it on CTA q (CTA 0 where the grid is smaller); the others count their part on
-    //     a monotone counter that CTA 0 waits for before the leaf
-    int foreign = 0;
-    for (int q = 0; q < 4; ++q) {
-      const int owner = q < G ? q : 0;
-      foreign += owner != 0;
-      if (owner != b) continue;
-      __syncthreads();
-      for (int idx = tid; idx < kDW * kDW; idx += kDThreads) sB[(idx >> 5) * kDLd + lane] = __ldcg(P + idx);
-      __syncthreads();
-      const int i = 8 * q + warp;
-      double* pc = a + (r0 + i) + (r0 + lane) * ld;
-      double s0 = lane <= i ? __ldcg(pc) : 0.0;
+    //      W_i = V_i T_i in place, i = j - 1, in strips of eight columns (a strip is one task's alone); on the CTAs that
+    //      have no rows first
+    auto inverse_rows = [&](int i) {
+      const int first = i / per * per * kDW, n = (i * kDW - first) / 8;
+      for (int t = G - 1 - b; t < n; t += G) {
+        const int cb = first + 8 * t;
+        double* T = w + (int64_t)(i * kDW) * ldw + cb;
+        const double* V = w + (int64_t)(i * kDW) * (ldw + 1);
+        __syncthreads();
+        const double tv = __ldcg(T + (int64_t)(tid >> 3) * ldw + (tid & 7));
+        double vv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) vv[u] = __ldcg(V + (int64_t)(warp + 8 * u) * ldw + lane);
+        sA[(tid & 7) * kDLd + (tid >> 3)] = tv;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sB[(warp + 8 * u) * kDLd + lane] = vv[u];
+        __syncthreads();
+        double acc = 0.0;
 #pragma unroll 8
-      for (int k = 0; k < kDW; ++k) s0 = fma(-sB[i * kDLd + k], sB[lane * kDLd + k], s0);
-      if (lane <= i) *pc = s0;
-    }
-    if (b != 0 && b < 4) {
-      __syncthreads();
-      if (tid == 0) {
-        __threadfence();
-        atomicAdd(leadcnt, 1u);
+        for (int k = 0; k < kDW; ++k) acc = fma(sB[lane * kDLd + k], sA[warp * kDLd + k], acc);
+        __syncthreads();
+        sA[warp * kDLd + lane] = acc;
+        __syncthreads();
+        put_inverse(g, i * kDW + (tid >> 3), cb + (tid & 7), sA[(tid & 7) * kDLd + (tid >> 3)]);
+      }
+    };
+    if (j > 0) inverse_rows(j - 1);
+    if (j == nsteps - 1) {  // V of the last leaf and the log-determinant parts, off the chain
+      for (int q = 0; q < 4; ++q)
+        if (b == (G > 1 ? 1 + q % nv : 0)) diag_leaf_inverse(g, j, q, sm.S);
+      for (int s4 = b; s4 < size / kDSub; s4 += G) {  // uniform over the CTA
+        __syncthreads();
+        if (tid < kDSub) {
+          const int64_t r = k0 + kDSub * s4 + tid;
+          sB[tid] = log(__ldcg(a + r + r * ld));
+        }
+        __syncthreads();
+        if (warp == 0) {  // in a fixed order
+          double s = (sB[lane] + sB[lane + 32]) + (sB[lane + 64] + sB[lane + 96]);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          if (lane == 0) g.logdet[s4] = s;
+        }
       }
     }
-    lead_target += (unsigned int)foreign;
-    if (b == 0) {
-      if (tid == 0) wait_at_least(leadcnt, lead_target, abort, g.st, 72);
-      __syncthreads();
-      diag_leaf(g, j + 1, S, done);
-    } else {
-      if (b == G - 1) diag_leaf_inverse(g, j, S);
-      // A_rc -= L_r L_c^T over 32-row blocks R and 16-wide column strips s <= 2 R + 1, but for the leaf's (R = 0):
-      // block R has 2 R + 2 tasks, numbered from R (R + 1) - 2 on; lanes along the rows of the column-major matrix.
-      // The CTA that forms V_j takes its share of the last ones.
-      const int nr = below / kDW, nt = nr * (nr + 1) - 2;
-      for (int t = b - 1; t < nt; t += G - 1) {
+    grp.sync();
+    // ---- (c) the next leaf: its rows spread over the first CTAs
+    const bool more = j + 1 < nsteps;
+    if (more) {
+      if (b < nl) {
+        __syncthreads();
+        double vv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) vv[u] = __ldcg(a + r0 + lane + (c0 + warp + 8 * u) * ld);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sB[lane * kDLd + warp + 8 * u] = vv[u];
+        __syncthreads();
+        const int nrow = kDW / nl;
+        for (int i = nrow * b + warp; i < nrow * (b + 1); i += kDThreads / 32) {
+          double* pc = a + (r0 + i) + (r0 + lane) * ld;
+          double s0 = lane <= i ? __ldcg(pc) : 0.0, s1 = 0.0;
+#pragma unroll
+          for (int k = 0; k < kDW; k += 2) {
+            s0 = fma(-sB[i * kDLd + k], sB[lane * kDLd + k], s0);
+            s1 = fma(-sB[i * kDLd + k + 1], sB[lane * kDLd + k + 1], s1);
+          }
+          if (lane <= i) *pc = s0 + s1;
+        }
+      }
+      grp.lead_sync();
+      if (b == 0) diag_leaf(g, j + 1, sm.S, sm.done);
+      for (int q = 0; q < 4; ++q)
+        if (b == (G > 1 ? G - 1 - q % nv : 0)) diag_leaf_inverse(g, j, q, sm.S);
+    }
+    //      Tiles of 32 lanes x 16, two of the 16 a warp: C(l, x) -= sum_k Y(l, k) X(x, k).
+    //      A_rc -= L_r L_c^T over 32-row blocks R and 16-wide column strips s <= 2 R + 1, but for the leaf's (R = 0):
+    //      block R has 2 R + 2 tiles, numbered from R (R + 1) - 2 on; lanes along the rows.
+    //      T_i -= L_i,j-1 W_j-1 for i >= j: lanes along the columns, 16 rows a tile.
+    //      CTA 0 comes to them three rounds late (the leaf), the CTAs of V_j one or two.
+    const int nr = more ? below / kDW : 0, nt = nr > 0 ? nr * (nr + 1) - 2 : 0;
+    const int ni = j > 0 ? min(i1 + per, nsteps) - j : 0, nc = j - i1;  // row blocks i, column blocks of W_j-1
+    const int ntiles = nt + (j > 0 ? 2 * ni * nc : 0);
+    const int late0 = more ? 3 : 0, lateV = more ? (nv > 2 ? 1 : 2) : 0;
+    int round = 0, base = 0;
+    auto next = [&]() {  // this CTA's next tile, -1: none
+      while (base < ntiles) {
+        const bool no0 = round < late0, noV = round < lateV;
+        const int t = base + b - (no0 ? 1 : 0);
+        const bool mine = !(no0 && b == 0) && !(noV && b >= G - nv) && t < ntiles;
+        base += G - (no0 ? 1 : 0) - (noV ? nv : 0);
+        ++round;
+        if (mine) return t;
+      }
+      return -1;
+    };
+    double va[2], vb[4], vc[2];
+    double* pc = nullptr;
+    int64_t cs = 0;
+    int lim = 0;  // C(lane, x) belongs to the tile if x <= lim
+    auto load = [&](int t) {
+      const double *px, *py;
+      int64_t ys;
+      if (t < nt) {
         int R = (int)sqrtf((float)(t + 2));
         while (R * (R + 1) > t + 2) --R;
         while ((R + 1) * (R + 2) <= t + 2) ++R;
         const int s = t + 2 - R * (R + 1);
-        double acc[2] = {0.0, 0.0};
-        tile_gemm<2>(acc, P + s * 16 * kDW, kDW, 1, P + R * kDW * kDW, kDW, 1, kDW, sA, sB);
-        const int i = R * kDW + lane;
-        double* pc = a + (r0 + i) + (r0 + s * 16 + warp) * ld;
-        const bool lo = s * 16 + warp <= i, hi = s * 16 + warp + 8 <= i;
-        const double v0 = lo ? __ldcg(pc) : 0.0, v1 = hi ? __ldcg(pc + 8 * ld) : 0.0;
-        if (lo) *pc = v0 - acc[0];
-        if (hi) pc[8 * ld] = v1 - acc[1];
+        px = a + r0 + 16 * s + c0 * ld;
+        py = a + r0 + kDW * R + c0 * ld;
+        ys = ld;
+        pc = a + r0 + kDW * R + lane + (r0 + 16 * s) * ld;
+        cs = ld;
+        lim = kDW * R + lane - 16 * s;
+      } else {
+        const int q = t - nt, row = j * kDW + q / nc * 16, col = (i1 + q % nc) * kDW;
+        px = a + k0 + row + (c0 - kDW) * ld;
+        py = w + (int64_t)(j - 1) * kDW * ldw + col;
+        ys = ldw;
+        pc = w + (int64_t)row * ldw + col + lane;
+        cs = ldw;
+        lim = 15;
       }
-    }
-    sync_all();
-  }
-
-  // ---------------- log-determinant parts, leaves of the inverse ----------------
-  for (int s4 = b; s4 < size / 128; s4 += G) {  // uniform over the CTA
-    __syncthreads();
-    if (tid < 128) {
-      const int64_t r = k0 + 128 * s4 + tid;
-      sB[tid] = log(__ldcg(a + r + r * ld));
-    }
-    __syncthreads();
-    if (warp == 0) {  // in a fixed order
-      double s = (sB[lane] + sB[lane + 32]) + (sB[lane + 64] + sB[lane + 96]);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) g.logdet[s4] = s;
+      for (int u = 0; u < 2; ++u) va[u] = __ldcg(px + (tid & 15) + ((tid >> 4) + 16 * u) * ld);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) vb[u] = __ldcg(py + lane + (warp + 8 * u) * ys);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) vc[u] = warp + 8 * u <= lim ? __ldcg(pc + (warp + 8 * u) * cs) : 0.0;
+    };
+    int t = next();
+    if (t >= 0) load(t);
+    while (t >= 0) {
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 2; ++u) sA[(tid & 15) * kDLd + (tid >> 4) + 16 * u] = va[u];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sB[lane * kDLd + warp + 8 * u] = vb[u];
+      double acc0 = vc[0], acc1 = vc[1];
+      double* out = pc + warp * cs;
+      const int64_t step = 8 * cs;
+      const int left = lim - warp;
+      __syncthreads();
+      t = next();
+      if (t >= 0) load(t);  // in flight during the products
+#pragma unroll 8
+      for (int k = 0; k < kDW; ++k) {
+        const double y = sB[lane * kDLd + k];
+        acc0 = fma(-sA[warp * kDLd + k], y, acc0);
+        acc1 = fma(-sA[(warp + 8) * kDLd + k], y, acc1);
+      }
+      if (left >= 0) *out = acc0;
+      if (left >= 8) out[step] = acc1;
     }
+    grp.sync();
+    if (!more) inverse_rows(j);
   }
-  if (b == G - 1) diag_leaf_inverse(g, nsteps - 1, S);
-  sync_all();  // the last leaf's inverse
-  double* w2 = g.w2;
-  // W2 <- zero above the diagonal, the 32-inverses on the diagonal (other lower entries later)
-  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < (int64_t)size * kDB; idx += (int64_t)G * kDThreads) {
-    const int r = (int)(idx / kDB), c = (int)(idx % kDB);
-    if (c >= size) continue;
-    if (c > r) {
-      w2[idx] = 0.0;
-    } else if (r / kDW == c / kDW) {
-      const double* V = g.scr + (int64_t)(r / kDW) * kDW * kDW;
-      w2[idx] = __ldcg(V + (r % kDW) * kDW + (c % kDW));
-    }
-  }
-  sync_all();
+}
 
-  // ---------------- inverse by doubling: widths h = 32, 64, 128, 256 ----------------
-  // Tasks run from the longest reductions to the shortest in the first half of the list and back in the second, so
-  // that a CTA with two has a long and a short one.
-  double* T = g.scr + kDiagT;  // h x h products, row-major
-  auto fold = [](int q, int n) { return q < n / 2 ? q : n - 1 - (q - n / 2); };
-  // (a smaller block is the last of its matrix: only its 128 sub-tile inverses are wanted)
-  for (int h = kDW; h < (size == kDB ? kDB : 128); h *= 2) {
-    const int pairs = size / (2 * h), nr = h / 8, nc = h / kDW;  // blocks of width 2h; tiles of one h x h product
-    // first product: T_p = L_BA W_A  (L_BA: rows p 2h + h .., columns p 2h ..; W_A lower, row-major in w2)
-    for (int t = b; t < pairs * nr * nc; t += G) {
-      const int p = t % pairs, q = t / pairs, ti = q % nr, tj = fold(q / nr, nc);
-      const int64_t o = (int64_t)p * 2 * h;  // block origin within the block
-      double acc[1] = {0.0};
-      // T(r, c) = sum_k L(o + h + r, o + k) W(o + k, o + c): W_A(k, c) = 0 for k < c
-      const int kstart = tj * kDW;
-      tile_gemm<1>(acc, a + (k0 + o + h + ti * 8) + (k0 + o + kstart) * ld, 1, ld,
-                w2 + (o + kstart) * kDB + (o + tj * kDW), 1, kDB, h - kstart, sA, sB);
-      double* Tp = T + (int64_t)p * h * h;
-      Tp[(ti * 8 + warp) * h + tj * kDW + lane] = acc[0];
-    }
-    sync_all();
-    // second product: W_BA = -W_B T_p  (W_B lower, row-major in w2 at (o + h, o + h), zero above its diagonal)
-    for (int t = b; t < pairs * nr * nc; t += G) {
-      const int p = t % pairs, q = t / pairs, tj = q % nc, ti = nr - 1 - fold(q / nc, nr);
-      const int64_t o = (int64_t)p * 2 * h;
-      const double* Tp = T + (int64_t)p * h * h;
-      double acc[1] = {0.0};
-      // W_BA(r, c) = -sum_k W_B(r, k) T(k, c): W_B(r, k) = 0 for k > r
-      const int kend = (ti * 8 + 8 + kDW - 1) / kDW * kDW;
-      tile_gemm<1>(acc, w2 + (o + h + ti * 8) * kDB + (o + h), kDB, 1, Tp + tj * kDW, 1, h, kend, sA, sB);
-      w2[(o + h + ti * 8 + warp) * kDB + o + tj * kDW + lane] = -acc[0];
-    }
-    sync_all();
-  }
+__global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_constant__ DiagArgs g, double* scr) {
+  __shared__ DiagSmem sm;
+  diag_body(g, GridGroup(scr, g.st), sm);
+}
 
-  // ---------------- the 128 sub-tile inverses (diagonal blocks of W2) ----------------
-  for (int64_t idx = (int64_t)b * kDThreads + tid; idx < (int64_t)size * 128; idx += (int64_t)G * kDThreads) {
-    const int s = (int)(idx / (128 * 128)), rc = (int)(idx % (128 * 128)), r = rc / 128, c = rc % 128;
-    g.w_sub[idx] = __ldcg(w2 + (int64_t)(128 * s + r) * kDB + 128 * s + c);
+// One 128 x 128 tile a cluster; with task.z also y = W z, y^T y and the row exponents of L.
+__global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const DiagTileTask* __restrict__ tasks) {
+  __shared__ DiagSmem sm;
+  ClusterGroup grp;
+  const int G = grp.size(), b = grp.rank(), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const DiagTileTask t = tasks[blockIdx.x / G];
+  const DiagArgs g{t.a, t.ld, t.k0, t.w, kDSub, kDSub, nullptr, t.logdet, t.st, kDSub};
+  diag_body(g, grp, sm);
+  grp.sync();
+  if (!t.z) return;
+  if (b == G - 1) {  // the exponents, two threads a row
+    const double* row = t.a + t.k0 + (tid >> 1) + t.k0 * t.ld;
+    int hi = 0;
+#pragma unroll 8
+    for (int c = 0; c < kDSub / 2; ++c) {
+      const int cc = 2 * c + (tid & 1);
+      if (cc <= tid >> 1) hi = max(hi, __double2hiint(__ldcg(row + cc * t.ld)) & 0x7FFFFFFF);
+    }
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, 1));
+    if (!(tid & 1)) t.rex[tid >> 1] = (hi >> 20) - 1022;
   }
+  if (b != 0) return;
+  double* zs = sm.S;
+  if (tid < kDSub) zs[tid] = t.z[tid];
+  __syncthreads();
+  double qs = 0.0;
+#pragma unroll 4
+  for (int r = warp; r < kDSub; r += 8) {
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s = fma(__ldcg(t.w + r * kDSub + lane + 32 * q), zs[lane + 32 * q], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) t.z[r] = s;
+    qs = fma(s, s, qs);
+  }
+  __syncthreads();
+  if (lane == 0) zs[warp] = qs;
+  __syncthreads();
+  if (tid == 0) {
+    double s = 0.0;
+    for (int q = 0; q < 8; ++q) s += zs[q];
+    *t.quad = s;
+  }
+}
+
+// The widest cluster with which every tile has its SMs at once: more CTAs shorten a tile, but tiles that queue cost
+// more.
+cudaError_t launch_diag128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks) {
+  if (ntasks <= 0) return cudaSuccess;
+  int G = 8;
+  while (G > 1 && G * ntasks > tc_num_sms()) G /= 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(ntasks * G));
+  cfg.blockDim = dim3(kDThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim = {(unsigned)G, 1, 1};
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, diag_tasks_kernel, d_tasks);
 }
 
 size_t diag_block_scratch_doubles() { return (size_t)kDiagScratch; }
@@ -487,10 +619,11 @@ cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0,
   });
   if (e != cudaSuccess) return e;
   if (grid < 2) grid = 2;  // CTA 0 runs the leaves; the updates need at least one more CTA
-  e = cudaMemsetAsync(scratch + kDiagBar, 0, 2 * sizeof(double), s);
+  e = cudaMemsetAsync(scratch, 0, kDiagScratch * sizeof(double), s);
   if (e != cudaSuccess) return e;
-  DiagArgs g{a, ld, k0, w_sub, logdet_part, w2, scratch, st, size};
-  void* args[] = {&g};
+  // (a smaller block is the last of its matrix: only its 128 sub-tile inverses are wanted)
+  DiagArgs g{a, ld, k0, w2, kDB, size == kDB ? kDB : kDSub, w_sub, logdet_part, st, size};
+  void* args[] = {&g, &scratch};
   // cooperative launch: every CTA is resident at once, so the grid barriers cannot wait on an
   // unscheduled CTA
   return cudaLaunchCooperativeKernel((const void*)diag_block_kernel, grid, kDThreads, args, smem, s);

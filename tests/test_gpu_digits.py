@@ -161,3 +161,15 @@ def test_batched_fp64_against_the_persistent_form(ns):
         low = batch(c, ns, 0, 0)
         assert exa.exa_workspace_bytes(c.handle) <= need
     assert np.all(np.abs(low - ref) <= 1e-10 * np.abs(ref))
+
+
+@pytest.mark.parametrize("nrep", [19, 20, 38, 39, 76, 77])
+def test_batched_fp64_at_every_cluster_width(nrep):
+    # 8, 4, 4, 2, 2 and 1 CTAs a diagonal tile on 152 SMs; the bound of the test above
+    import paper_1908_06936_gb300 as exa
+
+    ns = [1 + (37 * r) % 300 for r in range(nrep)]
+    with exa.Context() as c:
+        got = batch(c, ns, 0, 0)
+        ref = batch(c, ns, 32, 0)
+    assert np.all(np.abs(got - ref) <= 1e-10 * np.abs(ref))
