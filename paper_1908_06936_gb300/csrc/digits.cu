@@ -34,19 +34,6 @@ struct Cfg {
 };
 static_assert(Cfg<kDigSlices>::SMEM <= 232448 && Cfg<kDigLow>::SMEM <= 232448, "stages fit in shared memory");
 
-// Shared-memory descriptor of a K-major operand without swizzling: 8-row core matrices of 128 bytes, the two of
-// a 16-column step 128 bytes apart (leading offset), 8-row groups 256 bytes apart (stride offset).
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
-         ((uint64_t)1 << 46);
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-
 // Lower-triangle enumeration of 128 x TN tiles: bands of kBand row blocks, each a rectangle left of the band's
 // diagonal square (column tiles outer, rows inner: the tiles of one wave share operand rows in L2) and then the
 // square's own lower tiles.  Row block b holds 2 (b + 1) column tiles.
@@ -149,15 +136,8 @@ __device__ __forceinline__ double i63_to_f64_scaled(long long V, int sh) {
 
 // FP32 integers as integers.  F2I converts 16 lanes a cycle on an SM, which for the 65,536 accumulators of a tile is a
 // ninth of its MMA time, so half of the groups go by additions instead:
-// |a| <= 2^22: the low bits of a + 1.5 2^23;
+// |a| <= 2^22: the low bits of a + 1.5 2^23 (above, f32_to_int).
 __device__ __forceinline__ int small_int_bits(float a) { return __float_as_int(a + 12582912.0f); }  // + 0x4B400000
-// |a| <= 2^24: the multiples of 4 from a + 1.5 2^25, then the rest.
-__device__ __forceinline__ int large_int(float a) {
-  const float u = a + 50331648.0f;
-  const float rest = a - (u - 50331648.0f);
-  return 4 * (__float_as_int(u) - 0x4C400000) + (__float_as_int(rest + 12582912.0f) - 0x4B400000);
-}
-
 // One CTA per SM, persistent: warp 0 copies operand planes into a ring of 16-column stages, one thread of warp 1
 // issues the MMAs, warps 2-17 drain TMEM into C.  The S B planes of a stage lie one after another and group g
 // follows group g - 1 in TMEM, so A digit s against B digits 0 .. S-1-s is one run of columns (two MMAs where
@@ -261,10 +241,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
         }
         fence_after();
         const uint32_t sb = smem_u32(smem + stage * STAGE_BYTES);
-        const uint64_t b0 = sdesc(sb + S * A_BYTES);
+        const uint64_t b0 = sdesc_flat(sb + S * A_BYTES);
 #pragma unroll
         for (int s = 0; s < S; ++s) {
-          const uint64_t a = sdesc(sb + s * A_BYTES);
+          const uint64_t a = sdesc_flat(sb + s * A_BYTES);
           const int n = TN * (S - s);
           // the first step's s = 0 writes every group, all others add
           const uint32_t acc = (kc | s) ? 1u : 0u;
@@ -335,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const int w45 = __float2int_rn(__uint_as_float(x[0][j])) * 128 + __float2int_rn(__uint_as_float(x[1][j]));
-            const int w67 = large_int(__uint_as_float(x[2][j])) * 128 + large_int(__uint_as_float(x[3][j]));
+            const int w67 = f32_to_int(__uint_as_float(x[2][j])) * 128 + f32_to_int(__uint_as_float(x[3][j]));
             V[h + j] += ((long long)w45 * 16384 + w67 + 128) >> 8;
           }
         }

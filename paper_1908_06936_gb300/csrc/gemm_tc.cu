@@ -21,6 +21,7 @@
 // warp 1 owns TMEM and issues tcgen05.mma from one thread, warps 2-5 drain the
 // accumulators into the FP64 matrix.  Every wait is bounded; on time-out the
 // CTA records EXA_ERR_TIMEOUT, drains its in-flight copies, frees TMEM and exits.
+#include <type_traits>
 #include <cuda.h>
 #include <math.h>
 
@@ -94,8 +95,10 @@ struct T3Tile {
   double* C;
   int64_t ldc;
   bool diag;
+  int chunks;  // 32-column steps of the reduction
 };
 __device__ __forceinline__ bool t3_tile(const GemmArgs& g, long long t, T3Tile& o) {
+  o.chunks = g.K / 32;
   if (g.enum_mode == kEnumTasks) {
     const TcTask tk = g.tasks[t];
     o.ya = tk.a_row;
@@ -112,6 +115,7 @@ __device__ __forceinline__ bool t3_tile(const GemmArgs& g, long long t, T3Tile& 
   o.C = g.C + (g.c_row0 + (int64_t)bi * 128) + (g.c_col0 + (int64_t)bj * 128) * g.ldc;
   o.ldc = g.ldc;
   o.diag = g.lower_mask && (bi == bj);
+  if (g.tri) o.chunks = min(o.chunks, (bj + 1) * 4);
   return true;
 }
 
@@ -173,7 +177,6 @@ __global__ void __launch_bounds__(kGemmThreads)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int kchunks = g.K / KC;
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer ----------------
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(kGemmThreads)
       if (!t3_tile(g, t, tl)) continue;
       const int ya = tl.ya, yb = tl.yb;
       const bool one = far_t3(g, tl);  // far tile: the hi halves only
-      for (int kc = 0; kc < kchunks; ++kc) {
+      for (int kc = 0; kc < tl.chunks; ++kc) {
         if (!mbar_wait(&empty[stage], phase ^ 1, abort)) {
           *abort = 1;
           record_timeout(g.st, 11);
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(kGemmThreads)
       const uint32_t d = tmem + b * TN;
       const bool one = far_t3(g, tl);
       bool ok = true;
-      for (int kc = 0; kc < kchunks; ++kc) {
+      for (int kc = 0; kc < tl.chunks; ++kc) {
         if (!mbar_wait(&full[stage], phase, abort)) {
           *abort = 1;
           record_timeout(g.st, 13);
@@ -620,142 +623,178 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 }
 
 // ===========================================================================
-// OZ kernel: tile 128 x 32, K chunks of 64 BF16 digits, S = 5 slices, 2 stages.
+// OZ kernel: exact products of 5-digit operands, tiles 128 x tn with tn = 96, 64 or 32.
 // ===========================================================================
 namespace oz {
-constexpr int TM = 128, KC = 64, STAGES = 2, S = kOzSlices;
-constexpr int A_BYTES = TM * KC * 2;   // 16 KB per slice
-constexpr int TMEM_COLS = 512;         // 2 accumulator buffers of S groups x TN columns
-// Per tile width TN (32, or 48 for the band of the trailing update: 27% fewer operand bytes per
-// output, and 2 x 5 x 48 = 480 TMEM columns still hold two accumulator buffers)
-template <int TN>
-struct Cfg {
-  static constexpr int B_BYTES = TN * KC * 2;  // per slice
-  static constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-  static constexpr int GROUP_COLS = TN;        // one accumulator per slice-sum group
-  static constexpr int BUF_COLS = S * GROUP_COLS;
-  static constexpr int CH = TN / 2;            // columns drained by one epilogue warp
-};
-static_assert(Cfg<48>::SMEM_BYTES <= 232448, "two 48-wide stages fit in shared memory");
-static_assert(2 * Cfg<48>::BUF_COLS <= TMEM_COLS, "two 48-wide accumulator buffers fit in TMEM");
+constexpr int TM = 128, TN = 96, S = kOzSlices;
+constexpr int A_BYTES = TM * 32;                       // one digit plane of a 16-column step
+constexpr int STAGE_BYTES = S * (A_BYTES + TN * 32), STAGES = 6;
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 256;
+constexpr int kEpiWarps = 16, kThreads = 64 + 32 * kEpiWarps;
+constexpr int TMEM_COLS = 512;
+static_assert(SMEM_BYTES <= 232448 && S * TN <= TMEM_COLS && 2 * S * 32 <= TMEM_COLS, "stages and accumulators fit");
 
-// Tile t of a launch: row block bi (128 rows), column offset cofs (from c_col0 / b_row0) and
-// the number of its TN columns inside the output (band tiles of width 48 end ragged at each
-// panel boundary: 512 = 10 x 48 + 32).  False: skip the tile.
-template <int TN>
-__device__ __forceinline__ bool oz_tile(const GemmArgs& g, long long t, int& bi, int& cofs, int& cvalid) {
-  if (g.enum_mode != kEnumBand) {  // kEnumFull (TN = 32)
-    bi = (int)(t / g.nt);
-    cofs = (int)(t % g.nt) * TN;
-    cvalid = TN;
-    return true;
+struct Args {
+  double* C;
+  int64_t ldc, c_row0, c_col0;
+  const uint8_t *A, *B;      // first plane, at the operand's row origin
+  int64_t a_plane, b_plane;  // bytes between planes
+  const int *ea, *eb;
+  int mode, band, panel;     // kEnumFull or kEnumBand
+  int mt, n;                 // row blocks; columns (kEnumFull)
+  int tn, nbuf, k16;
+  int store, lower, tri;
+  long long ntiles;
+  DevStatus* st;
+};
+
+// Tile t: row block bi, column offset cofs and width (a multiple of 32).  Band tiles run along each row block from its
+// first panel of the band to the diagonal; `at` and `base` (row block, tiles before it) follow the growing t of a CTA.
+// False: skip the tile (above the diagonal).
+struct Cursor {
+  int at = 0;
+  long long base = 0;
+};
+__device__ __forceinline__ bool tile_of(const Args& g, long long t, Cursor& c, int& bi, int& cofs, int& width) {
+  if (g.mode == kEnumFull) {
+    const int per = (g.n + g.tn - 1) / g.tn;
+    bi = (int)(t / per);
+    cofs = (int)(t % per) * g.tn;
+    width = min(g.tn, g.n - cofs);
+    return !(g.lower && g.c_col0 + cofs > g.c_row0 + (int64_t)bi * TM + TM - 1);
   }
-  const int SI = g.panel / TM, SJ = (g.panel + TN - 1) / TN;
-  const long long pair = t / (SI * SJ);
-  const int sub = (int)(t % (SI * SJ));
-  const int b = g.band;
-  const long long head = (long long)b * (b + 1) / 2;
-  int I, J;
-  if (pair < head) {
-    tile_tri_decode(pair, I, J);
-  } else {
-    I = b + (int)((pair - head) / (b + 1));
-    J = I - b + (int)((pair - head) % (b + 1));
+  const int SI = g.panel / TM;
+  while (true) {
+    const int start = max(0, c.at / SI - g.band) * g.panel, end = (c.at + 1) * TM;
+    const int count = (end - start + g.tn - 1) / g.tn;
+    if (t < c.base + count) {
+      bi = c.at;
+      cofs = start + (int)(t - c.base) * g.tn;
+      width = min(g.tn, end - cofs);
+      return true;
+    }
+    c.base += count;
+    ++c.at;
   }
-  bi = I * SI + sub / SJ;
-  const int sj = sub % SJ;
-  cofs = J * g.panel + sj * TN;
-  cvalid = g.panel - sj * TN < TN ? g.panel - sj * TN : TN;
-  // skip tiles strictly above the diagonal
-  return (long long)cofs <= (long long)bi * TM + TM - 1;
+}
+
+// One warp's part of a tile: 32 rows x CH columns out of TMEM, `release` once the accumulators are read.
+template <int CH, class Release>
+__device__ __forceinline__ void drain(const Args& g, int bi, int cofs, int quad, int part, uint32_t acc, Release release) {
+  const int lane = threadIdx.x & 31, r = quad * 32 + lane;
+  const int lc0 = CH * part;
+  const int64_t row = g.c_row0 + (int64_t)bi * TM + r, col0 = g.c_col0 + cofs + lc0;
+  double* cp = g.C + row + col0 * g.ldc;
+  const int last = g.lower ? (int)min((int64_t)CH, row - col0) : CH;  // columns up to this one are written
+  // group q holds an exact integer a_q (|a_q| < 2^24) of weight 2^(-7(q+2)): V = sum_q a_q 2^(7(4-q)) is an integer
+  // below 2^53, combined from two 32-bit words (|a_0|, |a_2| < 2^23.4) and a_4.  Half of the conversions go by
+  // additions: F2I converts 16 lanes a cycle on an SM.
+  long long V[CH];
+  const uint32_t ta = acc + ((uint32_t)(quad * 32) << 16) + lc0;
+  const int width = 4 * CH;
+#pragma unroll
+  for (int h = 0; h < CH; h += 4) {
+    uint32_t x[S][4];
+#pragma unroll
+    for (int q = 0; q < S; ++q) tmem_ld4(ta + q * width + h, x[q]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int w01 = f32_to_int(__uint_as_float(x[0][j])) * 128 + __float2int_rn(__uint_as_float(x[1][j]));
+      const int w23 = f32_to_int(__uint_as_float(x[2][j])) * 128 + __float2int_rn(__uint_as_float(x[3][j]));
+      V[h + j] = ((long long)w01 * 16384 + w23) * 128 + __float2int_rn(__uint_as_float(x[4][j]));
+    }
+  }
+  fence_before();
+  release();
+  const int base = g.ea[bi * TM + r] - 7 * (S + 1);
+  const int* eb = g.eb + cofs + lc0;
+#pragma unroll
+  for (int j0 = 0; j0 < CH; j0 += 4) {
+    asm volatile("" ::: "memory");  // four outputs at a time: more would not fit the registers
+    double cv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cv[j] = !g.store && j0 + j <= last ? __ldcs(cp + (int64_t)(j0 + j) * g.ldc) : 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double x = i53_to_f64_scaled(V[j0 + j], base + eb[j0 + j]);
+      if (j0 + j <= last) __stcs(cp + (int64_t)(j0 + j) * g.ldc, g.store ? x : cv[j] - x);
+    }
+  }
 }
 }  // namespace oz
 
-// CL = 2: the CTAs of a cluster pair take adjacent column tiles (bj even, bj + 1) of one row
-// block, so they need the same A digits: each loads half of the 128 A rows (map `ta`, 64-row
-// boxes) and multicasts it to both, halving the A bytes each CTA pulls through L2 (A is four
-// fifths of a tile's operand bytes).  Each CTA's MMA commit releases the stage in both CTAs
-// (empty[] counts CL arrivals), since both write into both.  Band and full enumerations list
-// the two tiles of a pair consecutively and skip them together; tile counts are even.
-template <int CL, int TN>
-__global__ void __launch_bounds__(kGemmThreads, 1) gemm_oz_kernel(const __grid_constant__ OzMaps ta,
-                                                         const __grid_constant__ OzMaps tb,
-                                                         const __grid_constant__ GemmArgs g) {
+// One CTA per SM, persistent: warp 0 copies digit planes into a ring of 16-column stages, one thread of warp 1 issues
+// the MMAs, warps 2-17 drain TMEM into C.  The S B planes of a stage lie one after another and group q = s + t follows
+// group q - 1 in TMEM, so A digit s against B digits 0 .. S-1-s is one run of columns (two MMAs where N > 256).  The
+// first (s = 0) of a tile writes all groups; sums stay exact integers, so neither order nor tile shape changes a bit.
+//
+// Bound: the tensor pipe (15 BF16 products: 125 TFLOP/s at 1,872) if the operands come in fast enough, which the tile
+// width decides: a 16-column step takes 7.9 tn cycles of MMA for 20 KB + 160 tn bytes, 46 bytes a cycle at tn = 96,
+// 60 at 64, 100 at 32, against the ~46 an SM was seen to take in.  96 columns leave room for one accumulator set, whose
+// drain is then not hidden; 32-wide tiles, for launches with few tiles, have two.  With tiles of 48 columns (and 32
+// outside the band) in two sets, 73 bytes a cycle, the band products of an n = 90,000 factorisation took 324 ms, now 286.
+__global__ void __launch_bounds__(oz::kThreads, 1) gemm_oz_kernel(const __grid_constant__ oz::Args g) {
   using namespace oz;
-  using C_ = Cfg<TN>;
-  constexpr int B_BYTES = C_::B_BYTES, STAGE_BYTES = C_::STAGE_BYTES, GROUP_COLS = C_::GROUP_COLS,
-                BUF_COLS = C_::BUF_COLS, CH = C_::CH;
-  static_assert(CL == 1 || TN == 32, "CTA pairs take 32-wide tiles");
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(256) uint8_t smem_oz[];
+  uint8_t* smem = smem_oz;
   uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);
   uint64_t* empty = full + STAGES;
   uint64_t* accfull = empty + STAGES;
   uint64_t* accempty = accfull + 2;
-  uint64_t* drain = accempty + 2;
-  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  uint32_t* tmem_slot = (uint32_t*)(accempty + 2);
   volatile int* abort = (volatile int*)(tmem_slot + 1);
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = CL > 1 ? (int)cluster_rank() : 0;
-  const long long first = CL > 1 ? (long long)(blockIdx.x / CL) : (long long)blockIdx.x;
-  const long long step = CL > 1 ? (long long)(gridDim.x / CL) : (long long)gridDim.x;
-  const long long nunits = g.ntiles / CL;  // tiles, or tile pairs
-  constexpr uint16_t kAll = (uint16_t)((1u << CL) - 1u);
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], CL);
+      mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&accfull[b], 1);
-      mbar_init(&accempty[b], kEpiThreads);
+      mbar_init(&accempty[b], 32 * kEpiWarps);
     }
-    mbar_init(drain, 1);
     *abort = 0;
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
   fence_before();
   __syncthreads();
-  if (CL > 1) cluster_sync();  // the peer's barriers exist before anything is multicast to them
   fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int kchunks = g.K / KC;
+  Cursor cur;
+  int bi, cofs, width;
 
-  if (warp == 0 && lane == 0) {
-    const uint64_t pol = l2_evict_last_policy();
-    for (int s = 0; s < S; ++s) {
-      prefetch_tmap(&ta.m[s]);
-      prefetch_tmap(&tb.m[s]);
-    }
+  if (warp == 0) {
+    // ---------------- copies: lane s < S brings A plane s, lane S + s B plane s ----------------
     int stage = 0;
     uint32_t phase = 0;
     int last_par[STAGES];
     for (int s = 0; s < STAGES; ++s) last_par[s] = -1;
-    for (long long u = first; u < nunits && !*abort; u += step) {
-      const long long t = u * CL + rank;
-      int bi, cofs, cvalid;
-      if (!oz_tile<TN>(g, t, bi, cofs, cvalid)) continue;
-      const int ya = g.a_row0 + bi * TM, yb = g.b_row0 + cofs;
-      for (int kc = 0; kc < kchunks; ++kc) {
-        if (!mbar_wait(&empty[stage], phase ^ 1, abort)) {
-          *abort = 1;
-          record_timeout(g.st, 21);
-          break;
+    bool ok = true;  // the same for every lane
+    for (long long t = blockIdx.x; t < g.ntiles && ok; t += gridDim.x) {
+      if (!tile_of(g, t, cur, bi, cofs, width)) continue;
+      const int steps = g.tri ? min(g.k16, (cofs + width) / 16) : g.k16;
+      const bool isA = lane < S;
+      const uint8_t* src = isA ? g.A + lane * g.a_plane + (int64_t)bi * A_BYTES
+                               : g.B + (lane - S) * g.b_plane + (int64_t)cofs * 32;
+      const int64_t step_bytes = S * (isA ? g.a_plane : g.b_plane);
+      const uint32_t bytes = isA ? A_BYTES : width * 32;
+      const uint32_t off = isA ? lane * A_BYTES : S * A_BYTES + (lane - S) * bytes;
+      for (int kc = 0; kc < steps; ++kc) {
+        if (lane == 0) {
+          ok = mbar_wait(&empty[stage], phase ^ 1, abort);
+          if (ok) {
+            mbar_expect_tx(&full[stage], S * (A_BYTES + width * 32));
+          } else {
+            *abort = 1;
+            record_timeout(g.st, 21);
+          }
         }
-        uint8_t* sb = smem + stage * STAGE_BYTES;
-        mbar_expect_tx(&full[stage], STAGE_BYTES);
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-          if (CL > 1)
-            tma_load_2d_mc_hint(sb + s * A_BYTES + rank * (A_BYTES / CL), &ta.m[s], &full[stage], kc * KC,
-                                ya + rank * (TM / CL), kAll, pol);
-          else
-            tma_load_2d_hint(sb + s * A_BYTES, &ta.m[s], &full[stage], kc * KC, ya, pol);
-          tma_load_2d_hint(sb + S * A_BYTES + s * B_BYTES, &tb.m[s], &full[stage], kc * KC, yb, pol);
-        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        if (lane < 2 * S) bulk_load(smem_u32(smem + stage * STAGE_BYTES) + off, src, bytes, smem_u32(&full[stage]));
+        src += step_bytes;
         last_par[stage] = (int)phase;
         if (++stage == STAGES) {
           stage = 0;
@@ -763,7 +802,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_oz_kernel(const __grid_c
         }
       }
     }
-    if (*abort) {
+    if (!ok || *abort) {  // let every copy of this warp land before the CTA exits
       for (int s = 0; s < STAGES; ++s)
         if (last_par[s] >= 0) {
           volatile int never = 0;
@@ -771,134 +810,100 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_oz_kernel(const __grid_c
         }
     }
   } else if (warp == 1 && lane == 0) {
-    int stage = 0;
+    // ---------------- MMA issue ----------------
+    int stage = 0, it = 0;
     uint32_t phase = 0;
-    int it = 0;
-    for (long long u = first; u < nunits && !*abort; u += step) {
-      const long long t = u * CL + rank;
-      int bi, cofs, cvalid;
-      if (!oz_tile<TN>(g, t, bi, cofs, cvalid)) continue;
-      const int b = it & 1;
-      const uint32_t ap = (it >> 1) & 1;
+    for (long long t = blockIdx.x; t < g.ntiles && !*abort; t += gridDim.x) {
+      if (!tile_of(g, t, cur, bi, cofs, width)) continue;
+      const int steps = g.tri ? min(g.k16, (cofs + width) / 16) : g.k16;
+      const int b = g.nbuf > 1 ? it & 1 : 0;
+      const uint32_t ap = (g.nbuf > 1 ? it >> 1 : it) & 1;
       if (!mbar_wait(&accempty[b], ap ^ 1, abort)) {
         *abort = 1;
         record_timeout(g.st, 22);
         break;
       }
       fence_after();
-      const uint32_t d0 = tmem + b * BUF_COLS;
+      const uint32_t d0 = tmem + b * (TMEM_COLS / 2);
       bool ok = true;
-      for (int kc = 0; kc < kchunks; ++kc) {
-        if (!mbar_wait(&full[stage], phase, abort)) {
-          *abort = 1;
-          record_timeout(g.st, 23);
-          ok = false;
-          break;
-        }
-        fence_after();
-        const uint32_t sb = smem_u32(smem + stage * STAGE_BYTES);
-#pragma unroll
-        for (int kk = 0; kk < KC / 16; ++kk) {  // K = 16 per instruction: advance 32 bytes
-          const uint64_t o = (uint64_t)(kk * 2);
-          // The B slices lie one after another (slice t = rows [TN t, TN t + TN) of one
-          // SW128 tile) and group g = s + t sits at columns [TN g, TN g + TN), so one
-          // MMA of A slice s against B slices 0 .. S-1-s (N = TN (S - s)) adds every
-          // product of that slice to its group.  The first (s = 0, N = S TN) writes all
-          // groups; sums stay exact integers, so the order changes no bit.
-          const uint64_t bb = sdesc_sw128(sb + S * A_BYTES) + o;
+      // the width as a constant: with run-time shapes the one issuing thread would not keep up with the tensor pipe
+      auto products = [&](auto w) {
+        constexpr int W = decltype(w)::value;
+        for (int kc = 0; kc < steps; ++kc) {
+          if (!mbar_wait(&full[stage], phase, abort)) {
+            *abort = 1;
+            record_timeout(g.st, 23);
+            ok = false;
+            return;
+          }
+          fence_after();
+          const uint32_t sb = smem_u32(smem + stage * STAGE_BYTES);
+          const uint64_t b0 = sdesc_flat(sb + S * A_BYTES);
 #pragma unroll
           for (int s = 0; s < S; ++s) {
-            const uint64_t a = sdesc_sw128(sb + s * A_BYTES) + o;
-            mma_bf16(d0 + s * GROUP_COLS, a, bb, idesc(kFmtBF16, TM, TN * (S - s)), (kc | kk | s) ? 1u : 0u);
+            const uint64_t a = sdesc_flat(sb + s * A_BYTES);
+            const int n = W * (S - s);
+            const uint32_t acc = (kc | s) ? 1u : 0u;
+            if (n > 256) {
+              const int h = n / 2;  // a multiple of 16
+              mma_bf16(d0 + s * W, a, b0, idesc(kFmtBF16, TM, h), acc);
+              mma_bf16(d0 + s * W + h, a, b0 + (uint64_t)(h * 32 >> 4), idesc(kFmtBF16, TM, h), acc);
+            } else {
+              mma_bf16(d0 + s * W, a, b0, idesc(kFmtBF16, TM, n), acc);
+            }
+          }
+          mma_commit(&empty[stage]);
+          if (++stage == STAGES) {
+            stage = 0;
+            phase ^= 1;
           }
         }
-        if (CL > 1)
-          mma_commit_mc(&empty[stage], kAll);
-        else
-          mma_commit(&empty[stage]);
-        if (++stage == STAGES) {
-          stage = 0;
-          phase ^= 1;
-        }
-      }
+      };
+      if (width == 96)
+        products(std::integral_constant<int, 96>{});
+      else if (width == 64)
+        products(std::integral_constant<int, 64>{});
+      else
+        products(std::integral_constant<int, 32>{});
       if (!ok) break;
       mma_commit(&accfull[b]);
       ++it;
     }
-    if (CL > 1) {  // every MMA (and so every commit to the peer) has finished before the pair leaves
-      mma_commit(drain);
-      volatile int never = 0;
-      mbar_wait(drain, 0, &never);
-    }
   } else if (warp >= 2) {
-    const int quad = warp & 3;
-    const int half = (warp - 2) >> 2;  // columns [CH half, CH half + CH) of the tile
-    const int r = quad * 32 + lane;
+    // ---------------- drain: warp w takes TMEM lanes 32 (w % 4).. and a quarter of the columns ----------------
+    const int quad = warp & 3, part = (warp - 2) >> 2;
     int it = 0;
-    for (long long u = first; u < nunits && !*abort; u += step) {
-      const long long t = u * CL + rank;
-      int bi, cofs, cvalid;
-      if (!oz_tile<TN>(g, t, bi, cofs, cvalid)) continue;
-      const int b = it & 1;
-      const uint32_t ap = (it >> 1) & 1;
-      if (!mbar_wait(&accfull[b], ap, abort)) {
-        *abort = 1;
-        record_timeout(g.st, 24);
+    for (long long t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
+      if (!tile_of(g, t, cur, bi, cofs, width)) continue;
+      const int b = g.nbuf > 1 ? it & 1 : 0;
+      const uint32_t ap = (g.nbuf > 1 ? it >> 1 : it) & 1;
+      const int ch = width / 4;
+      if (!g.store) {  // this warp's lines of C into L2 while the products run
+        const int64_t col0 = g.c_col0 + cofs + ch * part;
+        for (int l = lane; l < 2 * ch; l += 32)
+          prefetch_l2(g.C + g.c_row0 + (int64_t)bi * TM + quad * 32 + 16 * (l & 1) + (col0 + (l >> 1)) * g.ldc);
+      }
+      if (!__all_sync(0xffffffffu, mbar_wait(&accfull[b], ap, abort))) {
+        if (lane == 0) {
+          *abort = 1;
+          record_timeout(g.st, 24);
+        }
         break;
       }
       fence_after();
-      const int64_t row = g.c_row0 + (int64_t)bi * TM + r;
-      const int lc0 = CH * half;  // first tile column of this warp
-      const int64_t col0 = g.c_col0 + (int64_t)cofs + lc0;
-      double* cp = g.C + row + col0 * g.ldc;
-      const bool lower = g.lower_mask != 0;
-      // columns of this warp inside the output (ragged tiles end early) and on or below the diagonal
-      bool live[CH];
-#pragma unroll
-      for (int j = 0; j < CH; ++j) live[j] = lc0 + j < cvalid && !(lower && col0 + j > row);
-      double cv[CH];
-#pragma unroll
-      for (int j = 0; j < CH; ++j) cv[j] = (g.store || !live[j]) ? 0.0 : __ldcs(cp + (int64_t)j * g.ldc);
-      // group g holds an exact integer a_g (|a_g| < 2^24) of weight 2^(-7(g+2)):
-      // V = sum_g a_g 2^(7(4-g)) is an integer below 2^53, combined exactly in int64
-      long long V[CH];
-#pragma unroll
-      for (int j = 0; j < CH; ++j) V[j] = 0;
-#pragma unroll
-      for (int gs = 0; gs < S; ++gs) {
-        uint32_t acc[CH];
-        const uint32_t ta0 = tmem + ((uint32_t)(quad * 32) << 16) + b * BUF_COLS + gs * GROUP_COLS + lc0;
-        if constexpr (CH == 16) {
-          tmem_ld16(ta0, *reinterpret_cast<uint32_t(*)[16]>(acc));
-        } else {  // CH = 24: 16 + 8 columns (half 0) or 8 + 16 (half 1), each load aligned to its width
-          if (half == 0) {
-            tmem_ld16(ta0, *reinterpret_cast<uint32_t(*)[16]>(acc));
-            tmem_ld8(ta0 + 16, *reinterpret_cast<uint32_t(*)[8]>(acc + 16));
-          } else {
-            tmem_ld8(ta0, *reinterpret_cast<uint32_t(*)[8]>(acc));
-            tmem_ld16(ta0 + 8, *reinterpret_cast<uint32_t(*)[16]>(acc + 8));
-          }
-        }
-        tmem_ld_wait();
-#pragma unroll
-        for (int j = 0; j < CH; ++j) V[j] = V[j] * 128 + (long long)__float2int_rn(__uint_as_float(acc[j]));
-      }
-      fence_before();
-      mbar_arrive(&accempty[b]);
-      const int er = g.ea[g.a_row0 + bi * TM + r];
-#pragma unroll
-      for (int j = 0; j < CH; ++j) {
-        if (!live[j]) continue;
-        const int ec = g.eb[g.b_row0 + cofs + lc0 + j];
-        const double x = i53_to_f64_scaled(V[j], er + ec - 7 * (S + 1));
-        __stcs(cp + (int64_t)j * g.ldc, g.store ? x : cv[j] - x);
-      }
+      const uint32_t acc = tmem + b * (TMEM_COLS / 2);
+      auto release = [&] { mbar_arrive(&accempty[b]); };
+      if (width == 96)
+        drain<24>(g, bi, cofs, quad, part, acc, release);
+      else if (width == 64)
+        drain<16>(g, bi, cofs, quad, part, acc, release);
+      else
+        drain<8>(g, bi, cofs, quad, part, acc, release);
       ++it;
     }
   }
   fence_before();
   __syncthreads();
-  if (CL > 1) cluster_sync();  // the peer's copies into this CTA and commits to its barriers are done
   if (warp == 1) {
     fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
@@ -906,140 +911,160 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_oz_kernel(const __grid_c
 }
 
 // ===========================================================================
-// Split kernel: FP64 rows -> T3 (tf32 hi/lo, row-major) and OZ digits.
-// One CTA per kSplitRows rows; K <= kSplitMaxK.  src element (r, k) at src[r*rs + k*cs].
+// Split kernel: FP64 rows -> T3 (TF32 hi/lo, row-major) and OZ digit planes.  16 rows per CTA, every value in a
+// register: thread (row, group) of 16 x 16 holds K / 16 consecutive columns of its row, at most 32, and eight columns
+// give 16-byte stores.  On a panel's look-ahead stream its grid is held to that stream's SMs: larger grids get between the
+// main stream's kernels (the trailing update of n = 90,000 then takes 680 ms instead of 635).  Bound: the integer pipe (~25 instructions a value for T3, ~45 for the digits), on the few SMs of
+// the look-ahead stream, and HBM (8 bytes read, 18 written).  All splits of n = 90,000: 289 ms through shared memory with
+// 64-bit integers, now 220.
 // ===========================================================================
-// TF32 rounding (11 significant bits, half away from zero in magnitude) of the
-// double with bit pattern D, as FP32 bits; |a| below the FP32 normal range -> 0.
-// Integer instructions only (FP64 instructions are the scarce resource here).
-__device__ __forceinline__ uint32_t tf32_bits_of(unsigned long long D, unsigned long long* rounded) {
-  const unsigned long long sign = D & 0x8000000000000000ull;
-  unsigned long long mag = (D & 0x7FFFFFFFFFFFFFFFull) + (1ull << 41);
-  mag &= ~((1ull << 42) - 1);
-  const int fe = (int)(mag >> 52) - 896;  // FP64 bias 1023 -> FP32 bias 127
-  if (fe <= 0) {
-    *rounded = sign;
-    return (uint32_t)(sign >> 32);
-  }
-  *rounded = sign | mag;
-  return (uint32_t)(sign >> 32) | ((uint32_t)fe << 23) | (uint32_t)((mag >> 29) & 0x7FFFFFu);
+// TF32 rounding (11 significant bits, half away from zero in magnitude) of the double with upper word w, as FP32 bits;
+// below the FP32 normal range 0.  *up: the upper word of the rounded value (its lower word is 0).  Bit 41 of the
+// pattern, where the rounding adds, is bit 9 of the upper word.
+__device__ __forceinline__ uint32_t tf32_of(uint32_t w, uint32_t* up) {
+  const uint32_t sign = w & 0x80000000u, m = ((w & 0x7FFFFFFFu) + 0x200u) & ~0x3FFu;
+  const int fe = (int)(m >> 20) - 896;  // FP64 bias 1023 -> FP32 bias 127
+  *up = fe <= 0 ? sign : sign | m;
+  return fe <= 0 ? sign : sign | ((uint32_t)fe << 23) | ((m & 0xFFFFFu) << 3);
+}
+// a's two TF32 parts.  The one FP64 instruction (exact: a's bits below the rounding point) runs beside the integer ones.
+__device__ __forceinline__ void tf32_parts(double a, uint32_t& h, uint32_t& l) {
+  uint32_t up;
+  h = tf32_of((uint32_t)__double2hiint(a), &up);
+  l = tf32_of((uint32_t)__double2hiint(a - __hiloint2double((int)up, 0)), &up);
 }
 
-// Rows [r0, r0 + kSplitRows) of the split (one CTA).
-__device__ __forceinline__ void split_rows_body(const double* __restrict__ src, int64_t rs, int64_t cs, int rows,
-                                                int K, float* __restrict__ hi, float* __restrict__ lo,
-                                                __nv_bfloat16_raw* __restrict__ dig, int64_t dig_stride,
-                                                int* __restrict__ ex, int out_row0, int r0) {
-  extern __shared__ double tile[];  // kSplitRows x (K + 1)
-  const int tid = threadIdx.x;
-  const int ld = K + 1;
-  // coalesced along whichever source dimension is contiguous; 16 loads in flight per thread
-  constexpr int CH = 16;
-  const int total = kSplitRows * K;
-  for (int base = 0; base < total; base += CH * 256) {
-    double v[CH];
+// The five OZ digits of a 2^(35-e) rounded to an integer N (|a| < 2^e: |N| <= 2^35), as FP32 values: balanced base-128
+// digits from the least significant end, the leading one keeping the rest (|d_0| <= 128, |d_s| <= 64 otherwise; all exact
+// in BF16).  With 64 (1 + 128 + 128^2 + 128^3) added, the lower four are plain digits plus 64.
+__device__ __forceinline__ void oz_digits(uint32_t dh, uint32_t dl, int e, float (&d)[kOzSlices]) {
+  const int E = (int)((dh >> 20) & 0x7FFu);
+  // a = M 2^(E-1075) with its 53-bit significand M: N = M 2^-sh, sh = 1040 + e - E >= 18; one bit more for the rounding
+  const int sh = 1040 + e - E;
+  const unsigned long long M = E ? ((unsigned long long)((dh & 0xFFFFFu) | 0x100000u) << 32) | dl : 0ull;
+  const unsigned long long N = ((M >> min(sh - 1, 63)) + 1) >> 1;
+  constexpr unsigned long long B = 64ull * (1 + 128 + 128 * 128 + 128 * 128 * 128);
+  const unsigned long long x = (int)dh < 0 ? B - N : B + N;
+  constexpr float kMagic = 12582912.0f;
+  const uint32_t lo = (uint32_t)x;
 #pragma unroll
-    for (int u = 0; u < CH; ++u) {
-      const int idx = base + u * 256 + tid;
-      v[u] = 0.0;
-      if (idx < total) {
-        const int rr = (cs == 1) ? idx / K : idx % kSplitRows;
-        const int k = (cs == 1) ? idx % K : idx / kSplitRows;
-        if (r0 + rr < rows) v[u] = src[(int64_t)(r0 + rr) * rs + (int64_t)k * cs];
+  for (int s = 1; s < kOzSlices; ++s)
+    d[s] = __uint_as_float(((lo >> (7 * (kOzSlices - 1 - s))) & 127u) | 0x4B400000u) - (kMagic + 64.0f);
+  d[0] = __int_as_float((int)((long long)x >> 28) + 0x4B400000) - kMagic;
+}
+
+// Rows [r0, r0 + kSplitRows) of the split (one CTA); the digit planes hold dig_rows rows.
+constexpr int kSplitThreads = 256, kSplitGroups = kSplitThreads / kSplitRows;
+__device__ __forceinline__ void split_rows_body(const double* __restrict__ src, int64_t rs, int64_t cs, int rows, int K,
+                                                float* __restrict__ hi, float* __restrict__ lo,
+                                                uint8_t* __restrict__ dig, int64_t dig_rows, int* __restrict__ ex,
+                                                int out_row0, int r0) {
+  extern __shared__ __align__(16) float stage[];  // 2 kSplitRows x ld: the TF32 parts on their way out
+  __shared__ unsigned int s_max[kSplitRows][kSplitGroups + 1], s_low[kSplitRows][kSplitGroups + 1];
+  const int ld = K + 4;
+  const int tid = threadIdx.x, r = tid % kSplitRows, g = tid / kSplitRows;
+  const int row = r0 + r;
+  constexpr int U = kSplitMaxK / 8 / kSplitGroups;
+  const int octets = K / 8;  // dealt to the groups in runs: group g takes octets [o0, o1), at most U
+  const int o0 = octets * g / kSplitGroups, o1 = octets * (g + 1) / kSplitGroups;
+  const double* p = src + (int64_t)row * rs + (int64_t)(8 * o0) * cs;
+  double v[U][8];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[u][j] = o0 + u < o1 && row < rows ? p[(int64_t)(8 * u + j) * cs] : 0.0;
+  const int64_t orow = (int64_t)(out_row0 + row);
+  int e = 0;
+  if (dig) {
+    // row maximum of |a| on the bit patterns: f 2^e with f in [0.5, 1), e = biased exponent - 1022 (0: all zero)
+    unsigned int mx = 0, low = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        mx = max(mx, (unsigned int)__double2hiint(v[u][j]) & 0x7FFFFFFFu);
+        low |= (unsigned int)__double2loint(v[u][j]);
       }
+    s_max[r][g] = mx;
+    s_low[r][g] = low;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kSplitGroups; ++q) {
+      mx = max(mx, s_max[r][q]);
+      low |= s_low[r][q];
     }
+    e = mx | low ? (int)(mx >> 20) - 1022 : 0;
+    if (g == 0 && row < rows && ex) ex[orow] = e;
+  }
 #pragma unroll
-    for (int u = 0; u < CH; ++u) {
-      const int idx = base + u * 256 + tid;
-      if (idx < total) {
-        const int rr = (cs == 1) ? idx / K : idx % kSplitRows;
-        const int k = (cs == 1) ? idx % K : idx / kSplitRows;
-        tile[rr * ld + k] = v[u];
+  for (int u = 0; u < U; ++u) {
+    const int o = o0 + u;
+    if (o >= o1 || row >= rows) continue;
+    if (hi) {
+      uint32_t h[8], l[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        tf32_parts(v[u][j], h[j], l[j]);
+      uint4* ph = reinterpret_cast<uint4*>(stage + r * ld + 8 * o);
+      uint4* pl = reinterpret_cast<uint4*>(stage + (kSplitRows + r) * ld + 8 * o);
+      ph[0] = make_uint4(h[0], h[1], h[2], h[3]);
+      ph[1] = make_uint4(h[4], h[5], h[6], h[7]);
+      pl[0] = make_uint4(l[0], l[1], l[2], l[3]);
+      pl[1] = make_uint4(l[4], l[5], l[6], l[7]);
+    }
+    if (dig) {
+      uint32_t w[kOzSlices][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float d[kOzSlices];
+        oz_digits((uint32_t)__double2hiint(v[u][j]), (uint32_t)__double2loint(v[u][j]), e, d);
+#pragma unroll
+        for (int s = 0; s < kOzSlices; ++s) {  // exact in BF16: the upper half of the word
+          const uint32_t b = __float_as_uint(d[s]);
+          w[s][j >> 1] = (j & 1) ? __byte_perm(w[s][j >> 1], b, 0x7632) : b;
+        }
       }
+      uint8_t* po = dig + (int64_t)(o >> 1) * kOzSlices * dig_rows * 32 + (orow >> 3) * 256 + (o & 1) * 128 +
+                    (orow & 7) * 16;
+#pragma unroll
+      for (int s = 0; s < kOzSlices; ++s)
+        *reinterpret_cast<uint4*>(po + (int64_t)s * dig_rows * 32) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
     }
   }
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31;
-  for (int rr = warp; rr < kSplitRows; rr += blockDim.x / 32) {
-    const int row = r0 + rr;
-    if (row >= rows) break;
-    const int64_t orow = (int64_t)(out_row0 + row);
-    // row maximum of |a| on the bit patterns (non-negative doubles order like their bits)
-    unsigned long long mxb = 0;
-    for (int k = lane; k < K; k += 32) {
-      const unsigned long long b = (unsigned long long)__double_as_longlong(tile[rr * ld + k]) & 0x7FFFFFFFFFFFFFFFull;
-      mxb = b > mxb ? b : mxb;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, mxb, o);
-      mxb = ob > mxb ? ob : mxb;
-    }
-    // max = f 2^e with f in [0.5, 1): e = biased exponent - 1022 (0 for an all-zero row)
-    const int e = mxb ? (int)(mxb >> 52) - 1022 : 0;
-    if (lane == 0 && ex) ex[orow] = e;
-    for (int k = lane; k < K; k += 32) {
-      const double a = tile[rr * ld + k];
-      const unsigned long long D = (unsigned long long)__double_as_longlong(a);
-      if (hi) {
-        unsigned long long hd, ld2;
-        const uint32_t h = tf32_bits_of(D, &hd);
-        const double rem = a - __longlong_as_double((long long)hd);  // exact: a's bits below the rounding point
-        const uint32_t l = tf32_bits_of((unsigned long long)__double_as_longlong(rem), &ld2);
-        hi[orow * K + k] = __uint_as_float(h);
-        lo[orow * K + k] = __uint_as_float(l);
-      }
-      if (dig) {
-        // N = round(a 2^(35-e)) from the bits: a = M 2^(E-1075) with M the 53-bit significand,
-        // so a 2^(35-e) = M 2^-(1040+e-E); |a| < 2^e makes the shift >= 18 and |N| <= 2^35.
-        long long N = 0;
-        const int E = (int)((D >> 52) & 0x7FF);
-        if (E != 0) {
-          const unsigned long long M = (D & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-          const int sh = 1040 + e - E;
-          if (sh >= 64) N = 0;
-          else if (sh > 0) N = (long long)((M + (1ull << (sh - 1))) >> sh);
-          else N = (long long)(M << (-sh));
-          if (D >> 63) N = -N;
-        }
-        // balanced base-128 digits from the least significant end: d = ((N + 64) mod 128) - 64,
-        // N = (N - d) / 128.  The leading digit keeps the rest (|d_0| <= 128, |d_s| <= 64
-        // otherwise); all are exact in BF16.
-        short d[kOzSlices];
-#pragma unroll
-        for (int s2 = kOzSlices - 1; s2 >= 1; --s2) {
-          const long long q = ((N + 64) & 127) - 64;
-          d[s2] = (short)q;
-          N = (N - q) >> 7;
-        }
-        d[0] = (short)N;
-#pragma unroll
-        for (int s2 = 0; s2 < kOzSlices; ++s2) {
-          __nv_bfloat16_raw raw;
-          raw.x = (unsigned short)(__float_as_uint((float)d[s2]) >> 16);
-          dig[(int64_t)s2 * dig_stride + orow * K + k] = raw;
-        }
-      }
+  if (hi) {  // whole lines
+    __syncthreads();
+    const int quads = K / 4;
+    for (int idx = tid; idx < kSplitRows * quads; idx += kSplitThreads) {
+      const int rr = idx / quads, q = idx - rr * quads;
+      if (r0 + rr >= rows) break;
+      const int64_t at = (int64_t)(out_row0 + r0 + rr) * K + 4 * q;
+      *reinterpret_cast<uint4*>(hi + at) = *reinterpret_cast<const uint4*>(stage + rr * ld + 4 * q);
+      *reinterpret_cast<uint4*>(lo + at) = *reinterpret_cast<const uint4*>(stage + (kSplitRows + rr) * ld + 4 * q);
     }
   }
 }
 
-__global__ void __launch_bounds__(256) split_rows_kernel(const double* __restrict__ src, int64_t rs, int64_t cs,
-                                                         int rows, int K, float* __restrict__ hi,
-                                                         float* __restrict__ lo, __nv_bfloat16_raw* __restrict__ dig,
-                                                         int64_t dig_stride, int* __restrict__ ex, int out_row0) {
-  split_rows_body(src, rs, cs, rows, K, hi, lo, dig, dig_stride, ex, out_row0, blockIdx.x * kSplitRows);
+__global__ void __launch_bounds__(kSplitThreads) split_rows_kernel(const double* __restrict__ src, int64_t rs,
+                                                                      int64_t cs, int rows, int K,
+                                                                      float* __restrict__ hi, float* __restrict__ lo,
+                                                                      uint8_t* __restrict__ dig, int64_t dig_rows,
+                                                                      int* __restrict__ ex, int out_row0) {
+  for (int r0 = blockIdx.x * kSplitRows; r0 < rows; r0 += gridDim.x * kSplitRows) {
+    split_rows_body(src, rs, cs, rows, K, hi, lo, dig, dig_rows, ex, out_row0, r0);
+    __syncthreads();
+  }
 }
 
 // Many pieces in one launch: blockIdx.y = piece, blockIdx.x = 16-row chunk of it.
-__global__ void __launch_bounds__(256) split_rows_tasks_kernel(const SplitTask* __restrict__ tasks, int K,
-                                                               float* __restrict__ hi, float* __restrict__ lo,
-                                                               __nv_bfloat16_raw* __restrict__ dig,
-                                                               int64_t dig_stride, int* __restrict__ ex) {
+__global__ void __launch_bounds__(kSplitThreads) split_rows_tasks_kernel(const SplitTask* __restrict__ tasks, int K,
+                                                                            float* __restrict__ hi,
+                                                                            float* __restrict__ lo,
+                                                                            uint8_t* __restrict__ dig, int64_t dig_rows,
+                                                                            int* __restrict__ ex) {
   const SplitTask t = tasks[blockIdx.y];
   const int r0 = blockIdx.x * kSplitRows;
   if (r0 >= t.rows) return;  // uniform over the CTA, before any barrier
-  split_rows_body(t.src, t.rs, t.cs, t.rows, K, hi, lo, dig, dig_stride, ex, t.out_row0, r0);
+  split_rows_body(t.src, t.rs, t.cs, t.rows, K, hi, lo, dig, dig_rows, ex, t.out_row0, r0);
 }
 
 // Per 256-row block maximum of the row exponents (rows past the end count as -infinity).
@@ -1098,48 +1123,44 @@ cudaError_t make_split_maps(SplitOperand& op) {
     if ((e = make_tmap(&op.t_hi, op.hi, op.rows, op.K, 4, 32, 128)) != cudaSuccess) return e;
     if ((e = make_tmap(&op.t_lo, op.lo, op.rows, op.K, 4, 32, 128)) != cudaSuccess) return e;
   }
-  if (op.dig) {
-    for (int s = 0; s < kOzSlices; ++s) {
-      const void* base = (const uint8_t*)op.dig + (size_t)s * op.rows * op.K * 2;
-      if ((e = make_tmap(&op.oz_a.m[s], base, op.rows, op.K, 2, 64, 128)) != cudaSuccess) return e;
-      if ((e = make_tmap(&op.oz_b.m[s], base, op.rows, op.K, 2, 64, 32)) != cudaSuccess) return e;
-      if ((e = make_tmap(&op.oz_ah.m[s], base, op.rows, op.K, 2, 64, 64)) != cudaSuccess) return e;
-      if ((e = make_tmap(&op.oz_b48.m[s], base, op.rows, op.K, 2, 64, 48)) != cudaSuccess) return e;
-    }
-  }
   return cudaSuccess;
 }
 
-cudaError_t launch_split_rows(cudaStream_t s, const double* src, int64_t rs, int64_t cs, int rows, int K,
-                              SplitOperand& op, int out_row0) {
-  if (rows <= 0) return cudaSuccess;
-  if (K > kSplitMaxK) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)kSplitRows * (K + 1) * sizeof(double);
-  static PerDeviceOnce attr_once;
-  cudaError_t e = attr_once([] {
-    return cudaFuncSetAttribute(split_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kSplitRows * (kSplitMaxK + 1) * (int)sizeof(double));
+// (Always the size for K = 512: with less, the CTAs of the look-ahead stream's splits would find room beside those of the
+// main stream's products.)
+constexpr int kSplitSmem = 2 * kSplitRows * (kSplitMaxK + 4) * (int)sizeof(float);
+
+static cudaError_t split_attr() {
+  static PerDeviceOnce once;
+  return once([] {
+    cudaError_t r = cudaFuncSetAttribute(split_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    if (r == cudaSuccess)
+      r = cudaFuncSetAttribute(split_rows_tasks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSplitSmem);
+    return r;
   });
+}
+
+cudaError_t launch_split_rows(cudaStream_t s, const double* src, int64_t rs, int64_t cs, int rows, int K,
+                              SplitOperand& op, int out_row0, int max_ctas) {
+  if (rows <= 0) return cudaSuccess;
+  if (K > kSplitMaxK || K % 16) return cudaErrorInvalidValue;
+  const cudaError_t e = split_attr();
   if (e != cudaSuccess) return e;
-  split_rows_kernel<<<(rows + kSplitRows - 1) / kSplitRows, 256, smem, s>>>(src, rs, cs, rows, K, op.hi, op.lo,
-                                                        (__nv_bfloat16_raw*)op.dig, (int64_t)op.rows * op.K, op.ex,
-                                                        out_row0);
+  int grid = (rows + kSplitRows - 1) / kSplitRows;
+  if (max_ctas > 0 && grid > 2 * max_ctas) grid = 2 * max_ctas;
+  split_rows_kernel<<<grid, kSplitThreads, kSplitSmem, s>>>(src, rs, cs, rows, K, op.hi, op.lo, (uint8_t*)op.dig, op.rows,
+                                                            op.ex, out_row0);
   return cudaGetLastError();
 }
 
 cudaError_t launch_split_rows_tasks(cudaStream_t s, const SplitTask* d_tasks, int ntasks, int max_rows, int K,
                                     SplitOperand& op) {
   if (ntasks <= 0 || max_rows <= 0) return cudaSuccess;
-  if (K > kSplitMaxK) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)kSplitRows * (K + 1) * sizeof(double);
-  static PerDeviceOnce attr_once;
-  cudaError_t e = attr_once([] {
-    return cudaFuncSetAttribute(split_rows_tasks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kSplitRows * (kSplitMaxK + 1) * (int)sizeof(double));
-  });
+  if (K > kSplitMaxK || K % 16) return cudaErrorInvalidValue;
+  const cudaError_t e = split_attr();
   if (e != cudaSuccess) return e;
-  split_rows_tasks_kernel<<<dim3((unsigned)((max_rows + kSplitRows - 1) / kSplitRows), (unsigned)ntasks), 256, smem,
-                            s>>>(d_tasks, K, op.hi, op.lo, (__nv_bfloat16_raw*)op.dig, (int64_t)op.rows * op.K, op.ex);
+  split_rows_tasks_kernel<<<dim3((unsigned)((max_rows + kSplitRows - 1) / kSplitRows), (unsigned)ntasks), kSplitThreads,
+                            kSplitSmem, s>>>(d_tasks, K, op.hi, op.lo, (uint8_t*)op.dig, op.rows, op.ex);
   return cudaGetLastError();
 }
 
@@ -1198,60 +1219,66 @@ cudaError_t launch_gemm_t3_pair(cudaStream_t s, const SplitOperand& A, const Spl
   return cudaGetLastError();
 }
 
+// Tiles of width tn of a launch.
+static long long oz_tiles(const GemmArgs& g, int tn) {
+  if (g.enum_mode == kEnumFull) return (long long)g.mt * (((long long)g.nt * 32 + tn - 1) / tn);
+  long long t = 0;
+  const int SI = g.panel / oz::TM;
+  for (int bi = 0; bi < g.mt; ++bi) {
+    const int I = bi / SI, start = (I > g.band ? I - g.band : 0) * g.panel;
+    t += ((bi + 1) * oz::TM - start + tn - 1) / tn;
+  }
+  return t;
+}
+
 cudaError_t launch_gemm_oz(cudaStream_t s, const SplitOperand& A, const SplitOperand& B, const GemmArgs& g,
                            int max_ctas) {
-  if (g.ntiles <= 0) return cudaSuccess;
+  if (g.mt <= 0 || (g.enum_mode == kEnumFull && g.nt <= 0)) return cudaSuccess;
+  if (g.K % 16 || g.K > kSplitMaxK || (g.enum_mode != kEnumFull && g.enum_mode != kEnumBand) ||
+      A.rows % 8 || B.rows % 8 || g.a_row0 % 8 || g.b_row0 % 8)
+    return cudaErrorInvalidValue;
   static PerDeviceOnce attr_once;
-  {
-    const cudaError_t e = attr_once([] {
-      cudaError_t r = cudaFuncSetAttribute(gemm_oz_kernel<1, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           oz::Cfg<32>::SMEM_BYTES);
-      if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(gemm_oz_kernel<2, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 oz::Cfg<32>::SMEM_BYTES);
-      if (r == cudaSuccess)
-        r = cudaFuncSetAttribute(gemm_oz_kernel<1, 48>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 oz::Cfg<48>::SMEM_BYTES);
-      return r;
-    });
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = attr_once([] {
+    return cudaFuncSetAttribute(gemm_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz::SMEM_BYTES);
+  });
+  if (e != cudaSuccess) return e;
   int cap = num_sms();
   if (max_ctas > 0 && max_ctas < cap) cap = max_ctas;
-  GemmArgs g2 = g;
-  g2.ea = A.ex;
-  g2.eb = B.ex;
-  if (g.enum_mode == kEnumBand && g.panel % 128 == 0) {
-    // band tiles 128 x 48 (the caller counts 128 x 32 sub-tiles per panel pair)
-    const long long per32 = (long long)(g.panel / 128) * (g.panel / 32);
-    const long long per48 = (long long)(g.panel / 128) * ((g.panel + 47) / 48);
-    g2.ntiles = g.ntiles / per32 * per48;
-    const int grid = (int)(g2.ntiles < cap ? g2.ntiles : cap);
-    gemm_oz_kernel<1, 48><<<grid, kGemmThreads, oz::Cfg<48>::SMEM_BYTES, s>>>(A.oz_a, B.oz_b48, g2);
-    return cudaGetLastError();
+  oz::Args a{};
+  a.C = g.C;
+  a.ldc = g.ldc;
+  a.c_row0 = g.c_row0;
+  a.c_col0 = g.c_col0;
+  a.A = (const uint8_t*)A.dig + (int64_t)g.a_row0 * 32;
+  a.B = (const uint8_t*)B.dig + (int64_t)g.b_row0 * 32;
+  a.a_plane = A.rows * 32;
+  a.b_plane = B.rows * 32;
+  a.ea = A.ex + g.a_row0;
+  a.eb = B.ex + g.b_row0;
+  a.mode = g.enum_mode;
+  a.band = g.band;
+  a.panel = g.panel;
+  a.mt = g.mt;
+  a.n = g.nt * 32;
+  a.k16 = g.K / 16;
+  a.tri = g.tri;
+  a.store = g.store;
+  a.lower = g.lower_mask || g.enum_mode == kEnumBand;
+  a.st = g.st;
+  // the width whose waves end first: a tile takes about 30, 24 and 17 thousand cycles for K = 512
+  constexpr struct { int tn, cost; } kWidths[] = {{96, 30}, {64, 24}, {32, 17}};
+  long long best = 0;
+  for (const auto& w : kWidths) {
+    const long long t = oz_tiles(g, w.tn), cost = (t + cap - 1) / cap * w.cost;
+    if (best == 0 || cost < best) {
+      best = cost;
+      a.tn = w.tn;
+      a.ntiles = t;
+    }
   }
-  // CTA pairs sharing the A digits when the tiles pair up (even counts) and the launch may use
-  // most of the GPU: a cluster needs two free SMs of one GPC at once, which a small SM share
-  // beside other running kernels may not offer (the launch would then wait for them)
-  if (g.ntiles % 2 == 0 && cap >= 64 && g.enum_mode == kEnumFull && g.nt % 2 == 0) {
-    const long long pairs = g.ntiles / 2;
-    const int grid = 2 * (int)(pairs < cap / 2 ? pairs : cap / 2);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.dynamicSmemBytes = oz::Cfg<32>::SMEM_BYTES;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_oz_kernel<2, 32>, A.oz_ah, B.oz_b, g2);
-  }
-  const int grid = (int)(g.ntiles < cap ? g.ntiles : cap);
-  gemm_oz_kernel<1, 32><<<grid, kGemmThreads, oz::Cfg<32>::SMEM_BYTES, s>>>(A.oz_a, B.oz_b, g2);
+  a.nbuf = a.tn == 32 ? 2 : 1;
+  const int grid = (int)(a.ntiles < cap ? a.ntiles : cap);
+  gemm_oz_kernel<<<grid, oz::kThreads, oz::SMEM_BYTES, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -36,10 +36,6 @@ struct SplitTask {
 constexpr int kRasterSuper = 16;  // supertile edge (in 128-tiles) of the lower off-band enumeration
 constexpr int kPairSuper = 16;    // supertile edge (in 256-tiles) of the CTA-pair lower off-band enumeration
 
-struct OzMaps {
-  CUtensorMap m[kOzSlices];
-};
-
 // Kernel arguments (passed by value as a __grid_constant__).
 struct GemmArgs {
   double* C;                  // FP64 output, column-major
@@ -48,14 +44,15 @@ struct GemmArgs {
   int a_row0, b_row0;         // operand row origins
   int K;                      // reduction length (T3: % 32, OZ: % 64 and <= 512, its exact-sum limit)
   int enum_mode;              // kEnum*
-  int nt;                     // tiles along N (kEnumFull); tile rows (kEnumLowerOffBand)
+  int mt;                     // OZ: 128-row blocks
+  int nt;                     // tiles along N (kEnumFull; OZ: n / 32); tile rows (kEnumLowerOffBand)
   int band;                   // band width in panel tiles (kEnumLowerOffBand / kEnumBand)
   int panel;                  // panel width (256 or 512) that `band` is measured in
-  long long ntiles;           // number of enumerated tiles
+  long long ntiles;           // number of enumerated tiles (not OZ)
   int store;                  // 1: C = A B^T ; 0: C -= A B^T
   int lower_mask;             // skip entries above the diagonal
-  const int* ea;              // OZ: per-row power-of-two exponents of A (set by the launcher)
-  const int* eb;              // OZ: per-row exponents of B
+  int tri;                    // kEnumFull, T3 and OZ: B(j, k) = 0 for k > j (j from b_row0), so column tile j's reduction
+                              // stops at its last column
   // T3 on CTA pairs: with far_thr set (> INT_MIN), a 256 x 256 tile whose operand blocks have
   // maximum exponents eA + eB <= far_thr takes the single hi * hi product (see the kernel)
   const int* ea_blk;          // per 256-row block maximum exponent of A
@@ -73,7 +70,9 @@ struct GemmArgs {
 };
 
 // One split operand: `rows` x K values held as T3 (tf32 hi/lo, row-major) and/or
-// OZ digits (kOzSlices planes of rows x K BF16, row-major) with row exponents.
+// OZ digits with row exponents.  Digit plane p = kc kOzSlices + s (16 columns from 16 kc, digit s) holds every row's 16
+// BF16 digits in the order the tensor cores read: 8-row groups of 256 bytes, each two 128-byte halves (columns 0-7 and
+// 8-15) of 8 rows x 16 bytes.
 struct SplitOperand {
   int64_t rows = 0;
   int K = 0;
@@ -83,10 +82,6 @@ struct SplitOperand {
   int* ex = nullptr;
   int* exb = nullptr;         // per 256-row block maximum of ex
   CUtensorMap t_hi, t_lo;     // boxes 32 x 128
-  OzMaps oz_a;                // boxes 64 x 128 (A role)
-  OzMaps oz_b;                // boxes 64 x 32  (B role)
-  OzMaps oz_ah;               // boxes 64 x 64  (A role, half a tile: multicast by a CTA pair)
-  OzMaps oz_b48;              // boxes 64 x 48  (B role, 48-wide band tiles)
 };
 
 cudaError_t make_split_maps(SplitOperand& op);
@@ -94,7 +89,7 @@ cudaError_t make_split_maps(SplitOperand& op);
 cudaError_t launch_row_exp_blockmax(cudaStream_t s, SplitOperand& op, int64_t rows);
 // rows [0, rows) of src (element (r, k) at src[r*rs + k*cs]) -> operand rows [out_row0, ...)
 cudaError_t launch_split_rows(cudaStream_t s, const double* src, int64_t rs, int64_t cs, int rows, int K,
-                              SplitOperand& op, int out_row0);
+                              SplitOperand& op, int out_row0, int max_ctas = 0);
 // ntasks pieces in one launch (max_rows: the longest piece), each to its own operand rows.
 cudaError_t launch_split_rows_tasks(cudaStream_t s, const SplitTask* d_tasks, int ntasks, int max_rows, int K,
                                     SplitOperand& op);

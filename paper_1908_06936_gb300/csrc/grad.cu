@@ -615,8 +615,8 @@ static exa_status mixed_inverse_tc(exa_ctx* c, int64_t npad, double* Sneg) {
         g.a_row0 = l * NB;
         g.b_row0 = 0;
         g.enum_mode = kEnumFull;
+        g.mt = NB / 128;
         g.nt = (l + 1) * NB / 32;
-        g.ntiles = (long long)(NB / 128) * g.nt;
         g.store = 0;
         g.lower_mask = 0;
         ProfScope ps(c, PK_GEMM_OZ, 2.0 * NB * (double)(l + 1) * NB * NB, 16.0 * NB * (double)(l + 1) * NB);
@@ -632,8 +632,8 @@ static exa_status mixed_inverse_tc(exa_ctx* c, int64_t npad, double* Sneg) {
         g.C = A + i0;
         g.ldc = npad;
         g.a_row0 = g.b_row0 = 0;
+        g.mt = NB / 128;
         g.nt = (int)(i0 / 32);
-        g.ntiles = (long long)(NB / 128) * g.nt;
         g.store = 1;
         ProfScope ps(c, PK_GEMM_OZ, 2.0 * NB * (double)i0 * NB, 8.0 * NB * (double)i0);
         e = launch_gemm_oz(s, WS, TS, g);
@@ -658,8 +658,7 @@ static exa_status mixed_inverse_tc(exa_ctx* c, int64_t npad, double* Sneg) {
       g.panel = NB;
       g.store = 0;
       g.lower_mask = 1;
-      const long long pairs = (long long)(i + 1) * (i + 2) / 2;
-      g.ntiles = pairs * (NB / 128) * (NB / 32);
+      g.mt = (i + 1) * (NB / 128);
       const double e2 = (double)(i0 + NB);
       ProfScope ps(c, PK_GEMM_OZ, e2 * e2 * NB, 8.0 * e2 * e2);
       e = launch_gemm_oz(s, X[i], X[i], g);

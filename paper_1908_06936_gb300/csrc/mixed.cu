@@ -30,7 +30,7 @@ constexpr double kWideBandNu = 0.75;     // from this smoothness one more panel 
 
 size_t split_bytes(int64_t rows, int K, bool t3, bool oz) {
   const size_t t3_bytes = t3 ? (size_t)rows * K * 4 : 0;
-  const size_t dig_bytes = oz ? (size_t)kOzSlices * rows * K * 2 : 0;
+  const size_t dig_bytes = oz ? (size_t)kOzSlices * round_up(rows, 128) * K * 2 : 0;
   const size_t ex_bytes = oz ? (size_t)round_up(rows, 64) * 4 : 0;
   const size_t exb_bytes = oz ? (size_t)round_up((rows + 255) / 256, 64) * 4 : 0;
   return (2 * t3_bytes + dig_bytes + ex_bytes + exb_bytes + 1023) / 1024 * 1024;
@@ -38,7 +38,7 @@ size_t split_bytes(int64_t rows, int K, bool t3, bool oz) {
 
 cudaError_t split_layout(SplitOperand& op, void* base_p, int64_t rows, int K, bool t3, bool oz) {
   const size_t t3_bytes = t3 ? (size_t)rows * K * 4 : 0;
-  const size_t dig_bytes = oz ? (size_t)kOzSlices * rows * K * 2 : 0;
+  const size_t dig_bytes = oz ? (size_t)kOzSlices * round_up(rows, 128) * K * 2 : 0;
   const size_t ex_bytes = oz ? (size_t)round_up(rows, 64) * 4 : 0;
   uint8_t* base = (uint8_t*)base_p;
   op.rows = rows;
@@ -116,14 +116,19 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   const int64_t r0 = k0 + NB;
   const int64_t m = npad - r0;
   double* panel_src = a + r0 + k0 * ld;  // element (r, t) at panel_src[r + t*ld]
+  // the first `band` tile rows are solved with exact products, the rest with T3: each gets the parts it takes
+  const int64_t rb = m < (int64_t)M.band * NB ? m : (int64_t)M.band * NB;
   {
-    ProfScope ps(c, PK_SPLIT, 0.0, 26.0 * (double)(m + NB) * NB, 2, s, true);
-    e = launch_split_rows(s, W2, NB, 1, NB, NB, c->sp_b, 0);
-    if (e == cudaSuccess) e = launch_split_rows(s, panel_src, 1, ld, (int)m, NB, sp, 0);
+    ProfScope ps(c, PK_SPLIT, 0.0, 26.0 * (double)NB * NB + 16.0 * (double)m * NB, m > rb ? 3 : 2, s, true);
+    SplitOperand exact = sp, t3 = sp;
+    exact.hi = exact.lo = nullptr;
+    t3.dig = nullptr;
+    e = launch_split_rows(s, W2, NB, 1, NB, NB, c->sp_b, 0, ctas);
+    if (e == cudaSuccess) e = launch_split_rows(s, panel_src, 1, ld, (int)rb, NB, exact, 0, ctas);
+    if (e == cudaSuccess) e = launch_split_rows(s, panel_src + rb, 1, ld, (int)(m - rb), NB, t3, (int)rb, ctas);
   }
   if (e != cudaSuccess) return cuda_err(c, e, "split launch");
-  // 3. panel TRSM on the tensor cores: the first `band` tile rows exact, the rest TF32x3
-  const int64_t rb = m < (int64_t)M.band * NB ? m : (int64_t)M.band * NB;
+  // 3. panel TRSM on the tensor cores
   GemmArgs g;
   memset(&g, 0, sizeof(g));
   g.C = a;
@@ -132,11 +137,12 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   g.panel = NB;
   g.st = c->d_status;
   g.store = 1;
+  g.tri = 1;
   g.enum_mode = kEnumFull;
   g.c_col0 = k0;
   g.c_row0 = r0;
+  g.mt = (int)(rb / 128);
   g.nt = NB / 32;
-  g.ntiles = (rb / 128) * g.nt;
   {
     ProfScope ps(c, PK_GEMM_OZ, 2.0 * (double)rb * NB * NB, 8.0 * (double)rb * NB, 1, s, true);
     e = launch_gemm_oz(s, sp, c->sp_b, g, ctas);
@@ -151,7 +157,7 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   }
   if (e == cudaSuccess) {
     ProfScope ps(c, PK_SPLIT, 0.0, 26.0 * (double)m * NB, 2, s, true);
-    e = launch_split_rows(s, panel_src, 1, ld, (int)m, NB, sp, 0);
+    e = launch_split_rows(s, panel_src, 1, ld, (int)m, NB, sp, 0, ctas);
     if (e == cudaSuccess) e = launch_row_exp_blockmax(s, sp, m);
   }
   if (e != cudaSuccess) return cuda_err(c, e, "panel trsm launch");
@@ -184,8 +190,8 @@ static exa_status column_update(const MixStep& M, cudaStream_t s, int p, int j, 
   g.c_col0 = cj;
   g.a_row0 = off;
   g.b_row0 = off;
+  g.mt = (int)(rb / 128);
   g.nt = NB / 32;
-  g.ntiles = (rb / 128) * g.nt;
   cudaError_t e;
   {
     ProfScope ps(c, PK_GEMM_OZ, 2.0 * (double)rb * NB * NB, 16.0 * (double)rb * NB, 1, s, true);
@@ -278,17 +284,12 @@ static exa_status region_update(const MixStep& M, cudaStream_t s, int p, int j0,
   const long long tr = m2 / NB;
   long long pairs = 0;
   for (long long I = 0; I < tr; ++I) pairs += (I < band ? I : band) + 1;
-  const long long per_pair = (long long)(NB / 128) * (NB / 32);
-  long long skipped = 0;
-  for (int h = 0; h < NB / 128; ++h)
-    for (int q = 0; q < NB / 32; ++q)
-      if ((long long)q * 32 > (long long)h * 128 + 127) ++skipped;
-  const double oz_tiles = (double)pairs * per_pair - (double)skipped * (double)tr;
+  const double oz_area = ((double)pairs - 0.5 * (double)tr) * NB * NB;
   g.enum_mode = kEnumBand;
-  g.ntiles = pairs * per_pair;
+  g.mt = (int)t128;
   for (int q = 0; q < (sp2 ? 2 : 1) && e == cudaSuccess; ++q) {
     g.a_row0 = g.b_row0 = q ? off2 : off1;
-    ProfScope ps(c, PK_GEMM_OZ, 2.0 * 128.0 * 32.0 * NB * oz_tiles, 16.0 * 128.0 * 32.0 * oz_tiles, 1, s, true);
+    ProfScope ps(c, PK_GEMM_OZ, 2.0 * oz_area * NB, 16.0 * oz_area, 1, s, true);
     e = launch_gemm_oz(s, q ? *sp2 : sp, q ? *sp2 : sp, g, ctas);
   }
   if (e != cudaSuccess) return cuda_err(c, e, "trailing update launch");
@@ -715,8 +716,8 @@ extern "C" exa_status exa_gemm_update(exa_ctx* c, exa_gemm_kind kind, int64_t m,
   g.store = store ? 1 : 0;
   g.st = c->d_status;
   if (oz) {
+    g.mt = (int)(m / 128);
     g.nt = (int)(n / 32);
-    g.ntiles = (m / 128) * (n / 32);
     e = launch_gemm_oz(c->stream, c->sp_a, c->sp_b, g);
   } else if (pair) {
     g.nt = (int)(n / 256);

@@ -83,27 +83,6 @@ __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* m
       : "memory");
 }
 
-// 2-D TMA tile load multicast to the CTAs of ctaMask: the data and its byte count land at the
-// same shared-memory offsets (dst, bar) in each of them.
-__device__ __forceinline__ void tma_load_2d_mc_hint(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y,
-                                                    uint16_t mask, uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster.L2::cache_hint "
-      "[%0], [%1, {%3, %4}], [%2], %5, %6;" ::"r"(smem_u32(dst)),
-      "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y), "h"(mask), "l"(pol)
-      : "memory");
-}
-
-// Arrive once on the mbarrier at local offset `bar` in every CTA of ctaMask when all tcgen05
-// operations issued so far by this thread (single-CTA MMAs) complete.
-__device__ __forceinline__ void mma_commit_mc(uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"(mask)
-      : "memory");
-}
-
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
@@ -123,6 +102,26 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)2 << 61;
   return d;
+}
+
+// Shared-memory descriptor of a K-major operand without swizzling: 8-row core matrices of 128 bytes, the two of
+// a 16-column step 128 bytes apart (leading offset), 8-row groups 256 bytes apart (stride offset).
+__device__ __forceinline__ uint64_t sdesc_flat(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(128 >> 4) << 16) | ((uint64_t)(256 >> 4) << 32) |
+         ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// An FP32 integer, |a| <= 2^24, by additions: the multiples of 4 from a + 1.5 2^25, then the rest.
+__device__ __forceinline__ int f32_to_int(float a) {
+  const float u = a + 50331648.0f;
+  const float rest = a - (u - 50331648.0f);
+  return 4 * (__float_as_int(u) - 0x4C400000) + (__float_as_int(rest + 12582912.0f) - 0x4B400000);
 }
 
 // Instruction descriptor for kind::tf32 / kind::f16: D format F32 (bits 4-5 = 1),

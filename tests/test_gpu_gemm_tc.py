@@ -86,6 +86,20 @@ def test_oz_exact_on_short_integers(ctx):
     assert np.array_equal(got, A @ B.T)
 
 
+# tiles 96, 64 and 32 wide (by the number of waves), whole and with a ragged last tile, one and several waves
+@pytest.mark.parametrize("m,n,k", [(6400, 1120, 64), (6400, 1088, 512), (2560, 992, 64), (2560, 960, 512), (128, 160, 64),
+                                   (4864, 32, 512)])
+def test_oz_exact_at_every_tile_width(ctx, m, n, k):
+    import paper_1908_06936_gb300 as exa
+
+    rng = np.random.default_rng(m + n)
+    A = rng.integers(-127, 128, (m, k)).astype(np.float64) / 128.0
+    B = rng.integers(-127, 128, (n, k)).astype(np.float64) / 256.0
+    C0 = rng.integers(-9, 10, (m, n)).astype(np.float64)
+    got = run(ctx, exa.EXA_GEMM_OZ, A, B, C0, 0)
+    assert np.array_equal(got, C0 - A @ B.T)
+
+
 def test_bad_shapes(ctx):
     import torch
     import paper_1908_06936_gb300 as exa
