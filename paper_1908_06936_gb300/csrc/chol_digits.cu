@@ -48,20 +48,17 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
   return ok;
 }
 
-// Grids of the diagonal block and what it takes on them (512 rows, measured): beyond 104 CTAs nothing is gained.
-constexpr struct { int ctas; double us; } kDiagGrids[] = {{104, 426.0}, {64, 464.0}, {32, 698.0}, {16, 1180.0}};
-
 // The look-ahead stream's share of the GPU beside a trailing update of m rows (m^2 512 operations at 42 TFLOP/s on the
-// whole GPU): the grid with which the later of the two ends first.
+// whole GPU): the grid of the diagonal block with which the later of the two ends first.
 static int side_share(int64_t m, int sms) {
   const double update_us = (double)m * (double)m * kNB / 42e6;
-  int best = kDiagGrids[0].ctas;
+  int best = kDiagCtas;
   double best_us = 0.0;
-  for (const auto& g : kDiagGrids) {
-    const double us = std::max(g.us, update_us * sms / (sms - g.ctas));
+  for (int ctas = kDiagCtas; ctas >= 16; ctas -= 8) {
+    const double us = std::max(diag_block_us(ctas), update_us * sms / (sms - ctas));
     if (best_us == 0.0 || us < best_us) {
       best_us = us;
-      best = g.ctas;
+      best = ctas;
     }
   }
   return best;
@@ -111,7 +108,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     }
     return e;
   };
-  cudaError_t e = diagonal(ms, 0, kDiagGrids[0].ctas);
+  cudaError_t e = diagonal(ms, 0, kDiagCtas);
   for (int k = 0; k + 1 < T && e == cudaSuccess; ++k) {
     const int64_t k0 = (int64_t)k * kNB, r0 = k0 + kNB, m = npad - r0;
     const double dm = (double)m;

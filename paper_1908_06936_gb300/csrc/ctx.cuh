@@ -19,7 +19,7 @@ struct DevBuf {
 
 constexpr int kNumEvents = 8;
 constexpr int kMixPanel = 512;     // panel width of the mixed-precision factorisation
-constexpr int kDiagCtas = 64;      // CTAs of one diagonal-block launch at most (mixed path)
+constexpr int kDiagCtas = 104;    // CTAs of one diagonal-block launch at most
 constexpr int kRedPartials = 512;  // partial sums of one two-stage reduction
 
 inline int64_t kPartialDoubles(int64_t npad, int nb) { return 2 * kRedPartials + (npad / 1024 + 2) * (int64_t)nb; }
@@ -32,7 +32,7 @@ struct exa_ctx {
   size_t ws_limit = 0;   // 0: unbounded
   size_t held_bytes = 0;
   int tile_nb = 128;     // FP64 tile
-  int lookahead_sms = 0;  // SMs reserved for the look-ahead stream (0: default)
+  int lookahead_sms = 0;  // SMs reserved for the look-ahead stream (0: by the rows left)
   int64_t late_rows = -1; // one-panel phase: below this many trailing rows the look-ahead share grows (-1: default)
   int late_sms = 0;       // ... linearly up to this many SMs at late_rows / 3 (0: default)
   int64_t fuse_min_rows = -1;  // two-panel trailing passes down to this many rows (0: off, < 0: default)

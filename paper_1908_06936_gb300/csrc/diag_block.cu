@@ -606,6 +606,17 @@ cudaError_t launch_diag128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, in
   return cudaLaunchKernelEx(&cfg, diag_tasks_kernel, d_tasks);
 }
 
+double diag_block_us(int ctas) {
+  static const struct { int ctas; double us; } kAt[] = {{16, 1180.0}, {32, 698.0}, {64, 464.0}, {104, 426.0}};
+  if (ctas <= kAt[0].ctas) return kAt[0].us * kAt[0].ctas / ctas;
+  for (int i = 1; i < 4; ++i)
+    if (ctas <= kAt[i].ctas) {  // linear in the reciprocal
+      const double f = (1.0 / ctas - 1.0 / kAt[i].ctas) / (1.0 / kAt[i - 1].ctas - 1.0 / kAt[i].ctas);
+      return kAt[i].us + f * (kAt[i - 1].us - kAt[i].us);
+    }
+  return kAt[3].us;
+}
+
 size_t diag_block_scratch_doubles() { return (size_t)kDiagScratch; }
 
 cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0, double* w_sub, double* logdet_part,

@@ -167,6 +167,8 @@ cudaError_t launch_diag128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, in
 // diag_block_scratch_doubles() doubles.  size: 512, or for the last block of a matrix a smaller multiple of 128
 // (then w2 is scratch: only the sub-tile inverses are formed).
 size_t diag_block_scratch_doubles();
+// What a 512 block takes on a grid (measured), microseconds.  Nothing is gained beyond 104 CTAs.
+double diag_block_us(int ctas);
 cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0, double* w_sub, double* logdet_part,
                               double* w2, double* scratch, DevStatus* st, int grid, int size = 512);
 

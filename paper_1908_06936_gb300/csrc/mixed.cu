@@ -20,9 +20,10 @@ constexpr double kIrQuadTol = 1e-8;   // refinement stops once q is final to thi
 // below the true error of the quadratic form on smooth fields (the residual of a preconditioned
 // step gathers in the directions where Sigma^-1 is large); they are taken 100 times over.
 constexpr double kIrQuadSafety = 100.0;
-constexpr int kLookaheadSMs = 20;         // SMs left to the look-ahead stream during a trailing update
+constexpr int kLookaheadSMs = 20;         // fewest SMs left to the look-ahead stream during a trailing update
 constexpr int64_t kFuseMinRows = 40960;   // two panels per trailing pass down to this many rows
-constexpr int64_t kLateRows = 61440;      // one-panel phase: the look-ahead share grows below this many rows
+constexpr int64_t kLateRows = 61440;      // where the caller sets one of the shares, the others' defaults: one-panel
+                                          // phase, the look-ahead share grows below this many rows
 constexpr int kLateSMs = 48;              // ... up to this many SMs
 constexpr double kExactThreshold = 0.8;  // tiles holding |Sigma_ij| >= 0.8 sigma^2 get exact products
 constexpr double kSmoothNu = 1.2;        // above this smoothness every tile gets exact products
@@ -103,8 +104,7 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   // 1. FP64 Cholesky of the diagonal block, its 128 sub-tile inverses and log sums, and
   // 2. its inverse W = L_kk^-1: one cooperative launch (diag_block.cu)
   {
-    // one CTA per SM of the look-ahead share, 64 at most (the block's parallel phases gain
-    // little beyond: 1.45 ms on 32 CTAs, 1.33 ms on 64)
+    // one CTA per SM of the look-ahead share
     const int grid = ctas > 0 ? (ctas < kDiagCtas ? ctas : kDiagCtas) : kDiagCtas;
     const double nb3 = (double)NB * NB * NB;
     ProfScope ps(c, PK_POTRF, 2.0 * nb3 / 3.0, 8.0 * (3.0 * NB * NB + 4.0 * nb * nb), 1, s, true);
@@ -296,7 +296,28 @@ static exa_status region_update(const MixStep& M, cudaStream_t s, int p, int j0,
   return EXA_OK;
 }
 
-// Mixed-precision tiled Cholesky with look-ahead on a side stream (kLookaheadSMs SMs
+// SMs for the look-ahead stream while the main stream updates m trailing rows from `panels` panels: with them the later
+// of the two streams ends first.  A panel of m rows takes the diagonal block and then ~1.6 us a row and SM (splits and
+// solves; a second panel also its column's update, 0.3), the update 3e-6 us m^2 a panel on 132 SMs (fitted to timelines
+// of n = 40,000 and 90,000).  Below 20 SMs the two streams' shares of the memory system no longer follow their SMs.
+// With 20 SMs, and 20 to 48 below 61,440 rows, n = 40,000 took 184 ms (now 177), n = 90,000 1,189 (1,178), the n = 10,000
+// gradient 42.6 (39.2).
+static int lookahead_share(int64_t m, int panels, int sms) {
+  int best = 0;
+  double best_us = 0.0;
+  for (int s = kLookaheadSMs; s <= kDiagCtas && s < sms - 2; s += 4) {
+    const double side = panels * (diag_block_us(s) + 1.6 * (double)m / s) + (panels - 1) * 0.3 * (double)m / s;
+    const double main = panels * 3e-6 * (double)m * (double)m * 132.0 / (sms - s);
+    const double us = side > main ? side : main;
+    if (best == 0 || us < best_us) {
+      best_us = us;
+      best = s;
+    }
+  }
+  return best;
+}
+
+// Mixed-precision tiled Cholesky with look-ahead on a side stream (some SMs
 // reserved for it during the big trailing updates).  Panel splits rotate through four
 // buffers (panel k in buffer k mod 4), so the side stream never overwrites operands
 // still in use.
@@ -346,7 +367,7 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   cudaStream_t ms = c->stream, ss = c->side;
   const int sms = tc_num_sms();
   const int side_ctas = c->lookahead_sms > 0 ? c->lookahead_sms : kLookaheadSMs;
-  const int main_ctas = sms - side_ctas;
+  const bool by_rows = c->lookahead_sms <= 0 && c->late_rows < 0 && c->late_sms <= 0;
   auto B = [&](int p) -> SplitOperand& { return *buf[p % nbuf]; };
   // panel 0 on the main stream
   if ((st = panel_factor(M, ms, 0, B(0), 0)) != EXA_OK) return st;
@@ -361,11 +382,12 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
           if ((st = column_update(M, ms, p, j, B(p), 0)) != EXA_OK) return st;
       cudaEventRecord(c->la_ev[0], ms);
       cudaStreamWaitEvent(ss, c->la_ev[0], 0);
-      if ((st = panel_factor(M, ss, k + 2, B(k + 2), side_ctas)) != EXA_OK) return st;
-      if ((st = column_update(M, ss, k + 2, k + 3, B(k + 2), side_ctas)) != EXA_OK) return st;
-      if ((st = panel_factor(M, ss, k + 3, B(k + 3), side_ctas)) != EXA_OK) return st;
+      const int side_k = by_rows ? lookahead_share(npad - (int64_t)(k + 4) * NB, 2, sms) : side_ctas;
+      if ((st = panel_factor(M, ss, k + 2, B(k + 2), side_k)) != EXA_OK) return st;
+      if ((st = column_update(M, ss, k + 2, k + 3, B(k + 2), side_k)) != EXA_OK) return st;
+      if ((st = panel_factor(M, ss, k + 3, B(k + 3), side_k)) != EXA_OK) return st;
       cudaEventRecord(c->la_ev[1], ss);
-      if ((st = region_update(M, ms, k, k + 4, B(k), &B(k + 1), main_ctas)) != EXA_OK) return st;
+      if ((st = region_update(M, ms, k, k + 4, B(k), &B(k + 1), sms - side_k)) != EXA_OK) return st;
       cudaStreamWaitEvent(ms, c->la_ev[1], 0);
     }
     // hand over to the one-panel loop: panel k applied to every column >= k+2 leaves
@@ -375,14 +397,14 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   }
   // As the trailing matrix shrinks, the main stream's update of it gets shorter than the
   // look-ahead stream's panel (FP64 diagonal block, panel solve, splits), which then sets
-  // the pace: below late_rows trailing rows the look-ahead stream's SM share grows linearly
-  // to late_sms (reached at late_rows / 3) and the main stream's shrinks by as much.
+  // the pace.  Where the caller has set the shares: below late_rows trailing rows the look-ahead
+  // stream's grows linearly to late_sms (reached at late_rows / 3), the main stream's shrinks by as much.
   const int64_t late_rows = c->late_rows < 0 ? kLateRows : c->late_rows;
   const int late_sms = c->late_sms > 0 ? c->late_sms : kLateSMs;
   for (; k + 1 < T; ++k) {
     const int64_t rows = npad - (int64_t)(k + 2) * NB;  // rows of the main stream's region update
-    int side_k = side_ctas;
-    if (late_rows > 0 && rows < late_rows && late_sms > side_ctas) {
+    int side_k = by_rows ? lookahead_share(rows, 1, sms) : side_ctas;
+    if (!by_rows && late_rows > 0 && rows < late_rows && late_sms > side_ctas) {
       const double f = fmin(1.0, (double)(late_rows - rows) / (double)(late_rows - late_rows / 3));
       side_k = side_ctas + (int)(f * (late_sms - side_ctas));
       side_k = side_k < sms - 2 ? side_k & ~1 : (sms - 2) & ~1;
