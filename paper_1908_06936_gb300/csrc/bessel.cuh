@@ -14,24 +14,40 @@ namespace exa {
 // exponentially (u -> +inf), so the trapezoid rule with h = 1/16 on [-110, 5]
 // is exact to rounding.  D(0) = Gamma'(1).  Written this way Gamma_1(mu) has no
 // cancellation as mu -> 0 (integer nu).
-__host__ __device__ inline double temme_D(double mu) {
-  const double h = 1.0 / 16.0;
-  double s = 0.0;
-  for (int k = -110 * 16; k <= 5 * 16; ++k) {
-    const double u = h * k;
-    const double w = mu * u;
-    double sh;  // sinh(mu u) / mu
-    if (fabs(w) < 1e-4)
-      sh = u * (1.0 + w * w / 6.0);
-    else
-      sh = sinh(w) / mu;
-    s += exp(u - exp(u)) * sh;
-  }
-  return s * h;
+// Node k's weight exp(u - e^u) and sinh(mu u) / mu.
+constexpr int kTemmeNode0 = -110 * 16, kTemmeNodes = 115 * 16 + 1;
+__device__ inline void temme_node(double mu, int k, double& weight, double& sh) {
+  const double u = (1.0 / 16.0) * k;
+  const double w = mu * u;
+  if (fabs(w) < 1e-4)
+    sh = u * (1.0 + w * w / 6.0);
+  else
+    sh = sinh(w) / mu;
+  weight = exp(u - exp(u));
 }
 
-// Per-theta constants (host, or device for parameters that live in device memory).
-__host__ __device__ inline void matern_params_hd(const double theta[3], MaternParams* p) {
+// D as its Chebyshev series in 8 mu^2 - 1 (D is even and analytic for |mu| < 1; |mu| <= 1/2 here; coefficients computed
+// in 60 digits from the Gamma functions, the first left out is 1.6e-17): the host's form.  The quadrature took 60 to 80
+// us of every evaluation before its first launch.
+inline double temme_D(double mu) {
+  static const double c[15] = {-0.7199084713786869458,   -0.1536487143301728609,   -0.01175117600821049204,
+                               -0.0008524878889197950983, -0.00006132983876749679187, -4.405228124551044456e-6,
+                               -3.163124672838448819e-7,  -2.271071938289958833e-8,  -1.630564460807760955e-9,
+                               -1.170693929941477657e-10, -8.405206378646443717e-12, -6.034667011897999149e-13,
+                               -4.332696033568137195e-14, -3.110735803020354621e-15, -2.233407822673698225e-16};
+  const double x = 8.0 * mu * mu - 1.0;
+  double b1 = 0.0, b2 = 0.0;
+  for (int j = 14; j >= 1; --j) {
+    const double b = 2.0 * x * b1 - b2 + c[j];
+    b2 = b1;
+    b1 = b;
+  }
+  return x * b1 - b2 + c[0];
+}
+
+// Per-theta constants (host, or device for parameters that live in device memory); D = D(matern_mu(nu)).
+__host__ __device__ inline double matern_mu(double nu) { return nu - (int)floor(nu + 0.5); }
+__host__ __device__ inline void matern_params_hd(const double theta[3], double D, MaternParams* p) {
   const double nu = theta[2];
   p->sigma2 = theta[0];
   p->beta = theta[1];
@@ -43,7 +59,7 @@ __host__ __device__ inline void matern_params_hd(const double theta[3], MaternPa
   p->nu = nu;
   p->logc = (1.0 - nu) * 0.69314718055994530942 - lgamma(nu);
   const int N = (int)floor(nu + 0.5);
-  const double mu = nu - N;
+  const double mu = matern_mu(nu);
   p->N = N;
   p->mu = mu;
   p->pad_ = 0;
@@ -53,7 +69,7 @@ __host__ __device__ inline void matern_params_hd(const double theta[3], MaternPa
   p->gp = tgamma(1.0 + mu);
   p->gm = tgamma(1.0 - mu);
   // Gamma_1 = D(mu) / (Gamma(1+mu) Gamma(1-mu)) and Gamma(1+mu) Gamma(1-mu) = 1 / sinc
-  p->gam1 = temme_D(mu) * sinc;
+  p->gam1 = D * sinc;
   p->gam2 = 0.5 * (1.0 / p->gm + 1.0 / p->gp);
   p->t_k2[0] = p->t_km[0] = p->t_kp[0] = 0.0;
   for (int k = 1; k <= kTemmeTerms; ++k) {

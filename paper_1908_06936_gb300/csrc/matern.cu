@@ -17,7 +17,9 @@ namespace exa {
 // Host side
 // ---------------------------------------------------------------------------
 
-void matern_params(const double theta[3], MaternParams* p) { matern_params_hd(theta, p); }
+void matern_params(const double theta[3], MaternParams* p) {
+  matern_params_hd(theta, temme_D(matern_mu(theta[2])), p);
+}
 
 // ---------------------------------------------------------------------------
 // Device side (K_nu itself lives in bessel.cuh)
