@@ -217,7 +217,7 @@ cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y
     ProfScope ps(c, PK_TRSV, 2.0 * rows * h, 8.0 * rows * h, c->wall_kept ? 3 + (npad - k0 > h) : 1);
     if (c->wall_kept)
       e = launch_block_fwd(c->stream, a + k0 + k0 * npad, npad, (int)h, npad - k0 - h, block_inverse(c, k0, (int)h),
-                           z + k0, y + k0, tmp);
+                           z + k0, y + k0, tmp, k0 == 0);
     else
       e = launch_trsv_fwd_step(c->stream, a, npad, npad, nb, (int)(k0 / nb), (const double*)c->w_all.p, y, z,
                                c->d_status);
@@ -235,7 +235,7 @@ cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y, double* 
     const double rows = c->wall_kept ? (double)end : (double)(npad - k0);
     ProfScope ps(c, PK_TRSV, 2.0 * rows * h, 8.0 * rows * h, c->wall_kept ? 3 + (k0 > 0) : 2);
     if (c->wall_kept)
-      e = launch_block_bwd(c->stream, a + k0, npad, k0, (int)h, block_inverse(c, k0, (int)h), y, tmp);
+      e = launch_block_bwd(c->stream, a + k0, npad, k0, (int)h, block_inverse(c, k0, (int)h), y, tmp, end == npad);
     else
       e = launch_trsv_bwd_step(c->stream, a, npad, npad, nb, (int)(k0 / nb), (const double*)c->w_all.p, y,
                                (double*)c->partial.p + 2 * kRedPartials, c->d_status);

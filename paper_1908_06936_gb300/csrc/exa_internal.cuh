@@ -192,11 +192,12 @@ cudaError_t launch_trsv_bwd_step(cudaStream_t s, const double* a, int64_t ld, in
 // One block step of either solve with the block's h x h inverse w (row-major, lower; h 128 or 512).  Forward, block at
 // lkk with `rest` rows below it: y <- L_kk^-1 z, then those rows of z (z[h ..]) -= L y; tmp: h doubles.  Backward, block
 // row at lrow (columns [0, k0 + h) of the factor's rows k0 ..): y[k0 ..] <- L_kk^-T y[k0 ..], then y[0, k0) -= L^T of
-// it; tmp: 2 h doubles.
+// it; tmp: 2 h doubles.  first: the first step of its solve (the others may start on the factor while the one before
+// them runs).
 cudaError_t launch_block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int h, int64_t rest, const double* w,
-                             double* z, double* y, double* tmp);
+                             double* z, double* y, double* tmp, bool first);
 cudaError_t launch_block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, int h, const double* w,
-                             double* y, double* tmp);
+                             double* y, double* tmp, bool first);
 
 // Deterministic reductions: out[0] = sum(v[i]^2) ; out[0] = sum(v[i]) over n values.
 cudaError_t launch_sumsq(cudaStream_t s, const double* v, int64_t n, double* partial, double* out);

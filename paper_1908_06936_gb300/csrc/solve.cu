@@ -645,31 +645,49 @@ namespace exa {
 // Block solves of the FP64 factor with the inverses of its 512-wide diagonal blocks (128-wide at the end): per block
 // three products with the block (y = W z, r = z - L_kk y, y += W r: an explicit inverse alone would leave cond(L_kk)
 // rounding errors) and one with the panel, each spread over the GPU.  A 128-row step with one launch each (above) was
-// one CTA's work and ~48 us: 4.7 ms of an n = 12,300 evaluation, 13 ms of a prediction at n = 10,000.
+// one CTA's work and ~48 us: 4.7 ms of an n = 12,300 evaluation (now 0.65), 13 ms of a prediction at n = 10,000 (1.0).
 // All sums in a fixed order.
 // ---------------------------------------------------------------------------
 
 // All loads of a thread are issued before its first multiply-add (masked ones count as 0): in a loop with a bound of
 // its own each waited for the one before, 12 us a kernel.
+//
+// A solve is a chain of such kernels, each a few microseconds, so what a kernel reads of the factor it reads while the one
+// before it still runs: all but the first of a solve are launched as programmatic dependents, and take the vectors after
+// `await_previous` (which waits for the whole preceding grid; each kernel does, so for all before it as well).  The solves of
+// an n = 12,300 evaluation: 0.88 ms without, 0.65 with.
+__device__ __forceinline__ void await_previous() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The H entries of a vector that the previous kernel wrote, into shared memory (from L2, once a CTA).
+template <int H>
+__device__ __forceinline__ void load_vector(const double* v, double* sh) {
+  await_previous();
+  for (int i = threadIdx.x; i < H; i += 256) sh[i] = __ldcg(v + i);
+  __syncthreads();
+}
 
 // out[r] = add[r] + sum_{t <= r} W(r, t) v[t], W row-major H x H: a warp per row.
 template <int H>
-__global__ void __launch_bounds__(256) block_lower_kernel(const double* __restrict__ W, const double* __restrict__ v,
-                                                          const double* __restrict__ add, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) block_lower_kernel(const double* __restrict__ W, const double* v,
+                                                          const double* add, double* out) {
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  double w[H / 32], x[H / 32];
+  __shared__ double x[H];
+  double w[H / 32];
 #pragma unroll
   for (int i = 0; i < H / 32; ++i) {
     const int t = lane + 32 * i;
     w[i] = t <= r ? W[(int64_t)r * H + t] : 0.0;
-    x[i] = v[t];
   }
+  load_vector<H>(v, x);
   double s = 0.0;
 #pragma unroll
-  for (int i = 0; i < H / 32; ++i) s = fma(w[i], x[i], s);
+  for (int i = 0; i < H / 32; ++i) s = fma(w[i], x[lane + 32 * i], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[r] = add ? add[r] + s : s;
+  if (lane == 0) out[r] = add ? __ldcg(add + r) + s : s;
 }
 
 // Sum of v over the CTA's 256 / R threads with the same tid mod R (R = 8, 32 or 128), on thread tid < R; fixed order.
@@ -696,112 +714,125 @@ __device__ __forceinline__ double sum_over_groups(double v) {
 // out[t] = add[t] + sum_{u >= t} W(u, t) v[u], W row-major H x H: eight columns a CTA, the rows split 32 ways (32
 // columns a CTA would be 4 us of one SM's FP64 pipe).
 template <int H>
-__global__ void __launch_bounds__(256) block_lower_t_kernel(const double* __restrict__ W, const double* __restrict__ v,
-                                                            const double* __restrict__ add, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) block_lower_t_kernel(const double* __restrict__ W, const double* v,
+                                                            const double* add, double* out) {
   constexpr int N = H / 32;
   const int t = blockIdx.x * 8 + (threadIdx.x & 7), u0 = (threadIdx.x >> 3) * N;
-  double w[N], x[N];
+  __shared__ double x[H];
+  double w[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    w[i] = u0 + i >= t ? W[(int64_t)(u0 + i) * H + t] : 0.0;
-    x[i] = v[u0 + i];
-  }
+  for (int i = 0; i < N; ++i) w[i] = u0 + i >= t ? W[(int64_t)(u0 + i) * H + t] : 0.0;
+  load_vector<H>(v, x);
   double s = 0.0;
 #pragma unroll
-  for (int i = 0; i < N; ++i) s = fma(w[i], x[i], s);
+  for (int i = 0; i < N; ++i) s = fma(w[i], x[u0 + i], s);
   s = sum_over_groups<8>(s);
-  if (threadIdx.x < 8) out[t] = add ? add[t] + s : s;
+  if (threadIdx.x < 8) out[t] = add ? __ldcg(add + t) + s : s;
 }
 
 // out[r] = z[r] - sum_{t < H} L(r, t) y[t] (lower: t <= r), L column-major, R rows a CTA, the columns split 256 / R
 // ways: 8 rows where there are too few for the GPU's FP64 pipes otherwise, 128 (1 KB of every column) for long panels.
 template <int H, int R>
 __global__ void __launch_bounds__(256) block_rows_kernel(const double* __restrict__ L, int64_t ld, int lower,
-                                                         const double* __restrict__ y, const double* __restrict__ z,
-                                                         double* __restrict__ out) {
+                                                         const double* y, const double* z, double* out) {
   constexpr int per = H * R / 256, N = per < 16 ? per : 16;
+  __shared__ double x[H];
   const int64_t r = (int64_t)blockIdx.x * R + threadIdx.x % R;
   const int t0 = (threadIdx.x / R) * per;
   double s = 0.0;
 #pragma unroll 1
   for (int c = 0; c < per; c += N) {
-    double l[N], x[N];
+    double l[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const int t = t0 + c + i;
       l[i] = !lower || t <= r ? L[r + t * ld] : 0.0;
-      x[i] = y[t];
     }
+    if (c == 0) load_vector<H>(y, x);
 #pragma unroll
-    for (int i = 0; i < N; ++i) s = fma(l[i], x[i], s);
+    for (int i = 0; i < N; ++i) s = fma(l[i], x[t0 + c + i], s);
   }
   s = sum_over_groups<R>(s);
-  if (threadIdx.x < R) out[r] = z[r] - s;
+  if (threadIdx.x < R) out[r] = __ldcg(z + r) - s;
 }
 
 // out[c] = z[c] - sum_{r < H} L(r, c) x[r] (lower: r >= c), L column-major: a warp per column.
 template <int H>
 __global__ void __launch_bounds__(256) block_cols_kernel(const double* __restrict__ L, int64_t ld, int lower,
-                                                         const double* __restrict__ x, const double* __restrict__ z,
-                                                         double* __restrict__ out) {
+                                                         const double* x, const double* z, double* out) {
   const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  double l[H / 32], v[H / 32];
+  __shared__ double v[H];
+  double l[H / 32];
 #pragma unroll
   for (int i = 0; i < H / 32; ++i) {
     const int r = lane + 32 * i;
     l[i] = !lower || r >= c ? L[r + c * ld] : 0.0;
-    v[i] = x[r];
   }
+  load_vector<H>(x, v);
   double s = 0.0;
 #pragma unroll
-  for (int i = 0; i < H / 32; ++i) s = fma(l[i], v[i], s);
+  for (int i = 0; i < H / 32; ++i) s = fma(l[i], v[lane + 32 * i], s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) out[c] = z[c] - s;
+  if (lane == 0) out[c] = __ldcg(z + c) - s;
+}
+
+// chained: after another kernel of the same solve.
+template <class... P, class... A>
+static cudaError_t launch_block(cudaStream_t s, bool chained, int64_t grid, void (*kernel)(P...), A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
 }
 
 template <int H>
 static cudaError_t block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int64_t rest, const double* w, double* z,
-                             double* y, double* tmp) {
-  block_lower_kernel<H><<<H / 8, 256, 0, s>>>(w, z, nullptr, y);
-  block_rows_kernel<H, 8><<<H / 8, 256, 0, s>>>(lkk, ld, 1, y, z, tmp);
-  block_lower_kernel<H><<<H / 8, 256, 0, s>>>(w, tmp, y, y);
+                             double* y, double* tmp, bool first) {
+  cudaError_t e = launch_block(s, !first, H / 8, block_lower_kernel<H>, w, z, nullptr, y);
+  if (e == cudaSuccess) e = launch_block(s, true, H / 8, block_rows_kernel<H, 8>, lkk, ld, 1, y, z, tmp);
+  if (e == cudaSuccess) e = launch_block(s, true, H / 8, block_lower_kernel<H>, w, tmp, y, y);
+  if (e != cudaSuccess || rest <= 0) return e;
   const double* l = lkk + H;
   double* zr = z + H;
   if (rest >= 32768)  // more than one 128-row CTA per SM
-    block_rows_kernel<H, 128><<<(unsigned)(rest / 128), 256, 0, s>>>(l, ld, 0, y, zr, zr);
-  else if (rest >= 4864)  // one 32-row CTA per SM
-    block_rows_kernel<H, 32><<<(unsigned)(rest / 32), 256, 0, s>>>(l, ld, 0, y, zr, zr);
-  else if (rest > 0)
-    block_rows_kernel<H, 8><<<(unsigned)(rest / 8), 256, 0, s>>>(l, ld, 0, y, zr, zr);
-  return cudaGetLastError();
+    return launch_block(s, true, rest / 128, block_rows_kernel<H, 128>, l, ld, 0, y, zr, zr);
+  if (rest >= 4864)  // one 32-row CTA per SM
+    return launch_block(s, true, rest / 32, block_rows_kernel<H, 32>, l, ld, 0, y, zr, zr);
+  return launch_block(s, true, rest / 8, block_rows_kernel<H, 8>, l, ld, 0, y, zr, zr);
 }
 
 template <int H>
 static cudaError_t block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, const double* w, double* y,
-                             double* tmp) {
+                             double* tmp, bool first) {
   const double* lkk = lrow + k0 * ld;
   double* v = y + k0;
   double* x = tmp + H;
-  block_lower_t_kernel<H><<<H / 8, 256, 0, s>>>(w, v, nullptr, x);
-  block_cols_kernel<H><<<H / 8, 256, 0, s>>>(lkk, ld, 1, x, v, tmp);
-  block_lower_t_kernel<H><<<H / 8, 256, 0, s>>>(w, tmp, x, v);
-  if (k0 > 0) block_cols_kernel<H><<<(unsigned)(k0 / 8), 256, 0, s>>>(lrow, ld, 0, v, y, y);
-  return cudaGetLastError();
+  cudaError_t e = launch_block(s, !first, H / 8, block_lower_t_kernel<H>, w, v, nullptr, x);
+  if (e == cudaSuccess) e = launch_block(s, true, H / 8, block_cols_kernel<H>, lkk, ld, 1, x, v, tmp);
+  if (e == cudaSuccess) e = launch_block(s, true, H / 8, block_lower_t_kernel<H>, w, tmp, x, v);
+  if (e == cudaSuccess && k0 > 0) e = launch_block(s, true, k0 / 8, block_cols_kernel<H>, lrow, ld, 0, v, y, y);
+  return e;
 }
 
 cudaError_t launch_block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int h, int64_t rest, const double* w,
-                             double* z, double* y, double* tmp) {
-  if (h == 512) return block_fwd<512>(s, lkk, ld, rest, w, z, y, tmp);
-  if (h == 128) return block_fwd<128>(s, lkk, ld, rest, w, z, y, tmp);
+                             double* z, double* y, double* tmp, bool first) {
+  if (h == 512) return block_fwd<512>(s, lkk, ld, rest, w, z, y, tmp, first);
+  if (h == 128) return block_fwd<128>(s, lkk, ld, rest, w, z, y, tmp, first);
   return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_block_bwd(cudaStream_t s, const double* lrow, int64_t ld, int64_t k0, int h, const double* w,
-                             double* y, double* tmp) {
-  if (h == 512) return block_bwd<512>(s, lrow, ld, k0, w, y, tmp);
-  if (h == 128) return block_bwd<128>(s, lrow, ld, k0, w, y, tmp);
+                             double* y, double* tmp, bool first) {
+  if (h == 512) return block_bwd<512>(s, lrow, ld, k0, w, y, tmp, first);
+  if (h == 128) return block_bwd<128>(s, lrow, ld, k0, w, y, tmp, first);
   return cudaErrorInvalidValue;
 }
 
