@@ -64,6 +64,28 @@ def test_covariance_and_loglik(ctx, model, nugget, metric, radius, theta):
     assert abs(lmx - l_ref) <= 1e-6 * abs(l_ref)
 
 
+def test_great_circle_covariance_over_all_arcs(ctx, model):
+    # arcs from 0 to 175 degrees along meridians, parallels and across a pole, several on both sides of the arcs where
+    # the series for the sines and the squared arc sine end; distances to a few roundings, so 1e-12 as above
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    theta = (1.3, 3000.0, 0.5)
+    model(0.0, 1, 0.0)
+    arcs = np.concatenate([[0.0], 10.0 ** np.linspace(-2, 2.2, 40), 28.6479 + np.linspace(-0.01, 0.01, 7),
+                           28.955 + np.linspace(-0.01, 0.01, 7), [57.2, 57.3, 90.0, 175.0]])
+    pts = [np.column_stack([np.zeros_like(arcs), -85.0 + arcs]), np.column_stack([10.0 + arcs, np.zeros_like(arcs)]),
+           np.column_stack([20.0 + arcs, np.full_like(arcs, 60.0)]), [[0.0, 90.0], [77.0, 89.9], [257.0, 89.9]]]
+    locs = np.ascontiguousarray(np.concatenate(pts))
+    n = len(locs)
+    S = torch.zeros(n * n, dtype=torch.float64, device="cuda")
+    ctx.check(exa.exa_covariance(ctx.handle, to_dev(locs), n, theta, S, n))
+    got = S.cpu().numpy().reshape(n, n).T
+    ref = oracle.covariance(locs, theta)
+    low = np.tril_indices(n)
+    assert np.allclose(got[low], ref[low], rtol=1e-12, atol=1e-300)
+
+
 @pytest.mark.parametrize("nugget,metric,radius,theta", CASES[:2])
 def test_gradient_prediction_fisher(ctx, model, nugget, metric, radius, theta):
     model(nugget, metric, radius)
