@@ -143,9 +143,10 @@ constexpr int STAGE_BYTES = 4 * OP_BYTES;       // A_hi, A_lo, B_hi, B_lo
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr uint32_t IDESC = idesc(kFmtTF32, TM, TN);
 constexpr int TMEM_COLS = 256;                  // 2 accumulator buffers x 128 columns
+constexpr int kThreads = 64 + 2 * kEpiThreads;  // eight epilogue warps for each accumulator
 }  // namespace t3
 
-__global__ void __launch_bounds__(kGemmThreads)
+__global__ void __launch_bounds__(t3::kThreads)
     gemm_t3_kernel(const __grid_constant__ CUtensorMap tA_hi, const __grid_constant__ CUtensorMap tA_lo,
                    const __grid_constant__ CUtensorMap tB_hi, const __grid_constant__ CUtensorMap tB_lo,
                    const __grid_constant__ GemmArgs g) {
@@ -273,51 +274,54 @@ __global__ void __launch_bounds__(kGemmThreads)
     }
   } else if (warp >= 2) {
     // ---------------- epilogue: TMEM -> FP64 C ----------------
-    // 8 warps: warp w drains TMEM lanes 32*(w%4).. (its row quarter) and column half (w-2)/4
+    // Two groups of 8 warps take the tiles in turn, one accumulator each: while one waits for C or stores it, the other
+    // subtracts (the three phases of one group, 64 KB read and written and 16,384 FP64 additions an SM, took 22,000
+    // cycles a tile one after another, the memory alone 11,000).  Warp w drains TMEM lanes 32*(w%4).. (its row quarter)
+    // and one column half.
     const int quad = warp & 3;
-    const int half = (warp - 2) >> 2;
+    const int b = (warp - 2) >> 3, half = ((warp - 2) >> 2) & 1;
     const int r = quad * 32 + lane;
     int it = 0;
     for (long long t = blockIdx.x; t < g.ntiles && !*abort; t += gridDim.x) {
       T3Tile tl;
       if (!t3_tile(g, t, tl)) continue;
-      const int b = it & 1;
-      const uint32_t ap = (it >> 1) & 1;
+      if ((it++ & 1) != b) continue;
+      const uint32_t ap = ((it - 1) >> 1) & 1;
+      const bool diag = tl.diag;
+      const int64_t ldc = tl.ldc;
+      double* cp = tl.C + r;
+      if (!g.store) {  // this warp's lines into L2 while the products run
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+          prefetch_l2(tl.C + quad * 32 + 16 * (lane & 1) + (int64_t)(half * 64 + l * 16 + (lane >> 1)) * ldc);
+      }
       if (!mbar_wait(&accfull[b], ap, abort)) {
         *abort = 1;
         record_timeout(g.st, 14);
         break;
       }
       fence_after();
-      const bool diag = tl.diag;
-      const int64_t ldc = tl.ldc;
-      double* cp = tl.C + r;
-      // two batches of 32 C loads in flight per thread (64 KB per SM), then drain TMEM
 #pragma unroll 1
-      for (int h2 = 0; h2 < 2; ++h2) {
-        const int cb = half * 64 + h2 * 32;
-        double cv[32];
+      for (int h4 = 0; h4 < 4; ++h4) {
+        const int cb = half * 64 + h4 * 16;
+        double cv[16];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) cv[j] = g.store ? 0.0 : __ldcs(cp + (int64_t)(cb + j) * ldc);
+        for (int j = 0; j < 16; ++j) cv[j] = g.store ? 0.0 : __ldcs(cp + (int64_t)(cb + j) * ldc);
+        uint32_t acc[16];
+        tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + b * TN + cb, acc);
+        tmem_ld_wait();
+        if (h4 == 3) {
+          fence_before();
+          mbar_arrive(&accempty[b]);
+        }
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          uint32_t acc[16];
-          tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + b * TN + cb + c * 16, acc);
-          tmem_ld_wait();
-          if (h2 == 1 && c == 1) {
-            fence_before();
-            mbar_arrive(&accempty[b]);
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int cc = cb + c * 16 + j;
-            if (diag && cc > r) continue;
-            const double v = f32_bits_to_f64(acc[j]);
-            __stcs(cp + (int64_t)cc * ldc, g.store ? v : cv[c * 16 + j] - v);
-          }
+        for (int j = 0; j < 16; ++j) {
+          const int cc = cb + j;
+          if (diag && cc > r) continue;
+          const double v = f32_bits_to_f64(acc[j]);
+          __stcs(cp + (int64_t)cc * ldc, g.store ? v : cv[j] - v);
         }
       }
-      ++it;
     }
   }
   fence_before();
@@ -1189,7 +1193,7 @@ cudaError_t launch_gemm_t3(cudaStream_t s, const SplitOperand& A, const SplitOpe
   int cap = num_sms();
   if (max_ctas > 0 && max_ctas < cap) cap = max_ctas;
   const int grid = (int)(g.ntiles < cap ? g.ntiles : cap);
-  gemm_t3_kernel<<<grid, kGemmThreads, t3::SMEM_BYTES, s>>>(A.t_hi, A.t_lo, B.t_hi, B.t_lo, g);
+  gemm_t3_kernel<<<grid, t3::kThreads, t3::SMEM_BYTES, s>>>(A.t_hi, A.t_lo, B.t_hi, B.t_lo, g);
   return cudaGetLastError();
 }
 
