@@ -123,16 +123,26 @@ __global__ void __launch_bounds__(256) potrf_diag_kernel(double* __restrict__ a,
 // panel).
 constexpr int kPotrfPW = 16;
 
-// The tile's log sum goes to *logdet_out.  Returns true (on every thread) when the tile was
-// factored; L then also sits in the first NB x (NB + 1) doubles of shared memory.
-template <int NB>
+// The tile's log sum goes to *logdet_out.  Returns true (on every thread) when the tile was factored; L then also sits at
+// the start of shared memory, element (i, j) at tile_at<NB, PACKED>(i, j): rows of NB + 1 doubles, or the packed lower
+// triangle (rows i (i + 1) / 2: free of bank conflicts along a column as well, and two CTAs fit an SM).
+template <int NB, bool PACKED>
+__device__ __forceinline__ int tile_at(int i, int j) {
+  return PACKED ? i * (i + 1) / 2 + j : i * (NB + 1) + j;
+}
+template <int NB, bool PACKED>
+constexpr int kTileDoubles = PACKED ? NB * (NB + 1) / 2 : NB * (NB + 1);
+
+template <int NB, bool PACKED>
 __device__ __forceinline__ bool potrf_blocked_body(double* __restrict__ a, int64_t ld, int64_t k0,
                                                    double* __restrict__ logdet_out, DevStatus* st) {
-  constexpr int PW = kPotrfPW, sd = NB + 1;
+  constexpr int PW = kPotrfPW;
   extern __shared__ double sm[];
-  double* S = sm;                // NB x sd, element (i, j) at S[i * sd + j]
-  double* lg = sm + NB * sd;     // NB logs
+  double* S = sm;
+  double* lg = sm + kTileDoubles<NB, PACKED>;  // NB logs
   __shared__ int s_bad, s_skip;
+  __shared__ double s_inv[PW];
+  auto at = [](int i, int j) { return tile_at<NB, PACKED>(i, j); };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) s_skip = failed(st) ? 1 : 0;  // one read, so that every thread takes the same path
   __syncthreads();
@@ -151,47 +161,73 @@ __device__ __forceinline__ bool potrf_blocked_body(double* __restrict__ a, int64
     }
 #pragma unroll
     for (int u = 0; u < CH; ++u) {
-      const int idx = tid + (c0 + u) * 256;
-      S[(idx % NB) * sd + idx / NB] = v[u];
+      const int idx = tid + (c0 + u) * 256, i = idx % NB, j = idx / NB;
+      if (i >= j) S[at(i, j)] = v[u];
     }
   }
   __syncthreads();
   // ---- factorisation ----
   for (int p = 0; p < NB; p += PW) {
+    // the panel's first 32 rows on warp 0, then the others, 32 a warp: every entry sees the same operations in the same
+    // order as if one warp took all rows column by column
     if (warp == 0) {
+      const int end = min(NB, p + 32);
       for (int j = p; j < p + PW; ++j) {
-        const double d = S[j * sd + j];
+        const double d = S[at(j, j)];
         if (!(d > 0.0) || !isfinite(d)) {  // warp-uniform
           if (lane == 0) s_bad = j;
           break;
         }
         const double lj = sqrt(d), inv = 1.0 / lj;
-        for (int i = j + 1 + lane; i < NB; i += 32) S[i * sd + j] *= inv;
+        const int i = p + lane;
+        if (i > j && i < end) S[at(i, j)] *= inv;
         __syncwarp();
-        if (lane == 0) S[j * sd + j] = lj;
-        for (int c = j + 1; c < p + PW; ++c) {
-          const double scj = S[c * sd + j];
-          for (int i = c + lane; i < NB; i += 32) S[i * sd + c] = fma(-S[i * sd + j], scj, S[i * sd + c]);
+        if (lane == 0) {
+          S[at(j, j)] = lj;
+          s_inv[j - p] = inv;
+        }
+        if (i < end) {
+          const double sij = i > j ? S[at(i, j)] : 0.0;
+          for (int c = j + 1; c < p + PW; ++c)
+            if (i >= c) S[at(i, c)] = fma(-sij, S[at(c, j)], S[at(i, c)]);
         }
         __syncwarp();
       }
     }
     __syncthreads();
     if (s_bad >= 0) break;
-    // trailing triangle (i >= l >= p + PW): S_il -= sum_{t in panel} S_it S_lt
+    {
+      const int i = p + 32 + 32 * (warp - 1) + lane;
+      if (warp > 0 && i < NB) {
+        double x[PW];
+#pragma unroll
+        for (int j = 0; j < PW; ++j) x[j] = S[at(i, p + j)];
+#pragma unroll
+        for (int j = 0; j < PW; ++j) {
+          x[j] *= s_inv[j];
+#pragma unroll
+          for (int c = j + 1; c < PW; ++c) x[c] = fma(-x[j], S[at(p + c, p + j)], x[c]);
+        }
+#pragma unroll
+        for (int j = 0; j < PW; ++j) S[at(i, p + j)] = x[j];
+      }
+    }
+    __syncthreads();
+    // trailing triangle (i >= l >= p + PW): S_il -= sum_{t in panel} S_it S_lt; rows a and m - 1 - a together hold m + 1
+    // entries
     const int q0 = p + PW, m = NB - q0;
-    for (int e = tid; e < m * m; e += 256) {
-      const int i = q0 + e % m, l = q0 + e / m;
-      if (i < l) continue;
-      const double* ri = S + i * sd + p;
-      const double* rl = S + l * sd + p;
+    for (int e = tid; e < m / 2 * (m + 1); e += 256) {
+      const int u = e / (m + 1), w = e - u * (m + 1);
+      const int i = q0 + (w <= u ? u : m - 1 - u), l = q0 + (w <= u ? w : w - u - 1);
+      const double* ri = S + at(i, p);
+      const double* rl = S + at(l, p);
       double s0 = 0.0, s1 = 0.0;
 #pragma unroll
       for (int t = 0; t < PW; t += 2) {
         s0 = fma(ri[t], rl[t], s0);
         s1 = fma(ri[t + 1], rl[t + 1], s1);
       }
-      S[i * sd + l] -= s0 + s1;
+      S[at(i, l)] -= s0 + s1;
     }
     __syncthreads();
   }
@@ -205,9 +241,9 @@ __device__ __forceinline__ bool potrf_blocked_body(double* __restrict__ a, int64
   // write L back (lower triangle) and the log-determinant part (fixed-order sum)
   for (int idx = tid; idx < NB * NB; idx += 256) {
     const int i = idx % NB, j = idx / NB;
-    if (i >= j) A[i + (int64_t)j * ld] = S[i * sd + j];
+    if (i >= j) A[i + (int64_t)j * ld] = S[at(i, j)];
   }
-  if (tid < NB) lg[tid] = log(S[tid * sd + tid]);
+  if (tid < NB) lg[tid] = log(S[at(tid, tid)]);
   __syncthreads();
   if (tid == 0) {
     double s = 0.0;
@@ -220,7 +256,7 @@ __device__ __forceinline__ bool potrf_blocked_body(double* __restrict__ a, int64
 template <int NB>
 __global__ void __launch_bounds__(256) potrf_diag_blocked_kernel(double* __restrict__ a, int64_t ld, int64_t k0,
                                                                  double* __restrict__ logdet_part, DevStatus* st) {
-  potrf_blocked_body<NB>(a, ld, k0, logdet_part + k0 / NB, st);
+  potrf_blocked_body<NB, false>(a, ld, k0, logdet_part + k0 / NB, st);
 }
 
 // W_k = L_kk^-1 (row-major, zeros above the diagonal) for the NB x NB diagonal tile that
@@ -293,17 +329,20 @@ __global__ void __launch_bounds__(256) trtri_rows_kernel(const double* __restric
 // [[W_A, 0], [L_BA, W_B]]^-1 = [[W_A, 0], [-W_B (L_BA W_A), W_B]] for widths 16, 32, 64, with
 // the products in shared memory.  Plain FP64 sums: W preconditions the FP64 refinement and
 // feeds TF32 panel solves, so the compensated row inverse of the single-field FP64 path (16
-// CTAs per tile) is not needed here, and one CTA per tile keeps a batch of hundreds of tiles
-// at one wave or two.
-constexpr int kInvSmem = 128 * 129 + 128 + 64 * 64;  // doubles: L, logs, one product
+// CTAs per tile) is not needed here, and one CTA per tile, two on an SM, keeps a batch of hundreds of tiles
+// at one wave.
+// Bound: FP64 instructions (2 multiply-adds a cycle on an SM) and, for few tiles, the columns' square roots and divisions.
+// 256 tiles of ragged fields: 0.53 ms a launch; one CTA an SM with all rows of a panel on one warp took 0.73.
+constexpr int kInvSmem = kTileDoubles<128, true> + 128 + 64 * 64;  // doubles: L, logs, one product
 
-__global__ void __launch_bounds__(256) potrf_inv128_tasks_kernel(const DiagTileTask* __restrict__ tasks) {
-  constexpr int NB = 128, sd = NB + 1, PW = 16;
+__global__ void __launch_bounds__(256, 2) potrf_inv128_tasks_kernel(const DiagTileTask* __restrict__ tasks) {
+  constexpr int NB = 128, PW = 16;
   const DiagTileTask t = tasks[blockIdx.x];
-  if (!potrf_blocked_body<NB>(t.a, t.ld, t.k0, t.logdet, t.st)) return;  // uniform over the CTA
+  if (!potrf_blocked_body<NB, true>(t.a, t.ld, t.k0, t.logdet, t.st)) return;  // uniform over the CTA
   extern __shared__ double sm[];
-  const double* S = sm;            // L(i, j) at S[i * sd + j]
-  double* T = sm + NB * sd + NB;   // products, at most 64 x 64
+  const double* S = sm;  // L(i, j) at S[at(i, j)]
+  auto at = [](int i, int j) { return tile_at<NB, true>(i, j); };
+  double* T = sm + kTileDoubles<NB, true> + NB;  // products, at most 64 x 64
   double* W = t.w;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   for (int idx = tid; idx < NB * NB; idx += 256) {
@@ -314,10 +353,10 @@ __global__ void __launch_bounds__(256) potrf_inv128_tasks_kernel(const DiagTileT
   {
     const int p0 = warp * PW;  // warp w inverts diagonal block w
     for (int c = PW - 1; c >= 0; --c) {
-      const double vcc = 1.0 / S[(p0 + c) * sd + p0 + c];
+      const double vcc = 1.0 / S[at(p0 + c, p0 + c)];
       if (lane > c && lane < PW) {
         double acc = 0.0;
-        for (int l = c + 1; l <= lane; ++l) acc = fma(W[(p0 + lane) * NB + p0 + l], S[(p0 + l) * sd + p0 + c], acc);
+        for (int l = c + 1; l <= lane; ++l) acc = fma(W[(p0 + lane) * NB + p0 + l], S[at(p0 + l, p0 + c)], acc);
         W[(p0 + lane) * NB + p0 + c] = -acc * vcc;
       }
       if (lane == c) W[(p0 + c) * NB + p0 + c] = vcc;
@@ -330,7 +369,7 @@ __global__ void __launch_bounds__(256) potrf_inv128_tasks_kernel(const DiagTileT
     for (int idx = tid; idx < pairs * h * h; idx += 256) {
       const int p = idx / (h * h), r = (idx / h) % h, c = idx % h, o = p * 2 * h;
       double acc = 0.0;
-      for (int k = c; k < h; ++k) acc = fma(S[(o + h + r) * sd + o + k], W[(o + k) * NB + o + c], acc);
+      for (int k = c; k < h; ++k) acc = fma(S[at(o + h + r, o + k)], W[(o + k) * NB + o + c], acc);
       T[idx] = acc;
     }
     __syncthreads();
