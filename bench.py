@@ -275,6 +275,10 @@ def class_roofline(st: dict, pk: dict) -> dict:
         ach, peak = flop_rate, pk["bf16"]
         bound, unit, note = "tensor", "TFLOP/s", "useful flops vs bf16 peak (15 bf16 MMAs per useful product)"
         extra["frac_of_digit_product_ceiling"] = 15.0 * ach / peak
+    elif name in ("gemm_fp64_digits",):
+        ach, peak = flop_rate, pk["bf16"]
+        bound, unit, note = "tensor", "TFLOP/s", "useful FP64 flops vs bf16 peak (36 bf16 MMAs per useful product)"
+        extra["frac_of_digit_product_ceiling"] = 36.0 * ach / peak
     elif name in ("syrk_update_fp64", "trsm_panel_fp64", "dgemm_small_fp64"):
         ach, peak = flop_rate, pk["fp64"]
         bound, unit, note = "tensor", "TFLOP/s", "FP64 DMMA"
@@ -307,7 +311,7 @@ def roofline(stats: list, pk: dict) -> dict:
     return class_roofline(dom, pk)
 
 
-# kernel classes of the mixed evaluation that run (wholly or partly) on the look-ahead stream, on 20 to 48
+# kernel classes of the mixed evaluation that run (wholly or partly) on the look-ahead stream, on 20 to 104
 # of the GPU's SMs beside the trailing update: their fraction of the whole GPU's peak is low by construction
 LOOKAHEAD_CLASSES = ("potrf_diag_fp64", "split_rows", "gemm_tf32x3_tc")
 

@@ -105,6 +105,10 @@ typedef struct {
 /* Create a context on the current CUDA device.
  *   cuda_stream      cudaStream_t to issue work on (NULL: the legacy default stream).
  *   workspace_bytes  upper bound on device memory the context may hold (0: no bound).
+ *                    FP64 evaluations use up to ~20 KB a row of the matrix beside it for digit
+ *                    operands and block inverses where the bound and the device allow it
+ *                    (they make the products run on the tensor cores), and give it up for
+ *                    a buffer that a call cannot do without.
  *   tile_nb          FP64 tile size, a multiple of 64 and <= 128 (0: library default).
  * Returns EXA_ERR_ARG on a bad tile size, EXA_ERR_CUDA if no device is usable. */
 exa_status exa_ctx_create(exa_ctx** ctx, void* cuda_stream, size_t workspace_bytes, int tile_nb);
@@ -211,7 +215,9 @@ exa_status exa_loglik_ex(exa_ctx* ctx, const double* d_locs, const double* d_z, 
  * through the Matern covariance of Eq. 3):
  *   dl/dtheta_k = 1/2 a^T (dSigma/dtheta_k) a - 1/2 tr(Sigma^-1 dSigma/dtheta_k),  a = Sigma^-1 z.
  * grad (host, 3 doubles).  dSigma/dtheta_k is regenerated entry by entry (never stored).
- *   EXA_FP64          FP64 factor, a, and Sigma^-1 = L^-T L^-1 on FP64 DMMA.  Holds two
+ *   EXA_FP64          FP64 factor, a, and Sigma^-1 = L^-T L^-1, with the products formed on
+ *                     the tensor cores from eight exact 7-bit digits (on FP64 DMMA with
+ *                     tile 64 or without room for the digits).  Holds two
  *                     n_pad^2 FP64 buffers (n_pad = n rounded up to the tile) when the
  *                     context can hold them; otherwise (workspace bound or cudaMalloc
  *                     failure) it holds one: L^-1 overwrites the factor and each tile of

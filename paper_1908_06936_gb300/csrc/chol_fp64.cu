@@ -1,5 +1,6 @@
-// Step a2 (FP64): right-looking tiled Cholesky, Sigma = L L^T (Section I;
-// the tile decomposition of Section II-A, Fig. 1(a)).
+// Step a2 on the FP64 units: right-looking tiled Cholesky, Sigma = L L^T (Section I;
+// the tile decomposition of Section II-A, Fig. 1(a)).  The path without room for digit operands
+// (chol_digits.cu) and of contexts with tile 64; and the diagonal tiles of the mixed batched form.
 //
 // For tile column k (k0 = k nb):
 //   potrf_diag  : L_kk = chol(A_kk) in shared memory (one CTA), then W_k = L_kk^-1

@@ -68,10 +68,8 @@ exa_status ensure_split(exa_ctx* c, SplitOperand& op, DevBuf& buf, int64_t rows,
 
 // ---------------------------------------------------------------------------
 // Mixed-precision tiled Cholesky (panel width kMixNB = 512).  For tile column k:
-//   1. FP64 factorisation of the 512 x 512 diagonal block as four 128 sub-tiles
-//      (POTRF with the sub-tile inverse, TRSM and SYRK within the block on DMMA),
-//      then its inverse W, block row by block row from the sub-tile inverses:
-//      W_ij = -W_ii sum_{l=j}^{i-1} L_il W_lj (small DMMA products).
+//   1. FP64 factorisation of the 512 x 512 diagonal block and its inverse W, with those
+//      of its four 128 sub-tiles: one cooperative launch (diag_block.cu).
 //   2. Panel TRSM  L_ik = A_ik W^T on the tensor cores: the first `band` tile
 //      rows with the exact OZ products, the rest with T3.
 //   3. Trailing update A_ij -= L_ik L_jk^T: tiles with I - J <= band (the
