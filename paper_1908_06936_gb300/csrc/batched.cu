@@ -822,7 +822,8 @@ struct BatchPlan {
   const void* tc_work = nullptr;
   const void* tc_meta = nullptr;
   int64_t ps_rows = 0;
-  SplitOperand ps, ws;
+  SplitOperand ps, ps2, ws;
+  bool fused = false;  // the lists take two panels a pass (ps2 holds the second's operand)
 };
 
 // Work-list order.  Every task gets its bottom level: the longest path, in
@@ -1093,7 +1094,8 @@ static exa_status batched_run(exa_ctx* c, int nrep, const int64_t* h_n, const do
 //   3. panel solve L_ik = A_ik W_k^T as ONE grouped tcgen05 launch of TF32x3 128 x 128 tiles;
 //   4. split of the solved panels (one launch);
 //   5. trailing update A_ij -= L_ik L_jk^T as ONE grouped tcgen05 launch over every replicate's
-//      trailing lower tiles.
+//      trailing lower tiles; with room for two panel operands an even panel updates the next
+//      column alone and the following one takes both over the rest, (A_ij - panel k) - panel k+1.
 // Then the FP64 refinement of x = Sigma^-1 z per replicate (as the FP32 form).  Everything is
 // stream-ordered with no host synchronisation (graph-capturable); the task lists depend only on
 // the replicate sizes and are uploaded when they change.
@@ -1186,13 +1188,39 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   double* wbuf = (double*)c->bt_work.p;
   double* ldpart = wbuf + wo;
   // task lists (rebuilt when the sizes or the buffers they point into change)
-  const bool rebuild = !same_shape || ps_new || P.tc_mat != c->bt_mat.p || P.tc_work != c->bt_work.p ||
+  const bool changed = !same_shape || ps_new || P.tc_mat != c->bt_mat.p || P.tc_work != c->bt_work.p ||
                        P.tc_meta != c->bt_meta.p;
+  // Two panels a pass over the trailing tiles, whose C traffic bounds the products (256 replicates: 54 ms at one panel a
+  // pass, 46 of them for C; now 47), where a second panel operand can be had beside everything else.
+  bool fused = false;
+  if (Tmax > 2 && (changed || P.fused)) {
+    if (changed) {  // room for the lists first: those of one panel a pass are the longer ones
+      int64_t nt = 0, nu = 0;
+      for (int r = 0; r < nrep; ++r) {
+        const int64_t T = meta[r].T;
+        nt += T;
+        nu += T * (T - 1) / 2 + (T - 1) * T * (T + 1) / 6;
+      }
+      const size_t lists = round_up(nt * (int64_t)sizeof(DiagTileTask), 256) +
+                           round_up(2 * (nt - nrep) * (int64_t)sizeof(SplitTask), 256) +
+                           round_up(nu * (int64_t)sizeof(TcTask), 256) + 256;
+      if ((st = ensure(c, c->bt_tasks, lists, "batched task lists")) != EXA_OK) return st;
+    }
+    fused = ensure(c, c->bt_ps2, split_bytes(ps_rows, NB, true, false) + 1024, "second panel operand", true) == EXA_OK &&
+            ensure_split(c, P.ps2, c->bt_ps2, ps_rows, NB, true, false) == EXA_OK;
+    if (!fused) c->err[0] = 0;
+  }
+  if (fused) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) c->ps2_captured = true;
+  }
+  const bool rebuild = changed || P.fused != fused;
   std::vector<DiagTileTask> diag;
   std::vector<SplitTask> spl;
   std::vector<TcTask> tc;
   if (rebuild) {
     P.steps.clear();
+    std::vector<int> before(nrep, 0);  // first operand row of each replicate in the panel before
     for (int k = 0; k < Tmax; ++k) {
       TcStep stp{};
       stp.diag_off = (int)diag.size();
@@ -1238,11 +1266,15 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
       for (int q = 0; q < stp.nset; ++q) {
         const BMeta& m = meta[set[q]];
         const int nbk = (int)(m.T - k - 1);
+        // fused: an even panel updates the next column alone, an odd one and the panel before it the rest together
+        const bool pair = fused && (k & 1);
+        const int row0 = pair ? before[set[q]] + NB : prow[q], shift = pair ? row0 - prow[q] : 0;
         for (int i = 0; i < nbk; ++i)
-          for (int j = 0; j <= i; ++j)
+          for (int j = 0; j <= (fused && !pair ? 0 : i); ++j)
             tc.push_back({mat + m.mo + (int64_t)(k + 1 + i) * NB + (int64_t)(k + 1 + j) * NB * m.npad, m.npad,
-                          prow[q] + i * NB, prow[q] + j * NB, i == j ? 1 : 0, 0});
+                          row0 + i * NB, row0 + j * NB, i == j ? 1 : 0, shift});
       }
+      for (int q = 0; q < stp.nset; ++q) before[set[q]] = prow[q];
       stp.nupd = (int)tc.size() - stp.upd_off;
       P.steps.push_back(stp);
     }
@@ -1297,6 +1329,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
     P.tc_work = c->bt_work.p;
     P.tc_meta = c->bt_meta.p;
     P.ps_rows = ps_rows;
+    P.fused = fused;
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(dCnt, 0, cnt_b + rst_b, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(DevStatus), s);
@@ -1324,6 +1357,8 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   g.st = c->d_status;
   for (size_t k = 0; k < P.steps.size() && e == cudaSuccess; ++k) {
     const TcStep& stp = P.steps[k];
+    const bool second = fused && (k & 1);
+    SplitOperand& panel = second ? P.ps2 : P.ps;
     {
       ProfScope ps(c, PK_POTRF, (double)stp.ndiag * NB * NB * NB * 2.0 / 3.0, 0.0, 1);
       e = launch_potrf128_tasks(s, dDiag + stp.diag_off, stp.ndiag);
@@ -1332,25 +1367,27 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
     {
       ProfScope ps(c, PK_SPLIT, 0.0, 16.0 * (double)(stp.ntrsm + stp.nset) * NB * NB, 2);
       e = launch_split_rows_tasks(s, dSpl + stp.wsplit_off, stp.nset, NB, NB, P.ws);
-      if (e == cudaSuccess) e = launch_split_rows_tasks(s, dSpl + stp.psplit_off, stp.nset, stp.max_m, NB, P.ps);
+      if (e == cudaSuccess) e = launch_split_rows_tasks(s, dSpl + stp.psplit_off, stp.nset, stp.max_m, NB, panel);
     }
     if (e == cudaSuccess) {
+      g.K2 = 0;
       g.tasks = dTc + stp.trsm_off;
       g.ntiles = stp.ntrsm;
       g.store = 1;
       ProfScope ps(c, PK_GEMM_T3, 2.0 * (double)stp.ntrsm * NB * NB * NB, 16.0 * (double)stp.ntrsm * NB * NB);
-      e = launch_gemm_t3(s, P.ps, P.ws, g);
+      e = launch_gemm_t3(s, panel, P.ws, g);
     }
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_SPLIT, 0.0, 16.0 * (double)stp.ntrsm * NB * NB);
-      e = launch_split_rows_tasks(s, dSpl + stp.psplit_off, stp.nset, stp.max_m, NB, P.ps);
+      e = launch_split_rows_tasks(s, dSpl + stp.psplit_off, stp.nset, stp.max_m, NB, panel);
     }
     if (e == cudaSuccess && stp.nupd > 0) {
       g.tasks = dTc + stp.upd_off;
       g.ntiles = stp.nupd;
       g.store = 0;
-      ProfScope ps(c, PK_GEMM_T3, 2.0 * (double)stp.nupd * NB * NB * NB, 16.0 * (double)stp.nupd * NB * NB);
-      e = launch_gemm_t3(s, P.ps, P.ps, g);
+      g.K2 = second ? NB : 0;
+      ProfScope ps(c, PK_GEMM_T3, 2.0 * (double)stp.nupd * NB * NB * (NB + g.K2), 16.0 * (double)stp.nupd * NB * NB);
+      e = launch_gemm_t3(s, P.ps, P.ps, g, 0, second ? &P.ps2 : nullptr);
     }
   }
   if (e != cudaSuccess) return cuda_err(c, e, "batched tensor-core factorisation");

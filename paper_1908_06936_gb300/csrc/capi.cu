@@ -57,6 +57,9 @@ static bool release_spare(exa_ctx* c) {
     cudaStreamSynchronize(c->stream);
     free_buf(c, c->mx_wall);
     c->wall_spare = c->wall_kept = false;
+  } else if (c->bt_ps2.p && !c->ps2_captured) {
+    cudaStreamSynchronize(c->stream);
+    free_buf(c, c->bt_ps2);
   } else {
     return false;
   }

@@ -82,6 +82,8 @@ struct exa_ctx {
   // batched
   exa::DevBuf bt_mat, bt_meta, bt_vec, bt_work, bt_mat2;
   exa::DevBuf bt_tasks, bt_ps, bt_ws;  // tensor-core batched form: task lists, panel and inverse split operands
+  exa::DevBuf bt_ps2;                  // ... and the second panel's, where there is room
+  bool ps2_captured = false;           // a captured graph may use bt_ps2
   exa::DevBuf bd_mat, bd_buf, bd_task;  // FP64 batched form on the tensor cores
   exa::DigPlan* dplan = nullptr;
   exa::BatchPlan* bplan = nullptr;  // cached work list of the last shape set

@@ -96,9 +96,11 @@ struct T3Tile {
   int64_t ldc;
   bool diag;
   int chunks;  // 32-column steps of the reduction
+  int shift;   // second operand: rows below ya, yb
 };
 __device__ __forceinline__ bool t3_tile(const GemmArgs& g, long long t, T3Tile& o) {
-  o.chunks = g.K / 32;
+  o.chunks = (g.K + g.K2) / 32;
+  o.shift = 0;
   if (g.enum_mode == kEnumTasks) {
     const TcTask tk = g.tasks[t];
     o.ya = tk.a_row;
@@ -106,6 +108,7 @@ __device__ __forceinline__ bool t3_tile(const GemmArgs& g, long long t, T3Tile& 
     o.C = tk.C;
     o.ldc = tk.ldc;
     o.diag = tk.lower != 0;
+    o.shift = tk.shift;
     return true;
   }
   int bi, bj;
@@ -142,13 +145,14 @@ constexpr int OP_BYTES = TM * KC * 4;           // 16 KB per operand tile
 constexpr int STAGE_BYTES = 4 * OP_BYTES;       // A_hi, A_lo, B_hi, B_lo
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
 constexpr uint32_t IDESC = idesc(kFmtTF32, TM, TN);
-constexpr int TMEM_COLS = 256;                  // 2 accumulator buffers x 128 columns
+constexpr int TMEM_COLS = 512;                  // 2 accumulator buffers x 128 columns, for each operand pair
 constexpr int kThreads = 64 + 2 * kEpiThreads;  // eight epilogue warps for each accumulator
 }  // namespace t3
 
 __global__ void __launch_bounds__(t3::kThreads)
     gemm_t3_kernel(const __grid_constant__ CUtensorMap tA_hi, const __grid_constant__ CUtensorMap tA_lo,
                    const __grid_constant__ CUtensorMap tB_hi, const __grid_constant__ CUtensorMap tB_lo,
+                   const __grid_constant__ CUtensorMap tS_hi, const __grid_constant__ CUtensorMap tS_lo,
                    const __grid_constant__ GemmArgs g) {
   using namespace t3;
   extern __shared__ uint8_t smem_raw[];
@@ -178,6 +182,7 @@ __global__ void __launch_bounds__(t3::kThreads)
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
+  const int kc1 = g.K / KC;  // chunks of the first operand pair
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer ----------------
@@ -203,11 +208,21 @@ __global__ void __launch_bounds__(t3::kThreads)
         }
         uint8_t* sb = smem + stage * STAGE_BYTES;
         mbar_expect_tx(&full[stage], one ? 2 * OP_BYTES : STAGE_BYTES);
-        tma_load_2d_hint(sb, &tA_hi, &full[stage], kc * KC, ya, pol);
-        tma_load_2d_hint(sb + 2 * OP_BYTES, &tB_hi, &full[stage], kc * KC, yb, pol);
-        if (!one) {
-          tma_load_2d_hint(sb + OP_BYTES, &tA_lo, &full[stage], kc * KC, ya, pol);
-          tma_load_2d_hint(sb + 3 * OP_BYTES, &tB_lo, &full[stage], kc * KC, yb, pol);
+        if (kc < kc1) {
+          tma_load_2d_hint(sb, &tA_hi, &full[stage], kc * KC, ya, pol);
+          tma_load_2d_hint(sb + 2 * OP_BYTES, &tB_hi, &full[stage], kc * KC, yb, pol);
+          if (!one) {
+            tma_load_2d_hint(sb + OP_BYTES, &tA_lo, &full[stage], kc * KC, ya, pol);
+            tma_load_2d_hint(sb + 3 * OP_BYTES, &tB_lo, &full[stage], kc * KC, yb, pol);
+          }
+        } else {
+          const int kx = (kc - kc1) * KC;
+          tma_load_2d_hint(sb, &tS_hi, &full[stage], kx, ya - tl.shift, pol);
+          tma_load_2d_hint(sb + 2 * OP_BYTES, &tS_hi, &full[stage], kx, yb - tl.shift, pol);
+          if (!one) {
+            tma_load_2d_hint(sb + OP_BYTES, &tS_lo, &full[stage], kx, ya - tl.shift, pol);
+            tma_load_2d_hint(sb + 3 * OP_BYTES, &tS_lo, &full[stage], kx, yb - tl.shift, pol);
+          }
         }
         last_par[stage] = (int)phase;
         if (++stage == STAGES) {
@@ -239,7 +254,6 @@ __global__ void __launch_bounds__(t3::kThreads)
         break;
       }
       fence_after();
-      const uint32_t d = tmem + b * TN;
       const bool one = far_t3(g, tl);
       bool ok = true;
       for (int kc = 0; kc < tl.chunks; ++kc) {
@@ -253,10 +267,12 @@ __global__ void __launch_bounds__(t3::kThreads)
         const uint32_t sb = smem_u32(smem + stage * STAGE_BYTES);
         const uint64_t ahi = sdesc_sw128(sb), alo = sdesc_sw128(sb + OP_BYTES);
         const uint64_t bhi = sdesc_sw128(sb + 2 * OP_BYTES), blo = sdesc_sw128(sb + 3 * OP_BYTES);
+        const uint32_t d = tmem + (kc < kc1 ? 0 : 2 * TN) + b * TN;
+        const bool start = kc == 0 || kc == kc1;
 #pragma unroll
         for (int kk = 0; kk < KC / 8; ++kk) {  // K = 8 per instruction: advance 32 bytes
           const uint64_t o = (uint64_t)(kk * 2);
-          mma_tf32(d, ahi + o, bhi + o, IDESC, (kc | kk) ? 1u : 0u);
+          mma_tf32(d, ahi + o, bhi + o, IDESC, start && kk == 0 ? 0u : 1u);
           if (!one) {
             mma_tf32(d, ahi + o, blo + o, IDESC, 1u);
             mma_tf32(d, alo + o, bhi + o, IDESC, 1u);
@@ -308,8 +324,15 @@ __global__ void __launch_bounds__(t3::kThreads)
 #pragma unroll
         for (int j = 0; j < 16; ++j) cv[j] = g.store ? 0.0 : __ldcs(cp + (int64_t)(cb + j) * ldc);
         uint32_t acc[16];
-        tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + b * TN + cb, acc);
+        const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + b * TN + cb;
+        tmem_ld16(ta, acc);
         tmem_ld_wait();
+        if (g.K2 > 0) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) cv[j] -= f32_bits_to_f64(acc[j]);
+          tmem_ld16(ta + 2 * TN, acc);
+          tmem_ld_wait();
+        }
         if (h4 == 3) {
           fence_before();
           mbar_arrive(&accempty[b]);
@@ -1182,8 +1205,10 @@ static int num_sms() {
 int tc_num_sms() { return num_sms(); }
 
 cudaError_t launch_gemm_t3(cudaStream_t s, const SplitOperand& A, const SplitOperand& B, const GemmArgs& g,
-                           int max_ctas) {
+                           int max_ctas, const SplitOperand* second) {
   if (g.ntiles <= 0) return cudaSuccess;
+  if (g.K2 > 0 && (!second || g.enum_mode != kEnumTasks || g.store)) return cudaErrorInvalidValue;
+  if (!second) second = &A;
   static PerDeviceOnce attr_once;
   {
     const cudaError_t e =
@@ -1193,7 +1218,8 @@ cudaError_t launch_gemm_t3(cudaStream_t s, const SplitOperand& A, const SplitOpe
   int cap = num_sms();
   if (max_ctas > 0 && max_ctas < cap) cap = max_ctas;
   const int grid = (int)(g.ntiles < cap ? g.ntiles : cap);
-  gemm_t3_kernel<<<grid, t3::kThreads, t3::SMEM_BYTES, s>>>(A.t_hi, A.t_lo, B.t_hi, B.t_lo, g);
+  gemm_t3_kernel<<<grid, t3::kThreads, t3::SMEM_BYTES, s>>>(A.t_hi, A.t_lo, B.t_hi, B.t_lo, second->t_hi,
+                                                                 second->t_lo, g);
   return cudaGetLastError();
 }
 

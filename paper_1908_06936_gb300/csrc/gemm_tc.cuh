@@ -23,7 +23,8 @@ struct TcTask {
   double* C;
   int64_t ldc;
   int a_row, b_row;
-  int lower, pad;
+  int lower;
+  int shift;  // launches with a second operand: its rows are a_row - shift and b_row - shift
 };
 
 // One piece of a batched split: rows [0, rows) of src (element (r, k) at src[r rs + k cs]) to
@@ -94,8 +95,10 @@ cudaError_t launch_split_rows(cudaStream_t s, const double* src, int64_t rs, int
 cudaError_t launch_split_rows_tasks(cudaStream_t s, const SplitTask* d_tasks, int ntasks, int max_rows, int K,
                                     SplitOperand& op);
 // max_ctas > 0 caps the persistent grid (to leave SMs to concurrent work).
+// second (task mode, g.K2 = its columns): C = (C - A B^T) - A2 B2^T, both A2 and B2 rows of `second`, each product in an
+// accumulator of its own, so that the result is that of two launches bit for bit.
 cudaError_t launch_gemm_t3(cudaStream_t s, const SplitOperand& A, const SplitOperand& B, const GemmArgs& g,
-                           int max_ctas = 0);
+                           int max_ctas = 0, const SplitOperand* second = nullptr);
 cudaError_t launch_gemm_oz(cudaStream_t s, const SplitOperand& A, const SplitOperand& B, const GemmArgs& g,
                            int max_ctas = 0);
 // T3 on CTA pairs, 256 x 256 tiles (kEnumFull with g.nt = n / 256, or kEnumLowerOffBand with

@@ -419,3 +419,32 @@ def test_batched_autotune_tc_form_reports_its_single_configuration(ctx):
         ref = oracle.loglik(locs[r_], zs[r_], (1.0, 0.1, 0.5))["l"]
         assert abs(got[r_] - ref) <= MIXED_TOL * abs(ref)
         assert abs(f32[r_] - ref) <= MIXED_TOL * abs(ref)
+
+
+@pytest.mark.parametrize("sides", [[11], [12, 3], [17, 12, 20, 16], [33, 5, 40, 36, 23]])
+def test_batched_tc_two_panels_a_pass_keep_the_bits(sides):
+    # tile columns 1 to 13, odd and even; a context bound one byte below what the call holds leaves no room for the second
+    # panel operand (which one or two tile columns do not need), and both forms apply the same updates to an entry in
+    # the same order
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    ns = [m * m for m in sides]
+    locs = [to_dev(synth.jittered_grid(m, m)) for m in sides]
+    z = [to_dev(synth.normals(n, 5)) for n in ns]
+    th = torch.tensor([(1.0, 0.1, 0.5)] * len(ns), dtype=torch.float64, device="cuda")
+
+    def evaluate(bound):
+        out = torch.empty(len(ns), dtype=torch.float64, device="cuda")
+        st = torch.empty(len(ns), dtype=torch.int32, device="cuda")
+        with exa.Context(workspace_bytes=bound) as c:
+            c.check(exa.exa_loglik_batched(c.handle, len(ns), ns, locs, z, th, exa.EXA_MIXED_TF32X3, out, st))
+            torch.cuda.synchronize()
+            assert np.all(st.cpu().numpy() == 0)
+            return out.cpu().numpy(), exa.exa_workspace_bytes(c.handle)
+
+    two, held = evaluate(0)
+    spare = max(ns) > 2 * 128
+    one, less = evaluate(held - 1 if spare else held)
+    assert less < held if spare else less == held
+    assert np.array_equal(two, one)
