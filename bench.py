@@ -326,7 +326,7 @@ def roofline_by_kernel(stats: list, pk: dict) -> list:
             continue
         row = {k: r.get(k) for k in keys}
         if r["kernel"] in LOOKAHEAD_CLASSES:
-            row["note"] += "; look-ahead stream work, on 20-48 SMs beside the trailing update (peak is the whole GPU's)"
+            row["note"] += "; look-ahead stream work, on 20-104 SMs beside the trailing update (peak is the whole GPU's)"
         out.append(row)
     return out
 
@@ -782,6 +782,9 @@ def run_ours(args, rank: int, world: int) -> dict | None:
             fp64 = {"evals_per_s": 1e3 / statistics.mean(ms), "ms_per_eval": statistics.mean(ms),
                     "chol_ms": rr["ms_chol"], "chol_tflops": (n ** 3 / 3.0) / (rr["ms_chol"] * 1e-3) / 1e12,
                     "chol_frac_of_fp64_peak": (n ** 3 / 3.0) / (rr["ms_chol"] * 1e-3) / 1e12 / peaks()["fp64"],
+                    # the products run on the tensor cores as 36 BF16 products of seven-bit digits each
+                    "chol_frac_of_digit_product_ceiling": 36.0 * (n ** 3 / 3.0) / (rr["ms_chol"] * 1e-3) / 1e12
+                    / peaks()["bf16"],
                     "loglik": rr["loglik"], "steps": args.fp64_steps,
                     "warmup": "one FP64 evaluation at n=1,600 (kernels loaded; the n=90,000 buffers are the mixed leg's)"}
         pk = peaks()
