@@ -173,3 +173,23 @@ def test_batched_fp64_at_every_cluster_width(nrep):
         got = batch(c, ns, 0, 0)
         ref = batch(c, ns, 32, 0)
     assert np.all(np.abs(got - ref) <= 1e-10 * np.abs(ref))
+
+
+@pytest.mark.parametrize("m", [23, 40, 64])
+def test_mixed_solves_without_room_for_the_block_inverses(m):
+    # one byte less than the evaluation holds leaves no room for the 512-wide block inverses: the same factor, solved by
+    # the persistent kernels.  Each quadratic form is final to 1e-8 by the refinement's stopping rule.
+    import paper_1908_06936_gb300 as exa
+    from gpu_util import to_dev
+    from paper_1908_06936_gb300 import synth
+
+    locs, z = to_dev(synth.jittered_grid(m, m)), to_dev(synth.normals(m * m, m))
+    theta = (1.0, 0.1, 0.5)
+    with exa.Context() as c:
+        a = c.loglik_ex(locs, z, theta, exa.EXA_MIXED_TF32X3)
+        held = exa.exa_workspace_bytes(c.handle)
+    with exa.Context(workspace_bytes=held - 1) as c:
+        b = c.loglik_ex(locs, z, theta, exa.EXA_MIXED_TF32X3)
+        assert exa.exa_workspace_bytes(c.handle) < held
+    assert a["logdet"] == b["logdet"]
+    assert abs(a["quad"] - b["quad"]) <= 2e-8 * abs(a["quad"])
