@@ -35,7 +35,7 @@ constexpr int kDSub = 128;      // sub-tile
 constexpr int kDW = 32;         // step
 constexpr int kDThreads = 256;
 constexpr int kDLd = kDW + 1;   // row stride of 32-wide tiles in shared memory (odd in doubles)
-constexpr int kDLead = 8;       // CTAs of a leaf's last update, at most (4 rows each)
+constexpr int kDLead = 8;       // CTAs of a leaf's last update, at most (then 4 rows each)
 constexpr int64_t kDiagScratch = 2;  // doubles: barrier counter, abort flag, lead counter
 constexpr long long kDiagSpin = 2000000000LL;  // bound of one barrier wait, SM clock cycles (~1 s)
 
@@ -436,8 +436,7 @@ __device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) sB[lane * kDLd + warp + 8 * u] = vv[u];
         __syncthreads();
-        const int nrow = kDW / nl;
-        for (int i = nrow * b + warp; i < nrow * (b + 1); i += kDThreads / 32) {
+        for (int i = kDW * b / nl + warp; i < kDW * (b + 1) / nl; i += kDThreads / 32) {  // (nl may not divide 32)
           double* pc = a + (r0 + i) + (r0 + lane) * ld;
           double s0 = lane <= i ? __ldcg(pc) : 0.0, s1 = 0.0;
 #pragma unroll
