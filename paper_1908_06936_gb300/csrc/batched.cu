@@ -1457,7 +1457,7 @@ __global__ void batched_fp64_finish_kernel(int nrep, const BMeta* __restrict__ M
   if (r >= nrep) return;
   const BMeta m = M[r];
   if (rstatus[r] == EXA_OK) {
-    if (st->timeout) rstatus[r] = EXA_ERR_TIMEOUT;
+    if (st->timeout || rst[r].timeout) rstatus[r] = EXA_ERR_TIMEOUT;
     else if (rst[r].info) rstatus[r] = EXA_ERR_NOT_SPD;
   }
   double ldet = 0.0, q = 0.0;

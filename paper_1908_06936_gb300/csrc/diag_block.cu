@@ -161,19 +161,6 @@ __device__ __forceinline__ double rsqrt_int(double d) {
   return __longlong_as_double((long long)(((Z + 256) >> 9) + ((unsigned long long)(unsigned int)((1021 - k) << 20) << 32)));
 }
 
-// A flag in shared memory between warps of one CTA: what was written before post is seen after await, which polls (a
-// few tens of cycles; an mbarrier wait takes longer to wake) and gives up after ~2^24 polls.
-__device__ __forceinline__ void post(int* flag, int v) {
-  asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(tc::smem_u32(flag)), "r"(v) : "memory");
-}
-__device__ __forceinline__ void await(const int* flag, int v) {
-  int got;
-  for (int n = 0; n < 1 << 24; ++n) {
-    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(got) : "r"(tc::smem_u32(flag)) : "memory");
-    if (got == v) return;
-  }
-}
-
 // D_j = chol of the 32 x 32 block at step j, on one CTA: a lane per row, the columns on four warps, one per SM quarter:
 // warp w holds columns 4 w .. 4 w + 3 and 16 + 4 w .. 16 + 4 w + 3.  Finished columns go to shared memory, where the
 // other warps wait for them (done[c] = j + 1) and subtract them from their own.  The chain per column is a product, a
@@ -193,6 +180,7 @@ __device__ void diag_leaf(const DiagArgs& g, int j, double* S, int* done) {
   __syncthreads();
   if (warp < 4) {
     double x0[4], x1[4];
+    int polls = tc::kFlagPolls;  // of all the waits below
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       x0[u] = S[(4 * warp + u) * kDLd + lane];
@@ -204,7 +192,7 @@ __device__ void diag_leaf(const DiagArgs& g, int j, double* S, int* done) {
 #pragma unroll
       for (int v = 0; v < 4; ++v) {
         const int c = 4 * q + v;
-        await(done + c, epoch);
+        tc::await(done + c, epoch, polls);
         const double* col = S + c * kDLd;
         const double lic = col[lane];
 #pragma unroll
@@ -239,7 +227,7 @@ __device__ void diag_leaf(const DiagArgs& g, int j, double* S, int* done) {
 #pragma unroll
         for (int v = u + 1; v < 4; ++v) x[v] = fma(-l, __shfl_sync(0xffffffffu, l, cb + v), x[v]);
         __syncwarp();
-        if (lane == 0) post(done + c, epoch);
+        if (lane == 0) tc::post(done + c, epoch);
       }
     };
     // the columns that this warp factors next come first; the later ones fill the time while other warps factor
@@ -250,6 +238,7 @@ __device__ void diag_leaf(const DiagArgs& g, int j, double* S, int* done) {
     factor(x0, 4 * warp);
     for (int q = max(warp - 1, 0); q < 4 + warp; ++q) subtract(x1, 16 + 4 * warp, q);
     factor(x1, 16 + 4 * warp);
+    tc::report_waits(polls, g.st, 73);
     if ((lane & 15) >> 2 == warp) g.w[(int64_t)(j * kDW + lane) * (g.ldw + 1)] = rr;
   }
   __syncthreads();

@@ -56,6 +56,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, volatile
   }
 }
 
+// A flag in shared memory between warps of one CTA: what was written before post is seen after await, which polls (a
+// few tens of cycles; an mbarrier wait takes longer to wake).  `polls` bounds a thread's waits together: once it has run
+// out (~0.3 s from kFlagPolls) they all return at once, and report_waits puts that into the status.
+constexpr int kFlagPolls = 1 << 24;
+__device__ __forceinline__ void post(int* flag, int v) {
+  asm volatile("st.release.cta.shared.b32 [%0], %1;" ::"r"(smem_u32(flag)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void await(const int* flag, int v, int& polls) {
+  int got;
+  do {
+    asm volatile("ld.acquire.cta.shared.b32 %0, [%1];" : "=r"(got) : "r"(smem_u32(flag)) : "memory");
+  } while (got != v && --polls > 0);
+}
+__device__ __forceinline__ void report_waits(int polls, DevStatus* st, int site) {
+  if (polls <= 0 && atomicExch(&st->timeout, 1) == 0) st->timeout_where = site;
+}
+
 // 2-D TMA tile load into shared memory, completion counted on `bar` (bytes).
 // x is the innermost coordinate (in elements), y the row.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y) {
