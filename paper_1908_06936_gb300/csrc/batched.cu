@@ -801,6 +801,89 @@ __global__ void __launch_bounds__(kIrThreads) batched_ir_kernel(
 // ---------------------------------------------------------------------------
 // host driver
 // ---------------------------------------------------------------------------
+// Pinned memory that the asynchronous copies of a call read after it has returned: calls take the slots of a ring in
+// turn, and one waits until the copies from its slot have run (those of the call kSlots before).  The copies of a
+// captured call read their slot at every replay, so it stays as it is for the life of the context; captures of the
+// same data share one.
+struct HostStage {
+  static constexpr int kSlots = 4;
+  struct Slot {
+    uint8_t* p = nullptr;
+    size_t bytes = 0, head = 0;
+    cudaEvent_t read = nullptr;
+  } ring[kSlots];
+  int at = 0;
+  bool capturing = false;  // the current call is being captured
+  std::vector<Slot> captured;
+};
+
+// *out: `bytes` of staging memory that starts with `head`, for copies on the context stream.  stage_end after the last.
+static exa_status stage_begin(exa_ctx* c, const std::vector<uint8_t>& head, size_t bytes, uint8_t** out) {
+  if (!c->stage) c->stage = new HostStage();
+  HostStage& S = *c->stage;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+  if (e != cudaSuccess) return cuda_err(c, e, "staging");
+  S.capturing = cap != cudaStreamCaptureStatusNone;
+  HostStage::Slot fresh, *slot = &fresh;
+  if (S.capturing) {
+    for (HostStage::Slot& q : S.captured)
+      if (bytes == head.size() && q.head == bytes && memcmp(q.p, head.data(), bytes) == 0) {
+        *out = q.p;
+        return EXA_OK;
+      }
+  } else {
+    S.at = (S.at + 1) % HostStage::kSlots;
+    slot = &S.ring[S.at];
+  }
+  // allowed while a stream captures, this one or another thread's: nothing here depends on captured work
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (slot->read) e = cudaEventSynchronize(slot->read);
+  if (e == cudaSuccess && !slot->read && !S.capturing) e = cudaEventCreateWithFlags(&slot->read, cudaEventDisableTiming);
+  if (e == cudaSuccess && slot->bytes < bytes) {
+    if (slot->p) cudaFreeHost(slot->p);
+    slot->p = nullptr;
+    slot->bytes = 0;
+    e = cudaMallocHost(&slot->p, bytes);
+    if (e == cudaSuccess) slot->bytes = bytes;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return set_err(c, EXA_ERR_NOMEM, "pinned staging");
+  }
+  if (e != cudaSuccess) return cuda_err(c, e, "staging");
+  memcpy(slot->p, head.data(), head.size());
+  slot->head = bytes == head.size() ? bytes : 0;
+  if (S.capturing) S.captured.push_back(*slot);
+  *out = slot->p;
+  return EXA_OK;
+}
+
+static cudaError_t stage_end(exa_ctx* c) {
+  HostStage& S = *c->stage;
+  return S.capturing ? cudaSuccess : cudaEventRecord(S.ring[S.at].read, c->stream);
+}
+
+static void release_stage(exa_ctx* c) {
+  if (!c->stage) return;
+  for (HostStage::Slot& q : c->stage->ring) {
+    if (q.read) cudaEventSynchronize(q.read);
+    if (q.read) cudaEventDestroy(q.read);
+    if (q.p) cudaFreeHost(q.p);
+  }
+  for (HostStage::Slot& q : c->stage->captured) cudaFreeHost(q.p);
+  delete c->stage;
+  c->stage = nullptr;
+}
+
+// The elements of v at byte `off` of a staging area's head.
+template <class T>
+static void put_head(std::vector<uint8_t>& head, size_t off, const std::vector<T>& v) {
+  memcpy(head.data() + off, v.data(), v.size() * sizeof(T));
+}
+
 struct TcStep {
   int diag_off, ndiag;       // DiagTileTask range
   int wsplit_off, psplit_off, nset, max_m;  // SplitTask ranges (inverse tiles, panels) and panel rows
@@ -810,6 +893,7 @@ struct TcStep {
 
 struct BatchPlan {
   std::vector<int64_t> ns;
+  bool replayed = false;  // a captured call uploads its lists: they reach the device at each replay, so every call does
   int nb = 0;
   int stall = 0;
   bool mixed = false;
@@ -946,7 +1030,7 @@ static exa_status batched_run(exa_ctx* c, int nrep, const int64_t* h_n, const do
                               const double* const* d_z, const double* d_theta, double* d_loglik, int32_t* d_status) {
   cudaStream_t s = c->stream;
   BatchPlan& P = *c->bplan;
-  const bool same = P.nb == NB && P.mixed == MIXED && P.stall == c->batched_stall && (int)P.ns.size() == nrep &&
+  const bool same = !P.replayed && P.nb == NB && P.mixed == MIXED && P.stall == c->batched_stall && (int)P.ns.size() == nrep &&
                     std::equal(P.ns.begin(), P.ns.end(), h_n);
   std::vector<BMeta> meta(nrep);
   int64_t mo = 0, wo = 0, co = 0, lo = 0, vo = 0, gt = 0;
@@ -1016,23 +1100,21 @@ static exa_status batched_run(exa_ctx* c, int nrep, const int64_t* h_n, const do
   BTask* dT = (BTask*)(base + meta_b + ord_b + par_b + tab_b + ctl_b + cnt_b);
   // the table nodes are scratch until the factorisation overwrites bt_work
   double* dNodes = (double*)c->bt_work.p;
-  // host staging (pinned, owned by the context so captured copies stay valid)
-  const size_t stage_need = meta_b + ord_b + (same ? 0 : task_b);
-  if (c->bt_stage_bytes < stage_need) {
-    if (c->bt_stage) cudaFreeHost(c->bt_stage);
-    c->bt_stage = nullptr;
-    c->bt_stage_bytes = 0;
-    if (cudaMallocHost(&c->bt_stage, stage_need) != cudaSuccess) return set_err(c, EXA_ERR_NOMEM, "pinned staging");
-    c->bt_stage_bytes = stage_need;
+  std::vector<uint8_t> head(meta_b + ord_b);
+  put_head(head, 0, meta);
+  put_head(head, meta_b, order);
+  uint8_t* hs = nullptr;
+  if ((st = stage_begin(c, head, meta_b + ord_b + (same ? 0 : task_b), &hs)) != EXA_OK) {
+    P.ns.clear();
+    return st;
   }
-  uint8_t* hs = (uint8_t*)c->bt_stage;
-  memcpy(hs, meta.data(), nrep * sizeof(BMeta));
-  memcpy(hs + meta_b, order.data(), nrep * sizeof(int));
   cudaError_t e = cudaMemcpyAsync(dM, hs, meta_b + ord_b, cudaMemcpyHostToDevice, s);
   if (!same && e == cudaSuccess) {
     memcpy(hs + meta_b + ord_b, tasks.data(), tasks.size() * sizeof(BTask));
     e = cudaMemcpyAsync(dT, hs + meta_b + ord_b, tasks.size() * sizeof(BTask), cudaMemcpyHostToDevice, s);
+    P.replayed = P.replayed || c->stage->capturing;
   }
+  if (e == cudaSuccess) e = stage_end(c);
   if (e == cudaSuccess) e = cudaMemsetAsync(dC, 0, ctl_b + cnt_b, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(DevStatus), s);
   if (e != cudaSuccess) return cuda_err(c, e, "batched setup");
@@ -1121,7 +1203,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   constexpr int NB = kTcNB;
   cudaStream_t s = c->stream;
   BatchPlan& P = *c->bplan;
-  const bool same_shape = P.tc && P.nb == NB && (int)P.ns.size() == nrep && std::equal(P.ns.begin(), P.ns.end(), h_n);
+  const bool same_shape = !P.replayed && P.tc && P.nb == NB && (int)P.ns.size() == nrep && std::equal(P.ns.begin(), P.ns.end(), h_n);
   std::vector<BMeta> meta(nrep);
   int64_t mo = 0, wo = 0, co = 0, lo = 0, vo = 0, gt = 0;
   int Tmax = 0;
@@ -1300,18 +1382,11 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   DiagTileTask* dDiag = (DiagTileTask*)c->bt_tasks.p;
   SplitTask* dSpl = (SplitTask*)((uint8_t*)c->bt_tasks.p + d_b);
   TcTask* dTc = (TcTask*)((uint8_t*)c->bt_tasks.p + d_b + s_b);
-  // host staging (pinned, owned by the context so captured copies stay valid)
-  const size_t stage_need = meta_b + ord_b + (rebuild ? d_b + s_b + t_b : 0);
-  if (c->bt_stage_bytes < stage_need) {
-    if (c->bt_stage) cudaFreeHost(c->bt_stage);
-    c->bt_stage = nullptr;
-    c->bt_stage_bytes = 0;
-    if (cudaMallocHost(&c->bt_stage, stage_need) != cudaSuccess) return set_err(c, EXA_ERR_NOMEM, "pinned staging");
-    c->bt_stage_bytes = stage_need;
-  }
-  uint8_t* hs = (uint8_t*)c->bt_stage;
-  memcpy(hs, meta.data(), nrep * sizeof(BMeta));
-  memcpy(hs + meta_b, order.data(), nrep * sizeof(int));
+  std::vector<uint8_t> head(meta_b + ord_b);
+  put_head(head, 0, meta);
+  put_head(head, meta_b, order);
+  uint8_t* hs = nullptr;
+  if ((st = stage_begin(c, head, meta_b + ord_b + (rebuild ? d_b + s_b + t_b : 0), &hs)) != EXA_OK) return st;
   cudaError_t e = cudaMemcpyAsync(dM, hs, meta_b + ord_b, cudaMemcpyHostToDevice, s);
   if (rebuild && e == cudaSuccess) {
     uint8_t* ht = hs + meta_b + ord_b;
@@ -1330,7 +1405,9 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
     P.tc_meta = c->bt_meta.p;
     P.ps_rows = ps_rows;
     P.fused = fused;
+    P.replayed = P.replayed || c->stage->capturing;
   }
+  if (e == cudaSuccess) e = stage_end(c);
   if (e == cudaSuccess) e = cudaMemsetAsync(dCnt, 0, cnt_b + rst_b, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(DevStatus), s);
   if (e != cudaSuccess) return cuda_err(c, e, "batched setup");
@@ -1476,10 +1553,9 @@ struct DigStep {
 
 struct DigPlan {
   std::vector<int64_t> ns;
+  bool replayed = false;   // as in BatchPlan
   std::vector<DigStep> steps;
   const void *mat = nullptr, *buf = nullptr, *task = nullptr;  // what the device lists point into
-  void* stage = nullptr;   // pinned; captured copies read it at replay, so no other form writes to it
-  size_t stage_bytes = 0;
 };
 
 // *done = false: its memory could not be had and nothing was launched.
@@ -1516,7 +1592,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     Tmax = m.T > Tmax ? (int)m.T : Tmax;
   }
   if (Tmax > 32000) return EXA_OK;
-  const bool same_shape = (int)P.ns.size() == nrep && std::equal(P.ns.begin(), P.ns.end(), h_n);
+  const bool same_shape = !P.replayed && (int)P.ns.size() == nrep && std::equal(P.ns.begin(), P.ns.end(), h_n);
   // one buffer: meta | params | tables | statuses | row exponents | inverses | log and quadratic parts | z | digits
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -1579,22 +1655,16 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
   DigitTask* dTask = (DigitTask*)(tb + d_b + s_b + z_b);
   const bool rebuild = !same_shape || P.mat != c->bd_mat.p || P.buf != c->bd_buf.p || P.task != c->bd_task.p;
   const size_t meta_b = round_up((int64_t)nrep * sizeof(BMeta), 256);
-  const size_t stage_need = meta_b + (rebuild ? d_b + s_b + z_b + t_b : 0);
-  if (P.stage_bytes < stage_need) {
-    if (P.stage) cudaFreeHost(P.stage);
-    P.stage = nullptr;
-    P.stage_bytes = 0;
-    if (cudaMallocHost(&P.stage, stage_need) != cudaSuccess) {
-      cudaGetLastError();
-      return EXA_OK;
-    }
-    P.stage_bytes = stage_need;
+  std::vector<uint8_t> head(meta_b);
+  put_head(head, 0, meta);
+  uint8_t* hs = nullptr;
+  const exa_status st = stage_begin(c, head, meta_b + (rebuild ? d_b + s_b + z_b + t_b : 0), &hs);
+  if (st == EXA_ERR_NOMEM) {
+    c->err[0] = 0;
+    return EXA_OK;
   }
-  uint8_t* hs = (uint8_t*)P.stage;
+  if (st != EXA_OK) return st;
   if (rebuild) {
-    // an earlier call's copies may still read the staging area
-    const cudaError_t es = cudaStreamSynchronize(s);
-    if (es != cudaSuccess) return cuda_err(c, es, "batched setup");
     P.steps.clear();
     P.ns.clear();
     DiagTileTask* hd = (DiagTileTask*)(hs + meta_b);
@@ -1661,11 +1731,13 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     P.buf = c->bd_buf.p;
     P.task = c->bd_task.p;
   }
-  memcpy(hs, meta.data(), nrep * sizeof(BMeta));
   *done = true;
   cudaError_t e = cudaMemcpyAsync(dM, hs, nrep * sizeof(BMeta), cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess && rebuild)
     e = cudaMemcpyAsync(tb, hs + meta_b, d_b + s_b + z_b + t_b, cudaMemcpyHostToDevice, s);
+  P.replayed = P.replayed || (rebuild && c->stage->capturing);
+  if (e != cudaSuccess) P.ns.clear();
+  if (e == cudaSuccess) e = stage_end(c);
   if (e == cudaSuccess) e = cudaMemsetAsync(dRst, 0, nrep * sizeof(DevStatus), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, sizeof(DevStatus), s);
   if (e != cudaSuccess) return cuda_err(c, e, "batched setup");
@@ -1737,13 +1809,10 @@ void release_batched_digits(exa_ctx* c) {
 }
 
 void release_batched(exa_ctx* c) {
-  if (c->bt_stage) cudaFreeHost(c->bt_stage);
-  c->bt_stage = nullptr;
-  c->bt_stage_bytes = 0;
+  release_stage(c);
   delete c->bplan;
   c->bplan = nullptr;
   release_batched_digits(c);
-  if (c->dplan && c->dplan->stage) cudaFreeHost(c->dplan->stage);
   delete c->dplan;
   c->dplan = nullptr;
 }

@@ -11,6 +11,7 @@ namespace exa {
 
 struct BatchPlan;
 struct DigPlan;
+struct HostStage;
 
 struct DevBuf {
   void* p = nullptr;
@@ -87,8 +88,7 @@ struct exa_ctx {
   exa::DevBuf bd_mat, bd_buf, bd_task;  // FP64 batched form on the tensor cores
   exa::DigPlan* dplan = nullptr;
   exa::BatchPlan* bplan = nullptr;  // cached work list of the last shape set
-  void* bt_stage = nullptr;         // pinned host staging for the work list / metadata
-  size_t bt_stage_bytes = 0;
+  exa::HostStage* stage = nullptr;  // pinned memory that the batched forms' copies read
   int batched_nb = 64;              // tile of the batched factorisation (32 or 64)
   int batched_ctas_per_sm = 0;      // 0: as many as fit
   long long batched_spin = 2000000000LL;  // bound of one dependency wait (SM cycles)
