@@ -1064,7 +1064,7 @@ static exa_status batched_run(exa_ctx* c, int nrep, const int64_t* h_n, const do
     for (int r = 0; r < nrep; ++r) Tmax = meta[r].T > Tmax ? (int)meta[r].T : Tmax;
     if (Tmax > 32000) return set_err(c, EXA_ERR_ARG, "replicate too large for the batched form");
     build_task_list(meta, MIXED, c->batched_stall != 0, tasks);
-    P.ns.assign(h_n, h_n + nrep);
+    P.ns.clear();  // until the list is on its way to the device
     P.nb = NB;
     P.stall = c->batched_stall;
     P.mixed = MIXED;
@@ -1104,14 +1104,12 @@ static exa_status batched_run(exa_ctx* c, int nrep, const int64_t* h_n, const do
   put_head(head, 0, meta);
   put_head(head, meta_b, order);
   uint8_t* hs = nullptr;
-  if ((st = stage_begin(c, head, meta_b + ord_b + (same ? 0 : task_b), &hs)) != EXA_OK) {
-    P.ns.clear();
-    return st;
-  }
+  if ((st = stage_begin(c, head, meta_b + ord_b + (same ? 0 : task_b), &hs)) != EXA_OK) return st;
   cudaError_t e = cudaMemcpyAsync(dM, hs, meta_b + ord_b, cudaMemcpyHostToDevice, s);
   if (!same && e == cudaSuccess) {
     memcpy(hs + meta_b + ord_b, tasks.data(), tasks.size() * sizeof(BTask));
     e = cudaMemcpyAsync(dT, hs + meta_b + ord_b, tasks.size() * sizeof(BTask), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) P.ns.assign(h_n, h_n + nrep);
     P.replayed = P.replayed || c->stage->capturing;
   }
   if (e == cudaSuccess) e = stage_end(c);
@@ -1301,6 +1299,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
   std::vector<SplitTask> spl;
   std::vector<TcTask> tc;
   if (rebuild) {
+    P.ns.clear();  // until the lists are on their way to the device
     P.steps.clear();
     std::vector<int> before(nrep, 0);  // first operand row of each replicate in the panel before
     for (int k = 0; k < Tmax; ++k) {
@@ -1394,7 +1393,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
     memcpy(ht + d_b, spl.data(), spl.size() * sizeof(SplitTask));
     memcpy(ht + d_b + s_b, tc.data(), tc.size() * sizeof(TcTask));
     e = cudaMemcpyAsync(c->bt_tasks.p, ht, d_b + s_b + t_b, cudaMemcpyHostToDevice, s);
-    P.ns.assign(h_n, h_n + nrep);
+    if (e == cudaSuccess) P.ns.assign(h_n, h_n + nrep);
     P.nb = NB;
     P.tc = true;
     P.mixed = true;
