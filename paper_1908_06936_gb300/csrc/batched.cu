@@ -1663,6 +1663,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     return EXA_OK;
   }
   if (st != EXA_OK) return st;
+  c->bd_captured = c->bd_captured || c->stage->capturing;
   if (rebuild) {
     P.steps.clear();
     P.ns.clear();

@@ -49,7 +49,8 @@ static void free_buf(exa_ctx* c, DevBuf& b) {
   b.bytes = 0;
 }
 
-// Gives up what its owner does without; false: nothing is held of that kind.
+// Gives up one kind of memory that its owner does without (no call takes such memory before its last request for what it
+// needs, or it asks for it anew); false: none is held.
 static bool release_spare(exa_ctx* c) {
   if (c->digits_held) {
     release_digits(c);
@@ -60,6 +61,13 @@ static bool release_spare(exa_ctx* c) {
   } else if (c->bt_ps2.p && !c->ps2_captured) {
     cudaStreamSynchronize(c->stream);
     free_buf(c, c->bt_ps2);
+  } else if ((c->bd_mat.p || c->bd_buf.p || c->bd_task.p) && !c->bd_captured) {
+    cudaStreamSynchronize(c->stream);
+    release_batched_digits(c);
+  } else if (c->gr_table.p || c->pr_m.p) {
+    cudaStreamSynchronize(c->stream);
+    free_buf(c, c->gr_table);
+    free_buf(c, c->pr_m);
   } else {
     return false;
   }
@@ -71,7 +79,8 @@ static bool release_spare(exa_ctx* c) {
 // optional ones back.
 exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool optional) {
   if (bytes <= b.bytes) return EXA_OK;
-  if (!optional && c->ws_limit && c->held_bytes - b.bytes + bytes > c->ws_limit) release_spare(c);
+  while (!optional && c->ws_limit && c->held_bytes - b.bytes + bytes > c->ws_limit && release_spare(c)) {
+  }
   const size_t held = c->held_bytes - b.bytes;
   if (c->ws_limit && held + bytes > c->ws_limit)
     return set_err(c, EXA_ERR_NOMEM, "workspace %s needs %zu bytes; context bound is %zu (held %zu)", name, bytes,
@@ -85,7 +94,7 @@ exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool op
   }
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
-  if (e != cudaSuccess && !optional && release_spare(c)) {
+  while (e != cudaSuccess && !optional && release_spare(c)) {
     cudaGetLastError();
     e = cudaMalloc(&p, bytes);
   }

@@ -86,6 +86,7 @@ struct exa_ctx {
   exa::DevBuf bt_ps2;                  // ... and the second panel's, where there is room
   bool ps2_captured = false;           // a captured graph may use bt_ps2
   exa::DevBuf bd_mat, bd_buf, bd_task;  // FP64 batched form on the tensor cores
+  bool bd_captured = false;             // a captured graph may use them
   exa::DigPlan* dplan = nullptr;
   exa::BatchPlan* bplan = nullptr;  // cached work list of the last shape set
   exa::HostStage* stage = nullptr;  // pinned memory that the batched forms' copies read
