@@ -1309,7 +1309,7 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
         const BMeta& m = meta[r];
         if (m.T <= k) continue;
         diag.push_back({mat + m.mo, m.npad, (int64_t)k * NB, ldpart + m.lo + k, wbuf + m.wo + (int64_t)k * NB * NB,
-                        dRst + r, nullptr, nullptr, nullptr});
+                        dRst + r});
       }
       stp.ndiag = (int)diag.size() - stp.diag_off;
       // replicates with a panel below tile k
@@ -1545,7 +1545,7 @@ __global__ void batched_fp64_finish_kernel(int nrep, const BMeta* __restrict__ M
 }
 
 struct DigStep {
-  int diag_off, ndiag, set_off, nset;     // DiagTileTask range; ZTask range, and the split tasks at twice its offsets
+  int diag_off, ndiag, set_off, nset;     // SolveTileTask range; ZTask range, and the split tasks at twice its offsets
   long long trsm_off, ntrsm, upd_off, nupd;
   int64_t max_m;
 };
@@ -1616,7 +1616,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     nset += T - 1;
     ntask += T * (T - 1) + (T - 1) * T * (T + 1) / 3;  // sum of 2 b (solves) and of b (b + 1) (updates), b < T
   }
-  const size_t d_b = round_up(nd * (int64_t)sizeof(DiagTileTask), 256);
+  const size_t d_b = round_up(nd * (int64_t)sizeof(SolveTileTask), 256);
   const size_t s_b = round_up(2 * nset * (int64_t)sizeof(DigitSplitTask), 256);
   const size_t z_b = round_up(nset * (int64_t)sizeof(ZTask), 256);
   const size_t t_b = round_up(ntask * (int64_t)sizeof(DigitTask), 256);
@@ -1648,7 +1648,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
   digit_layout(Ws, base + o_ws, (int64_t)nrep * NB, NB, kDigSlices);
   digit_layout(Ps, base + o_ps, ps_rows, NB, kDigSlices);
   uint8_t* tb = (uint8_t*)c->bd_task.p;
-  DiagTileTask* dDiag = (DiagTileTask*)tb;
+  SolveTileTask* dDiag = (SolveTileTask*)tb;
   DigitSplitTask* dSpl = (DigitSplitTask*)(tb + d_b);
   ZTask* dZ = (ZTask*)(tb + d_b + s_b);
   DigitTask* dTask = (DigitTask*)(tb + d_b + s_b + z_b);
@@ -1667,7 +1667,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
   if (rebuild) {
     P.steps.clear();
     P.ns.clear();
-    DiagTileTask* hd = (DiagTileTask*)(hs + meta_b);
+    SolveTileTask* hd = (SolveTileTask*)(hs + meta_b);
     DigitSplitTask* hp = (DigitSplitTask*)(hs + meta_b + d_b);
     ZTask* hz = (ZTask*)(hs + meta_b + d_b + s_b);
     DigitTask* ht = (DigitTask*)(hs + meta_b + d_b + s_b + z_b);
@@ -1684,8 +1684,9 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
       for (int r = 0; r < nrep; ++r) {
         const BMeta& m = meta[r];
         if (m.T <= k) continue;
-        hd[id++] = {mat + m.mo, m.npad, (int64_t)k * NB, ldpart + m.lo + k, wbuf + m.wo + (int64_t)k * NB * NB,
-                    dRst + r, zbuf + m.vo + (int64_t)k * NB, qpart + m.lo + k, dRex + r * NB};
+        hd[id++] = {{mat + m.mo, m.npad, (int64_t)k * NB, ldpart + m.lo + k, wbuf + m.wo + (int64_t)k * NB * NB,
+                     dRst + r},
+                    zbuf + m.vo + (int64_t)k * NB, qpart + m.lo + k, dRex + r * NB};
         if (m.T == k + 1) continue;
         set.push_back(r);
         prow.push_back(rows);

@@ -49,25 +49,29 @@ static void free_buf(exa_ctx* c, DevBuf& b) {
   b.bytes = 0;
 }
 
+void free_spare(exa_ctx* c, std::initializer_list<DevBuf*> bufs) {
+  cudaStreamSynchronize(c->stream);
+  for (DevBuf* b : bufs) free_buf(c, *b);
+}
+
 // Gives up one kind of memory that its owner does without (no call takes such memory before its last request for what it
 // needs, or it asks for it anew); false: none is held.
 static bool release_spare(exa_ctx* c) {
   if (c->digits_held) {
     release_digits(c);
   } else if (c->wall_spare) {
-    cudaStreamSynchronize(c->stream);
-    free_buf(c, c->mx_wall);
+    free_spare(c, {&c->mx_wall});
     c->wall_spare = c->wall_kept = false;
   } else if (c->bt_ps2.p && !c->ps2_captured) {
-    cudaStreamSynchronize(c->stream);
-    free_buf(c, c->bt_ps2);
+    free_spare(c, {&c->bt_ps2});
   } else if ((c->bd_mat.p || c->bd_buf.p || c->bd_task.p) && !c->bd_captured) {
     cudaStreamSynchronize(c->stream);
     release_batched_digits(c);
+  } else if (c->pred_spare) {
+    free_spare(c, {&c->pr_c, &c->pr_y});
+    c->pred_spare = false;
   } else if (c->gr_table.p || c->pr_m.p) {
-    cudaStreamSynchronize(c->stream);
-    free_buf(c, c->gr_table);
-    free_buf(c, c->pr_m);
+    free_spare(c, {&c->gr_table, &c->pr_m});
   } else {
     return false;
   }
@@ -387,14 +391,13 @@ exa_status loglik_fp64(exa_ctx* c, const double* d_locs, const double* d_z, cons
   const int T = (int)(npad / nb);
   exa_status st;
   if ((st = ensure(c, c->mat, (size_t)npad * npad * sizeof(double), "matrix")) != EXA_OK) return st;
-  if ((st = ensure(c, c->vec, (size_t)(2 * npad + kSolveScratch) * sizeof(double), "vectors")) != EXA_OK) return st;
+  if ((st = ensure(c, c->vec, (size_t)2 * npad * sizeof(double), "vectors")) != EXA_OK) return st;
   if ((st = ensure(c, c->partial, (size_t)(kPartialDoubles(npad, nb)) * sizeof(double), "partials")) != EXA_OK)
     return st;
   if ((st = reset_status(c)) != EXA_OK) return st;
   double* A = (double*)c->mat.p;
   double* zw = (double*)c->vec.p;  // working right-hand side
   double* y = zw + npad;           // L^-1 z
-  double* tmp = y + npad;
   double* part = (double*)c->partial.p;
   MaternParams P;
   model_params(c, theta, &P);
@@ -414,7 +417,7 @@ exa_status loglik_fp64(exa_ctx* c, const double* d_locs, const double* d_z, cons
     ProfScope ps(c, PK_OTHER, 0.0, 16.0 * (double)npad);
     e = launch_pad_vector(c->stream, d_z, n, npad, zw);
   }
-  if (e == cudaSuccess) e = solve_forward(c, npad, nb, zw, y, tmp);
+  if (e == cudaSuccess) e = solve_forward(c, npad, nb, zw, y);
   if (e == cudaSuccess) {
     ProfScope ps(c, PK_OTHER, 0.0, 8.0 * (double)npad, 4);
     e = launch_sumsq(c->stream, y, npad, part, c->d_scalars + 0);

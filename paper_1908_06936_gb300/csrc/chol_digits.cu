@@ -31,7 +31,7 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
     DevBuf* b;
     size_t bytes;
   } want[] = {{&c->mx_w2, (size_t)kNB * kNB * sizeof(double)},
-              {&c->mx_dscr, diag_block_scratch_doubles() * sizeof(double)},
+              {&c->mx_dscr, (diag_block_scratch_doubles() + kSolveScratch) * sizeof(double)},
               {&c->mx_wall, (size_t)(npad / kNB) * kNB * kNB * sizeof(double)},
               {&c->mx_split, below ? align256(digit_bytes(below, kNB, kDigSlices)) : 0},
               {&c->mx_split_b, below ? 2 * block_bytes(kDigSlices) + block_bytes(kDigLow) : 0},
@@ -208,8 +208,9 @@ const double* block_inverse(exa_ctx* c, int64_t k0, int h) {
   return h == kNB ? (const double*)c->mx_wall.p + k0 * kNB : (const double*)c->w_all.p + k0 * kSub;
 }
 
-cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y, double* tmp) {
+cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y) {
   const double* a = (const double*)c->mat.p;
+  double* tmp = (double*)c->mx_dscr.p + diag_block_scratch_doubles();  // with the block inverses only
   cudaError_t e = cudaSuccess;
   for (int64_t k0 = 0, h; k0 < npad && e == cudaSuccess; k0 += h) {
     h = !c->wall_kept ? nb : npad - k0 >= kNB ? kNB : kSub;
@@ -225,8 +226,9 @@ cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y
   return e;
 }
 
-cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y, double* tmp) {
+cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y) {
   const double* a = (const double*)c->mat.p;
+  double* tmp = (double*)c->mx_dscr.p + diag_block_scratch_doubles();
   const int64_t full = npad / kNB * kNB;  // the 128-wide blocks start here
   cudaError_t e = cudaSuccess;
   for (int64_t end = npad, h; end > 0 && e == cudaSuccess; end -= h) {

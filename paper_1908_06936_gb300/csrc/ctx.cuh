@@ -3,6 +3,8 @@
 
 #include <stddef.h>
 
+#include <initializer_list>
+
 #include "exa_internal.cuh"
 #include "gemm_tc.cuh"
 #include "prof.cuh"
@@ -62,7 +64,7 @@ struct exa_ctx {
   exa::DevBuf mx_vec;       // refinement vectors
   exa::DevBuf mx_w2;        // inverse of the panel-wide diagonal block (row-major)
   exa::DevBuf mx_wall;      // every panel's diagonal-block inverse, T x 512 x 512 (kept for the gradient)
-  exa::DevBuf mx_dscr;      // scratch of the cooperative diagonal-block factorisation
+  exa::DevBuf mx_dscr;      // scratch of the cooperative diagonal-block factorisation, then of the block solves
   int keep_block_inverses = 0;  // mixed factorisation: write block k's inverse to mx_wall + k 512^2 (2: if there is room)
   int ir_tight = 0;         // mixed refinement: iterate to rounding level (the gradient needs Sigma^-1 z)
   double ir_target = 0.0;   // mixed refinement: relative residual to reach (0: quadratic-form rule)
@@ -79,6 +81,7 @@ struct exa_ctx {
   exa::DevBuf gr_blocks;    // per-block gradient partial sums
   exa::DevBuf pr_c, pr_y;   // prediction: cross-covariance block and its solve block
   exa::DevBuf pr_m;         // prediction: partial sums of the means
+  bool pred_spare = false;  // pr_c and pr_y are between two predictions on the tensor cores, larger than the others'
   exa::DevBuf fs_m;         // Fisher information: Sigma^-1 D_k for k = 0, 1, 2
   // batched
   exa::DevBuf bt_mat, bt_meta, bt_vec, bt_work, bt_mat2;
@@ -117,6 +120,8 @@ namespace exa {
 exa_status set_err(exa_ctx* c, exa_status st, const char* fmt, ...);
 exa_status cuda_err(exa_ctx* c, cudaError_t e, const char* what);
 exa_status ensure(exa_ctx* c, DevBuf& b, size_t bytes, const char* name, bool optional = false);
+// Frees buffers that the context stream may still use.
+void free_spare(exa_ctx* c, std::initializer_list<DevBuf*> bufs);
 exa_status check_theta(exa_ctx* c, const double theta[3]);
 exa_status reset_status(exa_ctx* c);
 exa_status read_status(exa_ctx* c);
@@ -128,10 +133,10 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
 bool reserve_digits(exa_ctx* c, int64_t npad);
 void release_digits(exa_ctx* c);
 // y = L^-1 z (z overwritten) and y <- L^-T y with the FP64 factor in c->mat, by the block inverses its factorisation left
-// (of nb-wide tiles, or the digit path's); tmp: kSolveScratch doubles.
-constexpr int kSolveScratch = 1024;
-cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y, double* tmp);
-cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y, double* tmp);
+// (of nb-wide tiles, or the digit path's).
+constexpr int kSolveScratch = 1024;  // doubles, in mx_dscr after the diagonal block's
+cudaError_t solve_forward(exa_ctx* c, int64_t npad, int nb, double* z, double* y);
+cudaError_t solve_backward(exa_ctx* c, int64_t npad, int nb, double* y);
 // The digit path's inverse of the h x h diagonal block at k0 (row-major).
 const double* block_inverse(exa_ctx* c, int64_t k0, int h);
 // Sigma^-1 on the tensor cores: room for it (allocate = false: whether it is held), and the inverse in the lower

@@ -530,16 +530,16 @@ __global__ void __launch_bounds__(kDThreads) diag_block_kernel(const __grid_cons
   diag_body(g, GridGroup(scr, g.st), sm);
 }
 
-// One 128 x 128 tile a cluster; with task.z also y = W z, y^T y and the row exponents of L.
-__global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const DiagTileTask* __restrict__ tasks) {
+// One 128 x 128 tile a cluster, and y = W z, y^T y and the row exponents of L.
+__global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const SolveTileTask* __restrict__ tasks) {
   __shared__ DiagSmem sm;
   ClusterGroup grp;
   const int G = grp.size(), b = grp.rank(), tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const DiagTileTask t = tasks[blockIdx.x / G];
+  const SolveTileTask task = tasks[blockIdx.x / G];
+  const DiagTileTask& t = task.tile;
   const DiagArgs g{t.a, t.ld, t.k0, t.w, kDSub, kDSub, nullptr, t.logdet, t.st, kDSub};
   diag_body(g, grp, sm);
   grp.sync();
-  if (!t.z) return;
   if (b == G - 1) {  // the exponents, two threads a row
     const double* row = t.a + t.k0 + (tid >> 1) + t.k0 * t.ld;
     int hi = 0;
@@ -549,11 +549,11 @@ __global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const DiagTile
       if (cc <= tid >> 1) hi = max(hi, __double2hiint(__ldcg(row + cc * t.ld)) & 0x7FFFFFFF);
     }
     hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, 1));
-    if (!(tid & 1)) t.rex[tid >> 1] = (hi >> 20) - 1022;
+    if (!(tid & 1)) task.rex[tid >> 1] = (hi >> 20) - 1022;
   }
   if (b != 0) return;
   double* zs = sm.S;
-  if (tid < kDSub) zs[tid] = t.z[tid];
+  if (tid < kDSub) zs[tid] = task.z[tid];
   __syncthreads();
   double qs = 0.0;
 #pragma unroll 4
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const DiagTile
     for (int q = 0; q < 4; ++q) s = fma(__ldcg(t.w + r * kDSub + lane + 32 * q), zs[lane + 32 * q], s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) t.z[r] = s;
+    if (lane == 0) task.z[r] = s;
     qs = fma(s, s, qs);
   }
   __syncthreads();
@@ -572,13 +572,13 @@ __global__ void __launch_bounds__(kDThreads, 2) diag_tasks_kernel(const DiagTile
   if (tid == 0) {
     double s = 0.0;
     for (int q = 0; q < 8; ++q) s += zs[q];
-    *t.quad = s;
+    *task.quad = s;
   }
 }
 
 // The widest cluster with which every tile has its SMs at once: more CTAs shorten a tile, but tiles that queue cost
 // more.
-cudaError_t launch_diag128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks) {
+cudaError_t launch_diag128_tasks(cudaStream_t s, const SolveTileTask* d_tasks, int ntasks) {
   if (ntasks <= 0) return cudaSuccess;
   int G = 8;
   while (G > 1 && G * ntasks > tc_num_sms()) G /= 2;

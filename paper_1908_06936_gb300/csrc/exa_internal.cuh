@@ -151,8 +151,11 @@ struct DiagTileTask {
   double* logdet;
   double* w;
   DevStatus* st;
-  // diag128 only, with z != nullptr also: z (128 entries, the right-hand side here) <- y = W z, *quad = y^T y, and
-  // rex[i] the exponent e of row i of L (|L_ij| < 2^e)
+};
+// Also: z (128 entries, the right-hand side here) <- y = W z, *quad = y^T y, and rex[i] the exponent e of row i of L
+// (|L_ij| < 2^e).
+struct SolveTileTask {
+  DiagTileTask tile;
   double* z;
   double* quad;
   int* rex;
@@ -160,7 +163,7 @@ struct DiagTileTask {
 // A CTA a tile (the mixed path's: its likelihoods repeat the rounding of these tiles, so their arithmetic is kept), and
 // a cluster a tile.
 cudaError_t launch_potrf128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks);
-cudaError_t launch_diag128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks);
+cudaError_t launch_diag128_tasks(cudaStream_t s, const SolveTileTask* d_tasks, int ntasks);
 // FP64 Cholesky and inverse of the 512 x 512 diagonal block at (k0, k0) as one cooperative launch
 // of `grid` CTAs (>= 2): L in place, log sums of the four 128 sub-tiles into logdet_part[0..3], their
 // inverses (row-major) into w_sub, the block inverse (row-major) into w2; scratch holds

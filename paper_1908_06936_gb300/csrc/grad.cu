@@ -782,7 +782,7 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
   double* A = (double*)c->mat.p;
   cudaStream_t s = c->stream;
   // a = L^-T y (in place in y)
-  cudaError_t e = solve_backward(c, npad, nb, y, y + npad);
+  cudaError_t e = solve_backward(c, npad, nb, y);
   const bool digits = !one_buffer && c->wall_kept && reserve_inverse_digits(c, npad, false);
   if (!digits && (st = ensure(c, c->panel, (size_t)npad * nb * sizeof(double), "panel")) != EXA_OK) return st;
   if (!one_buffer) {

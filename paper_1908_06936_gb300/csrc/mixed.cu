@@ -352,7 +352,8 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   const int nbuf = fuse ? 4 : 2;
   if ((st = ensure_split(c, c->sp_b, c->mx_split_b, NB, NB, true, true)) != EXA_OK) return st;
   if ((st = ensure(c, c->mx_w2, (size_t)NB * NB * sizeof(double), "diagonal block inverse")) != EXA_OK) return st;
-  if ((st = ensure(c, c->mx_dscr, diag_block_scratch_doubles() * sizeof(double), "diagonal block scratch")) != EXA_OK)
+  if ((st = ensure(c, c->mx_dscr, (diag_block_scratch_doubles() + kSolveScratch) * sizeof(double),
+                   "diagonal block scratch")) != EXA_OK)
     return st;
   if ((st = ensure_side(c)) != EXA_OK) return st;
   if (c->keep_block_inverses) {  // last: 2 is a wish
@@ -422,14 +423,14 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
 
 // x = (L L^T)^-1 rhs with the FP64-stored factor: in 512-row block steps where the factorisation kept the block
 // inverses, else on 128-wide tiles with the sub-tile inverses (the upper tiles of a then hold L^T).  flags: scratch for
-// the persistent solves' flags; tmp: kSolveScratch doubles.
+// the persistent solves' flags.
 static cudaError_t solve_llt(exa_ctx* c, const double* a, int64_t ld, int64_t npad, const double* rhs, double* x,
-                             double* work, int* flags, double* tmp) {
+                             double* work, int* flags) {
   cudaError_t e = cudaMemcpyAsync(work, rhs, npad * sizeof(double), cudaMemcpyDeviceToDevice, c->stream);
   if (e != cudaSuccess) return e;
   if (c->wall_kept) {
-    e = solve_forward(c, npad, kMixSub, work, x, tmp);
-    return e == cudaSuccess ? solve_backward(c, npad, kMixSub, x, tmp) : e;
+    e = solve_forward(c, npad, kMixSub, work, x);
+    return e == cudaSuccess ? solve_backward(c, npad, kMixSub, x) : e;
   }
   ProfScope ps(c, PK_TRSV, 2.0 * (double)npad * (double)npad, 8.0 * (double)npad * (double)npad, 2);
   return launch_llt_solve_persistent(c->stream, a, ld, npad, (const double*)c->w_all.p, work, x, flags,
@@ -518,7 +519,7 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
   exa_status st;
   if ((st = ensure(c, c->mx_sigma, (size_t)npad * npad * sizeof(double), "FP64 covariance copy")) != EXA_OK)
     return st;
-  if ((st = ensure(c, c->mx_vec, (size_t)(6 * npad + kSolveScratch) * sizeof(double), "refinement vectors")) != EXA_OK)
+  if ((st = ensure(c, c->mx_vec, (size_t)6 * npad * sizeof(double), "refinement vectors")) != EXA_OK)
     return st;
   if ((st = ensure(c, c->partial, (size_t)(2 * kRedPartials + 2 * npad + 64) * sizeof(double), "partials")) != EXA_OK)
     return st;
@@ -533,7 +534,6 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
   double* d = r + npad;
   double* y = d + npad;
   double* work = y + npad;
-  double* tmp = work + npad;
   double* part = (double*)c->partial.p;
   double* red = part + 2 * kRedPartials;  // the solves' flags live after the reduction partials
   cudaStream_t s = c->stream;
@@ -557,7 +557,7 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
     ProfScope ps(c, PK_OTHER, 0.0, 8.0 * (double)npad * (double)npad);
     e = launch_transpose_lower_to_upper(s, A, npad, npad);
   }
-  if (e == cudaSuccess) e = solve_llt(c, A, npad, npad, zp, x, work, (int*)red, tmp);
+  if (e == cudaSuccess) e = solve_llt(c, A, npad, npad, zp, x, work, (int*)red);
   if (e != cudaSuccess) return cuda_err(c, e, "solve launch");
   // iterative refinement of x = Sigma^-1 z with the FP64 residual.  It stops when the
   // residual no longer halves or reaches rounding level, or once the quadratic form is final
@@ -595,7 +595,7 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
     rel_prev = rel;
     if (!(rel > (target > 0.0 ? target : 1e-15)) || it >= kMaxIt || rel > 0.5 * prev) break;
     prev = rel;
-    e = solve_llt(c, A, npad, npad, r, d, work, (int*)red, tmp);
+    e = solve_llt(c, A, npad, npad, r, d, work, (int*)red);
     // the variational estimate of q before x moves: with r = z - Sigma x and d = (L L^T)^-1 r,
     // q = z^T x + x^T r + r^T Sigma^-1 r, so q_hat = z^T x + x^T r + r^T d is off by
     // r^T (Sigma^-1 - (L L^T)^-1) r, second order in the residual (about the contraction

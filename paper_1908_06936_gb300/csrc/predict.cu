@@ -212,7 +212,7 @@ extern "C" exa_status exa_predict(exa_ctx* c, const double* d_locs, const double
   const double* W = (const double*)c->w_all.p;
   cudaStream_t s = c->stream;
   // a = L^-T y (in place)
-  cudaError_t e = solve_backward(c, npad, nb, y, y + npad);
+  cudaError_t e = solve_backward(c, npad, nb, y);
   if (e != cudaSuccess) return cuda_err(c, e, "prediction solve");
   MaternParams P;
   model_params(c, theta, &P);
@@ -237,9 +237,11 @@ extern "C" exa_status exa_predict(exa_ctx* c, const double* d_locs, const double
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return cuda_err(c, e, "prediction mean");
+  c->pred_spare = false;  // the buffers are this call's until it ends
   if (d_var && c->wall_kept && reserve_inverse_digits(c, npad, false, mc) &&
       ensure(c, c->pr_c, (size_t)npad * mc * sizeof(double), "prediction cross covariance", true) == EXA_OK &&
       ensure(c, c->pr_y, (size_t)(kDigMaxK + 1) * mc * sizeof(double), "prediction solve block", true) == EXA_OK) {
+    c->pred_spare = true;
     double* C = (double*)c->pr_c.p;
     double* Y = (double*)c->pr_y.p;
     double* acc = Y + (size_t)kDigMaxK * mc;
@@ -260,13 +262,12 @@ extern "C" exa_status exa_predict(exa_ctx* c, const double* d_locs, const double
     if (e != cudaSuccess) return cuda_err(c, e, "prediction variance");
   } else if (d_var) {
     c->err[0] = 0;
-    // variance: blocks of kPredCols new points
-    if ((st = ensure(c, c->pr_c, (size_t)npad * kPredCols * sizeof(double), "prediction cross covariance")) !=
-        EXA_OK)
-      return st;
-    if ((st = ensure(c, c->pr_y, (size_t)(nb + 1) * kPredCols * sizeof(double), "prediction solve block")) !=
-        EXA_OK)
-      return st;
+    // variance: blocks of kPredCols new points; what was sized for more goes first
+    const size_t c_bytes = (size_t)npad * kPredCols * sizeof(double);
+    const size_t y_bytes = (size_t)(nb + 1) * kPredCols * sizeof(double);
+    if (c->pr_c.bytes > c_bytes || c->pr_y.bytes > y_bytes) free_spare(c, {&c->pr_c, &c->pr_y});
+    if ((st = ensure(c, c->pr_c, c_bytes, "prediction cross covariance")) != EXA_OK) return st;
+    if ((st = ensure(c, c->pr_y, y_bytes, "prediction solve block")) != EXA_OK) return st;
     double* C = (double*)c->pr_c.p;
     double* Y = (double*)c->pr_y.p;
     double* acc = Y + (size_t)nb * kPredCols;

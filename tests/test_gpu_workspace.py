@@ -119,3 +119,80 @@ def test_every_kind_of_spare_memory_is_given_back():
     with exa.Context(workspace_bytes=bound) as c:
         before(c)
         assert abs(c.loglik(*large, theta) - ref) <= 1e-10 * abs(ref)
+
+
+def padded(n):
+    return -(-n // 128) * 128
+
+
+def fp64_units_bytes(n):
+    """What the FP64 evaluation on the FP64 units holds: the matrix, the tile inverses, the panel, log-determinant parts,
+    three vectors, the reductions' partial sums and the interpolation table."""
+    import paper_1908_06936_gb300 as exa
+
+    npad = padded(n)
+    with exa.Context() as c:
+        c.covariance(to_dev(synth.uniform_square(4, 1)), (1.0, 0.1, 0.5))
+        table = exa.exa_workspace_bytes(c.handle)
+    return 8 * (npad * npad + 2 * npad * 128 + npad // 128 + 3 * npad + 1024 + (npad // 1024 + 2) * 128) + table
+
+
+@pytest.mark.parametrize("n", [100, 700, 1300])
+def test_the_fp64_evaluation_needs_no_more_than_the_fp64_units(n):
+    import paper_1908_06936_gb300 as exa
+
+    locs, z = to_dev(synth.jittered_grid(37, n)[:n]), to_dev(synth.normals(n, n))
+    theta = (1.0, 0.1, 0.5)
+    with exa.Context() as c:
+        ref = c.loglik(locs, z, theta)
+    with exa.Context(workspace_bytes=fp64_units_bytes(n)) as c:
+        assert abs(c.loglik(locs, z, theta) - ref) <= 1e-10 * abs(ref)
+
+
+@pytest.mark.parametrize("n,m,extra", [(1300, 600, 0), (1300, 600, 4 << 20), (1300, 600, 12 << 20), (1300, 600, 24 << 20),
+                                       (700, 2048, 0), (700, 2048, 6 << 20), (700, 2048, 16 << 20)])
+def test_a_prediction_needs_no_more_than_the_fp64_units(n, m, extra):
+    # beside the evaluation: 512 columns of cross covariances and of a 128-row solve, and their sums; more room leaves
+    # some of the digit operands in, but not all
+    import paper_1908_06936_gb300 as exa
+
+    locs, z = to_dev(synth.jittered_grid(37, n)[:n]), to_dev(synth.normals(n, n))
+    new, theta = to_dev(synth.uniform_square(m, m + 1)), (1.0, 0.1, 0.5)
+    with exa.Context() as c:
+        ref = [t.cpu().numpy() for t in c.predict(locs, z, theta, new)]
+    bound = fp64_units_bytes(n) + 8 * 512 * (padded(n) + 129) + extra
+    with exa.Context(workspace_bytes=bound) as c:
+        got = [t.cpu().numpy() for t in c.predict(locs, z, theta, new)]
+        again = [t.cpu().numpy() for t in c.predict(locs, z, theta, new)]
+        assert exa.exa_workspace_bytes(c.handle) <= bound
+    for g, a, r, scale in zip(got, again, ref, (float(z.abs().max()), theta[0])):
+        assert np.all(np.abs(g - r) <= 1e-9 * scale) and np.all(np.abs(a - r) <= 1e-9 * scale)
+
+
+def test_fisher_needs_no_more_than_the_fp64_units():
+    # five padded matrices, the partial sums, the tile inverses, the panel, log-determinant parts and the table
+    import paper_1908_06936_gb300 as exa
+
+    n = 700
+    npad, locs, theta = padded(n), to_dev(synth.jittered_grid(27, 3)[:n]), (1.0, 0.1, 0.5)
+    with exa.Context() as c:
+        ref = c.fisher(locs, theta)
+    units = fp64_units_bytes(n) - 8 * (3 * npad + 1024 + (npad // 1024 + 2) * 128)
+    for extra in (0, 4 << 20, 9 << 20):
+        with exa.Context(workspace_bytes=units + 8 * (4 * npad * npad + (npad // 32) ** 2 * 6) + extra) as c:
+            assert np.all(np.abs(c.fisher(locs, theta) - ref) <= 1e-9 * np.abs(ref))
+
+
+def test_a_prediction_gives_way_to_a_larger_field():
+    # the prediction's blocks of 2,048 points go when the field needs their room; those of 512 points stay
+    import paper_1908_06936_gb300 as exa
+
+    n, large = 900, 2200
+    locs, z = to_dev(synth.jittered_grid(30, 1)), to_dev(synth.normals(n, 1))
+    new, theta = to_dev(synth.uniform_square(2048, 5)), (1.0, 0.1, 0.5)
+    big, zbig = to_dev(synth.jittered_grid(47, 2)[:large]), to_dev(synth.normals(large, 2))
+    with exa.Context() as c:
+        ref = c.loglik(big, zbig, theta)
+    with exa.Context(workspace_bytes=fp64_units_bytes(large) + 8 * 512 * (padded(n) + 129)) as c:
+        c.predict(locs, z, theta, new)
+        assert abs(c.loglik(big, zbig, theta) - ref) <= 1e-10 * abs(ref)
