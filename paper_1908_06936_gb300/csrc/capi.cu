@@ -57,11 +57,8 @@ void free_spare(exa_ctx* c, std::initializer_list<DevBuf*> bufs) {
 // Gives up one kind of memory that its owner does without (no call takes such memory before its last request for what it
 // needs, or it asks for it anew); false: none is held.
 static bool release_spare(exa_ctx* c) {
-  if (c->digits_held) {
+  if (c->operands_spare) {
     release_digits(c);
-  } else if (c->wall_spare) {
-    free_spare(c, {&c->mx_wall});
-    c->wall_spare = c->wall_kept = false;
   } else if (c->bt_ps2.p && !c->ps2_captured) {
     free_spare(c, {&c->bt_ps2});
   } else if ((c->bd_mat.p || c->bd_buf.p || c->bd_task.p) && !c->bd_captured) {
@@ -356,6 +353,7 @@ exa_status exa_loglik_ex(exa_ctx* c, const double* d_locs, const double* d_z, co
   exa_status st = check_theta(c, theta);
   if (st != EXA_OK) return st;
   if (prec == EXA_FP64 || prec == EXA_MIXED_TF32X3 || prec == EXA_MIXED_BF16X3) {
+    const OperandsSpare at_end{c};
     st = prec == EXA_FP64 ? loglik_fp64(c, d_locs, d_z, theta, n, out, nullptr)
                           : loglik_mixed(c, d_locs, d_z, theta, n, prec, out);
     prof_fold(c);  // the evaluation ended with a synchronise: recycle its timing events
@@ -460,6 +458,7 @@ extern "C" exa_status exa_simulate(exa_ctx* c, const double* d_locs, const doubl
   if (st != EXA_OK) return st;
   const int nb = c->tile_nb;
   const int64_t npad = round_up(n, prec == EXA_FP64 ? nb : kMixPanel);
+  const OperandsSpare at_end{c};
   if ((st = ensure(c, c->mat, (size_t)npad * npad * sizeof(double), "matrix")) != EXA_OK) return st;
   if ((st = reset_status(c)) != EXA_OK) return st;
   double* A = (double*)c->mat.p;

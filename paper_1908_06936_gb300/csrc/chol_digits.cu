@@ -40,7 +40,7 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
   for (auto& w : want) held += w.bytes > w.b->bytes ? w.bytes - w.b->bytes : 0;
   bool ok = !c->ws_limit || held <= c->ws_limit;
   for (auto& w : want) ok = ok && ensure(c, *w.b, w.bytes, "digit operands", true) == EXA_OK;
-  c->digits_held = true;
+  c->operands_spare = true;
   if (!ok) {
     c->err[0] = 0;
     release_digits(c);
@@ -253,7 +253,7 @@ void release_digits(exa_ctx* c) {
     b->p = nullptr;
     b->bytes = 0;
   }
-  c->digits_held = c->wall_spare = c->wall_kept = false;
+  c->operands_spare = c->wall_kept = false;
 }
 
 }  // namespace exa

@@ -59,8 +59,8 @@ struct exa_ctx {
   exa::DevBuf mx_split_b;   // split-precision operands (B role: inverse diagonal block / test B)
   exa::SplitOperand sp_a, sp_a2, sp_a3, sp_a4, sp_b;
   bool wall_kept = false;   // the last factorisation left its 512-wide block inverses in mx_wall
-  bool wall_spare = false;  // mx_wall is between two mixed evaluations, which do without it
-  bool digits_held = false; // the buffers of reserve_digits are the FP64 path's: given up for requests that need the room
+  bool operands_spare = false;  // the buffers that release_digits frees are the FP64 path's, which does without, or
+                                // between two calls: given up for requests that need the room
   exa::DevBuf mx_vec;       // refinement vectors
   exa::DevBuf mx_w2;        // inverse of the panel-wide diagonal block (row-major)
   exa::DevBuf mx_wall;      // every panel's diagonal-block inverse, T x 512 x 512 (kept for the gradient)
@@ -132,6 +132,11 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
 // be had, and those buffers are released.
 bool reserve_digits(exa_ctx* c, int64_t npad);
 void release_digits(exa_ctx* c);
+// At the end of a call its operand buffers are spare.
+struct OperandsSpare {
+  exa_ctx* c;
+  ~OperandsSpare() { c->operands_spare = true; }
+};
 // y = L^-1 z (z overwritten) and y <- L^-T y with the FP64 factor in c->mat, by the block inverses its factorisation left
 // (of nb-wide tiles, or the digit path's).
 constexpr int kSolveScratch = 1024;  // doubles, in mx_dscr after the diagonal block's

@@ -564,20 +564,31 @@ __global__ void __launch_bounds__(256) put_block_inverse_kernel(double* __restri
 //   S -= X_i^T X_i                   over the leading (i + 1) 512 square, lower triangle
 // so that Sneg = -X^T X = -Sigma^-1 of the factor.  The digit planes of every row block of X
 // are kept (about 5 n^2 bytes) and serve both its products.
+static std::vector<size_t> row_block_offsets(int T) {
+  std::vector<size_t> off(T + 1, 0);
+  for (int i = 0; i < T; ++i) off[i + 1] = off[i] + split_bytes((int64_t)(i + 1) * kMixPanel, kMixPanel, false, true);
+  return off;
+}
+
+static exa_status reserve_mixed_inverse(exa_ctx* c, int64_t npad) {
+  constexpr int NB = kMixPanel;
+  const size_t big = split_bytes(npad, NB, false, true), small = split_bytes(NB, NB, false, true);
+  exa_status st = ensure(c, c->gr_xsplit, row_block_offsets((int)(npad / NB)).back() + 1024, "digit planes of L^-1");
+  if (st == EXA_OK) st = ensure(c, c->gr_lsplit, 2 * big + small + 1024, "inverse operands");
+  if (st == EXA_OK) st = ensure(c, c->gr_t, (size_t)NB * npad * sizeof(double), "inverse row-block product");
+  return st;
+}
+
 static exa_status mixed_inverse_tc(exa_ctx* c, int64_t npad, double* Sneg) {
   constexpr int NB = kMixPanel;
   const int T = (int)(npad / NB);
   double* A = (double*)c->mat.p;
   const double* Wall = (const double*)c->mx_wall.p;
   cudaStream_t s = c->stream;
-  std::vector<size_t> off(T + 1, 0);
-  for (int i = 0; i < T; ++i) off[i + 1] = off[i] + split_bytes((int64_t)(i + 1) * NB, NB, false, true);
-  exa_status st;
-  if ((st = ensure(c, c->gr_xsplit, off[T] + 1024, "digit planes of L^-1")) != EXA_OK) return st;
-  const size_t big = split_bytes(npad, NB, false, true), small = split_bytes(NB, NB, false, true);
-  if ((st = ensure(c, c->gr_lsplit, 2 * big + small + 1024, "inverse operands")) != EXA_OK) return st;
-  if ((st = ensure(c, c->gr_t, (size_t)NB * npad * sizeof(double), "inverse row-block product")) != EXA_OK)
-    return st;
+  const std::vector<size_t> off = row_block_offsets(T);
+  const exa_status st = reserve_mixed_inverse(c, npad);
+  if (st != EXA_OK) return st;
+  const size_t big = split_bytes(npad, NB, false, true);
   auto align = [](void* p) { return (uint8_t*)(((uintptr_t)p + 1023) & ~(uintptr_t)1023); };
   uint8_t* xb = align(c->gr_xsplit.p);
   uint8_t* lb = align(c->gr_lsplit.p);
@@ -677,14 +688,25 @@ static exa_status loglik_grad_mixed(exa_ctx* c, const double* d_locs, const doub
                                     int64_t n, double* loglik, double grad[3]) {
   exa_result res;
   memset(&res, 0, sizeof(res));
+  const int64_t npad = round_up(n, kMixPanel);
+  const long long t64n = (n + 63) / 64;
+  const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
+  // what follows the evaluation asks for its memory before it, while the evaluation's operand buffers may still give
+  // back what another path left in them; without it the evaluation is made all the same
+  exa_status st = c->grad_inverse_fp64 ? ensure(c, c->panel, (size_t)npad * 128 * sizeof(double), "panel")
+                                       : reserve_mixed_inverse(c, npad);
+  if (st == EXA_OK) st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials");
+  if (st != EXA_OK) {
+    free_spare(c, {&c->gr_xsplit, &c->gr_lsplit, &c->gr_t, &c->gr_blocks});
+    c->err[0] = 0;
+  }
   c->keep_block_inverses = 1;
   c->ir_tight = 1;
-  exa_status st = loglik_mixed(c, d_locs, d_z, theta, n, EXA_MIXED_TF32X3, &res);
+  st = loglik_mixed(c, d_locs, d_z, theta, n, EXA_MIXED_TF32X3, &res);
   c->keep_block_inverses = 0;
   c->ir_tight = 0;
   if (st != EXA_OK) return st;
   *loglik = res.loglik;
-  const int64_t npad = round_up(n, kMixPanel);
   const double* x = (const double*)c->mx_vec.p + npad;  // refined Sigma^-1 z (loglik_mixed's layout)
   double* Sneg = (double*)c->mx_sigma.p;                // the FP64 copy of Sigma is no longer needed
   double ssign = -1.0;
@@ -697,8 +719,6 @@ static exa_status loglik_grad_mixed(exa_ctx* c, const double* d_locs, const doub
   } else if ((st = mixed_inverse_tc(c, npad, Sneg)) != EXA_OK) {
     return st;
   }
-  const long long t64n = (n + 63) / 64;
-  const size_t nblocks = (size_t)(t64n * (t64n + 1) / 2);
   if ((st = ensure(c, c->gr_blocks, nblocks * 3 * sizeof(double), "gradient partials")) != EXA_OK) return st;
   cudaError_t e;
   e = launch_gradient(c, d_locs, n, npad, theta, x, Sneg, ssign, (double*)c->gr_blocks.p, c->d_scalars + 8);
@@ -736,6 +756,7 @@ extern "C" exa_status exa_loglik_grad(exa_ctx* c, const double* d_locs, const do
                    (int)prec);
   exa_status st = check_theta(c, theta);
   if (st != EXA_OK) return st;
+  const OperandsSpare at_end{c};
   if (prec == EXA_MIXED_TF32X3) {
     st = loglik_grad_mixed(c, d_locs, d_z, theta, n, loglik, grad);
     prof_fold(c);

@@ -34,7 +34,7 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t row
   size_t held = c->held_bytes;
   for (auto& w : want) held += w.bytes > w.b->bytes ? w.bytes - w.b->bytes : 0;
   bool ok = !c->ws_limit || held <= c->ws_limit;
-  c->digits_held = true;  // given back to what the call cannot do without
+  c->operands_spare = true;  // given back to what the call cannot do without
   for (auto& w : want) ok = ok && ensure(c, *w.b, w.bytes, "digit operands", true) == EXA_OK;
   if (!ok) c->err[0] = 0;
   return ok;

@@ -66,6 +66,21 @@ exa_status ensure_split(exa_ctx* c, SplitOperand& op, DevBuf& buf, int64_t rows,
   return EXA_OK;
 }
 
+// From here on the split-operand buffers are the call's, not spare: `reserve` sizes them, and if memory runs out once
+// more with what earlier calls left in them given back.
+template <class F>
+static exa_status take_split_buffers(exa_ctx* c, F reserve) {
+  const bool spare = c->operands_spare;
+  c->operands_spare = c->wall_kept = false;
+  exa_status st = reserve();
+  if (st == EXA_ERR_NOMEM && spare) {
+    release_digits(c);
+    c->err[0] = 0;
+    st = reserve();
+  }
+  return st;
+}
+
 // ---------------------------------------------------------------------------
 // Mixed-precision tiled Cholesky (panel width kMixNB = 512).  For tile column k:
 //   1. FP64 factorisation of the 512 x 512 diagonal block and its inverse W, with those
@@ -343,23 +358,25 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   const int64_t fuse_rows = c->fuse_min_rows < 0 ? kFuseMinRows : c->fuse_min_rows;
   // the fused phase runs while rows (k + 4) NB .. npad number at least fuse_rows, from k = 0
   const bool fuse = fuse_rows > 0 && c->tc_pairs && T >= 4 && npad - 4 * (int64_t)NB >= fuse_rows;
-  c->digits_held = false;
-  c->wall_spare = c->wall_kept = false;
   SplitOperand* buf[4] = {&c->sp_a, &c->sp_a2, &c->sp_a3, &c->sp_a4};
   DevBuf* mem[4] = {&c->mx_split, &c->mx_split2, &c->mx_split3, &c->mx_split4};
-  for (int i = 0; i < (fuse ? 4 : 2); ++i)
-    if ((st = ensure_split(c, *buf[i], *mem[i], npad, NB, true, true)) != EXA_OK) return st;
   const int nbuf = fuse ? 4 : 2;
-  if ((st = ensure_split(c, c->sp_b, c->mx_split_b, NB, NB, true, true)) != EXA_OK) return st;
-  if ((st = ensure(c, c->mx_w2, (size_t)NB * NB * sizeof(double), "diagonal block inverse")) != EXA_OK) return st;
-  if ((st = ensure(c, c->mx_dscr, (diag_block_scratch_doubles() + kSolveScratch) * sizeof(double),
-                   "diagonal block scratch")) != EXA_OK)
-    return st;
+  const size_t wall = (size_t)T * NB * NB * sizeof(double);
+  st = take_split_buffers(c, [&] {
+    exa_status r = EXA_OK;
+    for (int i = 0; i < nbuf && r == EXA_OK; ++i) r = ensure_split(c, *buf[i], *mem[i], npad, NB, true, true);
+    if (r == EXA_OK) r = ensure_split(c, c->sp_b, c->mx_split_b, NB, NB, true, true);
+    if (r == EXA_OK) r = ensure(c, c->mx_w2, (size_t)NB * NB * sizeof(double), "diagonal block inverse");
+    if (r == EXA_OK)
+      r = ensure(c, c->mx_dscr, (diag_block_scratch_doubles() + kSolveScratch) * sizeof(double),
+                 "diagonal block scratch");
+    if (r == EXA_OK && c->keep_block_inverses == 1) r = ensure(c, c->mx_wall, wall, "diagonal block inverses");
+    return r;
+  });
+  if (st != EXA_OK) return st;
   if ((st = ensure_side(c)) != EXA_OK) return st;
-  if (c->keep_block_inverses) {  // last: 2 is a wish
-    st = ensure(c, c->mx_wall, (size_t)T * NB * NB * sizeof(double), "diagonal block inverses", true);
-    if (st != EXA_OK && c->keep_block_inverses == 1) return st;
-    c->wall_kept = st == EXA_OK;
+  if (c->keep_block_inverses) {  // 2 is a wish
+    c->wall_kept = ensure(c, c->mx_wall, wall, "diagonal block inverses", true) == EXA_OK;
     c->err[0] = 0;
   }
   MixStep M{c, a, ld, npad, band, T, far_thr};
@@ -544,7 +561,6 @@ exa_status loglik_mixed(exa_ctx* c, const double* d_locs, const double* d_z, con
   if (!keep) c->keep_block_inverses = 2;
   st = mixed_generate_factor(c, d_locs, n, theta, npad, prec, S, &band);
   c->keep_block_inverses = keep;
-  c->wall_spare = !keep && c->wall_kept;
   if (st != EXA_OK) return st;
   cudaEventRecord(c->ev[2], s);
   cudaError_t e;
@@ -713,14 +729,15 @@ extern "C" exa_status exa_gemm_update(exa_ctx* c, exa_gemm_kind kind, int64_t m,
     return set_err(c, EXA_ERR_ARG, "gemm shape m=%lld n=%lld k=%lld not supported", (long long)m, (long long)n,
                    (long long)k);
   const int k1 = (int)(k < kSplitMaxK ? k : kSplitMaxK), k2 = (int)(k - k1);
-  exa_status st;
-  c->digits_held = false;
-  if ((st = ensure_split(c, c->sp_a, c->mx_split, m, k1, !oz, oz)) != EXA_OK) return st;
-  if ((st = ensure_split(c, c->sp_b, c->mx_split_b, n, k1, !oz, oz)) != EXA_OK) return st;
-  if (k2 > 0) {
-    if ((st = ensure_split(c, c->sp_a2, c->mx_split2, m, k2, true, false)) != EXA_OK) return st;
-    if ((st = ensure_split(c, c->sp_a3, c->mx_split3, n, k2, true, false)) != EXA_OK) return st;
-  }
+  const OperandsSpare at_end{c};
+  exa_status st = take_split_buffers(c, [&] {
+    exa_status r = ensure_split(c, c->sp_a, c->mx_split, m, k1, !oz, oz);
+    if (r == EXA_OK) r = ensure_split(c, c->sp_b, c->mx_split_b, n, k1, !oz, oz);
+    if (r == EXA_OK && k2 > 0) r = ensure_split(c, c->sp_a2, c->mx_split2, m, k2, true, false);
+    if (r == EXA_OK && k2 > 0) r = ensure_split(c, c->sp_a3, c->mx_split3, n, k2, true, false);
+    return r;
+  });
+  if (st != EXA_OK) return st;
   if ((st = reset_status(c)) != EXA_OK) return st;
   cudaError_t e = launch_split_rows(c->stream, d_a, k, 1, (int)m, k1, c->sp_a, 0);
   if (e == cudaSuccess) e = launch_split_rows(c->stream, d_b, k, 1, (int)n, k1, c->sp_b, 0);

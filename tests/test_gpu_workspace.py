@@ -196,3 +196,63 @@ def test_a_prediction_gives_way_to_a_larger_field():
     with exa.Context(workspace_bytes=fp64_units_bytes(large) + 8 * 512 * (padded(n) + 129)) as c:
         c.predict(locs, z, theta, new)
         assert abs(c.loglik(big, zbig, theta) - ref) <= 1e-10 * abs(ref)
+
+
+# Calls on one context, and the bytes they left held when the FP64 calls ran on the FP64 units and the mixed ones without
+# the 512-wide block inverses.  ll, g, f, p, s: log-likelihood, gradient, Fisher information, prediction of 2,500 points,
+# simulation of n points in FP64; mx, gm, sm: the mixed ones; b32: FP64 batch in one launch, bt: mixed batch.
+SEQUENCES = [
+    ("ll1024 mx1500", 77165456),
+    ("ll1024 gm1024", 75418664),
+    ("ll1024 sm1500", 57900432),
+    ("mx1024 mx1500", 76747664),
+    ("mx1024 sm1500", 66065296),
+    ("g513 gm2100", 256875640),
+    ("f513 mx1500", 89874064),
+    ("mx513 gm400 btL b32S", 174693936),
+    ("p513 f100 gm513 s513", 78688160),
+    ("f513 gm400 s1024 s1024", 57964128),
+    ("mx400 p513 mx513 f2100", 232764080),
+    ("s100 g400 gm1024 sm513", 77110312),
+    ("p100 sm1024 mx513 ll1500", 58631048),
+]
+SMALL, LARGE = [20, 11, 26], [30, 41, 22, 36]
+
+
+def make(name):
+    import paper_1908_06936_gb300 as exa
+
+    theta = (1.0, 0.1, 0.5)
+    kind, size = name.rstrip("0123456789SL"), name.lstrip("bcdefghijklmnopqrstuvwxyz")
+    if name.startswith("b"):
+        def call(c):
+            c.check(exa.exa_ctx_set_batched(c.handle, 32 if name.startswith("b32") else 0, 0, 0, 0))
+            return evaluate(c, batch(SMALL if name.endswith("S") else LARGE), FP64 if name.startswith("b32") else TF32X3)
+        return call
+    n = int(size)
+    locs, z = to_dev(synth.jittered_grid(int(np.ceil(n ** 0.5)), n)[:n]), to_dev(synth.normals(n, n))
+    return {
+        "ll": lambda c: c.loglik(locs, z, theta),
+        "mx": lambda c: c.loglik(locs, z, theta, TF32X3),
+        "g": lambda c: c.loglik_grad(locs, z, theta)[1],
+        "gm": lambda c: c.loglik_grad(locs, z, theta, TF32X3)[1],
+        "f": lambda c: c.fisher(locs, theta),
+        "p": lambda c: c.predict(locs, z, theta, to_dev(synth.uniform_square(2500, 9)))[0].cpu().numpy(),
+        "s": lambda c: c.simulate(locs, z, theta).cpu().numpy(),
+        "sm": lambda c: c.simulate(locs, z, theta, TF32X3).cpu().numpy(),
+    }[kind]
+
+
+@pytest.mark.parametrize("calls,bound", SEQUENCES)
+def test_a_sequence_needs_no_more_than_without_the_spare_memory(calls, bound):
+    # the results are those of each call on a context of its own: to 1e-8 of the largest, the bar of the quadratic forms
+    import paper_1908_06936_gb300 as exa
+
+    with exa.Context(workspace_bytes=bound) as c:
+        for name in calls.split():
+            call = make(name)
+            got = np.asarray(call(c))
+            with exa.Context() as fresh:
+                ref = np.asarray(call(fresh))
+            assert np.all(np.abs(got - ref) <= 2e-8 * np.max(np.abs(ref))), name
+        assert exa.exa_workspace_bytes(c.handle) <= bound
