@@ -48,22 +48,6 @@ bool reserve_digits(exa_ctx* c, int64_t npad) {
   return ok;
 }
 
-// The look-ahead stream's share of the GPU beside a trailing update of m rows (m^2 512 operations at 42 TFLOP/s on the
-// whole GPU): the grid of the diagonal block with which the later of the two ends first.
-static int side_share(int64_t m, int sms) {
-  const double update_us = (double)m * (double)m * kNB / 42e6;
-  int best = kDiagCtas;
-  double best_us = 0.0;
-  for (int ctas = kDiagCtas; ctas >= 16; ctas -= 8) {
-    const double us = std::max(diag_block_us(ctas), update_us * sms / (sms - ctas));
-    if (best_us == 0.0 || us < best_us) {
-      best_us = us;
-      best = ctas;
-    }
-  }
-  return best;
-}
-
 // The factorisation of `a` (npad a multiple of 128).  *done = false: the workspace could not be had and nothing was
 // launched.
 exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* done) {
@@ -189,7 +173,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
     if (e != cudaSuccess) break;
     cudaEventRecord(c->la_ev[0], ms);
     cudaStreamWaitEvent(ss, c->la_ev[0], 0);
-    const int side = side_share(m, sms);
+    const int side = side_share(m, kNB, sms);
     e = diagonal(ss, k + 1, side);
     cudaEventRecord(c->la_ev[1], ss);
     if (e == cudaSuccess && m > w1) {

@@ -8,6 +8,7 @@
 #include "exa_internal.cuh"
 #include "gemm_tc.cuh"
 #include "prof.cuh"
+#include "shares.cuh"
 
 namespace exa {
 
@@ -22,7 +23,6 @@ struct DevBuf {
 
 constexpr int kNumEvents = 8;
 constexpr int kMixPanel = 512;     // panel width of the mixed-precision factorisation
-constexpr int kDiagCtas = 104;    // CTAs of one diagonal-block launch at most
 constexpr int kRedPartials = 512;  // partial sums of one two-stage reduction
 
 inline int64_t kPartialDoubles(int64_t npad, int nb) { return 2 * kRedPartials + (npad / 1024 + 2) * (int64_t)nb; }

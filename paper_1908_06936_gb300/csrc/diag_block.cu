@@ -26,6 +26,7 @@
 
 #include "exa_internal.cuh"
 #include "gemm_tc.cuh"
+#include "shares.cuh"
 #include "tc_common.cuh"
 
 namespace exa {
@@ -594,17 +595,6 @@ cudaError_t launch_diag128_tasks(cudaStream_t s, const SolveTileTask* d_tasks, i
   return cudaLaunchKernelEx(&cfg, diag_tasks_kernel, d_tasks);
 }
 
-double diag_block_us(int ctas) {
-  static const struct { int ctas; double us; } kAt[] = {{16, 1180.0}, {32, 698.0}, {64, 464.0}, {104, 426.0}};
-  if (ctas <= kAt[0].ctas) return kAt[0].us * kAt[0].ctas / ctas;
-  for (int i = 1; i < 4; ++i)
-    if (ctas <= kAt[i].ctas) {  // linear in the reciprocal
-      const double f = (1.0 / ctas - 1.0 / kAt[i].ctas) / (1.0 / kAt[i - 1].ctas - 1.0 / kAt[i].ctas);
-      return kAt[i].us + f * (kAt[i - 1].us - kAt[i].us);
-    }
-  return kAt[3].us;
-}
-
 size_t diag_block_scratch_doubles() { return (size_t)kDiagScratch; }
 
 cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0, double* w_sub, double* logdet_part,
@@ -617,7 +607,7 @@ cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0,
     return cudaFuncSetAttribute(diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (e != cudaSuccess) return e;
-  if (grid < 2) grid = 2;  // CTA 0 runs the leaves; the updates need at least one more CTA
+  grid = diag_grid(grid, tc_num_sms());
   e = cudaMemsetAsync(scratch, 0, kDiagScratch * sizeof(double), s);
   if (e != cudaSuccess) return e;
   // (a smaller block is the last of its matrix: only its 128 sub-tile inverses are wanted)

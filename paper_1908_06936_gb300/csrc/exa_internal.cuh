@@ -165,13 +165,11 @@ struct SolveTileTask {
 cudaError_t launch_potrf128_tasks(cudaStream_t s, const DiagTileTask* d_tasks, int ntasks);
 cudaError_t launch_diag128_tasks(cudaStream_t s, const SolveTileTask* d_tasks, int ntasks);
 // FP64 Cholesky and inverse of the 512 x 512 diagonal block at (k0, k0) as one cooperative launch
-// of `grid` CTAs (>= 2): L in place, log sums of the four 128 sub-tiles into logdet_part[0..3], their
+// of `grid` CTAs (held to 2 .. kDiagCtas and the GPU's SMs): L in place, log sums of the four 128 sub-tiles into logdet_part[0..3], their
 // inverses (row-major) into w_sub, the block inverse (row-major) into w2; scratch holds
 // diag_block_scratch_doubles() doubles.  size: 512, or for the last block of a matrix a smaller multiple of 128
 // (then w2 is scratch: only the sub-tile inverses are formed).
 size_t diag_block_scratch_doubles();
-// What a 512 block takes on a grid (measured), microseconds.  Nothing is gained beyond 104 CTAs.
-double diag_block_us(int ctas);
 cudaError_t launch_diag_block(cudaStream_t s, double* a, int64_t ld, int64_t k0, double* w_sub, double* logdet_part,
                               double* w2, double* scratch, DevStatus* st, int grid, int size = 512);
 

@@ -118,7 +118,7 @@ static exa_status panel_factor(const MixStep& M, cudaStream_t s, int k, SplitOpe
   // 2. its inverse W = L_kk^-1: one cooperative launch (diag_block.cu)
   {
     // one CTA per SM of the look-ahead share
-    const int grid = ctas > 0 ? (ctas < kDiagCtas ? ctas : kDiagCtas) : kDiagCtas;
+    const int grid = ctas > 0 ? ctas : kDiagCtas;
     const double nb3 = (double)NB * NB * NB;
     ProfScope ps(c, PK_POTRF, 2.0 * nb3 / 3.0, 8.0 * (3.0 * NB * NB + 4.0 * nb * nb), 1, s, true);
     e = launch_diag_block(s, a, ld, k0, W + (k0 / nb) * (int64_t)nb * nb, LD + k0 / nb, W2, (double*)c->mx_dscr.p,
