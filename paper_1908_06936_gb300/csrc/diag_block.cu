@@ -428,13 +428,14 @@ __device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
         __syncthreads();
         for (int i = kDW * b / nl + warp; i < kDW * (b + 1) / nl; i += kDThreads / 32) {  // (nl may not divide 32)
           double* pc = a + (r0 + i) + (r0 + lane) * ld;
-          double s0 = lane <= i ? __ldcg(pc) : 0.0, s1 = 0.0;
+          const double a0 = lane <= i ? __ldcg(pc) : 0.0;
+          double s0 = 0.0, s1 = 0.0;
 #pragma unroll
           for (int k = 0; k < kDW; k += 2) {
-            s0 = fma(-sB[i * kDLd + k], sB[lane * kDLd + k], s0);
-            s1 = fma(-sB[i * kDLd + k + 1], sB[lane * kDLd + k + 1], s1);
+            s0 = fma(sB[i * kDLd + k], sB[lane * kDLd + k], s0);
+            s1 = fma(sB[i * kDLd + k + 1], sB[lane * kDLd + k + 1], s1);
           }
-          if (lane <= i) *pc = s0 + s1;
+          if (lane <= i) *pc = a0 - (s0 + s1);
         }
       }
       grp.lead_sync();
@@ -446,6 +447,7 @@ __device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
     //      A_rc -= L_r L_c^T over 32-row blocks R and 16-wide column strips s <= 2 R + 1, but for the leaf's (R = 0):
     //      block R has 2 R + 2 tiles, numbered from R (R + 1) - 2 on; lanes along the rows.
     //      T_i -= L_i,j-1 W_j-1 for i >= j: lanes along the columns, 16 rows a tile.
+    //      The products of a step are summed from zero: taken off C one by one, each would round at C's size.
     //      CTA 0 comes to them three rounds late (the leaf), the CTAs of V_j one or two.
     const int nr = more ? below / kDW : 0, nt = nr > 0 ? nr * (nr + 1) - 2 : 0;
     const int ni = j > 0 ? min(i1 + per, nsteps) - j : 0, nc = j - i1;  // row blocks i, column blocks of W_j-1
@@ -505,7 +507,8 @@ __device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
       for (int u = 0; u < 2; ++u) sA[(tid & 15) * kDLd + (tid >> 4) + 16 * u] = va[u];
 #pragma unroll
       for (int u = 0; u < 4; ++u) sB[lane * kDLd + warp + 8 * u] = vb[u];
-      double acc0 = vc[0], acc1 = vc[1];
+      double acc0 = 0.0, acc1 = 0.0;
+      const double c0v = vc[0], c1v = vc[1];
       double* out = pc + warp * cs;
       const int64_t step = 8 * cs;
       const int left = lim - warp;
@@ -515,11 +518,11 @@ __device__ void diag_body(const DiagArgs& g, Group grp, DiagSmem& sm) {
 #pragma unroll 8
       for (int k = 0; k < kDW; ++k) {
         const double y = sB[lane * kDLd + k];
-        acc0 = fma(-sA[warp * kDLd + k], y, acc0);
-        acc1 = fma(-sA[(warp + 8) * kDLd + k], y, acc1);
+        acc0 = fma(sA[warp * kDLd + k], y, acc0);
+        acc1 = fma(sA[(warp + 8) * kDLd + k], y, acc1);
       }
-      if (left >= 0) *out = acc0;
-      if (left >= 8) out[step] = acc1;
+      if (left >= 0) *out = c0v - acc0;
+      if (left >= 8) out[step] = c1v - acc1;
     }
     grp.sync();
     if (!more) inverse_rows(j);
