@@ -6,7 +6,9 @@
 //      R = A_ik - X L_kk^T, L_ik = X + R W^T.  Multiplying by an explicit inverse alone leaves an error of
 //      cond(L_kk) rounding units in A_ik, which grows with the block: on a 512 block of a smooth field it was three
 //      times the error of the 128-wide panels; with the correction it is a rounding unit.  R is that much smaller
-//      than A_ik, so its product needs two digits.  The digits are relative to a row's largest value, while column
+//      than A_ik, and its product has to hold 1 / cond(L_kk) of itself: four digits.  (With two, the log-determinant of
+//      1,024 points was off by 3e-7 at nu = 2.5, range 0.2, and by 4e-2 at nu = 3.5, where now 7e-9 and 8e-6; the panels
+//      of 128 rows left 3e-8 and 4e-5.)  The digits are relative to a row's largest value, while column
 //      c of A_ik and of W^T goes with the size of row c of L_kk: both products run on A_ic 2^-e_c and W_.c 2^e_c
 //      with e_c that row's exponent, so that a badly scaled matrix loses nothing;
 //   3. A_ij -= L_ik L_jk^T over the trailing lower triangle: the next diagonal block first, then, while the

@@ -26,9 +26,10 @@ constexpr int kEpiWarps = 16, kThreads = 64 + 32 * kEpiWarps;
 
 template <int S>
 struct Cfg {
+  static_assert(S == 4 || S == 8, "the drain's words");
   static constexpr int A_BYTES = TM * 32, B_BYTES = TN * 32;  // one digit plane of a 16-column step
   static constexpr int STAGE_BYTES = S * (A_BYTES + B_BYTES);
-  static constexpr int STAGES = S == kDigSlices ? 4 : 12;
+  static constexpr int STAGES = S == kDigSlices ? 4 : 9;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 512;
   static constexpr int TMEM_COLS = S * TN;  // group g in columns [TN g, TN g + TN)
 };
@@ -288,25 +289,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
         break;
       }
       fence_after();
-      // groups 2p and 2p + 1 hold exact integers of weights 2^(-12-14p), 2^(-19-14p): a 32-bit word for both (S = 8: at
-      // most 7 2^28 + 2^24), a 64-bit one for groups 0-3 and one for 4-7, and V for all, in units of 2^8 of the last
+      // groups 2p and 2p + 1 hold exact integers of weights 2^(-12-14p), 2^(-19-14p): a 32-bit word for both (at most
+      // 7 2^28 + 2^24), a 64-bit one for groups 0-3 (S = 4: V, in units of the last) and one for 4-7, and V for all, in
+      // units of 2^8 of the last
       long long V[CH];
       const uint32_t ta = tmem + ((uint32_t)(quad * 32) << 16) + half * CH;
 #pragma unroll
       for (int h = 0; h < CH; h += 4) {
-        constexpr int H = S < 4 ? S : 4;
-        uint32_t x[H][4];
+        uint32_t x[4][4];
 #pragma unroll
-        for (int p = 0; p < H; ++p) tmem_ld4(ta + p * TN + h, x[p]);
+        for (int p = 0; p < 4; ++p) tmem_ld4(ta + p * TN + h, x[p]);
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const int w01 = small_int_bits(__uint_as_float(x[0][j])) * 128 + small_int_bits(__uint_as_float(x[1][j])) -
                           (int)(129u * 0x4B400000u);
-          V[h + j] = w01;
-          if constexpr (S == 8)
-            V[h + j] = ((long long)w01 * 16384 + (__float2int_rn(__uint_as_float(x[2][j])) * 128 +
-                                                  __float2int_rn(__uint_as_float(x[3][j])))) << 20;
+          V[h + j] = (long long)w01 * 16384 + (__float2int_rn(__uint_as_float(x[2][j])) * 128 +
+                                               __float2int_rn(__uint_as_float(x[3][j])));
+          if constexpr (S == 8) V[h + j] = V[h + j] << 20;
         }
         if constexpr (S == 8) {
 #pragma unroll
@@ -388,7 +388,7 @@ __device__ __forceinline__ void digits_of(double a, int e, float (&d)[S]) {
   const unsigned int mh = E ? ((unsigned int)hi & 0xFFFFFu) | 0x100000u : 0u, ml = E ? (unsigned int)__double2loint(a) : 0u;
   const unsigned long long M = (((unsigned long long)mh << 32) | ml) << 10;  // below 2^63
   const unsigned long long N = ((M >> min(sh + 9, 63)) + 1) >> 1;
-  constexpr unsigned long long B = S == 8 ? 64ull * ((1ull << 49) - 1) / 127 : 64ull;
+  constexpr unsigned long long B = 64ull * ((1ull << (7 * (S - 1))) - 1) / 127;
   const unsigned long long x = hi < 0 ? B - N : B + N;
   constexpr float kMagic = 12582912.0f;
   // digits 1 .. S-1 from the 28 bits of each half

@@ -8,7 +8,7 @@ struct exa_ctx;
 namespace exa {
 
 constexpr int kDigSlices = 8;    // 7-bit digits per value of a full-precision operand (55 bits below the row maximum)
-constexpr int kDigLow = 2;       // digits of a correction operand (13 bits below its row maximum)
+constexpr int kDigLow = 4;       // digits of a correction operand (27 bits below its row maximum)
 constexpr int kDigMaxK = 512;    // longest reduction of one pass (its digit sums stay below 2^24)
 constexpr int kDigTN = 64;       // output tile: 128 x kDigTN
 

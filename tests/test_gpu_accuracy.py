@@ -29,3 +29,18 @@ def test_diagonal_block_rounds_once_a_step(seed):
     l = np.triu(buf.cpu().numpy()).T.astype(np.longdouble)
     resid = ((l * l).sum(1) - np.diag(a))[384:] / np.diag(a)[384:]
     assert np.sqrt(np.mean(resid.astype(float) ** 2)) <= 4 * U
+
+
+@pytest.mark.parametrize("nu,beta,bound", [(2.5, 0.2, 1.2e-7), (3.5, 0.15, 3e-5)])
+def test_log_determinant_of_smooth_fields(nu, beta, bound):
+    # 1,024 points, against the FP64 units (tile 64).  In 80-bit arithmetic 128-wide panels on the FP64 units leave
+    # errors of 3.1e-8 and 5.4e-6 (root mean square of 16 fields), panels with a correction from two digits 3.4e-7 and
+    # 2.0e-3, from four 7e-9 and 8e-7.  Bound: four times the FP64 units' own, and a margin for four fields.
+    import paper_1908_06936_gb300 as exa
+
+    diff = []
+    for seed in range(1, 5):
+        locs, z = to_dev(synth.jittered_grid(32, seed)), to_dev(synth.normals(1024, seed))
+        with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as units:
+            diff.append(c.loglik_ex(locs, z, (1.0, beta, nu))["logdet"] - units.loglik_ex(locs, z, (1.0, beta, nu))["logdet"])
+    assert np.sqrt(np.mean(np.square(diff))) <= bound, diff
