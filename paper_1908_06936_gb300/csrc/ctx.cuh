@@ -149,9 +149,10 @@ const double* block_inverse(exa_ctx* c, int64_t k0, int h);
 // rows: of the second operand where it has more than npad (prediction points).
 bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate = true, int64_t rows = 0);
 // Digits of the h x h diagonal block at k0 of the factor in c->mat (Dl) and of its inverse with column k scaled by row
-// k's exponent of Dl (Dw), in mx_split_b.
+// k's exponent of Dl (Dw; Dwl: the same for a correction's product), in mx_split_b.
 struct DigitOperand;
-cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl);
+cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl,
+                                DigitOperand* Dwl = nullptr);
 cudaError_t inverse_digits(exa_ctx* c, int64_t npad, double* x);
 // The look-ahead stream and its events.
 exa_status ensure_side(exa_ctx* c);

@@ -25,7 +25,7 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t row
     size_t bytes;
   } want[] = {{&c->mx_split, digit_bytes(npad, kNB, kDigSlices)},
               {&c->mx_split2, digit_bytes(rows, kNB, kDigSlices)},
-              {&c->mx_split_b, 2 * align256(digit_bytes(kNB, kNB, kDigSlices))}};
+              {&c->mx_split_b, 2 * align256(digit_bytes(kNB, kNB, kDigSlices)) + align256(digit_bytes(kNB, kNB, kDigLow))}};
   if (!allocate) {
     bool have = true;
     for (auto& w : want) have = have && w.b->bytes >= w.bytes;
@@ -40,13 +40,19 @@ bool reserve_inverse_digits(exa_ctx* c, int64_t npad, bool allocate, int64_t row
   return ok;
 }
 
-cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl) {
+cudaError_t split_block_inverse(exa_ctx* c, int64_t npad, int64_t k0, int h, DigitOperand& Dw, DigitOperand& Dl,
+                                DigitOperand* Dwl) {
   const double* a = (const double*)c->mat.p + k0 + k0 * npad;
   const double* w = block_inverse(c, k0, h);
   digit_layout(Dl, c->mx_split_b.p, h, h, kDigSlices);
-  digit_layout(Dw, (uint8_t*)c->mx_split_b.p + align256(digit_bytes(kNB, kNB, kDigSlices)), h, h, kDigSlices);
+  const size_t one = align256(digit_bytes(kNB, kNB, kDigSlices));
+  digit_layout(Dw, (uint8_t*)c->mx_split_b.p + one, h, h, kDigSlices);
   cudaError_t e = launch_digit_split(c->stream, a, 1, npad, h, h, kDigSlices, Dl, 0, true);
   if (e == cudaSuccess) e = launch_digit_split(c->stream, w, h, 1, h, h, kDigSlices, Dw, 0, true, Dl.ex, 1);
+  if (e == cudaSuccess && Dwl) {
+    digit_layout(*Dwl, (uint8_t*)c->mx_split_b.p + 2 * one, h, h, kDigLow);
+    e = launch_digit_split(c->stream, w, h, 1, h, h, kDigLow, *Dwl, 0, true, Dl.ex, 1);
+  }
   return e;
 }
 

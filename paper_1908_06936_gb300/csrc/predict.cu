@@ -125,8 +125,11 @@ __global__ void krige_var_kernel(const double* __restrict__ acc, double sigma2, 
 }
 
 // acc[c] = |L^-1 C(:, c)|^2 for mc columns (a multiple of 64) of C (npad rows, ld npad, overwritten) as digit
-// products, block row by block row: Y_k = W_k C_k, C_rest -= L_rest,k Y_k.  Y: 512 x mc scratch.  On the FP64 units
-// the products took 221 ms for 2,048 points and n = 10,000.
+// products, block row by block row: Y_k = W_k C_k, corrected once as in the factorisation's panel solve (Y_k += W_k R,
+// R = C_k - L_kk Y_k), C_rest -= L_rest,k Y_k.  Y: 512 x mc scratch.  Without the correction the variances were off by
+// cond(L_kk) rounding units: 529 points, 3e-15 at nu = 0.5 and 7e-13 at nu = 2.5, range 0.2; 128-wide inverses on the FP64
+// units 9e-16 and 2e-14, now 9e-16 and 2e-15.  It takes 2.2 of 29.7 ms for 2,048 points and n = 10,000, where the
+// products took 221 ms on the FP64 units.
 static cudaError_t variance_digits(exa_ctx* c, int64_t npad, int64_t mc, double* C, double* Y, double* acc) {
   const double* A = (const double*)c->mat.p;
   cudaStream_t s = c->stream;
@@ -135,11 +138,12 @@ static cudaError_t variance_digits(exa_ctx* c, int64_t npad, int64_t mc, double*
     h = npad - k0 >= kDigMaxK ? kDigMaxK : 128;
     const int64_t rest = npad - k0 - h;
     const double dh = (double)h, dm = (double)mc;
-    DigitOperand Dw, Dl, Dc, D;
+    DigitOperand Dw, Dl, Dwl, Dc, Dr, D;
     digit_layout(Dc, c->mx_split2.p, mc, (int)h, kDigSlices);
+    digit_layout(Dr, c->mx_split2.p, mc, (int)h, kDigLow);
     {
-      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * dh * (dm + dh), 3);
-      e = split_block_inverse(c, npad, k0, (int)h, Dw, Dl);
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * dh * (dm + dh), 4);
+      e = split_block_inverse(c, npad, k0, (int)h, Dw, Dl, &Dwl);
       if (e == cudaSuccess) e = launch_digit_split(s, C + k0, npad, 1, mc, (int)h, kDigSlices, Dc, 0, false, Dl.ex, -1);
     }
     DigitGemm g{};
@@ -156,6 +160,34 @@ static cudaError_t variance_digits(exa_ctx* c, int64_t npad, int64_t mc, double*
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_GEMM_DIG, dh * dh * dm, 8.0 * dh * dm);
       e = launch_gemm_digits(s, g);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * dh * dm, 1);
+      e = launch_digit_split(s, Y, h, 1, mc, (int)h, kDigSlices, Dc);
+    }
+    if (e == cudaSuccess) {  // R in C_k's place
+      DigitGemm r = g;
+      r.C = C + k0;
+      r.Cin = r.C;
+      r.ldc = r.ldcin = npad;
+      r.A = Dl;
+      r.neg = 1;
+      ProfScope ps(c, PK_GEMM_DIG, dh * dh * dm, 16.0 * dh * dm);
+      e = launch_gemm_digits(s, r);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_SPLIT, 0.0, 16.0 * dh * dm, 1);
+      e = launch_digit_split(s, C + k0, npad, 1, mc, (int)h, kDigLow, Dr, 0, false, Dl.ex, -1);
+    }
+    if (e == cudaSuccess) {
+      DigitGemm r = g;
+      r.Cin = Y;
+      r.ldcin = h;
+      r.A = Dwl;
+      r.B = Dr;
+      r.S = kDigLow;
+      ProfScope ps(c, PK_GEMM_DIG, dh * dh * dm, 16.0 * dh * dm);
+      e = launch_gemm_digits(s, r);
     }
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_OTHER, 0.0, 8.0 * dh * dm);

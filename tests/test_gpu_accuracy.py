@@ -44,3 +44,21 @@ def test_log_determinant_of_smooth_fields(nu, beta, bound):
         with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as units:
             diff.append(c.loglik_ex(locs, z, (1.0, beta, nu))["logdet"] - units.loglik_ex(locs, z, (1.0, beta, nu))["logdet"])
     assert np.sqrt(np.mean(np.square(diff))) <= bound, diff
+
+
+@pytest.mark.parametrize("nu,beta,bound", [(0.5, 0.1, 2.5e-15), (1.0, 0.05, 2.5e-15), (2.5, 0.1, 3e-14), (2.5, 0.2, 1e-13)])
+def test_kriging_variance_against_the_fp64_units(nu, beta, bound):
+    # 1,024 points, the largest difference from tile 64 (the FP64 units).  In 80-bit arithmetic with one and the same
+    # factor, 128-wide inverses on the FP64 units leave 9.3e-16, 1.2e-15, 1.1e-14 and 2.2e-14, 512-wide ones as digit
+    # products 4.0e-15, 4.2e-15, 2.7e-13 and 1.1e-12, and once corrected 6e-16, 8e-16, 5e-16 and 1e-15.  Bound: the FP64
+    # units' error and a margin for the maximum over three fields and for the two factors.
+    import paper_1908_06936_gb300 as exa
+
+    diff = []
+    for seed in range(1, 4):
+        locs, z = to_dev(synth.jittered_grid(32, seed)), to_dev(synth.normals(1024, seed))
+        new = to_dev(synth.uniform_square(256, seed + 50))
+        with exa.Context(tile_nb=128) as c, exa.Context(tile_nb=64) as units:
+            a, b = (x.predict(locs, z, (1.0, beta, nu), new)[1].cpu().numpy() for x in (c, units))
+        diff.append(np.max(np.abs(a - b)))
+    assert max(diff) <= bound, diff
