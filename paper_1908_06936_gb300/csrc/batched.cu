@@ -1487,9 +1487,14 @@ static exa_status batched_run_tc(exa_ctx* c, int nrep, const int64_t* h_n, const
 // and y = L^-1 z carried along (the diagonal kernel finishes y_k, one launch per step takes L_rest,k y_k off the
 // rest), so that no refinement and no second copy of Sigma is needed.  Per step k:
 //   1. Cholesky and inverse W_k of the diagonal tiles, y_k = W_k z_k, the row exponents of L_kk;
-//   2. digits of the W_k and of the panels, column c of the panel and of W scaled by row c's exponent;
-//   3. L_ik = A_ik W_k^T, one grouped launch; 4. z_i -= L_ik y_k and the digits of L_ik;
+//   2. digits of the W_k, the L_kk and the panels, column c of the panel and of W scaled by row c's exponent;
+//   3. X = A_ik W_k^T and one correction as in the single-field panel solve, R = A_ik - X L_kk^T in A's place and
+//      L_ik = X + R W_k^T in X's, each one grouped launch (L_ik is not read after this step, so it stays there);
+//   4. z_i -= L_ik y_k and the digits of L_ik;
 //   5. A_ij -= L_ik L_jk^T, one grouped launch.
+// Without the correction the likelihoods of smooth fields were off by cond(L_kk) rounding units (529 points, nu = 2.5,
+// range 0.2: 8e-10 relative, the persistent form 2e-10, now 8e-11).  It takes 6.4 of the 38.1 ms of 32 fields of 400 to
+// 6,400 points.
 // On the FP64 units (the persistent form) 32 fields of 400 to 6,400 points took 542 ms in the factorisation.
 // ---------------------------------------------------------------------------
 struct ZTask {
@@ -1545,8 +1550,8 @@ __global__ void batched_fp64_finish_kernel(int nrep, const BMeta* __restrict__ M
 }
 
 struct DigStep {
-  int diag_off, ndiag, set_off, nset;     // SolveTileTask range; ZTask range, and the split tasks at twice its offsets
-  long long trsm_off, ntrsm, upd_off, nupd;
+  int diag_off, ndiag, set_off, nset;     // SolveTileTask range; ZTask range, and the split tasks at four times its offsets
+  long long trsm_off, ntrsm, upd_off, nupd;  // X, then as many each of R and L
   int64_t max_m;
 };
 
@@ -1603,21 +1608,23 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
   const size_t o_tab = take(nrep * sizeof(MaternTable)), o_rst = take(nrep * sizeof(DevStatus));
   const size_t o_rex = take((size_t)nrep * NB * sizeof(int)), o_w = take(wo * sizeof(double));
   const size_t o_ld = take(lo * sizeof(double)), o_q = take(lo * sizeof(double)), o_z = take(vo * sizeof(double));
-  const size_t o_ws = take(digit_bytes((int64_t)nrep * NB, NB, kDigSlices));
+  const size_t o_ws = take(digit_bytes((int64_t)2 * nrep * NB, NB, kDigSlices));  // W and L_kk
+  const size_t o_wl = take(digit_bytes((int64_t)nrep * NB, NB, kDigLow));
+  const size_t o_x = take((size_t)ps_rows * NB * sizeof(double));
   constexpr int64_t kNodes = kTabSeg * (kTabDeg + 1);
   const size_t nodes_b = (size_t)nrep * kNodes * sizeof(double);  // scratch before the first panel
   const size_t ps_b = digit_bytes(ps_rows, NB, kDigSlices);
   const size_t o_ps = take(ps_b > nodes_b ? ps_b : nodes_b);
-  // task lists: diagonal tiles | splits (W, panel) | z | products
+  // task lists: diagonal tiles | splits (W, L_kk, panel, X) | z | products
   long long nd = 0, nset = 0, ntask = 0;
   for (int r = 0; r < nrep; ++r) {
     const long long T = meta[r].T;
     nd += T;
     nset += T - 1;
-    ntask += T * (T - 1) + (T - 1) * T * (T + 1) / 3;  // sum of 2 b (solves) and of b (b + 1) (updates), b < T
+    ntask += 3 * T * (T - 1) + (T - 1) * T * (T + 1) / 3;  // sum of 6 b (solves) and of b (b + 1) (updates), b < T
   }
   const size_t d_b = round_up(nd * (int64_t)sizeof(SolveTileTask), 256);
-  const size_t s_b = round_up(2 * nset * (int64_t)sizeof(DigitSplitTask), 256);
+  const size_t s_b = round_up(4 * nset * (int64_t)sizeof(DigitSplitTask), 256);
   const size_t z_b = round_up(nset * (int64_t)sizeof(ZTask), 256);
   const size_t t_b = round_up(ntask * (int64_t)sizeof(DigitTask), 256);
   struct {
@@ -1644,9 +1651,12 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
   double* qpart = (double*)(base + o_q);
   double* zbuf = (double*)(base + o_z);
   double* mat = (double*)c->bd_mat.p;
-  DigitOperand Ws, Ps;
-  digit_layout(Ws, base + o_ws, (int64_t)nrep * NB, NB, kDigSlices);
+  DigitOperand Ws, Wl, Ps, Pl;  // Pl in Ps's place
+  digit_layout(Ws, base + o_ws, (int64_t)2 * nrep * NB, NB, kDigSlices);
+  digit_layout(Wl, base + o_wl, (int64_t)nrep * NB, NB, kDigLow);
   digit_layout(Ps, base + o_ps, ps_rows, NB, kDigSlices);
+  digit_layout(Pl, base + o_ps, ps_rows, NB, kDigLow);
+  double* xbuf = (double*)(base + o_x);  // X_i of replicate q: mr x NB, column-major, from entry prow NB
   uint8_t* tb = (uint8_t*)c->bd_task.p;
   SolveTileTask* dDiag = (SolveTileTask*)tb;
   DigitSplitTask* dSpl = (DigitSplitTask*)(tb + d_b);
@@ -1699,22 +1709,30 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
         const BMeta& m = meta[r];
         const int64_t mr = m.npad - (int64_t)(k + 1) * NB;
         const double* panel = mat + m.mo + (int64_t)(k + 1) * NB + (int64_t)k * NB * m.npad;
-        // the W's at 2 set_off .., the panels after them
-        hp[2 * stp.set_off + q] = {wbuf + m.wo + (int64_t)k * NB * NB, NB, 1, NB, (int64_t)q * NB, dRex + r * NB, 1, 1};
-        hp[2 * stp.set_off + stp.nset + q] = {panel, 1, m.npad, mr, prow[q], dRex + r * NB, -1, 0};
-        hz[iset++] = {panel, m.npad, mr, zbuf + m.vo + (int64_t)k * NB};
+        double* x = xbuf + (int64_t)prow[q] * NB;
+        // the W's at 4 set_off .., then the L's, the panels and the X's
+        DigitSplitTask* sp = hp + 4 * stp.set_off + q;
+        sp[0] = {wbuf + m.wo + (int64_t)k * NB * NB, NB, 1, NB, (int64_t)q * NB, dRex + r * NB, 1, 1};
+        sp[stp.nset] = {panel - NB, 1, m.npad, NB, (int64_t)(stp.nset + q) * NB, nullptr, 0, 1};
+        sp[2 * stp.nset] = {panel, 1, m.npad, mr, prow[q], dRex + r * NB, -1, 0};
+        sp[3 * stp.nset] = {x, 1, mr, mr, prow[q], nullptr, 0, 0};
+        hz[iset++] = {x, mr, mr, zbuf + m.vo + (int64_t)k * NB};
         stp.max_m = mr > stp.max_m ? mr : stp.max_m;
       }
       stp.trsm_off = it;
-      for (int q = 0; q < stp.nset; ++q) {
-        const BMeta& m = meta[set[q]];
-        double* panel = mat + m.mo + (int64_t)(k + 1) * NB + (int64_t)k * NB * m.npad;
-        for (int64_t i = 0; i < m.T - k - 1; ++i)
-          for (int h = 0; h < NB / kDigTN; ++h)
-            ht[it++] = {panel + i * NB + (int64_t)h * kDigTN * m.npad, m.npad, prow[q] + (int)i * NB,
-                        q * NB + h * kDigTN, kDigStore, 0};
+      for (int part = 0; part < 3; ++part) {  // X, R, L
+        for (int q = 0; q < stp.nset; ++q) {
+          const BMeta& m = meta[set[q]];
+          const int64_t mr = m.npad - (int64_t)(k + 1) * NB, ld = part == 1 ? m.npad : mr;
+          double* to = part == 1 ? mat + m.mo + (int64_t)(k + 1) * NB + (int64_t)k * NB * m.npad
+                                 : xbuf + (int64_t)prow[q] * NB;
+          for (int64_t i = 0; i < m.T - k - 1; ++i)
+            for (int h = 0; h < NB / kDigTN; ++h)
+              ht[it++] = {to + i * NB + (int64_t)h * kDigTN * ld, ld, prow[q] + (int)i * NB,
+                          (part == 1 ? stp.nset + q : q) * NB + h * kDigTN, part == 0 ? kDigStore : kDigPlain, 0};
+        }
+        if (part == 0) stp.ntrsm = it - stp.trsm_off;
       }
-      stp.ntrsm = it - stp.trsm_off;
       stp.upd_off = it;
       for (int q = 0; q < stp.nset; ++q) {
         const BMeta& m = meta[set[q]];
@@ -1765,20 +1783,39 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
       e = launch_diag128_tasks(s, dDiag + stp.diag_off, stp.ndiag);
     }
     if (e != cudaSuccess || stp.nset == 0) continue;
-    const DigitSplitTask* spl = dSpl + 2 * stp.set_off;
+    const DigitSplitTask* spl = dSpl + 4 * stp.set_off;
+    const DigitSplitTask *spl_panel = spl + 2 * stp.nset, *spl_x = spl + 3 * stp.nset;
+    const DigitTask* solve = dTask + stp.trsm_off;
     const double panel_e = (double)stp.ntrsm * NB * kDigTN;  // panel entries
     {
-      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * (panel_e + (double)stp.nset * NB * NB), 2);
-      e = launch_digit_split_tasks(s, spl, stp.nset, NB, NB, Ws);
-      if (e == cudaSuccess) e = launch_digit_split_tasks(s, spl + stp.nset, stp.nset, stp.max_m, NB, Ps, true);
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * panel_e + 64.0 * (double)stp.nset * NB * NB, 3);
+      e = launch_digit_split_tasks(s, spl, 2 * stp.nset, NB, NB, kDigSlices, Ws);
+      if (e == cudaSuccess) e = launch_digit_split_tasks(s, spl, stp.nset, NB, NB, kDigLow, Wl);
+      if (e == cudaSuccess) e = launch_digit_split_tasks(s, spl_panel, stp.nset, stp.max_m, NB, kDigSlices, Ps);
     }
-    if (e == cudaSuccess) {
+    if (e == cudaSuccess) {  // X
       ProfScope ps(c, PK_GEMM_DIG, panel_e * NB, 8.0 * panel_e);
-      e = launch_gemm_digits_tasks(s, dTask + stp.trsm_off, stp.ntrsm, NB, Ps, Ws, false, c->d_status);
+      e = launch_gemm_digits_tasks(s, solve, stp.ntrsm, NB, kDigSlices, Ps, Ws, false, c->d_status);
     }
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * panel_e);
-      e = launch_digit_split_tasks(s, spl + stp.nset, stp.nset, stp.max_m, NB, Ps, false);
+      e = launch_digit_split_tasks(s, spl_x, stp.nset, stp.max_m, NB, kDigSlices, Ps);
+    }
+    if (e == cudaSuccess) {  // R
+      ProfScope ps(c, PK_GEMM_DIG, panel_e * NB, 16.0 * panel_e);
+      e = launch_gemm_digits_tasks(s, solve + stp.ntrsm, stp.ntrsm, NB, kDigSlices, Ps, Ws, true, c->d_status);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_SPLIT, 0.0, 16.0 * panel_e);
+      e = launch_digit_split_tasks(s, spl_panel, stp.nset, stp.max_m, NB, kDigLow, Pl);
+    }
+    if (e == cudaSuccess) {  // L
+      ProfScope ps(c, PK_GEMM_DIG, panel_e * NB, 16.0 * panel_e);
+      e = launch_gemm_digits_tasks(s, solve + 2 * stp.ntrsm, stp.ntrsm, NB, kDigLow, Pl, Wl, false, c->d_status);
+    }
+    if (e == cudaSuccess) {
+      ProfScope ps(c, PK_SPLIT, 0.0, 24.0 * panel_e);
+      e = launch_digit_split_tasks(s, spl_x, stp.nset, stp.max_m, NB, kDigSlices, Ps);
     }
     if (e == cudaSuccess) {
       ProfScope ps(c, PK_TRSV, 2.0 * panel_e, 8.0 * panel_e);
@@ -1788,7 +1825,7 @@ static exa_status batched_run_digits(exa_ctx* c, int nrep, const int64_t* h_n, c
     if (e == cudaSuccess) {
       const double upd = (double)stp.nupd * NB * kDigTN;
       ProfScope ps(c, PK_GEMM_DIG, 2.0 * upd * NB, 16.0 * upd);
-      e = launch_gemm_digits_tasks(s, dTask + stp.upd_off, stp.nupd, NB, Ps, Ps, true, c->d_status);
+      e = launch_gemm_digits_tasks(s, dTask + stp.upd_off, stp.nupd, NB, kDigSlices, Ps, Ps, true, c->d_status);
     }
   }
   if (e != cudaSuccess) return cuda_err(c, e, "batched factorisation");

@@ -489,12 +489,12 @@ __global__ void __launch_bounds__(kSplitThreads) digit_split_kernel(const double
 }
 
 // Many pieces in one launch: blockIdx.y = piece, blockIdx.x = 16-row chunk of it.
+template <int S>
 __global__ void __launch_bounds__(kSplitThreads) digit_split_tasks_kernel(const DigitSplitTask* __restrict__ tasks,
-                                                                          int K, int scaled, DigitOperand op) {
+                                                                          int K, DigitOperand op) {
   const DigitSplitTask t = tasks[blockIdx.y];
   if ((int64_t)blockIdx.x * kRows >= t.rows) return;  // uniform over the CTA, before any barrier
-  split_body<kDigSlices>(t.src, t.rs, t.cs, t.rows, K, t.lower, scaled ? t.colex : nullptr, t.colsign, op,
-                         t.out_row0);
+  split_body<S>(t.src, t.rs, t.cs, t.rows, K, t.lower, t.colex, t.colsign, op, t.out_row0);
 }
 
 }  // namespace dig
@@ -530,11 +530,17 @@ cudaError_t launch_digit_split(cudaStream_t s, const double* src, int64_t rs, in
 }
 
 cudaError_t launch_digit_split_tasks(cudaStream_t s, const DigitSplitTask* d_tasks, int ntasks, int64_t max_rows,
-                                     int K, const DigitOperand& op, bool scaled) {
+                                     int K, int S, const DigitOperand& op) {
   if (ntasks <= 0 || max_rows <= 0) return cudaSuccess;
-  if (K <= 0 || K % 16 || K > kDigMaxK) return cudaErrorInvalidValue;
-  dig::digit_split_tasks_kernel<<<dim3((unsigned)ceil_div(max_rows, dig::kRows), (unsigned)ntasks), dig::kSplitThreads, 0,
-                                  s>>>(d_tasks, K, scaled, op);
+  if (K <= 0 || K % 16 || K > kDigMaxK || (S != kDigSlices && S != kDigLow)) return cudaErrorInvalidValue;
+  constexpr int kMaxY = 65535;  // of a grid
+  for (int t = 0; t < ntasks; t += kMaxY) {
+    const dim3 grid((unsigned)ceil_div(max_rows, dig::kRows), (unsigned)(ntasks - t < kMaxY ? ntasks - t : kMaxY));
+    if (S == kDigSlices)
+      dig::digit_split_tasks_kernel<kDigSlices><<<grid, dig::kSplitThreads, 0, s>>>(d_tasks + t, K, op);
+    else
+      dig::digit_split_tasks_kernel<kDigLow><<<grid, dig::kSplitThreads, 0, s>>>(d_tasks + t, K, op);
+  }
   return cudaGetLastError();
 }
 
@@ -587,7 +593,7 @@ cudaError_t launch_gemm_digits(cudaStream_t s, const DigitGemm& g, int max_ctas)
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K,
+cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K, int S,
                                      const DigitOperand& A, const DigitOperand& B, bool neg, DevStatus* st) {
   if (ntasks <= 0) return cudaSuccess;
   if (K <= 0 || K % 16 || K > kDigMaxK) return cudaErrorInvalidValue;
@@ -605,7 +611,9 @@ cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, l
   a.ntiles = ntasks;
   a.sign = neg ? 0x80000000u : 0u;
   a.st = st;
-  return gemm_impl<kDigSlices>(s, a, 0);
+  if (S == kDigSlices) return gemm_impl<kDigSlices>(s, a, 0);
+  if (S == kDigLow) return gemm_impl<kDigLow>(s, a, 0);
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace exa

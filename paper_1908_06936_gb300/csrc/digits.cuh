@@ -67,9 +67,9 @@ struct DigitTask {
   int a_row, b_row;
   int diag, pad;
 };
-cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K,
+cudaError_t launch_gemm_digits_tasks(cudaStream_t s, const DigitTask* d_tasks, long long ntasks, int K, int S,
                                      const DigitOperand& A, const DigitOperand& B, bool neg, DevStatus* st);
-// One piece of a grouped split (the arguments of launch_digit_split); scaled = false: without the column exponents.
+// One piece of a grouped split (the arguments of launch_digit_split).
 struct DigitSplitTask {
   const double* src;
   int64_t rs, cs, rows, out_row0;
@@ -77,6 +77,6 @@ struct DigitSplitTask {
   int colsign, lower;
 };
 cudaError_t launch_digit_split_tasks(cudaStream_t s, const DigitSplitTask* d_tasks, int ntasks, int64_t max_rows,
-                                     int K, const DigitOperand& op, bool scaled = true);
+                                     int K, int S, const DigitOperand& op);
 
 }  // namespace exa

@@ -62,3 +62,29 @@ def test_kriging_variance_against_the_fp64_units(nu, beta, bound):
             a, b = (x.predict(locs, z, (1.0, beta, nu), new)[1].cpu().numpy() for x in (c, units))
         diff.append(np.max(np.abs(a - b)))
     assert max(diff) <= bound, diff
+
+
+@pytest.mark.parametrize("nu,beta,bound", [(2.5, 0.2, 4e-10), (3.5, 0.15, 2.5e-8)])
+def test_batched_log_likelihood_of_smooth_fields(nu, beta, bound):
+    # eight fields of 529 points, relative difference from the persistent form (root mean square).  In 80-bit arithmetic
+    # the persistent form's 64-wide tiles leave 1.3e-10 and 5.5e-9 (16 fields), 128-wide inverses as digit products
+    # 6.8e-10 and 8.2e-8, and once corrected 3.6e-11 and 1.4e-9.  Bound: the persistent form's error, and a factor of 3
+    # to 4.5 for the smaller sample.
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    locs = [to_dev(synth.jittered_grid(23, seed)) for seed in range(1, 9)]
+    z = [to_dev(synth.normals(529, seed)) for seed in range(1, 9)]
+    theta = to_dev(np.tile([1.0, beta, nu], 8))
+    got = []
+    with exa.Context() as c:
+        for ctas in (0, 1):
+            out = torch.empty(8, dtype=torch.float64, device="cuda")
+            st = torch.empty(8, dtype=torch.int32, device="cuda")
+            c.check(exa.exa_ctx_set_batched(c.handle, 64, ctas, 0, 0))
+            c.check(exa.exa_loglik_batched(c.handle, 8, [529] * 8, locs, z, theta, exa.EXA_FP64, out, st))
+            torch.cuda.synchronize()
+            assert np.all(st.cpu().numpy() == 0)
+            got.append(out.cpu().numpy())
+    rel = (got[0] - got[1]) / got[1]
+    assert np.sqrt(np.mean(rel ** 2)) <= bound, rel
