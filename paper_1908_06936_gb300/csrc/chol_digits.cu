@@ -67,6 +67,7 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
   c->wall_kept = true;
   double* X = (double*)c->mx_split2.p;
   cudaStream_t ms = c->stream, ss = c->side;
+  SideJoin streams(ms, ss, c->la_ev);
   const int sms = tc_num_sms();
   DigitOperand Dw, Dl, Dwl;
   if (T > 1) {
@@ -173,18 +174,17 @@ exa_status factor_digits(exa_ctx* c, double* a, int64_t ld, int64_t npad, bool* 
       e = launch_gemm_digits(ms, u);
     }
     if (e != cudaSuccess) break;
-    cudaEventRecord(c->la_ev[0], ms);
-    cudaStreamWaitEvent(ss, c->la_ev[0], 0);
+    streams.fork();
     const int side = side_share(m, kNB, sms);
     e = diagonal(ss, k + 1, side);
-    cudaEventRecord(c->la_ev[1], ss);
+    streams.side_done();
     if (e == cudaSuccess && m > w1) {
       ProfScope ps(c, PK_GEMM_DIG, (dm * dm - (double)w1 * w1) * kNB, 8.0 * (dm * dm - (double)w1 * w1));
       u.m = u.n = m;
       u.skip = w1;
       e = launch_gemm_digits(ms, u, sms - side);
     }
-    cudaStreamWaitEvent(ms, c->la_ev[1], 0);
+    streams.join();
   }
   if (e != cudaSuccess) return cuda_err(c, e, "Cholesky launch");
   return EXA_OK;

@@ -9,6 +9,7 @@
 #include "gemm_tc.cuh"
 #include "prof.cuh"
 #include "shares.cuh"
+#include "side_join.cuh"
 
 namespace exa {
 

@@ -381,6 +381,7 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
   }
   MixStep M{c, a, ld, npad, band, T, far_thr};
   cudaStream_t ms = c->stream, ss = c->side;
+  SideJoin streams(ms, ss, c->la_ev);
   const int sms = tc_num_sms();
   const int side_ctas = c->lookahead_sms > 0 ? c->lookahead_sms : kLookaheadSMs;
   const bool by_rows = c->lookahead_sms <= 0 && c->late_rows < 0 && c->late_sms <= 0;
@@ -396,15 +397,14 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
       for (int j = k + 2; j <= k + 3; ++j)
         for (int p = k; p <= k + 1; ++p)
           if ((st = column_update(M, ms, p, j, B(p), 0)) != EXA_OK) return st;
-      cudaEventRecord(c->la_ev[0], ms);
-      cudaStreamWaitEvent(ss, c->la_ev[0], 0);
+      streams.fork();
       const int side_k = by_rows ? lookahead_share(npad - (int64_t)(k + 4) * NB, 2, sms) : side_ctas;
       if ((st = panel_factor(M, ss, k + 2, B(k + 2), side_k)) != EXA_OK) return st;
       if ((st = column_update(M, ss, k + 2, k + 3, B(k + 2), side_k)) != EXA_OK) return st;
       if ((st = panel_factor(M, ss, k + 3, B(k + 3), side_k)) != EXA_OK) return st;
-      cudaEventRecord(c->la_ev[1], ss);
+      streams.side_done();
       if ((st = region_update(M, ms, k, k + 4, B(k), &B(k + 1), sms - side_k)) != EXA_OK) return st;
-      cudaStreamWaitEvent(ms, c->la_ev[1], 0);
+      streams.join();
     }
     // hand over to the one-panel loop: panel k applied to every column >= k+2 leaves
     // panel k+1 factored and the columns >= k+2 holding every panel before k+1
@@ -427,13 +427,12 @@ exa_status factor_mixed(exa_ctx* c, double* a, int64_t ld, int64_t npad, exa_pre
     }
     // block column k+1 first (everything the side stream needs), on the whole GPU
     if ((st = column_update(M, ms, k, k + 1, B(k), 0)) != EXA_OK) return st;
-    cudaEventRecord(c->la_ev[0], ms);
-    cudaStreamWaitEvent(ss, c->la_ev[0], 0);
+    streams.fork();
     if ((st = panel_factor(M, ss, k + 1, B(k + 1), side_k)) != EXA_OK) return st;
-    cudaEventRecord(c->la_ev[1], ss);
+    streams.side_done();
     // the rest of the trailing matrix on the remaining SMs
     if ((st = region_update(M, ms, k, k + 2, B(k), nullptr, sms - side_k)) != EXA_OK) return st;
-    cudaStreamWaitEvent(ms, c->la_ev[1], 0);
+    streams.join();
   }
   return EXA_OK;
 }
