@@ -138,7 +138,7 @@ __device__ __forceinline__ double i63_to_f64_scaled(long long V, int sh) {
 // FP32 integers as integers.  F2I converts 16 lanes a cycle on an SM, which for the 65,536 accumulators of a tile is a
 // ninth of its MMA time, so half of the groups go by additions instead:
 // |a| <= 2^22: the low bits of a + 1.5 2^23 (above, f32_to_int).
-__device__ __forceinline__ int small_int_bits(float a) { return __float_as_int(a + 12582912.0f); }  // + 0x4B400000
+__device__ __forceinline__ uint32_t small_int_bits(float a) { return __float_as_uint(a + 12582912.0f); }  // + 0x4B400000
 // One CTA per SM, persistent: warp 0 copies operand planes into a ring of 16-column stages, one thread of warp 1
 // issues the MMAs, warps 2-17 drain TMEM into C.  The S B planes of a stage lie one after another and group g
 // follows group g - 1 in TMEM, so A digit s against B digits 0 .. S-1-s is one run of columns (two MMAs where
@@ -302,8 +302,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_digits_kernel(const __grid_c
         tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int w01 = small_int_bits(__uint_as_float(x[0][j])) * 128 + small_int_bits(__uint_as_float(x[1][j])) -
-                          (int)(129u * 0x4B400000u);
+          const int w01 = (int)(small_int_bits(__uint_as_float(x[0][j])) * 128u +  // modulo 2^32
+                                small_int_bits(__uint_as_float(x[1][j])) - 129u * 0x4B400000u);
           V[h + j] = (long long)w01 * 16384 + (__float2int_rn(__uint_as_float(x[2][j])) * 128 +
                                                __float2int_rn(__uint_as_float(x[3][j])));
           if constexpr (S == 8) V[h + j] = V[h + j] << 20;
