@@ -4,6 +4,7 @@
 // Both are HBM-bound: the solve streams the lower triangle once.  All
 // reductions run in a fixed order, so FP64 results are bitwise reproducible.
 #include "exa_internal.cuh"
+#include "gemm_tc.cuh"
 
 namespace exa {
 
@@ -804,7 +805,7 @@ static cudaError_t block_fwd(cudaStream_t s, const double* lkk, int64_t ld, int6
   double* zr = z + H;
   if (rest >= 32768)  // more than one 128-row CTA per SM
     return launch_block(s, true, rest / 128, block_rows_kernel<H, 128>, l, ld, 0, y, zr, zr);
-  if (rest >= 4864)  // one 32-row CTA per SM
+  if (rest >= 32 * (int64_t)tc_num_sms())  // one 32-row CTA per SM
     return launch_block(s, true, rest / 32, block_rows_kernel<H, 32>, l, ld, 0, y, zr, zr);
   return launch_block(s, true, rest / 8, block_rows_kernel<H, 8>, l, ld, 0, y, zr, zr);
 }
