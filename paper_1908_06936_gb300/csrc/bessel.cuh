@@ -227,8 +227,8 @@ __device__ __forceinline__ int table_segment(double s) {
 
 // Table construction.  Segment sgi covers [lo, lo + w) of s with lo = 2^e (1 + sub / kTabSub),
 // w = 2^e / kTabSub.  Node id = sgi (kTabDeg + 1) + k is f at the k-th Chebyshev point.
-__device__ __forceinline__ void segment_geometry(int sgi, double& centre, double& half, int e0 = kTabE0) {
-  const int e = e0 + sgi / kTabSub, sub = sgi % kTabSub;
+__device__ __forceinline__ void segment_geometry(int sgi, double& centre, double& half) {
+  const int e = kTabE0 + sgi / kTabSub, sub = sgi % kTabSub;
   const double lo = ldexp(1.0 + (double)sub / kTabSub, e);
   const double w = ldexp(1.0 / kTabSub, e);
   centre = lo + 0.5 * w;

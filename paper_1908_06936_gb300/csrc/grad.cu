@@ -237,18 +237,50 @@ __device__ __forceinline__ void matern_derivs(const GradParams& G, double r, dou
   d2 = sig * (lnx - 0.69314718055994530942 - G.psi_nu) + P.sigma2 * exp(base - x) * dknu_dnu_scaled(P.nu, x);
 }
 
-// Per-theta interpolation table of the three derivatives in s = (r / beta)^2, laid out as the generator's (degree-8
-// polynomials on 1/64 octave pieces) over a longer range: 2^-24 <= s < 2^16, x = r / beta from 2^-12 to 256.  The
-// exact derivatives take a quadrature of ~100 exponentials an entry (3.1 ns an entry, 156 ms at n = 10,000); from
-// the table an entry is ~33 FP64 operations.  Below and above the range the exact routine applies.
-constexpr int kDerE0 = -24, kDerOct = 40, kDerSeg = kDerOct * kTabSub;
+// Per-theta interpolation table of the three derivatives in s = (r / beta)^2: degree-8 polynomials as the generator's, over
+// 2^-24 <= s < 2^14, x = r / beta from 2^-12 to 128.  The exact derivatives take a quadrature of ~100 exponentials an entry
+// (3.1 ns an entry, 156 ms at n = 10,000); from the table an entry is ~33 FP64 operations.  Below and above the range the
+// exact routine applies.
+// Pieces an octave: 64 for x < 32, 256 up to 64 and 512 up to 128, because a piece's exponential range grows with x.  The
+// interpolation's largest error, relative to the derivative itself (40-digit arithmetic, nu = 0.5 to 2.5): 1e-18 at x = 16,
+// 2e-17 at 23 and 3e-16 at 32; from 64 pieces it would be 9e-14 at 64 and 4e-11 at 128, and falls with the ninth power of
+// their number: below 2e-17 in the finer octaves.
+constexpr int kDerE0 = -24;
+struct DerivBand {
+  int octave, end, bits;  // octaves [octave, end) from 2^kDerE0, 2^bits pieces each
+  int first;              // number of its first piece
+};
+constexpr DerivBand kDerBand[3] = {{0, 34, 6, 0}, {34, 36, 8, 34 << 6}, {36, 38, 9, (34 << 6) + (2 << 8)}};
+constexpr int kDerOct = kDerBand[2].end, kDerSeg = kDerBand[2].first + ((kDerOct - kDerBand[2].octave) << kDerBand[2].bits);
 struct DerivTable {
   double seg[kDerSeg][2];                 // -centre / half-width, 1 / half-width
   double a[kDerSeg][3][kTabDeg + 1];
 };
 constexpr int kDerNodes = kDerSeg * (kTabDeg + 1);
-// Building it costs ~23,000 exact evaluations; below this many entries they are evaluated one by one.
-constexpr int64_t kDerMinEntries = 4 * (int64_t)kDerNodes;
+// Building the table costs ~33,000 exact evaluations; below this many entries (n < 429) they are evaluated one by one.
+constexpr int64_t kDerMinEntries = 92160;
+
+// Piece of s, octave o = its exponent less kDerE0 (0 <= o < kDerOct).
+__device__ __forceinline__ int deriv_segment(double s, unsigned int o) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(s);
+  constexpr DerivBand b0 = kDerBand[0], b1 = kDerBand[1], b2 = kDerBand[2];
+  const int b = o < b1.octave ? b0.bits : o < b2.octave ? b1.bits : b2.bits;
+  const int first = o < b1.octave ? b0.first - ((1023 + kDerE0 + b0.octave) << b0.bits)
+                    : o < b2.octave ? b1.first - ((1023 + kDerE0 + b1.octave) << b1.bits)
+                                    : b2.first - ((1023 + kDerE0 + b2.octave) << b2.bits);
+  return (int)(bits >> (52 - b)) + first;
+}
+
+__device__ __forceinline__ void deriv_geometry(int sgi, double& centre, double& half) {
+  constexpr DerivBand b0 = kDerBand[0], b1 = kDerBand[1], b2 = kDerBand[2];
+  const int first = sgi < b1.first ? b0.first : sgi < b2.first ? b1.first : b2.first;
+  const int octave = sgi < b1.first ? b0.octave : sgi < b2.first ? b1.octave : b2.octave;
+  const int b = sgi < b1.first ? b0.bits : sgi < b2.first ? b1.bits : b2.bits;
+  const int q = sgi - first, e = kDerE0 + octave + (q >> b);
+  const double w = ldexp(1.0, e - b), lo = ldexp((double)((1 << b) + (q & ((1 << b) - 1))), e - b);
+  centre = lo + 0.5 * w;
+  half = 0.5 * w;
+}
 
 __global__ void __launch_bounds__(64) deriv_nodes_kernel(const __grid_constant__ GradParams G,
                                                          double* __restrict__ nodes) {
@@ -256,7 +288,7 @@ __global__ void __launch_bounds__(64) deriv_nodes_kernel(const __grid_constant__
   if (id >= kDerNodes) return;
   const int sgi = id / (kTabDeg + 1), k = id % (kTabDeg + 1);
   double centre, half, d0, d1, d2;
-  segment_geometry(sgi, centre, half, kDerE0);
+  deriv_geometry(sgi, centre, half);
   const double tk = cos(3.14159265358979323846 * (k + 0.5) / (kTabDeg + 1));
   matern_derivs(G, sqrt(centre + half * tk) * G.m.beta, d0, d1, d2);
   nodes[id] = d0;
@@ -272,7 +304,7 @@ __global__ void __launch_bounds__(64) deriv_coef_kernel(const double* __restrict
   segment_polynomial(nodes + f * kDerNodes + sgi * (kTabDeg + 1), T->a[sgi][f]);
   if (f == 0) {
     double centre, half;
-    segment_geometry(sgi, centre, half, kDerE0);
+    deriv_geometry(sgi, centre, half);
     T->seg[sgi][0] = -centre / half;
     T->seg[sgi][1] = 1.0 / half;
   }
@@ -289,15 +321,15 @@ __device__ __forceinline__ void matern_derivs_tab(const GradParams& G, const Der
   const double s = r2 * G.m.ib2;
   const unsigned int se = (unsigned int)((unsigned long long)__double_as_longlong(s) >> 52);
   // negative, zero, subnormal, infinite and NaN values all fall outside
-  if (!T || se - (unsigned int)(1023 + kDerE0) >= (unsigned int)kDerOct) {
+  const unsigned int o = se - (unsigned int)(1023 + kDerE0);
+  if (!T || o >= (unsigned int)kDerOct) {
     double e[3];
     matern_derivs_exact(G, r2, e);
 #pragma unroll
     for (int k = K0; k < K1; ++k) d[k - K0] = e[k];
     return;
   }
-  const int sgi = (int)((unsigned long long)__double_as_longlong(s) >> (52 - kTabSubBits)) -
-                  ((1023 + kDerE0) << kTabSubBits);
+  const int sgi = deriv_segment(s, o);
   const double t = fma(s, __ldg(&T->seg[sgi][1]), __ldg(&T->seg[sgi][0]));
 #pragma unroll
   for (int k = K0; k < K1; ++k) {

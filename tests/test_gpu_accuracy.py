@@ -88,3 +88,28 @@ def test_batched_log_likelihood_of_smooth_fields(nu, beta, bound):
             got.append(out.cpu().numpy())
     rel = (got[0] - got[1]) / got[1]
     assert np.sqrt(np.mean(rel ** 2)) <= bound, rel
+
+
+@pytest.mark.parametrize("x", [20.0, 31.0, 40.0, 63.0, 64.5, 70.0, 90.0, 91.0, 120.0, 150.0])
+def test_range_derivative_of_far_points(x):
+    # A 21 x 22 grid with spacing x beta, nu = 1/2: Sigma = sigma^2 (I + E) with E of size exp(-x), so its inverse is
+    # (I - E) / sigma^2 to exp(-2 x), and dl/dbeta = 1/2 sum_ij (a_i a_j - S_ij) D_ij, D = sigma^2 (r / beta^2) exp(-r / beta),
+    # is carried by the pairs at distance x and a few more.  An entry is off by the rounding of r^2 / beta^2 (2 u
+    # relative, x u in the exponential), of the piece's coordinate (no more) and of the polynomial: 4 x u of the sum of the
+    # absolute values bounds it with room for the sum.
+    import paper_1908_06936_gb300 as exa
+
+    sigma2, beta = 1.3, 0.01
+    i, j = np.meshgrid(np.arange(21), np.arange(22), indexing="ij")
+    locs = np.stack([i.ravel(), j.ravel()], 1) * (x * beta)
+    z = synth.normals(len(locs), 7)
+    with exa.Context() as c:
+        g = c.loglik_grad(to_dev(locs), to_dev(z), (sigma2, beta, 0.5))[1]
+    r = np.sqrt(((locs[:, None].astype(np.longdouble) - locs[None]) ** 2).sum(-1))
+    e = np.exp(-r / np.longdouble(beta))
+    d = sigma2 * r / np.longdouble(beta) ** 2 * e
+    e[np.diag_indices(len(e))] = 0
+    ez = (e * z[None]).sum(1)
+    a = (z - ez + (e * ez[None]).sum(1)) / sigma2
+    terms = 0.5 * (a[:, None] * a[None] + e / sigma2) * d  # D is zero on the diagonal
+    assert abs(float(g[1] - terms.sum())) <= 4 * x * U * float(np.abs(terms).sum())
