@@ -107,8 +107,10 @@ typedef struct {
  *   workspace_bytes  upper bound on device memory the context may hold (0: no bound).
  *                    FP64 evaluations use up to ~20 KB a row of the matrix beside it for digit
  *                    operands and block inverses where the bound and the device allow it
- *                    (they make the products run on the tensor cores), and give it up for
- *                    a buffer that a call cannot do without.
+ *                    (they make the products run on the tensor cores).  This and all other
+ *                    memory that calls do without is given up, within a call and between
+ *                    calls, for a buffer that a call cannot do without (but for what a
+ *                    captured graph uses).
  *   tile_nb          FP64 tile size, a multiple of 64 and <= 128 (0: library default).
  * Returns EXA_ERR_ARG on a bad tile size, EXA_ERR_CUDA if no device is usable. */
 exa_status exa_ctx_create(exa_ctx** ctx, void* cuda_stream, size_t workspace_bytes, int tile_nb);
@@ -278,8 +280,10 @@ exa_status exa_ctx_set_gradient_inverse(exa_ctx* ctx, int fp64);
  * Stream-asynchronous: returns once the work is enqueued; device memory is
  * allocated on the first call for a shape set, so make that call before any
  * CUDA-graph capture, after which the sequence can be captured and replayed
- * with new d_theta.  Calls that overlap on the GPU share the context's
- * buffers and must not run concurrently.                                     */
+ * with new d_theta.  The host arrays are read before the call returns, and a
+ * call that waits behind others on its stream, or a captured one at each replay,
+ * works on the pointers it was given.  Calls that overlap on the GPU share the
+ * context's buffers and must not run concurrently.                           */
 exa_status exa_loglik_batched(exa_ctx* ctx, int32_t nrep, const int64_t* h_n, const double* const* d_locs,
                               const double* const* d_z, const double* d_theta, exa_prec prec, double* d_loglik,
                               int32_t* d_status);
