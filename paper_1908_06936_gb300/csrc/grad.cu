@@ -257,7 +257,8 @@ struct DerivTable {
   double a[kDerSeg][3][kTabDeg + 1];
 };
 constexpr int kDerNodes = kDerSeg * (kTabDeg + 1);
-// Building the table costs ~33,000 exact evaluations; below this many entries (n < 429) they are evaluated one by one.
+// Building the table costs ~33,000 exact evaluations; below this many entries (gradients below n = 429) they are evaluated
+// one by one.
 constexpr int64_t kDerMinEntries = 92160;
 
 // Piece of s, octave o = its exponent less kDerE0 (0 <= o < kDerOct).

@@ -121,3 +121,25 @@ def test_lists_built_under_capture_are_not_taken_for_built(prec, tile):
             check(g.replay, small, ref)
             check(lambda: big.call(c, prec), big, ref_big)
             check(lambda: big.call(c, prec), big, ref_big)
+
+
+def test_more_panels_than_a_grid_has_rows():
+    # 33,000 fields with a panel: the splits of W and of L, one piece each a field, exceed the 65,535 of a grid's y dimension
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    nrep, n = 33000, 129
+    locs = [to_dev(synth.jittered_grid(12, s)[:n]) for s in range(3)]
+    z = [to_dev(synth.normals(n, s)) for s in range(3)]
+    theta = to_dev(np.tile([1.0, 0.1, 0.5], nrep))
+    out = torch.zeros(nrep, dtype=torch.float64, device="cuda")
+    status = torch.zeros(nrep, dtype=torch.int32, device="cuda")
+    pick = [r % 3 for r in range(nrep)]
+    with exa.Context() as c:
+        ref = np.array([c.loglik(l, y, (1.0, 0.1, 0.5)) for l, y in zip(locs, z)])
+        c.check(exa.exa_loglik_batched(c.handle, nrep, [n] * nrep, [locs[k] for k in pick], [z[k] for k in pick], theta,
+                                       exa.EXA_FP64, out, status))
+        torch.cuda.synchronize()
+    assert np.all(status.cpu().numpy() == 0)
+    got = out.cpu().numpy()
+    assert np.all(np.abs(got - ref[pick]) <= 1e-10 * np.abs(ref[pick]))
