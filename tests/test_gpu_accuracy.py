@@ -113,3 +113,28 @@ def test_range_derivative_of_far_points(x):
     a = (z - ez + (e * ez[None]).sum(1)) / sigma2
     terms = 0.5 * (a[:, None] * a[None] + e / sigma2) * d  # D is zero on the diagonal
     assert abs(float(g[1] - terms.sum())) <= 4 * x * U * float(np.abs(terms).sum())
+
+
+@pytest.mark.parametrize("m,nu,beta", [(20, 3.5, 1.0), (32, 3.0, 1.0), (32, 3.5, 0.3), (32, 4.5, 0.2), (45, 3.0, 0.5), (45, 3.5, 0.3)])
+def test_smooth_fields_that_the_fp64_units_factor(m, nu, beta):
+    # close to the limit of FP64, a lost digit shows as a failed pivot: what the FP64 units (tile 64, persistent batch)
+    # factor, the digit products factor too
+    import torch
+    import paper_1908_06936_gb300 as exa
+
+    theta = (1.0, beta, nu)
+    for seed in (1, 2):
+        locs, z = to_dev(synth.jittered_grid(m, seed)), to_dev(synth.normals(m * m, seed))
+        with exa.Context(tile_nb=64) as units:
+            ok = exa.exa_loglik_ex(units.handle, locs, z, theta, m * m, exa.EXA_FP64, exa.ExaResult()) == exa.EXA_OK
+        with exa.Context() as c:
+            st = exa.exa_loglik_ex(c.handle, locs, z, theta, m * m, exa.EXA_FP64, exa.ExaResult())
+            assert st == exa.EXA_OK or not ok, seed
+            statuses = []
+            for ctas in (1, 0):
+                out = torch.empty(1, dtype=torch.float64, device="cuda")
+                s = torch.empty(1, dtype=torch.int32, device="cuda")
+                c.check(exa.exa_ctx_set_batched(c.handle, 64, ctas, 0, 0))
+                c.check(exa.exa_loglik_batched(c.handle, 1, [m * m], [locs], [z], to_dev(np.array(theta)), exa.EXA_FP64, out, s))
+                statuses.append(int(s.item()))
+            assert statuses[1] == exa.EXA_OK or statuses[0] != exa.EXA_OK, seed
